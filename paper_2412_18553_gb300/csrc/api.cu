@@ -154,13 +154,13 @@ static te_status host_check(const Handle* h, const te_cluster* c, te_precision p
   return TE_OK;
 }
 
-// Host checks (descriptor, sizes, pointers), then the device-side value
-// checks (finite entries, max eps_o < min eps_v) launched on s: no host
-// synchronisation, the result is reported by te_sync.
-static te_status validate(Handle* h, const te_cluster* c, te_precision p, cudaStream_t s, int64_t cluster = 0) {
-  te_status st = host_check(h, c, p);
-  if (st != TE_OK) return st;
-  const cudaError_t e = launch_check_inputs(c, cluster, h->d_err, h->num_sms, s);
+// The device-side value checks (finite entries, max eps_o < min eps_v)
+// launched on s: no host synchronisation, the result is reported by te_sync.
+// The tensor-core paths make them themselves, in the pass that finds their
+// scales; this launch is for the others and for calls without triples.
+static te_status check_values(Handle* h, const te_cluster* c, cudaStream_t s, int64_t cluster = 0,
+                              const te_df* df = nullptr) {
+  const cudaError_t e = launch_check_inputs(c, cluster, h->d_err, h->num_sms, s, df);
   ++h->n_launches;
   if (e != cudaSuccess) return fail(TE_ECUDA, "input check launch: %s", cudaGetErrorString(e));
   return TE_OK;
@@ -317,9 +317,8 @@ void tune_save(Handle* h) {
 te_status ensure_workspace_public(Handle* h, size_t bytes) { return ensure_workspace(h, bytes); }
 te_status ensure_triples_public(Handle* h, int nocc) { return ensure_triples(h, nocc); }
 
-// The descriptor and factors of t_energy_df; then the device value checks
-// (Bov and Bvv instead of ovvv).
-static te_status validate_df(Handle* h, const te_cluster* c, const te_df* df, te_precision p, cudaStream_t s) {
+// The descriptor and factors of t_energy_df.
+static te_status host_check_df(Handle* h, const te_cluster* c, const te_df* df, te_precision p) {
   te_status st = host_check(h, c, p, false);
   if (st != TE_OK) return st;
   if (!df) return fail(TE_EINVAL, "null density-fitting factor descriptor");
@@ -330,15 +329,15 @@ static te_status validate_df(Handle* h, const te_cluster* c, const te_df* df, te
     return fail(TE_EUNSUPPORTED, "ovvv from density-fitting factors needs a tensor-core mode (TE_OZAKI, "
                                  "TE_BF16X3, TE_TF32X3 or TE_TF32)");
   if (c->nvir > 2047) return fail(TE_EUNSUPPORTED, "ovvv from density-fitting factors needs nvir <= 2047");
-  const cudaError_t e = launch_check_inputs(c, 0, h->d_err, h->num_sms, s, df);
-  ++h->n_launches;
-  if (e != cudaSuccess) return fail(TE_ECUDA, "input check launch: %s", cudaGetErrorString(e));
   return TE_OK;
 }
 
 static te_status run_any(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin,
                          int64_t t_end, double* e_tri_out, double* e_total_out, cudaStream_t s) {
-  if (p == TE_FP64) return run_fp64(h, c, t_begin, t_end, e_tri_out, e_total_out, s);
+  if (p == TE_FP64) {
+    const te_status st = check_values(h, c, s);
+    return st != TE_OK ? st : run_fp64(h, c, t_begin, t_end, e_tri_out, e_total_out, s);
+  }
   return run_tc(h, c, p, t_begin, t_end, e_tri_out, e_total_out, s);
 }
 
@@ -405,13 +404,13 @@ te_status t_energy_triples(te_handle hh, const te_cluster* c, te_precision p, in
   cudaStream_t s = reinterpret_cast<cudaStream_t>(ss);
   if (!h) return fail(TE_EINVAL, "null handle");
   DeviceGuard g(h->device);
-  te_status st = validate(h, c, p, s);
+  te_status st = host_check(h, c, p);
   if (st != TE_OK) return st;
   const int64_t nt = num_unique_triples(c->nocc);
   if (t_begin < 0 || t_end > nt || t_begin > t_end)
     return fail(TE_EINVAL, "triple range [%lld,%lld) outside [0,%lld)", (long long)t_begin,
                 (long long)t_end, (long long)nt);
-  if (t_begin == t_end) return TE_OK;
+  if (t_begin == t_end) return check_values(h, c, s);
   if (!e_triples) return fail(TE_EINVAL, "null e_triples");
   return run_any(h, c, p, t_begin, t_end, e_triples, nullptr, s);
 }
@@ -422,10 +421,12 @@ te_status t_energy(te_handle hh, const te_cluster* c, te_precision p, double* e_
   if (!h) return fail(TE_EINVAL, "null handle");
   if (!e_out) return fail(TE_EINVAL, "null e_out");
   DeviceGuard g(h->device);
-  te_status st = validate(h, c, p, s);
+  te_status st = host_check(h, c, p);
   if (st != TE_OK) return st;
   const int64_t nt = num_unique_triples(c->nocc);
   if (nt == 0) {
+    st = check_values(h, c, s);
+    if (st != TE_OK) return st;
     if (cudaMemsetAsync(e_out, 0, sizeof(double), s) != cudaSuccess)
       return fail(TE_ECUDA, "memset failed");
     return TE_OK;
@@ -440,10 +441,12 @@ te_status t_energy_df(te_handle hh, const te_cluster* c, const te_df* df, te_pre
   if (!h) return fail(TE_EINVAL, "null handle");
   if (!e_out) return fail(TE_EINVAL, "null e_out");
   DeviceGuard g(h->device);
-  te_status st = validate_df(h, c, df, p, s);
+  te_status st = host_check_df(h, c, df, p);
   if (st != TE_OK) return st;
   const int64_t nt = num_unique_triples(c->nocc);
   if (nt == 0) {
+    st = check_values(h, c, s, 0, df);
+    if (st != TE_OK) return st;
     if (cudaMemsetAsync(e_out, 0, sizeof(double), s) != cudaSuccess) return fail(TE_ECUDA, "memset failed");
     return TE_OK;
   }
@@ -456,13 +459,13 @@ te_status t_energy_df_triples(te_handle hh, const te_cluster* c, const te_df* df
   cudaStream_t s = reinterpret_cast<cudaStream_t>(ss);
   if (!h) return fail(TE_EINVAL, "null handle");
   DeviceGuard g(h->device);
-  te_status st = validate_df(h, c, df, p, s);
+  te_status st = host_check_df(h, c, df, p);
   if (st != TE_OK) return st;
   const int64_t nt = num_unique_triples(c->nocc);
   if (t_begin < 0 || t_end > nt || t_begin > t_end)
     return fail(TE_EINVAL, "triple range [%lld,%lld) outside [0,%lld)", (long long)t_begin, (long long)t_end,
                 (long long)nt);
-  if (t_begin == t_end) return TE_OK;
+  if (t_begin == t_end) return check_values(h, c, s, 0, df);
   if (!e_triples) return fail(TE_EINVAL, "null e_triples");
   return run_tc(h, c, p, t_begin, t_end, e_triples, nullptr, s, df);
 }
@@ -538,7 +541,7 @@ te_status t_energy_batched(te_handle hh, const te_cluster* cs, int64_t n, te_pre
     return fail(TE_ECUDA, "begin capture: %s", cudaGetErrorString(cudaGetLastError()));
   h->capturing = true;
   const int64_t l0 = h->n_launches;
-  for (int64_t x = 0; x < n && st == TE_OK; ++x) st = validate(h, cs + x, p, h->cap_stream, x);
+  for (int64_t x = 0; x < n && st == TE_OK && p == TE_FP64; ++x) st = check_values(h, cs + x, h->cap_stream, x);
   if (st == TE_OK && p != TE_FP64) st = run_tc_batched(h, cs, n, p, e_out, h->cap_stream);
   for (int64_t x = 0; x < n && st == TE_OK && p == TE_FP64; ++x) {
     const int64_t nt = num_unique_triples(cs[x].nocc);
@@ -547,7 +550,7 @@ te_status t_energy_batched(te_handle hh, const te_cluster* cs, int64_t n, te_pre
         st = fail(TE_ECUDA, "memset failed");
       ++h->n_launches;
     } else {
-      st = run_any(h, cs + x, p, 0, nt, nullptr, e_out + x, h->cap_stream);
+      st = run_fp64(h, cs + x, 0, nt, nullptr, e_out + x, h->cap_stream);
     }
   }
   h->capturing = false;
@@ -584,17 +587,20 @@ static te_status vjp_range(Handle* h, const te_cluster* c, te_precision p, int64
   if (!gr) return fail(TE_EINVAL, "null gradient descriptor");
   if (!(gE == gE) || gE > 1e300 || gE < -1e300) return fail(TE_EINVAL, "non-finite gE");
   if (h->capturing) return fail(TE_EINVAL, "the adjoint cannot run inside the library's graph capture");
-  te_status st = validate(h, c, p, s, cluster);
+  te_status st = host_check(h, c, p);
   if (st != TE_OK) return st;
   const int64_t nt = num_unique_triples(c->nocc);
   if (t_begin < 0 || t_end > nt || t_begin > t_end)
     return fail(TE_EINVAL, "triple range [%lld,%lld) outside [0,%lld)", (long long)t_begin, (long long)t_end,
                 (long long)nt);
   // float64: DFMA contractions; the tensor-core modes: exact-slice contractions
-  if (p == TE_FP64) return run_vjp_fp64(h, c, t_begin, t_end, gE, e_out, gr, s);
+  if (p == TE_FP64) {
+    st = check_values(h, c, s, cluster);
+    return st != TE_OK ? st : run_vjp_fp64(h, c, t_begin, t_end, gE, e_out, gr, s);
+  }
   if (h->cc_major != 10 && h->cc_major != 11)
     return fail(TE_EUNSUPPORTED, "the tensor-core adjoint needs an sm_100-family GPU");
-  return run_vjp_tc(h, c, t_begin, t_end, gE, e_out, gr, s);
+  return run_vjp_tc(h, c, t_begin, t_end, gE, e_out, gr, s, cluster);
 }
 
 te_status t_energy_vjp(te_handle hh, const te_cluster* c, te_precision p, double gE, double* e_out,
@@ -667,10 +673,11 @@ te_status t_energy_frag(te_handle hh, const te_cluster* c, const double* cf, te_
     return fail(TE_EUNSUPPORTED, "the projected energy runs in TE_FP64 or TE_OZAKI (got %d)", (int)p);
   if (h->capturing) return fail(TE_EINVAL, "t_energy_frag cannot run inside a graph capture");
   DeviceGuard g(h->device);
-  te_status st = validate(h, c, p, s);
+  te_status st = host_check(h, c, p);
   if (st != TE_OK) return st;
   if (p == TE_OZAKI && h->cc_major != 10 && h->cc_major != 11)
     return fail(TE_EUNSUPPORTED, "exact-slice contractions need an sm_100-family GPU");
+  if (p == TE_FP64 && (st = check_values(h, c, s)) != TE_OK) return st;
   return run_frag(h, c, cf, p, e_out, e_triples, s);
 }
 

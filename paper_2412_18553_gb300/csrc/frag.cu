@@ -186,11 +186,10 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
     ca.t2 = W.t2C;
     ca.ooov = W.ooovC;
     cb.t2 = W.t2C2;
-    st = tc_prepare_slices(c, W.slices[0], &S0, h->num_sms, s);
-    if (st == TE_OK) st = tc_prepare_slices(&ca, W.slices[1], &SA, h->num_sms, s);
-    if (st == TE_OK) st = tc_prepare_slices(&cb, W.slices[2], &SB, h->num_sms, s);
+    st = tc_prepare_slices(c, W.slices[0], &S0, h->num_sms, s, 4, h->d_err, 0, &h->n_launches);
+    if (st == TE_OK) st = tc_prepare_slices(&ca, W.slices[1], &SA, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
+    if (st == TE_OK) st = tc_prepare_slices(&cb, W.slices[2], &SB, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
     if (st != TE_OK) return st;
-    h->n_launches += 18;
   }
   // exact slices: the tcgen05 view GEMM (view_tc.cu) over the six segment
   // views of each slice set, encoded once

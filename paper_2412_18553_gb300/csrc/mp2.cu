@@ -338,8 +338,13 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     if (q.t2) t2 = q.t2;
     if (q.gamma_oo) goo = q.gamma_oo;
     if (q.gamma_vv) gvv = q.gamma_vv;
-    // input values: finite, max eps_o < min eps_v (reported by te_sync)
-    e = launch_check_mp2(c.eps_o, o, c.eps_v, v, c.Bov, P * ov, x, h->d_err, h->num_sms, s);
+    // input values: finite, max eps_o < min eps_v (reported by te_sync); the
+    // same pass finds max |Bov|, the scale of its slices
+    __nv_bfloat16* bs = oz ? reinterpret_cast<__nv_bfloat16*>(take((size_t)P * ov * 8)) : nullptr;
+    unsigned int* mx = oz ? reinterpret_cast<unsigned int*>(take(64)) : nullptr;
+    if (oz) e = cudaMemsetAsync(mx, 0, 4, s);
+    if (e == cudaSuccess)
+      e = launch_check_mp2(c.eps_o, o, c.eps_v, v, c.Bov, P * ov, x, h->d_err, h->num_sms, s, mx);
     ++h->n_launches;
     // (ia|jb) = sum_P B[P,i,a] B[P,j,b]: rows (i,a), columns (j,b), K = P
     if (e == cudaSuccess) e = cudaMemsetAsync(ovov, 0, (size_t)ov * ov * 8, s);
@@ -348,8 +353,6 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
         e = gemm_strided(GemmView{c.Bov, c.Bov, ovov, o, v, ov, P, 1, v, 1, ov, 0, ov, 0, 1, v * ov, ov, 1, 1.0},
                          h->num_sms, scratch, cap, s, &h->n_launches);
     } else {
-      __nv_bfloat16* bs = reinterpret_cast<__nv_bfloat16*>(take((size_t)P * ov * 8));
-      unsigned long long* mx = reinterpret_cast<unsigned long long*>(take(64));
       int* ex = reinterpret_cast<int*>(mx + 3);
       if (e == cudaSuccess) e = slice_planes(c.Bov, P * ov, 4, mx, ex, bs, s, &h->n_launches);
       if (e == cudaSuccess)

@@ -84,7 +84,7 @@ __device__ __forceinline__ void orbit_values(const AdjArgs& A, int a, int b, int
 // 2^(e - 7 NS - 1).  Zeros and subnormals give N = 0; non-finite x gives
 // unspecified digits.
 template <int NS>
-__device__ __forceinline__ void slice_digits(double x, int e, float* d) {
+__device__ __forceinline__ void slice_digits_int(double x, int e, int* d) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int E = (int)((bits >> 52) & 0x7FFull);
   long long N = 0;
@@ -97,11 +97,17 @@ __device__ __forceinline__ void slice_digits(double x, int e, float* d) {
   }
 #pragma unroll
   for (int k = NS - 1; k > 0; --k) {
-    const int dk = (int)((N + 64) & 127) - 64;
-    d[k] = (float)dk;
-    N = (N - dk) >> 7;
+    d[k] = (int)((N + 64) & 127) - 64;
+    N = (N - d[k]) >> 7;
   }
-  d[0] = (float)N;
+  d[0] = (int)N;
+}
+template <int NS>
+__device__ __forceinline__ void slice_digits(double x, int e, float* d) {
+  int n[NS];
+  slice_digits_int<NS>(x, e, n);
+#pragma unroll
+  for (int k = 0; k < NS; ++k) d[k] = (float)n[k];
 }
 
 // C[m,n] += alpha sum_k A[m,k] B[k,n], m = (m1, m2) and k = (k1, k2) with a
@@ -140,10 +146,10 @@ cudaError_t gemm_strided(const GemmView& g, int num_sms, double* scratch, int64_
                          int64_t* launches);
 cudaError_t gemm_oz(const OzView& g, int num_sms, double* scratch, int64_t scratch_cap, cudaStream_t s,
                     int64_t* launches);
-// NS (4 or 5) 7-bit slice planes of x[0..n) with one power-of-two scale:
-// *ex = e with 2^e > max |x| (the max's bits go to *mx), slice s at planes +
-// s n.  Two launches.
-cudaError_t slice_planes(const double* x, int64_t n, int ns, unsigned long long* mx, int* ex,
+// NS (4 or 5) 7-bit slice planes of x[0..n) with one power-of-two scale: x =
+// 2^e sum_s m_s 2^-7(s+1) + r, |r| <= 2^(e - 7 NS - 1), 2^e > max |x|, whose
+// high word is *xhi (launch_absmax); e goes to *ex, slice s to planes + s n.
+cudaError_t slice_planes(const double* x, int64_t n, int ns, const unsigned int* xhi, int* ex,
                          __nv_bfloat16* planes, cudaStream_t s, int64_t* launches);
 // doubles of split-K scratch gemm_oz needs for an M x N output over K
 int64_t gemm_oz_scratch(int64_t M, int64_t N, int64_t K, int num_sms);

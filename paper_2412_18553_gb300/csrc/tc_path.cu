@@ -33,19 +33,12 @@
 #include <cstring>
 
 #include "energy_tc.h"
+#include "prep_tc.h"
 #include "ptx_sm100.cuh"
 #include "strided.h"
 #include "tc_path.h"
 
 namespace te {
-
-// TC_OZAKI: four 7-bit slices, ten slice products (K = 2 (v + o) <= 1024).
-// TC_OZAKI6: five 6-bit slices, fifteen slice products (K <= 4096); chosen
-// for the same user mode when the K axis is too long for 7-bit slices.
-// TC_SLICE4, TC_SLICE5: four or five 7-bit slices, the operand form of the
-// strided exact-slice GEMMs (no contraction kernel of their own), cut from the
-// integer N = round(x 2^(7 NS - s)) in balanced base-128 digits.
-enum TcMode { TC_TF32 = 0, TC_BF16X3 = 1, TC_TF32X3 = 2, TC_OZAKI = 3, TC_OZAKI6 = 4, TC_SLICE5 = 5, TC_SLICE4 = 6 };
 
 constexpr int OZ_K_MAX7 = 1024;  // K * 2^14 < 2^24: exact level-2/3 sums with 7-bit slices
 constexpr int OZ_K_MAX6 = 4096;  // K * 2^12 < 2^24 with 6-bit slices
@@ -62,262 +55,6 @@ static int tc_mode_of(te_precision p, int o, int v, int ozaki_bits) {
       return 2 * (v + o) <= OZ_K_MAX7 ? TC_OZAKI : TC_OZAKI6;
   }
 }
-
-__host__ __device__ constexpr bool is_ozaki(int mode) {
-  return mode == TC_OZAKI || mode == TC_OZAKI6 || mode == TC_SLICE5 || mode == TC_SLICE4;
-}
-
-template <int MODE>
-struct ModeTraits {
-  static constexpr bool tf32 = (MODE == TC_TF32 || MODE == TC_TF32X3);
-  static constexpr int nparts =
-      (MODE == TC_TF32) ? 1
-                        : ((MODE == TC_OZAKI || MODE == TC_SLICE4) ? 4 : ((MODE == TC_OZAKI6 || MODE == TC_SLICE5) ? 5 : 2));
-  static constexpr int nacc = is_ozaki(MODE) ? 3 : 1;   // accumulators per tile
-  static constexpr int beta = MODE == TC_OZAKI6 ? 6 : 7;  // bits per slice
-};
-
-constexpr int MAX_PARTS = 5;
-
-// ---------------------------------------------------------------------------
-// operand preparation
-// ---------------------------------------------------------------------------
-
-// Round x to the nearest value with `bits` significant bits (Veltkamp split).
-// __dmul_rn / __dsub_rn keep the compiler from contracting into an FMA.
-template <int BITS>
-__device__ __forceinline__ double round_sig(double x) {
-  const double c = __dmul_rn(x, (double)((1ull << (53 - BITS)) + 1ull));
-  return __dsub_rn(c, __dsub_rn(c, x));
-}
-
-struct Parts {
-  void* p[MAX_PARTS];
-};
-
-// Element `idx` of every part plane.  For OZAKI, `scale` is 2^-s of the array.
-template <int MODE>
-__device__ __forceinline__ void split_store(double x, const Parts& parts, int64_t idx, double scale) {
-  if (MODE == TC_BF16X3) {
-    const double h = round_sig<8>(x);
-    const double l = round_sig<8>(x - h);
-    reinterpret_cast<__nv_bfloat16*>(parts.p[0])[idx] = __float2bfloat16_rn((float)h);
-    reinterpret_cast<__nv_bfloat16*>(parts.p[1])[idx] = __float2bfloat16_rn((float)l);
-  } else if (MODE == TC_SLICE4 || MODE == TC_SLICE5) {
-    // integer digits of x 2^-s (slice_digits): no float64 arithmetic, against
-    // five float64 operations per slice for the repeated rounding below
-    constexpr int NS = ModeTraits<MODE>::nparts;
-    const int e = 1023 - (int)((((unsigned long long)__double_as_longlong(scale)) >> 52) & 0x7FFull);  // scale = 2^-e
-    float d[NS];
-    slice_digits<NS>(x, e, d);
-#pragma unroll
-    for (int k = 0; k < NS; ++k)
-      reinterpret_cast<__nv_bfloat16*>(parts.p[k])[idx] = __float2bfloat16_rn(ldexpf(d[k], -7 * (k + 1)));
-  } else if (is_ozaki(MODE)) {
-    constexpr int BETA = ModeTraits<MODE>::beta, NS = ModeTraits<MODE>::nparts;
-    double t = x * scale;  // |t| < 1, exact power-of-two scaling
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      t = t * (double)(1 << BETA);
-      const double m = rint(t);
-      t = t - m;
-      // m 2^-BETA(k+1) is exact in BF16 (|m| <= 2^BETA)
-      reinterpret_cast<__nv_bfloat16*>(parts.p[k])[idx] =
-          __float2bfloat16_rn((float)(m * (1.0 / (double)(1ull << (BETA * (k + 1))))));
-    }
-  } else {
-    const double h = round_sig<11>(x);
-    reinterpret_cast<float*>(parts.p[0])[idx] = (float)h;
-    if (MODE == TC_TF32X3) reinterpret_cast<float*>(parts.p[1])[idx] = (float)round_sig<11>(x - h);
-  }
-}
-
-__device__ __forceinline__ double scale_of(const int* exps, int which) {
-  return exps ? ldexp(1.0, -exps[which]) : 1.0;
-}
-
-// Slice-interleaved operand planes: rows come in groups of G (one occupied
-// index, or one occupied pair), and a group's slices are consecutive blocks,
-// [group][slice][G rows][Kp].  parts.p[s] points at slice s of group 0, so a
-// row's element for every slice sits at the same index from its part.
-__device__ __forceinline__ int64_t slice_index(int64_t row, int64_t k, int64_t G, int NS, int64_t Kp) {
-  return (row / G) * (NS * G * Kp) + (row % G) * Kp + k;
-}
-
-// dst[row][kp] = src[row][k] (k < K) or 0, rows x Kp, slice-interleaved by
-// groups of G rows; gexp (nullable): one scale exponent per group instead of
-// exps[which]
-template <int MODE>
-__global__ void k_split_rows(const double* __restrict__ src, Parts parts, int64_t rows, int K, int Kp, int64_t G,
-                             const int* exps, int which, const int* __restrict__ gexp = nullptr) {
-  const double sc = scale_of(exps, which);
-  const int64_t n = rows * Kp;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(idx % Kp);
-    const int64_t row = idx / Kp;
-    const double x = k < K ? src[row * K + k] : 0.0;
-    split_store<MODE>(x, parts, slice_index(row, k, G, ModeTraits<MODE>::nparts, Kp),
-                      gexp ? ldexp(1.0, -gexp[row / G]) : sc);
-  }
-}
-
-// t2L[q][x][y][l] = t2[l][q][x][y], l padded to op; gexp (nullable): one
-// exponent per q
-template <int MODE>
-__global__ void k_split_t2L(const double* __restrict__ t2, Parts parts, int o, int v, int op, const int* exps,
-                            int which, const int* __restrict__ gexp = nullptr) {
-  const double sc = scale_of(exps, which);
-  const int64_t n = (int64_t)o * v * v * op;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int l = (int)(idx % op);
-    int64_t rest = idx / op;
-    const int y = (int)(rest % v);
-    rest /= v;
-    const int x = (int)(rest % v);
-    const int q = (int)(rest / v);
-    const double val = l < o ? t2[(((int64_t)l * o + q) * v + x) * v + y] : 0.0;
-    split_store<MODE>(val, parts, slice_index(idx / op, l, (int64_t)v * v, ModeTraits<MODE>::nparts, op),
-                      gexp ? ldexp(1.0, -gexp[q]) : sc);
-  }
-}
-
-// nooT[p][r][z][l] = -ooov[p][l][r][z], l padded to op; gexp (nullable): one
-// exponent per (p, r), at p o + r
-template <int MODE>
-__global__ void k_split_noo(const double* __restrict__ ooov, Parts parts, int o, int v, int op, const int* exps,
-                            int which, const int* __restrict__ gexp = nullptr) {
-  const double sc = scale_of(exps, which);
-  const int64_t n = (int64_t)o * o * v * op;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int l = (int)(idx % op);
-    int64_t rest = idx / op;
-    const int z = (int)(rest % v);
-    rest /= v;
-    const int r = (int)(rest % o);
-    const int p = (int)(rest / o);
-    const double val = l < o ? -ooov[(((int64_t)p * o + l) * o + r) * v + z] : 0.0;
-    split_store<MODE>(val, parts, slice_index(idx / op, l, v, ModeTraits<MODE>::nparts, op),
-                      gexp ? ldexp(1.0, -gexp[p * o + r]) : sc);
-  }
-}
-
-// ovs32[i][a][j][b] = 1/2 (ovov[i,a,j,b] + ovov[j,b,i,a]), b padded to vq
-__global__ void k_ovs32(const double* __restrict__ ovov, float* __restrict__ ovs32, int o, int v, int vq) {
-  const int64_t n = (int64_t)o * v * o * vq;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(idx % vq);
-    int64_t rest = idx / vq;
-    const int j = (int)(rest % o);
-    rest /= o;
-    const int a = (int)(rest % v);
-    const int i = (int)(rest / v);
-    float val = 0.f;
-    if (b < v)
-      val = (float)(0.5 * (ovov[(((int64_t)i * v + a) * o + j) * v + b] +
-                           ovov[(((int64_t)j * v + b) * o + i) * v + a]));
-    ovs32[idx] = val;
-  }
-}
-
-// t1_32[i][a] = t1[i][a] as float32, a padded to vq
-__global__ void k_small_copies(const double* __restrict__ t1, float* __restrict__ t1_32, int o, int v, int vq) {
-  const int64_t n = (int64_t)o * vq;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int a = (int)(idx % vq);
-    const int i = (int)(idx / vq);
-    t1_32[idx] = a < v ? (float)t1[(int64_t)i * v + a] : 0.f;
-  }
-}
-
-// max |x| of three arrays (bit patterns of non-negative doubles order as integers)
-__global__ void k_maxabs(const double* __restrict__ a, int64_t na, const double* __restrict__ b, int64_t nb,
-                         const double* __restrict__ c, int64_t nc, unsigned long long* out) {
-  const double* src[3] = {a, b, c};
-  const int64_t n[3] = {na, nb, nc};
-  for (int w = 0; w < 3; ++w) {
-    double m = 0.0;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n[w];
-         idx += (int64_t)gridDim.x * blockDim.x)
-      m = fmax(m, fabs(src[w][idx]));
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(out + w, (unsigned long long)__double_as_longlong(m));
-  }
-}
-
-// Scale exponents: every segment of the K axis gets the unit 2^U.
-// exps = {s_ovvv, s_t2, s_t2L, s_nooT, U}
-__global__ void k_exponents(const unsigned long long* maxbits, int* exps) {
-  int e[3];
-  for (int w = 0; w < 3; ++w) {
-    const double m = __longlong_as_double((long long)maxbits[w]);
-    int ex = 0;
-    if (m > 0.0) frexp(m, &ex);  // m < 2^ex
-    e[w] = ex;
-  }
-  const int Eovvv = e[0], Et2 = e[1], Eooov = e[2];
-  const int U = max(Eovvv + Et2, Et2 + Eooov);
-  exps[0] = U - Et2;    // ovvv slices
-  exps[1] = Et2;        // t2 slices
-  exps[2] = U - Eooov;  // t2L slices
-  exps[3] = Eooov;      // nooT slices
-  exps[4] = U;
-}
-
-// max |x| per row group of the strided GEMMs' operands, one bit pattern per
-// group (atomicMax of non-negative doubles).  Elements are enumerated group
-// by group, in chunks of `chunk` per block iteration:
-//   mode 0 ovvv[p][x][y][d]   group p       (groups of v^3)
-//   mode 1 t2[r][q][z][d]     group r o + q (groups of v^2)
-//   mode 2 t2[l][q][x][y]     group q       (the t2L view; groups of o v^2)
-//   mode 3 ooov[p][l][r][z]   group p o + r (the nooT view; groups of o v)
-__global__ void __launch_bounds__(256) k_group_maxabs(const double* __restrict__ src, int mode, int o, int v,
-                                                      int64_t gsize, int64_t ngroups, int64_t chunk,
-                                                      unsigned long long* __restrict__ out) {
-  const int64_t cpg = (gsize + chunk - 1) / chunk;
-  const int64_t v2 = (int64_t)v * v;
-  __shared__ double red[8];
-  for (int64_t cid = blockIdx.x; cid < ngroups * cpg; cid += gridDim.x) {
-    const int64_t g = cid / cpg, i0 = (cid % cpg) * chunk, i1 = min(gsize, i0 + chunk);
-    double m = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-      int64_t a;
-      if (mode <= 1) {
-        a = g * gsize + i;
-      } else if (mode == 2) {  // i = l v^2 + xy
-        a = ((i / v2) * o + g) * v2 + i % v2;
-      } else {                 // g = p o + r, i = l v + z
-        const int64_t p = g / o, r = g % o;
-        a = (((p * o) + i / v) * o + r) * v + i % v;
-      }
-      m = fmax(m, fabs(src[a]));
-    }
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
-      if (m > 0.0) atomicMax(out + g, (unsigned long long)__double_as_longlong(m));
-    }
-    __syncthreads();
-  }
-}
-
-// exps[g] = e with 2^e > max of group g (0 for an all-zero group)
-__global__ void k_group_exps(const unsigned long long* __restrict__ bits, int64_t n, int* __restrict__ exps) {
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-    const double m = __longlong_as_double((long long)bits[g]);
-    int ex = 0;
-    if (m > 0.0) frexp(m, &ex);
-    exps[g] = ex;
-  }
-}
-
-static int gridn(int64_t n) { return (int)std::min<int64_t>(std::max<int64_t>(1, (n + 255) / 256), 16384); }
 
 // ---------------------------------------------------------------------------
 // the GEMM kernel
@@ -969,7 +706,7 @@ struct TcBuffers {
   void *a[MAX_PARTS], *b[MAX_PARTS], *l[MAX_PARTS], *n[MAX_PARTS];
   float *ovs32, *t1_32;
   double* etri;
-  unsigned long long* maxbits;
+  unsigned int* maxhi;  // high words of max |ovvv|, |t2|, |ooov|
   int* exps;
 };
 
@@ -1002,7 +739,7 @@ static size_t tc_carve_cluster(char* base, const TcPlan& pl, int64_t o, int64_t 
   b->ovs32 = static_cast<float*>(take((size_t)o * v * o * pl.vq * 4));
   b->t1_32 = static_cast<float*>(take((size_t)o * pl.vq * 4));
   b->etri = static_cast<double*>(take((size_t)std::max<int64_t>(1, ntri) * 8));
-  b->maxbits = static_cast<unsigned long long*>(take(4 * 8));
+  b->maxhi = static_cast<unsigned int*>(take(4 * 4));
   b->exps = static_cast<int*>(take(8 * 4));
   return (off + 1023) & ~size_t(1023);
 }
@@ -1130,7 +867,7 @@ constexpr int64_t DF_KBLOCK = 1024;                       // exact level-0/1 sum
 // contraction only writes after every operand is ready (stream order).
 struct DfScratch {
   __nv_bfloat16 *bov = nullptr, *bvv = nullptr;  // DF_NS planes each
-  unsigned long long* mx = nullptr;              // max |Bov|, max |Bvv| (bits)
+  unsigned int* mx = nullptr;                    // max |Bov|, max |Bvv| (high words)
   int* ex = nullptr;                             // their scale exponents
   double* stage = nullptr;                       // nst slabs of v^3
   double* part = nullptr;                        // split-K partial tiles
@@ -1150,7 +887,7 @@ static size_t df_carve(char* base, int o, int v, int64_t naux, int num_sms, DfSc
   d->nst = (int)std::max<size_t>(1, std::min<size_t>((size_t)o, DF_STAGE_BYTES / (v3 * 8)));
   d->bov = reinterpret_cast<__nv_bfloat16*>(take((size_t)DF_NS * naux * o * v * 2));
   d->bvv = reinterpret_cast<__nv_bfloat16*>(take((size_t)DF_NS * naux * v * v * 2));
-  d->mx = reinterpret_cast<unsigned long long*>(take(16));
+  d->mx = reinterpret_cast<unsigned int*>(take(16));
   d->ex = reinterpret_cast<int*>(take(8));
   d->stage = reinterpret_cast<double*>(take((size_t)d->nst * v3 * 8));
   // the largest split-K scratch over the slab counts and K blocks that occur
@@ -1184,64 +921,78 @@ static cudaError_t df_form(const te_df* df, int o, int v, int p0, int ne, const 
   return cudaSuccess;
 }
 
-// Operand planes of one cluster.  With df, ovvv comes from the factors (the
-// slabs are formed once for the maximum in the exact-slice modes, once for
-// the slices: the same bits both times); else from c->ovvv.
-template <int MODE>
-static cudaError_t launch_prep_tc(const te_cluster* c, const TcPlan& pl, const TcBuffers& b, const te_df* df,
-                                  const DfScratch* dfs, int num_sms, cudaStream_t s, int64_t* launches) {
+// Operand planes of one cluster: one pass over the inputs for the value
+// checks (err set) and the largest magnitudes, then one launch that cuts every
+// operand.  With df, ovvv comes from the factors (the slabs are formed once
+// for the maximum in the exact-slice modes, once for the slices: the same bits
+// both times); else from c->ovvv.
+static cudaError_t launch_prep_tc(int mode, const te_cluster* c, const TcPlan& pl, const TcBuffers& b,
+                                  const te_df* df, const DfScratch* dfs, unsigned int* err, int64_t cluster,
+                                  int num_sms, cudaStream_t s, int64_t* launches) {
   const int o = (int)c->nocc, v = (int)c->nvir;
-  const int64_t v3 = (int64_t)v * v * v;
-  const int* ex = nullptr;
+  const int64_t v2 = (int64_t)v * v, v3 = v2 * v;
+  const bool oz = is_ozaki(mode);
   cudaError_t e = cudaSuccess;
+  if (oz || df || err) {
+    MaxOut mo{};
+    if (oz) {
+      mo.ovvv = df ? nullptr : b.maxhi;
+      mo.t2 = b.maxhi + 1;
+      mo.ooov = b.maxhi + 2;
+      if ((e = cudaMemsetAsync(b.maxhi, 0, 4 * 4, s)) != cudaSuccess) return e;
+    }
+    if (df) {
+      mo.bov = dfs->mx;
+      mo.bvv = dfs->mx + 1;
+      if ((e = cudaMemsetAsync(dfs->mx, 0, 2 * 4, s)) != cudaSuccess) return e;
+    }
+    e = launch_check_inputs(c, cluster, err, num_sms, s, df, &mo);
+    ++*launches;
+    if (e != cudaSuccess) return e;
+  }
   if (df) {
     e = slice_planes(df->Bov, df->naux * o * v, DF_NS, dfs->mx, dfs->ex, dfs->bov, s, launches);
-    if (e == cudaSuccess) e = slice_planes(df->Bvv, df->naux * v * v, DF_NS, dfs->mx + 1, dfs->ex + 1, dfs->bvv, s, launches);
-    if (e != cudaSuccess) return e;
-  }
-  if (is_ozaki(MODE)) {
-    cudaMemsetAsync(b.maxbits, 0, 4 * 8, s);
-    k_maxabs<<<1024, 256, 0, s>>>(df ? nullptr : c->ovvv, df ? 0 : (int64_t)o * v3, c->t2, (int64_t)o * o * v * v,
-                                  c->ooov, (int64_t)o * o * o * v, b.maxbits);
-    ++*launches;
-    for (int p0 = 0; df && p0 < o; p0 += dfs->nst) {
+    if (e == cudaSuccess) e = slice_planes(df->Bvv, df->naux * v2, DF_NS, dfs->mx + 1, dfs->ex + 1, dfs->bvv, s, launches);
+    for (int p0 = 0; oz && p0 < o && e == cudaSuccess; p0 += dfs->nst) {
       const int ne = std::min(dfs->nst, o - p0);
       e = df_form(df, o, v, p0, ne, *dfs, num_sms, s, launches);
-      if (e != cudaSuccess) return e;
-      k_maxabs<<<1024, 256, 0, s>>>(dfs->stage, (int64_t)ne * v3, nullptr, 0, nullptr, 0, b.maxbits);
+      const MaxArray a{dfs->stage, 1, (int64_t)ne * v3, 0, b.maxhi, nullptr, 0, 0u};
+      if (e == cudaSuccess) e = launch_absmax(&a, 1, nullptr, 0, nullptr, 0, 0, nullptr, num_sms, s);
       ++*launches;
     }
-    k_exponents<<<1, 1, 0, s>>>(b.maxbits, b.exps);
-    ++*launches;
-    ex = b.exps;
+    if (e != cudaSuccess) return e;
   }
-  const Parts A{{b.a[0], b.a[1], b.a[2], b.a[3], b.a[4]}}, B{{b.b[0], b.b[1], b.b[2], b.b[3], b.b[4]}};
-  const Parts Lp{{b.l[0], b.l[1], b.l[2], b.l[3], b.l[4]}}, N{{b.n[0], b.n[1], b.n[2], b.n[3], b.n[4]}};
-  if (!df) {
-    k_split_rows<MODE><<<gridn((int64_t)o * v * v * pl.vp), 256, 0, s>>>(c->ovvv, A, (int64_t)o * v * v, v, pl.vp,
-                                                                         (int64_t)v * v, ex, 0);
-    ++*launches;
+  SplitScales sc{};
+  if (oz) {
+    sc.maxhi = b.maxhi;
+    sc.exps = b.exps;
   }
+  auto parts = [](void* const* p) { return Parts{{p[0], p[1], p[2], p[3], p[4]}}; };
+  const int64_t ov = (int64_t)o * v;
+  SplitJob jobs[SPLIT_MAX_JOBS] = {};
+  int n = 0;
+  if (!df) jobs[n++] = SplitJob{SPLIT_ROWS, c->ovvv, parts(b.a), nullptr, v, pl.vp, o * v2, 1, 0, 0, v2, 1, 0, nullptr, 0};
+  jobs[n++] = SplitJob{SPLIT_ROWS, c->t2, parts(b.b), nullptr, v, pl.vp, (int64_t)o * o * v, 1, 0, 0, v, 1, 1, nullptr, 0};
+  // t2L[q][x][y][l] = t2[l,q,x,y]; nooT[p][r][z][l] = -ooov[p,l,r,z]
+  jobs[n++] = SplitJob{SPLIT_COLS, c->t2, parts(b.l), nullptr, o, pl.op, v2, o, v2, o * v2, v2, 1, 2, nullptr, 0};
+  jobs[n++] = SplitJob{SPLIT_COLS, c->ooov, parts(b.n), nullptr, o, pl.op, ov, o, o * ov, ov, v, -1, 3, nullptr, 0};
+  jobs[n++] = SplitJob{SPLIT_OVS, c->ovov, Parts{}, b.ovs32, v, pl.vq, o, 1, 0, 0, 1, 1, 0, nullptr, 0};
+  jobs[n++] = SplitJob{SPLIT_COPY, c->t1, Parts{}, b.t1_32, v, pl.vq, o, 1, 0, 0, 1, 1, 0, nullptr, 0};
+  e = launch_split(mode, jobs, n, sc, s);
+  ++*launches;
   // one occupied index's slices of ovvv: nparts consecutive [v^2][vp] blocks
-  const size_t group = (size_t)pl.nparts * v * v * pl.vp * pl.es;
-  for (int p0 = 0; df && p0 < o; p0 += dfs->nst) {
+  const size_t group = (size_t)pl.nparts * v2 * pl.vp * pl.es;
+  for (int p0 = 0; df && p0 < o && e == cudaSuccess; p0 += dfs->nst) {
     const int ne = std::min(dfs->nst, o - p0);
     e = df_form(df, o, v, p0, ne, *dfs, num_sms, s, launches);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) break;
     Parts Ap{};
-    for (int k = 0; k < MAX_PARTS; ++k) Ap.p[k] = A.p[k] ? static_cast<char*>(A.p[k]) + (size_t)p0 * group : nullptr;
-    k_split_rows<MODE><<<gridn((int64_t)ne * v * v * pl.vp), 256, 0, s>>>(dfs->stage, Ap, (int64_t)ne * v * v, v,
-                                                                          pl.vp, (int64_t)v * v, ex, 0);
+    for (int k = 0; k < MAX_PARTS; ++k) Ap.p[k] = b.a[k] ? static_cast<char*>(b.a[k]) + (size_t)p0 * group : nullptr;
+    const SplitJob slab{SPLIT_ROWS, dfs->stage, Ap, nullptr, v, pl.vp, ne * v2, 1, 0, 0, v2, 1, 0, nullptr, 0};
+    e = launch_split(mode, &slab, 1, sc, s);
     ++*launches;
   }
-  k_split_rows<MODE><<<gridn((int64_t)o * o * v * pl.vp), 256, 0, s>>>(c->t2, B, (int64_t)o * o * v, v, pl.vp,
-                                                                       (int64_t)v, ex, 1);
-  k_split_t2L<MODE><<<gridn((int64_t)o * v * v * pl.op), 256, 0, s>>>(c->t2, Lp, o, v, pl.op, ex, 2);
-  k_split_noo<MODE><<<gridn((int64_t)o * o * v * pl.op), 256, 0, s>>>(c->ooov, N, o, v, pl.op, ex, 3);
-  k_ovs32<<<gridn((int64_t)o * v * o * pl.vq), 256, 0, s>>>(c->ovov, b.ovs32, o, v, pl.vq);
-  k_small_copies<<<gridn((int64_t)o * pl.vq), 256, 0, s>>>(c->t1, b.t1_32, o, v, pl.vq);
-  *launches += 5;
-  return cudaGetLastError();
+  return e;
 }
 
 template <int MODE>
@@ -1260,16 +1011,6 @@ static cudaError_t launch_gemm_any(int mode, const TcMapSet& M, const TcParams& 
   if (mode == TC_TF32) return launch_gemm_tc<TC_TF32>(M, P, smem, grid_cap, s);
   if (mode == TC_OZAKI) return launch_gemm_tc<TC_OZAKI>(M, P, smem, grid_cap, s);
   return launch_gemm_tc<TC_OZAKI6>(M, P, smem, grid_cap, s);
-}
-
-static cudaError_t launch_prep_any(int mode, const te_cluster* c, const TcPlan& pl, const TcBuffers& b,
-                                   const te_df* df, const DfScratch* dfs, int num_sms, cudaStream_t s,
-                                   int64_t* launches) {
-  if (mode == TC_BF16X3) return launch_prep_tc<TC_BF16X3>(c, pl, b, df, dfs, num_sms, s, launches);
-  if (mode == TC_TF32X3) return launch_prep_tc<TC_TF32X3>(c, pl, b, df, dfs, num_sms, s, launches);
-  if (mode == TC_TF32) return launch_prep_tc<TC_TF32>(c, pl, b, df, dfs, num_sms, s, launches);
-  if (mode == TC_OZAKI) return launch_prep_tc<TC_OZAKI>(c, pl, b, df, dfs, num_sms, s, launches);
-  return launch_prep_tc<TC_OZAKI6>(c, pl, b, df, dfs, num_sms, s, launches);
 }
 
 // One cluster of a run: its plan, buffers, tensor maps and triple range.
@@ -1471,8 +1212,8 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
 
 // Plan, buffers (carved from base), operand preparation and maps of one job.
 static te_status setup_job(Handle* h, TcState* st, const te_cluster* c, int mode, int64_t t_begin, int64_t t_end,
-                           const TcPlan& pl, char* base, TcJob* J, cudaStream_t s, const te_df* df = nullptr,
-                           const DfScratch* dfs = nullptr) {
+                           const TcPlan& pl, char* base, TcJob* J, int64_t cluster, cudaStream_t s,
+                           const te_df* df = nullptr, const DfScratch* dfs = nullptr) {
   J->c = c;
   J->pl = pl;
   J->o = (int)c->nocc;
@@ -1484,7 +1225,7 @@ static te_status setup_job(Handle* h, TcState* st, const te_cluster* c, int mode
   J->tiles_per_triple = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
   tc_carve_cluster(base, pl, J->o, J->v, num_unique_triples(J->o), &J->b);
   J->shares = J->b.etri;
-  const cudaError_t e = launch_prep_any(mode, c, pl, J->b, df, dfs, h->num_sms, s, &h->n_launches);
+  const cudaError_t e = launch_prep_tc(mode, c, pl, J->b, df, dfs, h->d_err, cluster, h->num_sms, s, &h->n_launches);
   if (e != cudaSuccess) return fail(TE_ECUDA, "operand split launch: %s", cudaGetErrorString(e));
   te_status rs = build_maps(st, pl, J->o, J->v, J->b, &J->maps);
   if (rs != TE_OK) return rs;
@@ -1516,22 +1257,8 @@ size_t tc_slices_bytes(int o, int v, int ns) {
   return al(NS * na * es) + al(NS * nb * es) + al(NS * nl * es) + al(NS * nn * es) + al(ng * 8) + al(ng * 4) + 1024;
 }
 
-template <int MODE>
-static void launch_slice_set(const te_cluster* c, int vp, int op, const Parts& pa, const Parts& pb, const Parts& pL,
-                             const Parts& pN, const int* e_ovvv, const int* e_t2, const int* e_t2L,
-                             const int* e_nooT, cudaStream_t s) {
-  const int o = (int)c->nocc, v = (int)c->nvir;
-  const int64_t v2 = (int64_t)v * v;
-  k_split_rows<MODE><<<gridn((int64_t)o * v * v * vp), 256, 0, s>>>(c->ovvv, pa, (int64_t)o * v * v, v, vp, v2,
-                                                                    nullptr, 0, e_ovvv);
-  k_split_rows<MODE><<<gridn((int64_t)o * o * v * vp), 256, 0, s>>>(c->t2, pb, (int64_t)o * o * v, v, vp,
-                                                                    (int64_t)v, nullptr, 1, e_t2);
-  k_split_t2L<MODE><<<gridn((int64_t)o * v * v * op), 256, 0, s>>>(c->t2, pL, o, v, op, nullptr, 2, e_t2L);
-  k_split_noo<MODE><<<gridn((int64_t)o * o * v * op), 256, 0, s>>>(c->ooov, pN, o, v, op, nullptr, 3, e_nooT);
-}
-
 te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, int num_sms, cudaStream_t s,
-                            int ns) {
+                            int ns, unsigned int* err, int64_t cluster, int64_t* launches) {
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int vp = round_up(v, 16), op = round_up(o, 16);
   if (ns != 4 && ns != 5) return fail(TE_EINVAL, "slice count %d (4 or 5)", ns);
@@ -1552,7 +1279,7 @@ te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, in
   char* L = take(NS * nl * es);
   char* N = take(NS * nn * es);
   const int64_t oo = (int64_t)o * o, ng = 2 * (int64_t)o + 2 * oo;
-  auto* maxbits = reinterpret_cast<unsigned long long*>(take((size_t)ng * 8));
+  auto* hi = reinterpret_cast<unsigned int*>(take((size_t)ng * 8));  // largest magnitudes, laid out as exps
   int* exps = reinterpret_cast<int*>(take((size_t)ng * 4));
   int* e_ovvv = exps;           // [o]
   int* e_t2 = e_ovvv + o;       // [o o]
@@ -1567,17 +1294,24 @@ te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, in
   }
   // one scale per row group (each strided GEMM reads one group of each
   // operand), so a block far below the array's largest keeps its 28 bits
-  cudaMemsetAsync(maxbits, 0, (size_t)ng * 8, s);
-  const int64_t v2 = (int64_t)v * v, chunk = 65536;
-  const int gm = 4 * std::max(1, num_sms);
-  k_group_maxabs<<<gm, 256, 0, s>>>(c->ovvv, 0, o, v, v2 * v, o, chunk, maxbits);
-  k_group_maxabs<<<gm, 256, 0, s>>>(c->t2, 1, o, v, v2, oo, chunk, maxbits + o);
-  k_group_maxabs<<<gm, 256, 0, s>>>(c->t2, 2, o, v, (int64_t)o * v2, o, chunk, maxbits + o + oo);
-  k_group_maxabs<<<gm, 256, 0, s>>>(c->ooov, 3, o, v, (int64_t)o * v, oo, chunk, maxbits + 2 * o + oo);
-  k_group_exps<<<(unsigned)((ng + 255) / 256), 256, 0, s>>>(maxbits, ng, exps);
-  if (NS == 5) launch_slice_set<TC_SLICE5>(c, vp, op, pa, pb, pL, pN, e_ovvv, e_t2, e_t2L, e_nooT, s);
-  else launch_slice_set<TC_SLICE4>(c, vp, op, pa, pb, pL, pN, e_ovvv, e_t2, e_t2L, e_nooT, s);
-  if (cudaGetLastError() != cudaSuccess) return fail(TE_ECUDA, "slice preparation launch failed");
+  const int64_t v2 = (int64_t)v * v, ov = (int64_t)o * v;
+  MaxOut mo{};
+  mo.groups = true;
+  mo.ovvv = hi;
+  mo.t2 = hi + o;
+  mo.t2L = hi + o + oo;
+  mo.ooov = hi + 2 * o + oo;
+  cudaError_t e = cudaMemsetAsync(hi, 0, (size_t)ng * 4, s);
+  if (e == cudaSuccess) e = launch_check_inputs(c, cluster, err, num_sms, s, nullptr, &mo);
+  const SplitScales sc{nullptr, nullptr, hi, exps, (int)ng};
+  const SplitJob jobs[4] = {
+      {SPLIT_ROWS, c->ovvv, pa, nullptr, v, vp, o * v2, 1, 0, 0, v2, 1, 0, e_ovvv, 0},
+      {SPLIT_ROWS, c->t2, pb, nullptr, v, vp, (int64_t)o * o * v, 1, 0, 0, v, 1, 0, e_t2, 0},
+      {SPLIT_COLS, c->t2, pL, nullptr, o, op, v2, o, v2, o * v2, v2, 1, 0, e_t2L, 0},
+      {SPLIT_COLS, c->ooov, pN, nullptr, o, op, ov, o, o * ov, ov, v, -1, 0, e_nooT, 0}};
+  if (e == cudaSuccess) e = launch_split(NS == 5 ? TC_SLICE5 : TC_SLICE4, jobs, 4, sc, s);
+  *launches += 2;
+  if (e != cudaSuccess) return fail(TE_ECUDA, "slice preparation launch failed: %s", cudaGetErrorString(e));
   out->ovvv = A;
   out->t2 = B;
   out->t2L = L;
@@ -1689,7 +1423,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
     const size_t cbytes = tc_carve_cluster(wbase, pl, o, v, nt, &J.b);
     cudaError_t e = cudaSuccess;
     if (!prepped) {  // the operand planes sit first in the workspace for every candidate
-      e = launch_prep_any(mode, c, pl, J.b, nullptr, nullptr, h->num_sms, s, &h->n_launches);
+      e = launch_prep_tc(mode, c, pl, J.b, nullptr, nullptr, nullptr, 0, h->num_sms, s, &h->n_launches);
       prepped = true;
     }
     if (e != cudaSuccess || build_maps(st, pl, o, v, J.b, &J.maps) != TE_OK) continue;
@@ -1768,7 +1502,7 @@ te_status run_tc(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023));
   std::vector<TcJob> jobs(1);
   if (df) df_carve(base + cbytes, o, v, df->naux, h->num_sms, &dfs);  // over the G pool, before its first use
-  rs = setup_job(h, st, c, mode, t_begin, t_end, pl, base, &jobs[0], s, df, df ? &dfs : nullptr);
+  rs = setup_job(h, st, c, mode, t_begin, t_end, pl, base, &jobs[0], 0, s, df, df ? &dfs : nullptr);
   if (rs != TE_OK) return rs;
   if (e_tri_out) jobs[0].shares = e_tri_out;  // shares[t - t_begin]
   else jobs[0].shares = jobs[0].b.etri;
@@ -1842,14 +1576,16 @@ te_status run_tc_batched(Handle* h, const te_cluster* cs, int64_t n, te_precisio
     rs = check_k(mode, o, v);
     if (rs != TE_OK) return rs;
     const int64_t nt = num_unique_triples(o);
-    if (nt == 0) {
-      if (cudaMemsetAsync(e_out + x, 0, sizeof(double), s) != cudaSuccess) return fail(TE_ECUDA, "memset failed");
-      ++h->n_launches;
+    if (nt == 0) {  // no triples: the value checks alone
+      if (launch_check_inputs(cs + x, x, h->d_err, h->num_sms, s) != cudaSuccess ||
+          cudaMemsetAsync(e_out + x, 0, sizeof(double), s) != cudaSuccess)
+        return fail(TE_ECUDA, "check or memset launch failed");
+      h->n_launches += 2;
       continue;
     }
     const TcPlan pl = make_plan(h, o, v, mode, nt);
     TcJob J;
-    rs = setup_job(h, st, cs + x, mode, 0, nt, pl, base + off, &J, s);
+    rs = setup_job(h, st, cs + x, mode, 0, nt, pl, base + off, &J, x, s);
     if (rs != TE_OK) return rs;
     TcBuffers bb;
     off += tc_carve_cluster(nullptr, pl, o, v, nt, &bb);

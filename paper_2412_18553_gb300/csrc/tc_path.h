@@ -42,6 +42,8 @@ struct SliceSet {
 // Bytes the slice planes need; tc_prepare_slices lays them out from base
 // (256-byte aligned) and launches the slicing on s.
 size_t tc_slices_bytes(int o, int v, int ns = 4);
+// With err set, the pass over the inputs that finds the scales also makes the
+// value checks of launch_check_inputs.
 te_status tc_prepare_slices(const te_cluster* c, void* base, SliceSet* out, int num_sms, cudaStream_t s,
-                            int ns = 4);
+                            int ns, unsigned int* err, int64_t cluster, int64_t* launches);
 }  // namespace te

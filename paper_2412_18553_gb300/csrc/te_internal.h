@@ -27,12 +27,22 @@ enum : unsigned int {
 // site (1..7 the array, 8 the eps ordering, 9 and 10 the density-fitting
 // factors) and `cluster` in the error word.  With df, ovvv is not checked
 // (not read) and Bov, Bvv are.
+// Where the pass also leaves the largest magnitudes it saw (high words of the
+// float64, cleared by the caller; null members are not wanted): of whole
+// arrays, or with `groups` of ovvv[p], t2[r,q], ooov[p,:,r,:] and, for t2L,
+// t2[:,q].
+struct MaxOut {
+  unsigned int *ovvv, *t2, *ooov, *bov, *bvv, *t2L;
+  bool groups;
+};
+// err null: the magnitudes only, no checks.
 cudaError_t launch_check_inputs(const te_cluster* c, int64_t cluster, unsigned int* err, int num_sms,
-                                cudaStream_t s, const te_df* df = nullptr);
+                                cudaStream_t s, const te_df* df = nullptr, const MaxOut* out = nullptr);
 // The same for the MP2 step's inputs (eps_o, eps_v, and the DF factor's ov
-// block of nB entries, site 9).
+// block of nB entries, site 9); max_bov as in MaxOut.
 cudaError_t launch_check_mp2(const double* eps_o, int64_t o, const double* eps_v, int64_t v, const double* Bov,
-                             int64_t nB, int64_t cluster, unsigned int* err, int num_sms, cudaStream_t s);
+                             int64_t nB, int64_t cluster, unsigned int* err, int num_sms, cudaStream_t s,
+                             unsigned int* max_bov = nullptr);
 
 // One occupied triple of the canonical unique list.
 struct Triple {
@@ -149,9 +159,10 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
 // workspace bytes of the two adjoints (vjp.cu)
 size_t vjp_fp64_bytes(int64_t o, int64_t v);
 size_t vjp_tc_bytes(int64_t o, int64_t v, int num_sms);
-// the same with the contractions on the tensor cores in exact BF16 slices (vjp.cu)
+// the same with the contractions on the tensor cores in exact BF16 slices
+// (vjp.cu); makes the value checks, which the float64 adjoint leaves to its caller
 te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_end, double gE,
-                     double* e_out, te_cluster_grad* g, cudaStream_t s);
+                     double* e_out, te_cluster_grad* g, cudaStream_t s, int64_t cluster);
 
 constexpr int ENERGY_TB = 8;  // virtual block edge of the energy kernel
 inline int64_t energy_num_blocks(int64_t v) { return (v + ENERGY_TB - 1) / ENERGY_TB; }

@@ -624,50 +624,6 @@ cudaError_t gemm_oz(const OzView& g, int num_sms, double* scratch, int64_t scrat
   return cudaGetLastError();
 }
 
-// max |x| as the bit pattern of a non-negative double (they order as integers)
-__global__ void k_maxabs_bits(const double* __restrict__ x, int64_t n, unsigned long long* out) {
-  double m = 0.0;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x)
-    m = fmax(m, fabs(x[idx]));
-  for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
-}
-
-// NS 7-bit BF16 slices of x (slice s at planes + s n): x = 2^e sum_s m_s
-// 2^-7(s+1) + r, 2^e > max |x|, |r| <= 2^(e - 7 NS - 1)
-template <int NS>
-__global__ void k_slice_planes(const double* __restrict__ x, int64_t n, const unsigned long long* __restrict__ xmax,
-                               int* __restrict__ e_out, __nv_bfloat16* __restrict__ planes) {
-  const double mx = __longlong_as_double((long long)*xmax);
-  int ex = 0;
-  if (mx > 0.0) frexp(mx, &ex);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *e_out = ex;
-  const double sc = ldexp(1.0, -ex);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double t = x[i] * sc;  // |t| < 1
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      t = t * 128.0;
-      const double m = rint(t);
-      t = t - m;
-      planes[k * n + i] = __float2bfloat16_rn((float)(m * (1.0 / (double)(1ull << (7 * (k + 1))))));
-    }
-  }
-}
-
-cudaError_t slice_planes(const double* x, int64_t n, int ns, unsigned long long* mx, int* ex,
-                         __nv_bfloat16* planes, cudaStream_t s, int64_t* launches) {
-  if (ns != 4 && ns != 5) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(mx, 0, 8, s);
-  if (e != cudaSuccess) return e;
-  const int grid = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 255) / 256), 8192);
-  k_maxabs_bits<<<std::min(grid, 1024), 256, 0, s>>>(x, n, mx);
-  if (ns == 5) k_slice_planes<5><<<grid, 256, 0, s>>>(x, n, mx, ex, planes);
-  else k_slice_planes<4><<<grid, 256, 0, s>>>(x, n, mx, ex, planes);
-  *launches += 2;
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------------------
 // Y and denominator reductions for one triple
 // ---------------------------------------------------------------------------
@@ -1107,7 +1063,7 @@ size_t vjp_tc_bytes(int64_t o, int64_t v, int num_sms) {
 // Outputs of the same launch are disjoint: the contributions to one output
 // slab (or pair block) are the segments of one job.
 te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_end, double gE,
-                     double* e_out, te_cluster_grad* g, cudaStream_t s) {
+                     double* e_out, te_cluster_grad* g, cudaStream_t s, int64_t cluster) {
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int64_t v2 = (int64_t)v * v, v3 = v2 * v, nt = num_unique_triples(o);
   te_status st = ensure_workspace_public(h, vjp_tc_bytes(o, v, h->num_sms));
@@ -1119,7 +1075,7 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
   const int64_t vp = Z.vp;
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023));
   SliceSet S;
-  st = tc_prepare_slices(c, base, &S, h->num_sms, s, ns);
+  st = tc_prepare_slices(c, base, &S, h->num_sms, s, ns, h->d_err, cluster, &h->n_launches);
   if (st != TE_OK) return st;
   char* p = base + ((tc_slices_bytes(o, v, ns) + 1023) & ~size_t(1023));
   auto takeb = [&](size_t bytes) {
