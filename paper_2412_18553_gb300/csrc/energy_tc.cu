@@ -32,15 +32,6 @@ constexpr int TB = 8;
 constexpr int WARPS = 16;                 // compute warps: one orbit candidate (a,b,c) of 8^3 per thread
 constexpr int THREADS = (WARPS + 1) * 32;  // + one producer warp
 
-template <int N>
-struct Pos {
-  static constexpr int s0 = (N <= 1) ? 0 : (N <= 3) ? 1 : 2;
-  static constexpr int s1 = (N == 0) ? 1 : (N == 1) ? 2 : (N == 2) ? 0 : (N == 3) ? 2 : (N == 4) ? 0 : 1;
-  static constexpr int s2 = 3 - s0 - s1;
-  static constexpr int r1 = (N == 0) ? 3 : (N == 1) ? 5 : (N == 2) ? 1 : (N == 3) ? 4 : (N == 4) ? 0 : 2;
-  static constexpr int r2 = (N == 0) ? 4 : (N == 1) ? 2 : (N == 2) ? 5 : (N == 3) ? 0 : (N == 4) ? 3 : 1;
-};
-
 template <int CW>
 struct Layout {
   static constexpr uint32_t cube_bytes = TB * TB * TB * 4 * CW;
@@ -49,8 +40,6 @@ struct Layout {
   static constexpr uint32_t t1 = 9 * 128;
   static constexpr uint32_t eps = 640;  // dAB[64] = e_ijk - e_a - e_b, epsC[8] (FP64, written by the producer)
   static constexpr uint32_t buf = cubes + ovs + t1 + eps;
-  // W~ (CW planes) and Y (one plane) of the item's 6 block orders, assembled once per item
-  static constexpr uint32_t asm_bytes = 6 * 512 * 4 * (CW + 1);
   static constexpr uint32_t tx = 18 * cube_bytes + 18 * TB * TB * 4 + 9 * TB * 4;
 };
 
@@ -102,74 +91,6 @@ __device__ __forceinline__ df df_scale(df a, float k) {  // k a small integer
   return df_norm(p, __fadd_rn(e, __fmul_rn(a.l, k)));
 }
 
-// G value of block g at cube `pid`, local (x, y, z): hi and lo parts.
-template <int CW>
-__device__ __forceinline__ void gval(const float* cube, int g, int pid, int x, int y, int z, float& hi,
-                                     float& lo) {
-  const float* p = cube + (g * 6 + pid) * (TB * TB * TB * CW) + cube_off(x, y, z);
-  hi = p[0];
-  lo = (CW == 2) ? p[TB * TB * TB] : 0.f;
-}
-
-template <int S>
-__device__ __forceinline__ int pick(int la, int lb, int lc) {
-  return S == 0 ? la : (S == 1 ? lb : lc);
-}
-
-// deviation of W~ at position N from position 0, and Y at position N
-template <int CW, int N>
-__device__ __forceinline__ float w_dev(const float* cube, int la, int lb, int lc) {
-  constexpr int s0 = Pos<N>::s0, s1 = Pos<N>::s1, s2 = Pos<N>::s2;
-  const int x = pick<s0>(la, lb, lc), y = pick<s1>(la, lb, lc), z = pick<s2>(la, lb, lc);
-  float h0, l0, hn, ln, d = 0.f, dl = 0.f;
-  // G0[x][y][z] at cube N, minus G0[a][b][c] at cube 0
-  gval<CW>(cube, 0, N, x, y, z, hn, ln);
-  gval<CW>(cube, 0, 0, la, lb, lc, h0, l0);
-  d += hn - h0;
-  dl += ln - l0;
-  // G1[y][z][x] at cube r1(N), minus G1[b][c][a] at cube 3
-  gval<CW>(cube, 1, Pos<N>::r1, y, z, x, hn, ln);
-  gval<CW>(cube, 1, 3, lb, lc, la, h0, l0);
-  d += hn - h0;
-  dl += ln - l0;
-  // G2[z][x][y] at cube r2(N), minus G2[c][a][b] at cube 4
-  gval<CW>(cube, 2, Pos<N>::r2, z, x, y, hn, ln);
-  gval<CW>(cube, 2, 4, lc, la, lb, h0, l0);
-  d += hn - h0;
-  dl += ln - l0;
-  return d + dl;
-}
-
-// double-float deviation of W~ at position N from position 0 (CW = 2)
-template <int N>
-__device__ __forceinline__ df w_dev_df(const float* cube, int la, int lb, int lc) {
-  constexpr int s0 = Pos<N>::s0, s1 = Pos<N>::s1, s2 = Pos<N>::s2;
-  const int x = pick<s0>(la, lb, lc), y = pick<s1>(la, lb, lc), z = pick<s2>(la, lb, lc);
-  float h0, l0, hn, ln;
-  gval<2>(cube, 0, N, x, y, z, hn, ln);
-  gval<2>(cube, 0, 0, la, lb, lc, h0, l0);
-  df acc = df_two_sum(hn, -h0);
-  float lsum = __fsub_rn(ln, l0);
-  gval<2>(cube, 1, Pos<N>::r1, y, z, x, hn, ln);
-  gval<2>(cube, 1, 3, lb, lc, la, h0, l0);
-  acc = df_add(acc, df_two_sum(hn, -h0));
-  lsum = __fadd_rn(lsum, __fsub_rn(ln, l0));
-  gval<2>(cube, 2, Pos<N>::r2, z, x, y, hn, ln);
-  gval<2>(cube, 2, 4, lc, la, lb, h0, l0);
-  acc = df_add(acc, df_two_sum(hn, -h0));
-  lsum = __fadd_rn(lsum, __fsub_rn(ln, l0));
-  return df_add(acc, df{lsum, 0.f});
-}
-
-template <int N>
-__device__ __forceinline__ float y_at(const float* ovsS, const float* t1S, int la, int lb, int lc) {
-  constexpr int s0 = Pos<N>::s0, s1 = Pos<N>::s1, s2 = Pos<N>::s2;
-  const int x = pick<s0>(la, lb, lc), y = pick<s1>(la, lb, lc), z = pick<s2>(la, lb, lc);
-  return ovsS[((0 * 3 + s0) * 3 + s1) * 64 + x * 8 + y] * t1S[(2 * 3 + s2) * 32 + z] +
-         ovsS[((1 * 3 + s1) * 3 + s2) * 64 + y * 8 + z] * t1S[(0 * 3 + s0) * 32 + x] +
-         ovsS[((2 * 3 + s0) * 3 + s2) * 64 + x * 8 + z] * t1S[(1 * 3 + s1) * 32 + y];
-}
-
 struct EnergyMaps {
   CUtensorMap ovs[TC_MAX_CL];  // per cluster: ovs32 [o][v][o][vq], 4D (b, j, a, i)
   CUtensorMap t1[TC_MAX_CL];   // per cluster: t1 [o][vq], 2D (a, i)
@@ -181,7 +102,7 @@ struct EnergyParams {
   EnergyCl cl[TC_MAX_CL];
   TcPiece pc[TC_MAX_PIECES];  // G: orbit-major [slot][bt][g][pid][CW planes][512, swizzled] from pc.gbuf
   const Triple* triples;
-  double* partials;  // [global slot][grid][WARPS]: the warps' sums of a triple's items
+  double* partials;  // [slot][first item of the block][WARPS]: the warps' sums of a triple's items
   unsigned int* err;
   unsigned long long wait_ns;
 };
@@ -191,22 +112,31 @@ struct PieceTable {
   TcPiece pc[TC_MAX_PIECES];
 };
 
-// A block's items: for each piece, for each of its triples, the block
-// triples bt = blockIdx.x, blockIdx.x + gridDim.x, ... (< nbt), in order.
-// Which items of a triple a block takes, and in which order, depends on the
-// triple's nbt and the grid size alone (the grid is always one block per SM),
-// not on the launch's other pieces: a triple's float64 sums have the same bits
-// in a single-cluster call and in a batch.
+// A block's items: item bt of canonical triple t belongs to block (t nbt + bt)
+// mod gridDim.x, so consecutive triples follow each other around the blocks
+// without a gap (restarting every triple at block 0 left 11% of the block
+// slots empty at nvir = 120: 680 items on 152 blocks).  Which items of a
+// triple a block takes, and in which order, depends on t, nbt and the grid
+// size alone (the grid is always one block per SM), not on the launch's other
+// pieces: a triple's float64 sums have the same bits in a single-cluster call
+// and in a batch.
 struct ItemCursor {
-  int q, ls;   // piece, triple slot within the piece
-  int64_t bt;  // block triple
+  int q, ls;      // piece, triple slot within the piece
+  int64_t bt;     // block triple
+  int64_t first;  // the block's first block triple of this triple
 };
+
+__device__ __forceinline__ int64_t cursor_first(const TcPiece& pc, int ls) {
+  const int64_t r = ((int64_t)blockIdx.x - (pc.t0 + ls) * pc.nbt) % (int64_t)gridDim.x;
+  return r < 0 ? r + gridDim.x : r;
+}
 
 __device__ __forceinline__ void cursor_settle(const EnergyParams& P, ItemCursor& c) {
   while (c.q < P.npieces) {
     const TcPiece& pc = P.pc[c.q];
+    if (c.bt < 0) c.bt = c.first = cursor_first(pc, c.ls);
     if (c.bt < pc.nbt) return;
-    c.bt = blockIdx.x;  // no (more) items of this triple for this block
+    c.bt = -1;  // no (more) items of this triple for this block
     if (++c.ls >= pc.ns) {
       c.ls = 0;
       ++c.q;
@@ -221,8 +151,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                          ~uintptr_t(127));
-  float* asmW = reinterpret_cast<float*>(smem + 2 * L::buf);           // [CW planes][6][512] then Y [6][512]
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + 2 * L::buf + L::asm_bytes);  // [2]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + 2 * L::buf);    // [2]
   uint64_t* empty = full + 2;                                         // [2], one arrival per compute warp
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + 2);
   int* meta = const_cast<int*>(reinterpret_cast<volatile int*>(abort_flag) + 1);  // [2][8]: X, Y, Z, slot, v, item
@@ -243,7 +172,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t ephase = 0u, pending = 0u, fphase = 0u;  // one bit per buffer
     int b = 0;
     bool ok = true;
-    ItemCursor cur{0, 0, (int64_t)blockIdx.x};
+    ItemCursor cur{0, 0, -1, -1};
     cursor_settle(P, cur);
     for (; ok && cur.q < P.npieces; cur.bt += gridDim.x, cursor_settle(P, cur), b ^= 1) {
       // buffer b free: all compute warps done with the item it held
@@ -330,36 +259,38 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (((pending >> q) & 1u) && !ok) ptx::mbar_wait(&full[q], ((fphase >> q) & 1u) ^ 1u, P.wait_ns);
   } else {
     // ---------------- compute warps ----------------
-    // Each item in two phases.  A: every thread forms, at its own local point
-    // (la, lb, lc) of each of the 6 block orders P, W~ = G0 + G1 + G2 (as an FP32
-    // pair for CW = 2) and Y, into the assembled area; the G buffer is then
-    // released to the producer.  B: every thread takes the orbit (a,b,c) =
-    // its local point in block order 0 and reads W~ and Y at its 6 positions.
+    // A thread takes the orbit (a,b,c) = its local point of the block triple.
+    // With pid m a block order and A_m the same permutation of (la, lb, lc) in
+    // cube m, W~ at position n is G0[A_n] + G1[A_r1(n)] + G2[A_r2(n)]: six
+    // offsets address all 36 words, each read once, and no value crosses
+    // threads.  (An earlier form assembled W~ and Y of the six orders in shared
+    // memory first: 24 more stores and 18 more loads per thread, and two
+    // block-wide barriers per item.)  The buffer goes back to the producer as
+    // soon as the words are in registers.
     uint32_t phase = 0u;  // one bit per buffer
     int b = 0;
     const int la = (tid >> 6), lb = (tid >> 3) & 7, lc = tid & 7;
-    const int o_own = cube_off(la, lb, lc), o_g1 = cube_off(lb, lc, la), o_g2 = cube_off(lc, la, lb);
     int pos_off[6];
 #pragma unroll
     for (int n = 0; n < 6; ++n) {
       const int u = n <= 1 ? la : (n <= 3 ? lb : lc);
       const int w = (n == 0 || n == 5) ? lb : ((n == 1 || n == 3) ? lc : la);
-      const int z = 3 * 0 + ((n == 0 || n == 2) ? lc : ((n == 1 || n == 4) ? lb : la));
-      pos_off[n] = n * 512 + cube_off(u, w, z);
+      const int z = (n == 0 || n == 2) ? lc : ((n == 1 || n == 4) ? lb : la);
+      pos_off[n] = n * 512 * CW + cube_off(u, w, z);
     }
-    float* asmY = asmW + CW * 6 * 512;
     // this thread's float64 sum over its items of the current triple slot; the
     // warp's sum (fixed shuffle order) goes to the partials when the slot
     // changes (a block takes a triple's items one after another)
     double acc = 0.0;
     int cur_slot = -1;
+    int64_t cur_first = 0;
     auto flush = [&]() {
       double a = acc;
       for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-      if (lane == 0) P.partials[((int64_t)cur_slot * gridDim.x + blockIdx.x) * WARPS + warp] = a;
+      if (lane == 0) P.partials[((int64_t)cur_slot * gridDim.x + cur_first) * WARPS + warp] = a;
       acc = 0.0;
     };
-    ItemCursor cur{0, 0, (int64_t)blockIdx.x};
+    ItemCursor cur{0, 0, -1, -1};
     cursor_settle(P, cur);
     for (; cur.q < P.npieces; cur.bt += gridDim.x, cursor_settle(P, cur), b ^= 1) {
       int got = 0;
@@ -380,6 +311,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (slot != cur_slot) {
         if (cur_slot >= 0) flush();
         cur_slot = slot;
+        cur_first = cur.first;
       }
       const unsigned char* base = smem + (size_t)b * L::buf;
       const float* cube = reinterpret_cast<const float*>(base);
@@ -388,55 +320,61 @@ __global__ void __launch_bounds__(THREADS, 1)
       const double* dAB = reinterpret_cast<const double*>(base + L::cubes + L::ovs + L::t1);
       const double D = dAB[la * 8 + lb] - dAB[64 + lc];
 
-      // ---- phase A ----
+      const int a = bx * TB + la, bb = by * TB + lb, c = bz * TB + lc;
+      const bool valid = a < vcl && bb < vcl && c < vcl && !(bx == by && la < lb) && !(by == bz && lb < lc);
+      float wh[6], wl[6], y[6];
+      if (valid) {
+        float t1v[3][3];  // [i, j, k][slot of the virtual]
 #pragma unroll
-      for (int Pn = 0; Pn < 6; ++Pn) {
-        const int r1 = Pn == 0 ? 3 : Pn == 1 ? 5 : Pn == 2 ? 1 : Pn == 3 ? 4 : Pn == 4 ? 0 : 2;
-        const int r2 = Pn == 0 ? 4 : Pn == 1 ? 2 : Pn == 2 ? 5 : Pn == 3 ? 0 : Pn == 4 ? 3 : 1;
-        const int s0 = Pn <= 1 ? 0 : (Pn <= 3 ? 1 : 2);
-        const int s1 = Pn == 0 ? 1 : Pn == 1 ? 2 : Pn == 2 ? 0 : Pn == 3 ? 2 : Pn == 4 ? 0 : 1;
-        const int s2 = 3 - s0 - s1;
-        const float* g0 = cube + (0 * 6 + Pn) * 512 * CW;
-        const float* g1 = cube + (1 * 6 + r1) * 512 * CW;
-        const float* g2 = cube + (2 * 6 + r2) * 512 * CW;
-        const int wo = Pn * 512 + o_own;
-        if constexpr (CW == 2) {
-          df wv = df_two_sum(g0[o_own], g1[o_g1]);
-          wv = df_add(wv, df{g2[o_g2], 0.f});
-          wv = df_norm(wv.h, __fadd_rn(wv.l, __fadd_rn(__fadd_rn(g0[512 + o_own], g1[512 + o_g1]), g2[512 + o_g2])));
-          asmW[wo] = wv.h;
-          asmW[6 * 512 + wo] = wv.l;
-        } else {
-          asmW[wo] = (g0[o_own] + g1[o_g1]) + g2[o_g2];
+        for (int q = 0; q < 3; ++q) {
+          t1v[q][0] = t1S[(q * 3 + 0) * 32 + la];
+          t1v[q][1] = t1S[(q * 3 + 1) * 32 + lb];
+          t1v[q][2] = t1S[(q * 3 + 2) * 32 + lc];
         }
-        // Y at (x, y, z) = (la, lb, lc) of blocks (s0, s1, s2):
-        //   ovs(i,x,j,y) t1(k,z) + ovs(j,y,k,z) t1(i,x) + ovs(i,x,k,z) t1(j,y)
-        asmY[wo] = ovsS[((0 * 3 + s0) * 3 + s1) * 64 + la * 8 + lb] * t1S[(2 * 3 + s2) * 32 + lc] +
-                   ovsS[((1 * 3 + s1) * 3 + s2) * 64 + lb * 8 + lc] * t1S[(0 * 3 + s0) * 32 + la] +
-                   ovsS[((2 * 3 + s0) * 3 + s2) * 64 + la * 8 + lc] * t1S[(1 * 3 + s1) * 32 + lb];
+#pragma unroll
+        for (int n = 0; n < 6; ++n) {
+          const int r1 = n == 0 ? 3 : n == 1 ? 5 : n == 2 ? 1 : n == 3 ? 4 : n == 4 ? 0 : 2;
+          const int r2 = n == 0 ? 4 : n == 1 ? 2 : n == 2 ? 5 : n == 3 ? 0 : n == 4 ? 3 : 1;
+          const int s0 = n <= 1 ? 0 : (n <= 3 ? 1 : 2);
+          const int s1 = n == 0 ? 1 : n == 1 ? 2 : n == 2 ? 0 : n == 3 ? 2 : n == 4 ? 0 : 1;
+          const int s2 = 3 - s0 - s1;
+          const int x = s0 == 0 ? la : (s0 == 1 ? lb : lc), yy = s1 == 0 ? la : (s1 == 1 ? lb : lc),
+                    z = s2 == 0 ? la : (s2 == 1 ? lb : lc);
+          const float* g0 = cube + pos_off[n];
+          const float* g1 = cube + 6 * 512 * CW + pos_off[r1];
+          const float* g2 = cube + 12 * 512 * CW + pos_off[r2];
+          if constexpr (CW == 2) {
+            df wv = df_two_sum(g0[0], g1[0]);
+            wv = df_add(wv, df{g2[0], 0.f});
+            wv = df_norm(wv.h, __fadd_rn(wv.l, __fadd_rn(__fadd_rn(g0[512], g1[512]), g2[512])));
+            wh[n] = wv.h;
+            wl[n] = wv.l;
+          } else {
+            wh[n] = (g0[0] + g1[0]) + g2[0];
+            wl[n] = 0.f;
+          }
+          // Y at (x, y, z) = positions (s0, s1, s2):
+          //   ovs(i,x,j,y) t1(k,z) + ovs(j,y,k,z) t1(i,x) + ovs(i,x,k,z) t1(j,y)
+          y[n] = fmaf(ovsS[((2 * 3 + s0) * 3 + s2) * 64 + x * 8 + z], t1v[1][s1],
+                      fmaf(ovsS[((1 * 3 + s1) * 3 + s2) * 64 + yy * 8 + z], t1v[0][s0],
+                           __fmul_rn(ovsS[((0 * 3 + s0) * 3 + s1) * 64 + x * 8 + yy], t1v[2][s2])));
+        }
       }
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&empty[b]);  // this warp no longer reads buffer b
-      asm volatile("bar.sync 1, %0;" ::"n"(WARPS * 32) : "memory");
-
-      // ---- phase B ----
-      const int a = bx * TB + la, bb = by * TB + lb, c = bz * TB + lc;
-      const bool valid = a < vcl && bb < vcl && c < vcl && !(bx == by && la < lb) && !(by == bz && lb < lc);
       if (valid) {
         // orbit weight A (Eq. E_corr_CCSD_T): 1, 1/2 or 1/6
         const bool all3 = (a == bb && bb == c), two = (a == bb || bb == c);
         const double r0 = (double)__frcp_rn((float)D);
         const double r1 = fma(r0, fma(-D, r0, 1.0), r0);  // 1/D to ~1e-14 (one Newton step)
-        const float y0 = asmY[pos_off[0]];
         if constexpr (CW == 2) {
-          const float h0 = asmW[pos_off[0]], l0 = asmW[6 * 512 + pos_off[0]];
           df wd[5], vd[5];
 #pragma unroll
           for (int n = 1; n < 6; ++n) {
-            df d = df_two_sum(asmW[pos_off[n]], -h0);
-            d = df_norm(d.h, __fadd_rn(d.l, __fsub_rn(asmW[6 * 512 + pos_off[n]], l0)));
+            df d = df_two_sum(wh[n], -wh[0]);
+            d = df_norm(d.h, __fadd_rn(d.l, __fsub_rn(wl[n], wl[0])));
             wd[n - 1] = d;
-            vd[n - 1] = df_add(d, df{__fsub_rn(asmY[pos_off[n]], y0), 0.f});
+            vd[n - 1] = df_add(d, df{__fsub_rn(y[n], y[0]), 0.f});
           }
           const df w1 = wd[0], w2 = wd[1], w3 = wd[2], w4 = wd[3], w5 = wd[4];
           const df v1 = vd[0], v2 = vd[1], v3 = vd[2], v4 = vd[3], v5 = vd[4];
@@ -454,12 +392,11 @@ __global__ void __launch_bounds__(THREADS, 1)
           acc = fma((double)T.h, r1, acc);
           acc = fma((double)T.l, r1, acc);
         } else {
-          const float W0 = asmW[pos_off[0]];
           float w[5], vv[5];
 #pragma unroll
           for (int n = 1; n < 6; ++n) {
-            w[n - 1] = asmW[pos_off[n]] - W0;
-            vv[n - 1] = w[n - 1] + (asmY[pos_off[n]] - y0);
+            w[n - 1] = wh[n] - wh[0];
+            vv[n - 1] = w[n - 1] + (y[n] - y[0]);
           }
           const float Ae = w[2] + w[3], Ao = w[0] + w[1] + w[4];
           const float Se = vv[2] + vv[3], So = vv[0] + vv[1] + vv[4];
@@ -469,7 +406,6 @@ __global__ void __launch_bounds__(THREADS, 1)
           acc = fma(Tw, r1, acc);
         }
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(WARPS * 32) : "memory");  // assembled area free
     }
     if (cur_slot >= 0) flush();
   }
@@ -484,7 +420,7 @@ int64_t energy_tc_grid(int num_sms, int64_t items) {
 }
 
 size_t energy_tc_smem(int cw) {
-  const size_t buf = cw == 2 ? Layout<2>::buf + Layout<2>::asm_bytes / 2 : Layout<1>::buf + Layout<1>::asm_bytes / 2;
+  const size_t buf = cw == 2 ? Layout<2>::buf : Layout<1>::buf;
   return 2 * buf + 128 + 512;
 }
 
@@ -508,9 +444,7 @@ cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s) {
   P.wait_ns = e.wait_ns;
   const size_t smem = energy_tc_smem(e.cw);
   const int64_t grid = energy_tc_grid(e.num_sms, P.items);
-  // a block writes a slot's partials only if it took one of its items
-  cudaError_t err = cudaMemsetAsync(P.partials, 0, (size_t)e.nslots * grid * WARPS * sizeof(double), s);
-  if (err != cudaSuccess) return err;
+  cudaError_t err;
   if (e.cw == 2) {
     err = cudaFuncSetAttribute(k_energy_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
@@ -523,9 +457,13 @@ cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// One block per G slot of the launch: the slot's grid x WARPS partials summed
-// in a fixed order (thread t takes t, t + 256, ..., then a fixed tree, with
-// Neumaier compensation), times m/3, into its piece's shares.
+// One block per slot: the partials of the blocks that took items of the triple
+// (the first min(grid, nbt) x WARPS of the slot) summed in a fixed order
+// (thread t takes t, t + 256, ..., then a fixed tree, with Neumaier
+// compensation), times m/3, into its piece's shares.  A block is a chain of
+// latencies (12 us for 2432 partials, whatever the launch holds), so one
+// launch takes the slots of many rounds: at nocc=16 nvir=120, 200 launches of
+// four slots were 2.5 ms of a 50 ms call.
 __device__ __forceinline__ void neumaier(double& s, double& c, double x) {
   const double t = s + x;
   if (fabs(s) >= fabs(x)) c += (s - t) + x;
@@ -533,7 +471,7 @@ __device__ __forceinline__ void neumaier(double& s, double& c, double x) {
   s = t;
 }
 
-__global__ void __launch_bounds__(256) k_reduce_pieces(const double* __restrict__ partials, int nper,
+__global__ void __launch_bounds__(256) k_reduce_pieces(const double* __restrict__ partials, int grid,
                                                        const Triple* __restrict__ triples,
                                                        const __grid_constant__ PieceTable T) {
   const int gslot = blockIdx.x;
@@ -541,7 +479,8 @@ __global__ void __launch_bounds__(256) k_reduce_pieces(const double* __restrict_
   while (q + 1 < T.n && T.pc[q + 1].slot0 <= gslot) ++q;
   const TcPiece& pc = T.pc[q];
   const int local = gslot - pc.slot0;
-  const double* x = partials + (int64_t)gslot * nper;
+  const int nper = (int)min((int64_t)grid, pc.nbt) * WARPS;
+  const double* x = partials + (int64_t)gslot * grid * WARPS;
   __shared__ double ss[256], cc[256];
   double sum = 0.0, c = 0.0;
   for (int i = threadIdx.x; i < nper; i += blockDim.x) neumaier(sum, c, x[i]);
@@ -560,13 +499,13 @@ __global__ void __launch_bounds__(256) k_reduce_pieces(const double* __restrict_
   if (threadIdx.x == 0) pc.shares[local] = (ss[0] + cc[0]) * ((double)triples[pc.t0 + local].m / 3.0);
 }
 
-cudaError_t launch_reduce_pieces(const double* partials, int nper, const Triple* triples,
+cudaError_t launch_reduce_pieces(const double* partials, int grid, const Triple* triples,
                                  const TcPiece* pieces, int npieces, int nslots, cudaStream_t s) {
   PieceTable T;
   std::memset(&T, 0, sizeof(T));
   T.n = npieces;
   for (int q = 0; q < npieces; ++q) T.pc[q] = pieces[q];
-  k_reduce_pieces<<<(unsigned)nslots, 256, 0, s>>>(partials, nper, triples, T);
+  k_reduce_pieces<<<(unsigned)nslots, 256, 0, s>>>(partials, grid, triples, T);
   return cudaGetLastError();
 }
 

@@ -745,15 +745,19 @@ static size_t tc_carve_cluster(char* base, const TcPlan& pl, int64_t o, int64_t 
 }
 
 // Workspace of one run: the clusters' parts, then the G pool, then the
-// energy partials: per G slot of a launch, one float64 sum per block (one
-// block per SM) and compute warp.
+// energy partials: per triple, one float64 sum per block (one block per SM)
+// and compute warp, for the rounds up to the next share reduction.
 struct TcPool {
   int64_t pool_floats;
   int64_t max_slots;  // G slots per launch
+  int64_t par_slots;  // energy partials held until their share reduction (at least max_slots)
 };
 
+// Triples whose partials wait for one share reduction: about 20 MB of them.
+constexpr int64_t TC_PAR_SLOTS = 1024;
+
 static size_t tc_partial_bytes(const TcPool& q, int num_sms) {
-  return (size_t)q.max_slots * std::max(1, num_sms) * ENERGY_TC_WARPS * sizeof(double);
+  return (size_t)q.par_slots * std::max(1, num_sms) * ENERGY_TC_WARPS * sizeof(double);
 }
 
 static size_t tc_shared_bytes(const TcPool& q, int num_sms) {
@@ -1089,8 +1093,10 @@ static te_status gemm_params(const Handle* h, const std::vector<TcJob>& jobs, co
 
 // Runs the jobs' triples in rounds: each round fills the G pool with pieces
 // (up to TC_MAX_CL clusters, TC_MAX_PIECES pieces, one TMEM buffering), then
-// launches the contraction, the energy epilogue and the share reduction once.
-// Then each job's total.  Pieces follow the jobs' order.
+// launches the contraction and the energy epilogue once.  The shares are
+// reduced when the partials of par_slots triples or TC_MAX_PIECES runs of
+// triples have come together, and at the end; then each job's total.  Pieces
+// follow the jobs' order.
 static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float* pool, const TcPool& pq,
                             double* partials, cudaStream_t s) {
   const double nprod = (mode == TC_TF32) ? 1.0 : (mode == TC_OZAKI ? 10.0 : (mode == TC_OZAKI6 ? 15.0 : 3.0));
@@ -1102,6 +1108,17 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
   TcParams* P = new TcParams;
   EnergyLaunch* EL = new EnergyLaunch;
   te_status st = TE_OK;
+  const int egrid = (int)energy_tc_grid(h->num_sms, 0);
+  std::vector<TcPiece> held;  // runs of triples whose partials wait for the share reduction
+  int nheld = 0;              // their slots
+  auto reduce_held = [&]() {
+    if (held.empty()) return;
+    const cudaError_t e = launch_reduce_pieces(partials, egrid, h->d_triples, held.data(), (int)held.size(), nheld, s);
+    ++h->n_launches;
+    if (e != cudaSuccess) st = fail(TE_ECUDA, "share reduction launch: %s", cudaGetErrorString(e));
+    held.clear();
+    nheld = 0;
+  };
   while (st == TE_OK) {
     while (j < jobs.size() && t >= jobs[j].t_end) {
       ++j;
@@ -1157,6 +1174,18 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
       st = fail(TE_ENOMEM, "G pool smaller than one triple's G blocks");
       break;
     }
+    if (nheld + nslots > pq.par_slots || held.size() + pcs.size() > (size_t)TC_MAX_PIECES) reduce_held();
+    if (st != TE_OK) break;
+    for (const TcPiece& pc : pcs) {
+      // a run that continues the last one (same cluster, next triple) joins it
+      if (!held.empty() && held.back().shares + held.back().ns == pc.shares && held.back().t0 + held.back().ns == pc.t0 &&
+          held.back().nbt == pc.nbt) {
+        held.back().ns += pc.ns;
+      } else {
+        held.push_back(pc);
+        held.back().slot0 = nheld + pc.slot0;
+      }
+    }
     size_t smem = 0;
     st = gemm_params(h, jobs, jl, ncl, pcs.data(), (int)pcs.size(), tiles, mode, P, MS, &smem);
     if (st != TE_OK) break;
@@ -1175,7 +1204,8 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     }
     for (size_t q = 0; q < pcs.size(); ++q) EL->pc[q] = pcs[q];
     EL->triples = h->d_triples;
-    EL->partials = partials;
+    EL->partials = partials + (int64_t)nheld * egrid * ENERGY_TC_WARPS;
+    nheld += nslots;
     EL->err = h->d_err;
     EL->wait_ns = h->wait_limit_ns;
     if (h->log)
@@ -1190,12 +1220,10 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
       e = launch_energy_tc(*EL, s);
       prof_end(h, pm, s);
     }
-    if (e == cudaSuccess)
-      e = launch_reduce_pieces(partials, (int)(energy_tc_grid(h->num_sms, items) * ENERGY_TC_WARPS), h->d_triples,
-                               pcs.data(), (int)pcs.size(), nslots, s);
-    h->n_launches += 3;
+    h->n_launches += 2;
     if (e != cudaSuccess) st = fail(TE_ECUDA, "tensor-core path launch: %s", cudaGetErrorString(e));
   }
+  if (st == TE_OK) reduce_held();
   delete MS;
   delete P;
   delete EL;
@@ -1245,6 +1273,7 @@ static TcPool single_pool(const TcPlan& pl, int v) {
   TcPool q;
   q.pool_floats = (int64_t)pl.nslots * g_slot_floats(v, pl.cw);
   q.max_slots = pl.nslots;
+  q.par_slots = std::max<int64_t>(pl.nslots, TC_PAR_SLOTS);
   return q;
 }
 
@@ -1531,6 +1560,7 @@ static TcPool batch_pool(Handle* h, const te_cluster* cs, int64_t n, int mode_p)
   TcPool q;
   q.pool_floats = std::max(biggest, std::min<int64_t>(need, BATCH_POOL_BYTES / 4));
   q.max_slots = 2048;
+  q.par_slots = q.max_slots;
   return q;
 }
 
