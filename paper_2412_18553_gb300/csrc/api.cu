@@ -177,9 +177,11 @@ struct Fp64Plan {
 };
 
 static int fp64_slots(const Handle* h, int64_t v, int64_t ntri) {
-  const int64_t tiles = ((v * v + 63) / 64) * ((v + 63) / 64) * 3;
-  int64_t want = (8LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
-  const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(1536LL << 20) / (24 * v * v * v));
+  // about 32 CTAs per SM and launch (two to four run at a time): the last wave
+  // is then a small part of it; at most 512 MiB of G
+  const int64_t tiles = 3 * gemm_fp64_tiles(v);
+  int64_t want = (32LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
+  const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(512LL << 20) / (24 * v * v * v));
   want = std::min<int64_t>({want, mem_cap, 4096, std::max<int64_t>(1, ntri)});
   return (int)std::max<int64_t>(1, want);
 }

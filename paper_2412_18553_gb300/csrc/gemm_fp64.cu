@@ -17,6 +17,7 @@
 // with t2L[q][x][y][l] = t2[l,q,x,y] and nooT[p][r][z][l] = -ooov[p,l,r,z].
 // Each of the six terms of the permutation operator P appears exactly once in
 // the three G blocks (S1/S2 carry the sum over d, S3/S4 the sum over l).
+#include "dfma_tile.cuh"
 #include "te_internal.h"
 
 namespace te {
@@ -94,19 +95,20 @@ cudaError_t launch_prep_fp64(const te_cluster* c, Prepared* P, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// DFMA GEMM: one CTA = 64 rows (x,y) x 64 columns z of one G block
+// DFMA GEMM: one CTA = 32 RM rows (x,y) x 8 NB columns z of one G block
+// (dfma_tile.cuh).  The float64 units bound it: 12 v^3 (v + o) flops per triple
+// at 1.25 TFLOP/s (3.3 ms).  nocc=8 nvir=40, whole energy: 8.18 ms with 64 x 64 tiles
+// (40 columns on 64, K of 40 and 8 on 48 and 16), 4.01 ms with 128 x 40.
 // ---------------------------------------------------------------------------
 
-constexpr int FT = 64;  // tile edge
-constexpr int FK = 16;  // K chunk
-
-__global__ void __launch_bounds__(256)
+template <int RM, int NB>
+__global__ void __launch_bounds__(DT_THREADS)
 k_gemm_fp64(const double* __restrict__ ovvv, const double* __restrict__ t2,
             const double* __restrict__ t2L, const double* __restrict__ nooT,
             const Triple* __restrict__ triples, int64_t t0, int o, int v,
             double* __restrict__ gbuf) {
-  __shared__ double As[FK][FT + 1];
-  __shared__ double Bs[FK][FT + 1];
+  __shared__ DfmaSmem<RM, NB> S;
+  constexpr int TM = 32 * RM, TN = 8 * NB;
   const int tid = threadIdx.x;
   const int slot = blockIdx.z / 3;
   const int g = blockIdx.z % 3;
@@ -117,88 +119,76 @@ k_gemm_fp64(const double* __restrict__ ovvv, const double* __restrict__ t2,
   else { p = T.k; q = T.i; r = T.j; }
   const int64_t v2 = (int64_t)v * v;
   const int64_t v3 = v2 * v;
-  const int64_t row0 = (int64_t)blockIdx.x * FT;
-  const int col0 = blockIdx.y * FT;
+  const int64_t row0 = (int64_t)blockIdx.x * TM;
+  const int col0 = blockIdx.y * TN;
 
-  // loader coordinates: 64 rows x 16 k, 4 consecutive k per thread
-  const int lrow = tid >> 2;
-  const int lk = (tid & 3) * 4;
-  const int64_t R = row0 + lrow;
-  const bool rvalid = R < v2;
-  const int rx = rvalid ? (int)(R / v) : 0;
-  const int ry = rvalid ? (int)(R % v) : 0;
-  const int zc = col0 + lrow;
-  const bool cvalid = zc < v;
-
-  const int tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  // loader: 16 threads per row take its 16 k; the row's (x, y) stays the same
+  const int lk = tid & 15, lr = tid >> 4;
+  int rx[2 * RM], ry[2 * RM];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int i = 0; i < 2 * RM; ++i) {
+    const int64_t R = row0 + lr + 16 * i;
+    rx[i] = R < v2 ? (int)(R / v) : -1;
+    ry[i] = R < v2 ? (int)(R % v) : 0;
+  }
+  double acc[RM][NB];
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+  for (int a = 0; a < RM; ++a)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[a][b] = 0.0;
 
   for (int seg = 0; seg < 4; ++seg) {
-    const double* Arow;
-    const double* Brow;
+    const bool swap = seg == 1 || seg == 2;  // rows (y, x)
+    const double *A, *B;
     int K;
-    if (seg == 0) {
-      Arow = ovvv + (int64_t)p * v3 + ((int64_t)rx * v + ry) * v;
-      Brow = t2 + ((int64_t)r * o + q) * v2 + (int64_t)zc * v;
-      K = v;
-    } else if (seg == 1) {
-      Arow = ovvv + (int64_t)q * v3 + ((int64_t)ry * v + rx) * v;
-      Brow = t2 + ((int64_t)r * o + p) * v2 + (int64_t)zc * v;
-      K = v;
-    } else if (seg == 2) {
-      Arow = t2L + (int64_t)p * v2 * o + ((int64_t)ry * v + rx) * o;
-      Brow = nooT + ((int64_t)q * o + r) * v * o + (int64_t)zc * o;
-      K = o;
-    } else {
-      Arow = t2L + (int64_t)q * v2 * o + ((int64_t)rx * v + ry) * o;
-      Brow = nooT + ((int64_t)p * o + r) * v * o + (int64_t)zc * o;
-      K = o;
-    }
-    for (int k0 = 0; k0 < K; k0 += FK) {
+    if (seg == 0) { A = ovvv + (int64_t)p * v3; B = t2 + ((int64_t)r * o + q) * v2; K = v; }
+    else if (seg == 1) { A = ovvv + (int64_t)q * v3; B = t2 + ((int64_t)r * o + p) * v2; K = v; }
+    else if (seg == 2) { A = t2L + (int64_t)p * v2 * o; B = nooT + ((int64_t)q * o + r) * v * o; K = o; }
+    else { A = t2L + (int64_t)q * v2 * o; B = nooT + ((int64_t)p * o + r) * v * o; K = o; }
+    for (int k0 = 0; k0 < K; k0 += DT_K) {
+      const int kk = k0 + lk;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int kk = k0 + lk + u;
-        As[lk + u][lrow] = (rvalid && kk < K) ? Arow[kk] : 0.0;
-        Bs[lk + u][lrow] = (cvalid && kk < K) ? Brow[kk] : 0.0;
+      for (int i = 0; i < 2 * RM; ++i) {
+        const int64_t row = swap ? (int64_t)ry[i] * v + rx[i] : (int64_t)rx[i] * v + ry[i];
+        S.a[lk][lr + 16 * i] = (rx[i] >= 0 && kk < K) ? A[row * K + kk] : 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < (TN + 15) / 16; ++i) {
+        const int c = lr + 16 * i;
+        if (c < TN) S.b[lk][c] = (col0 + c < v && kk < K) ? B[(int64_t)(col0 + c) * K + kk] : 0.0;
       }
       __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < FK; ++kk) {
-        double av[4], bv[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) av[a] = As[kk][ty * 4 + a];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx * 4 + b];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-      }
+      dfma_chunk<RM, NB>(S, min(DT_K, K - k0), acc);
       __syncthreads();
     }
   }
   double* out = gbuf + ((int64_t)slot * 3 + g) * v3;
+  const int tx = tid & 7, ty = tid >> 3;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int64_t Ro = row0 + ty * 4 + a;
+  for (int a = 0; a < RM; ++a) {
+    const int64_t Ro = row0 + ty + 32 * a;
     if (Ro >= v2) continue;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int z = col0 + tx * 4 + b;
+    for (int b = 0; b < NB; ++b) {
+      const int z = col0 + tx + 8 * b;
       if (z < v) out[Ro * v + z] = acc[a][b];
     }
   }
 }
 
+int64_t gemm_fp64_tiles(int64_t v) {
+  const DfmaPick t = dfma_pick(v * v, v);
+  return t.tiles_m * t.tiles_n;
+}
+
 cudaError_t launch_gemm_fp64(const Prepared* P, const Triple* d_triples, int64_t t0, int nslots,
                              double* gbuf, cudaStream_t s) {
-  const int64_t v2 = (int64_t)P->v * P->v;
-  dim3 grid((unsigned)((v2 + FT - 1) / FT), (unsigned)((P->v + FT - 1) / FT), (unsigned)(3 * nslots));
-  k_gemm_fp64<<<grid, 256, 0, s>>>(P->ovvv, P->t2, P->t2L, P->nooT, d_triples, t0, P->o, P->v, gbuf);
+  const DfmaPick t = dfma_pick((int64_t)P->v * P->v, P->v);
+  const dim3 grid((unsigned)t.tiles_m, (unsigned)t.tiles_n, (unsigned)(3 * nslots));
+  dfma_dispatch(t, [&](auto rm, auto nb) {
+    k_gemm_fp64<decltype(rm)::value, decltype(nb)::value>
+        <<<grid, DT_THREADS, 0, s>>>(P->ovvv, P->t2, P->t2L, P->nooT, d_triples, t0, P->o, P->v, gbuf);
+  });
   return cudaGetLastError();
 }
 

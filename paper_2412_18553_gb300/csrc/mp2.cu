@@ -350,7 +350,7 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     if (e == cudaSuccess) e = cudaMemsetAsync(ovov, 0, (size_t)ov * ov * 8, s);
     if (!oz) {
       if (e == cudaSuccess)
-        e = gemm_strided(GemmView{c.Bov, c.Bov, ovov, o, v, ov, P, 1, v, 1, ov, 0, ov, 0, 1, v * ov, ov, 1, 1.0},
+        e = gemm_strided(GemmView{c.Bov, c.Bov, ovov, o, v, ov, P, 1, v, 1, ov, 0, ov, 0, 1, v * ov, ov, 1, 1.0, true},
                          h->num_sms, scratch, cap, s, &h->n_launches);
     } else {
       int* ex = reinterpret_cast<int*>(mx + 3);

@@ -121,6 +121,7 @@ struct GemmView {
   int64_t b_k1, b_k2, b_n;
   int64_t c_m1, c_m2, c_n;
   double alpha;
+  bool symmetric = false;  // A and B are the same view and C[m,n] and C[n,m] two elements: half the tiles
 };
 
 // the same over NS BF16 slice planes per operand (slice s at base + s *

@@ -24,6 +24,7 @@
 #include <initializer_list>
 #include <vector>
 
+#include "dfma_tile.cuh"
 #include "strided.h"
 #include "tc_path.h"
 #include "te_internal.h"
@@ -129,90 +130,80 @@ __global__ void __launch_bounds__(256) k_adjoint(AdjArgs A) {
 // ---------------------------------------------------------------------------
 
 
-constexpr int GT = 64, GK = 16;
-
-// (k1, k2) of k = k1 K2 + k2, advanced by GK per step without division
-struct KCursor {
-  int k1, k2;
-  __device__ __forceinline__ void init(int k, int K2) {
-    k1 = k / K2;
-    k2 = k - k1 * K2;
-  }
-  __device__ __forceinline__ void step(int K2) {
-    k2 += GK;
-    while (k2 >= K2) {
-      k2 -= K2;
-      ++k1;
-    }
-  }
-};
-
-__global__ void __launch_bounds__(256) k_gemm_strided(GemmView g, int kchunk, double* __restrict__ part) {
-  __shared__ double As[GK][GT + 1];
-  __shared__ double Bs[GK][GT + 1];
+// One CTA = 32 RM x 8 NB outputs of one K range (dfma_tile.cuh).  a_fast,
+// b_fast: the loader's threads run along k when the view is contiguous there,
+// else along the rows (columns).  With `sym` (the output is symmetric, both
+// operands the same view, no K split) only the tiles that reach m >= n are
+// computed, and each of their elements with m >= n is written at (m, n) and at
+// (n, m): a product of the same two factors in the same K order, so the
+// mirrored bits are those the other half would have had.  The float64 units
+// bound every launch; eight clusters' MP2 step (nocc 8 .. 20, nvir = 8 nocc,
+// three contractions each): 56.1 ms with 64 x 64 tiles and both halves of
+// (ia|jb), 29.1 ms now.
+template <int RM, int NB>
+__global__ void __launch_bounds__(DT_THREADS) k_gemm_strided(const __grid_constant__ GemmView g, int kchunk,
+                                                             double* __restrict__ part, int a_fast, int b_fast,
+                                                             int sym) {
+  constexpr int TM = 32 * RM, TN = 8 * NB;
+  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
+  if (sym && m0 + TM <= n0) return;
+  __shared__ DfmaSmem<RM, NB> S;
   const int tid = threadIdx.x;
-  const int M = (int)(g.M1 * g.M2), K = (int)(g.K1 * g.K2), K2 = (int)g.K2;
-  const int m0 = blockIdx.x * GT, n0 = blockIdx.y * GT;
+  const int M = (int)(g.M1 * g.M2), N = (int)g.N, K = (int)(g.K1 * g.K2), K2 = (int)g.K2, M2 = (int)g.M2;
   const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-  const int tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  double acc[RM][NB];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < RM; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  // loader: 64 rows (m or n) x 16 k; thread (lr, lk .. lk+3)
-  const int lr = tid >> 2, lk = (tid & 3) * 4;
-  const int am = m0 + lr;
-  const bool am_ok = am < M;
-  const int64_t a_row = am_ok ? (int64_t)(am / (int)g.M2) * g.a_m1 + (int64_t)(am % (int)g.M2) * g.a_m2 : 0;
-  const int bn = n0 + lr;
-  const bool bn_ok = bn < (int)g.N;
-  const int64_t b_col = bn_ok ? (int64_t)bn * g.b_n : 0;
-  KCursor cur[4];
+    for (int b = 0; b < NB; ++b) acc[a][b] = 0.0;
+  for (int k0 = kb; k0 < ke; k0 += DT_K) {
 #pragma unroll
-  for (int u = 0; u < 4; ++u) cur[u].init(kb + lk + u, K2);
-  for (int k0 = kb; k0 < ke; k0 += GK) {
+    for (int i = 0; i < 2 * RM; ++i) {
+      const int e = tid + DT_THREADS * i;
+      const int kk = a_fast ? e & 15 : e / TM, r = a_fast ? e >> 4 : e % TM;
+      const int m = m0 + r, k = k0 + kk;
+      double x = 0.0;
+      if (m < M && k < ke) {
+        const int m1 = m / M2, k1 = k / K2;
+        x = g.A[m1 * g.a_m1 + (m - m1 * M2) * g.a_m2 + k1 * g.a_k1 + (k - k1 * K2) * g.a_k2];
+      }
+      S.a[kk][r] = x;
+    }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const bool k_ok = k0 + lk + u < ke;
-      const int64_t ka = (int64_t)cur[u].k1 * g.a_k1 + (int64_t)cur[u].k2 * g.a_k2;
-      const int64_t kbo = (int64_t)cur[u].k1 * g.b_k1 + (int64_t)cur[u].k2 * g.b_k2;
-      As[lk + u][lr] = (am_ok && k_ok) ? g.A[a_row + ka] : 0.0;
-      Bs[lk + u][lr] = (bn_ok && k_ok) ? g.B[b_col + kbo] : 0.0;
-      cur[u].step(K2);
+    for (int i = 0; i < (TN * DT_K + DT_THREADS - 1) / DT_THREADS; ++i) {
+      const int e = tid + DT_THREADS * i;
+      if (e >= TN * DT_K) break;
+      const int kk = b_fast ? e & 15 : e / TN, c = b_fast ? e >> 4 : e % TN;
+      const int n = n0 + c, k = k0 + kk;
+      double x = 0.0;
+      if (n < N && k < ke) {
+        const int k1 = k / K2;
+        x = g.B[n * g.b_n + k1 * g.b_k1 + (k - k1 * K2) * g.b_k2];
+      }
+      S.b[kk][c] = x;
     }
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[kk][ty * 4 + a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx * 4 + b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-    }
+    dfma_chunk<RM, NB>(S, min(DT_K, ke - k0), acc);
     __syncthreads();
   }
+  const int tx = tid & 7, ty = tid >> 3;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int m = m0 + ty * 4 + a;
+  for (int a = 0; a < RM; ++a) {
+    const int m = m0 + ty + 32 * a;
     if (m >= M) continue;
-    if (part) {  // split K: this split's tile, row-major [M][N]
-      double* prow = part + ((int64_t)blockIdx.z * M + m) * g.N;
+    const int64_t crow = (int64_t)(m / M2) * g.c_m1 + (int64_t)(m % M2) * g.c_m2;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int n = n0 + tx * 4 + b;
-        if (n < g.N) prow[n] = acc[a][b];
-      }
-    } else {
-      const int64_t crow = (int64_t)(m / (int)g.M2) * g.c_m1 + (int64_t)(m % (int)g.M2) * g.c_m2;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int n = n0 + tx * 4 + b;
-        if (n < g.N) g.C[crow + n * g.c_n] += g.alpha * acc[a][b];
+    for (int b = 0; b < NB; ++b) {
+      const int n = n0 + tx + 8 * b;
+      if (n >= N) continue;
+      if (part) {  // split K: this split's tile, row-major [M][N]
+        part[((int64_t)blockIdx.z * M + m) * N + n] = acc[a][b];
+      } else if (!sym) {
+        g.C[crow + n * g.c_n] += g.alpha * acc[a][b];
+      } else if (m >= n) {
+        const double x = g.alpha * acc[a][b];
+        g.C[crow + n * g.c_n] += x;
+        if (m > n) g.C[(int64_t)(n / M2) * g.c_m1 + (int64_t)(n % M2) * g.c_m2 + m * g.c_n] += x;
       }
     }
   }
@@ -236,7 +227,7 @@ __global__ void k_splitk_add(GemmView g, int nsplit, const double* __restrict__ 
 // blocks per SM, each split at least 8 K steps; the scratch holds `cap`
 // doubles.
 static int num_splits(int64_t tiles, int64_t K, int64_t MN, int num_sms, int64_t cap) {
-  const int64_t steps = (K + GK - 1) / GK;
+  const int64_t steps = (K + DT_K - 1) / DT_K;
   int64_t want = (2LL * num_sms + tiles - 1) / tiles;
   want = std::min<int64_t>(want, std::max<int64_t>(1, steps / 8));
   want = std::min<int64_t>(want, std::max<int64_t>(1, cap / std::max<int64_t>(1, MN)));
@@ -246,13 +237,19 @@ static int num_splits(int64_t tiles, int64_t K, int64_t MN, int num_sms, int64_t
 cudaError_t gemm_strided(const GemmView& g, int num_sms, double* scratch, int64_t scratch_cap, cudaStream_t s,
                          int64_t* launches) {
   const int64_t M = g.M1 * g.M2, K = g.K1 * g.K2;
-  const int64_t tm = (M + GT - 1) / GT, tn = (g.N + GT - 1) / GT;
-  const int ns = num_splits(tm * tn, K, M * g.N, num_sms, scratch_cap);
-  const int64_t steps = (K + GK - 1) / GK;
-  const int kchunk = (int)(((steps + ns - 1) / ns) * GK);
+  const DfmaPick t = dfma_pick(M, g.N);
+  const int ns = num_splits(t.tiles_m * t.tiles_n, K, M * g.N, num_sms, scratch_cap);
+  const int64_t steps = (K + DT_K - 1) / DT_K;
+  const int kchunk = (int)(((steps + ns - 1) / ns) * DT_K);
   const int nsplit = (int)((K + kchunk - 1) / kchunk);
-  dim3 grid((unsigned)tm, (unsigned)tn, (unsigned)nsplit);
-  k_gemm_strided<<<grid, 256, 0, s>>>(g, kchunk, nsplit > 1 ? scratch : nullptr);
+  const dim3 grid((unsigned)t.tiles_m, (unsigned)t.tiles_n, (unsigned)nsplit);
+  const bool a_fast = (g.K2 > 1 ? g.a_k2 : g.a_k1) == 1, b_fast = (g.K2 > 1 ? g.b_k2 : g.b_k1) == 1;
+  const int sym = g.symmetric && nsplit == 1 ? 1 : 0;
+  double* part = nsplit > 1 ? scratch : nullptr;
+  dfma_dispatch(t, [&](auto rm, auto nb) {
+    k_gemm_strided<decltype(rm)::value, decltype(nb)::value>
+        <<<grid, DT_THREADS, 0, s>>>(g, kchunk, part, a_fast ? 1 : 0, b_fast ? 1 : 0, sym);
+  });
   ++*launches;
   if (nsplit > 1) {
     const int64_t MN = M * g.N;
