@@ -5,20 +5,25 @@
 // item's 18 G cubes (3 G blocks x 6 block orders) are contiguous and arrive
 // by one bulk copy; the 18 8x8 blocks of the symmetrised ovov the item uses
 // and 9 t1 rows come by TMA (few, large copies: the copy engine's per-copy
-// cost, not HBM, limited a layout that needed 54 copies per item).  A
-// producer warp issues the loads into a double buffer; one thread per
-// orbit candidate (a,b,c) of the 8^3 block triple.  G is either FP32 (BF16X3/TF32/TF32X3) or an FP32 pair
-// hi + lo (OZAKI), CW = 1 or 2 floats per element.
+// cost, not HBM, limited a layout that needed 54 copies per item).  A ring of
+// two to four buffers has a producer warp each: an item's decode, its loads of
+// the triple and the orbital energies and its float64 table are one chain of
+// some thousand cycles, which a single producer could not keep ahead of the
+// sixteen compute warps.  One thread per orbit candidate (a,b,c) of the 8^3
+// block triple.
 //
-// Orbit sum without cancellation: the 6x6 coefficient matrix C of R between
-// the six orbit positions (T = sum_nm W_n C_nm V_m) has zero row and column
-// sums, so T is unchanged when W_0 and V_0 are subtracted from every
-// position.  The deviations w_n = W_n - W_0 are formed G block by G block
-// (differences of close FP32 numbers are nearly exact), so the symmetric
-// part of W~, which R annihilates, never enters a rounded product.
-//   T = 3 sum_n w_n v_n + Ae Se + Ao So - 2 (Ae So + Ao Se)
-// D, its reciprocal (FP32 seed + one Newton step in FP64: error ~1e-14),
-// A T / D and the sums are FP64.
+// Orbit sum.  R's coefficient pattern between the six orbit positions has zero
+// row and column sums, so only differences of W~ enter, and the symmetric part
+// of W~, which R annihilates, never enters a rounded product.  With the even
+// positions e = (0, 3, 4), the odd ones o = (1, 2, 5), d1 = w_e0 - w_e1,
+// d2 = w_e1 - w_e2 (o alike), d' the same of V = W~ + Y, and X, X' the sums over
+// the even positions less those over the odd ones:
+//   T = sum_{e,o} [d1 (2 d1' + d2') + d2 (d1' + 2 d2')] + 2 X X',
+// five products (the form 3 sum w v + Ae Se + Ao So - 2 (Ae So + Ao Se) over the
+// deviations from position 0 takes nine).  W~, the differences and the products
+// are FP32 pairs whose high parts are summed without error (two-sum,
+// two-product) and whose low parts collect the rest.  D, its reciprocal (FP32
+// seed + one Newton step in FP64: error ~1e-14), A T / D and the sums are FP64.
 #include <cstring>
 
 #include "energy_tc.h"
@@ -30,18 +35,25 @@ namespace {
 
 constexpr int TB = 8;
 constexpr int WARPS = 16;                 // compute warps: one orbit candidate (a,b,c) of 8^3 per thread
-constexpr int THREADS = (WARPS + 1) * 32;  // + one producer warp
 
-template <int CW>
+template <int FMT>
 struct Layout {
-  static constexpr uint32_t cube_bytes = TB * TB * TB * 4 * CW;
+  static constexpr uint32_t cube_bytes = g_cube_floats(FMT) * 4;
   static constexpr uint32_t cubes = 18 * cube_bytes;
   static constexpr uint32_t ovs = 27 * TB * TB * 4;
   static constexpr uint32_t t1 = 9 * 128;
   static constexpr uint32_t eps = 640;  // dAB[64] = e_ijk - e_a - e_b, epsC[8] (FP64, written by the producer)
   static constexpr uint32_t buf = cubes + ovs + t1 + eps;
+  // A consumer holds a buffer for most of an item's arithmetic, and a copy
+  // takes about as long: two buffers left the warps waiting for half the time
+  // at nvir = 320.  As many as 227 KB hold, at most four.
+  static constexpr int nbuf = FMT == G_F32 ? 4 : (FMT == G_PAIR ? 2 : 3);
   static constexpr uint32_t tx = 18 * cube_bytes + 18 * TB * TB * 4 + 9 * TB * 4;
+  static constexpr size_t smem = (size_t)nbuf * buf + 128 + 512;
+  static constexpr int threads = (WARPS + nbuf) * 32;  // one producer warp per buffer
 };
+static_assert(Layout<G_F32>::smem <= 227 * 1024 && Layout<G_PAIR>::smem <= 227 * 1024 &&
+                  Layout<G_MIXED>::smem <= 227 * 1024, "shared memory of one block");
 
 __device__ __forceinline__ void decode_bt(int64_t bt, int* blk) {
   // bt = X(X+1)(X+2)/6 + Y(Y+1)/2 + Z, X >= Y >= Z >= 0 (FP32 estimate, exact integer fix-up)
@@ -57,16 +69,30 @@ __device__ __forceinline__ void decode_bt(int64_t bt, int* blk) {
   blk[2] = (int)(rem - (int64_t)y * (y + 1) / 2);
 }
 
-// ---- double-float (pair of FP32) arithmetic: error-free transformations ----
-// Knuth two-sum, FMA two-product; the rn intrinsics forbid contraction.
+// ---- pairs of FP32 (value h + l): error-free transformations ----
+// Knuth two-sum, FMA two-product; the rn intrinsics forbid contraction.  The
+// pairs are not renormalised: l stays a small correction of what was summed
+// into h, and a difference whose h cancels keeps its l.
 struct df {
   float h, l;
 };
 
-__device__ __forceinline__ df df_two_sum(float a, float b) {
+__device__ __forceinline__ df two_sum(float a, float b) {
   const float s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);
   return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+
+__device__ __forceinline__ df df_add(df a, df b) {
+  const df s = two_sum(a.h, b.h);
+  return {s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+
+__device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df{-b.h, -b.l}); }
+
+__device__ __forceinline__ df df_addf(df a, float b) {
+  const df s = two_sum(a.h, b);
+  return {s.h, __fadd_rn(s.l, a.l)};
 }
 
 __device__ __forceinline__ df df_norm(float h, float l) {
@@ -74,21 +100,54 @@ __device__ __forceinline__ df df_norm(float h, float l) {
   return {s, __fsub_rn(l, __fsub_rn(s, h))};
 }
 
-__device__ __forceinline__ df df_add(df a, df b) {
-  const df s = df_two_sum(a.h, b.h);
-  return df_norm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-
-__device__ __forceinline__ df df_mul(df a, df b) {
+// acc += a b
+__device__ __forceinline__ void df_fma(df& acc, df a, df b) {
   const float p = __fmul_rn(a.h, b.h);
-  const float e = fmaf(a.h, b.h, -p);
-  return df_norm(p, __fadd_rn(e, __fadd_rn(__fmul_rn(a.h, b.l), __fmul_rn(a.l, b.h))));
+  float e = fmaf(a.h, b.h, -p);
+  e = fmaf(a.h, b.l, e);
+  e = fmaf(a.l, b.h, e);
+  e = fmaf(a.l, b.l, e);
+  const df s = two_sum(acc.h, p);
+  acc.h = s.h;
+  acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
 }
 
-__device__ __forceinline__ df df_scale(df a, float k) {  // k a small integer
-  const float p = __fmul_rn(a.h, k);
-  const float e = fmaf(a.h, k, -p);
-  return df_norm(p, __fadd_rn(e, __fmul_rn(a.l, k)));
+// 2 a + b and a + 2 b
+__device__ __forceinline__ df df_2ab(df a, df b) { return df_add(df{2.f * a.h, 2.f * a.l}, b); }
+
+// float64 conversions share the two float64 lanes with the arithmetic (64 issue
+// cycles of a scheduler each); the usual range is converted by integer
+// operations instead (same bits).  The rare conversions are volatile so that
+// the compiler does not issue them ahead of their branch.
+__device__ __forceinline__ double cvt_double(float f) {
+  double d;
+  asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
+  return d;
+}
+__device__ __forceinline__ float cvt_float(double d) {
+  float f;
+  asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(d));
+  return f;
+}
+__device__ __forceinline__ double to_double(float f) {
+  const uint32_t u = __float_as_uint(f), m = u & 0x7FFFFFFFu;
+  if (m - 0x00800000u < 0x7F000000u)  // normal
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(m << 29));
+  return cvt_double(f);
+}
+
+// 1/D to ~1e-14: FP32 seed of D rounded to nearest, one Newton step
+__device__ __forceinline__ double recip(double D) {
+  const uint32_t h = (uint32_t)__double2hiint(D), m = h & 0x7FFFFFFFu;
+  double r0;
+  if (m - ((1023u - 100u) << 20) < (200u << 20)) {  // 2^-100 <= |D| < 2^100
+    const unsigned long long b = (((unsigned long long)m << 32) | (uint32_t)__double2loint(D)) + (1ull << 28);
+    const float f = __frcp_rn(__uint_as_float((h & 0x80000000u) | ((uint32_t)(b >> 29) - (896u << 23))));
+    r0 = to_double(f);
+  } else {
+    r0 = cvt_double(__frcp_rn(cvt_float(D)));
+  }
+  return fma(r0, fma(-D, r0, 1.0), r0);
 }
 
 struct EnergyMaps {
@@ -100,7 +159,7 @@ struct EnergyParams {
   int ncl, npieces;
   int64_t items;
   EnergyCl cl[TC_MAX_CL];
-  TcPiece pc[TC_MAX_PIECES];  // G: orbit-major [slot][bt][g][pid][CW planes][512, swizzled] from pc.gbuf
+  TcPiece pc[TC_MAX_PIECES];  // G: orbit-major [slot][bt][g][pid][cube] from pc.gbuf
   const Triple* triples;
   double* partials;  // [slot][first item of the block][WARPS]: the warps' sums of a triple's items
   unsigned int* err;
@@ -144,21 +203,25 @@ __device__ __forceinline__ void cursor_settle(const EnergyParams& P, ItemCursor&
   }
 }
 
-template <int CW>
-__global__ void __launch_bounds__(THREADS, 1)
+// Bound by instruction issue (59% of cycles; float64 pipe and HBM 45% each).
+// nocc=32 nvir=320: 177 us per triple; 272 us with the assembled area, 8-byte G
+// and one producer warp, 240 us with one producer for three buffers.
+template <int FMT>
+__global__ void __launch_bounds__(Layout<FMT>::threads, 1)
     k_energy_tc(const __grid_constant__ EnergyMaps M, const __grid_constant__ EnergyParams P) {
-  using L = Layout<CW>;
+  using L = Layout<FMT>;
+  constexpr int NB = L::nbuf, CUBE = g_cube_floats(FMT);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                          ~uintptr_t(127));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + 2 * L::buf);    // [2]
-  uint64_t* empty = full + 2;                                         // [2], one arrival per compute warp
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + 2);
-  int* meta = const_cast<int*>(reinterpret_cast<volatile int*>(abort_flag) + 1);  // [2][8]: X, Y, Z, slot, v, item
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + NB * L::buf);  // [NB]
+  uint64_t* empty = full + NB;                                       // [NB], one arrival per compute warp
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + NB);
+  int* meta = const_cast<int*>(reinterpret_cast<volatile int*>(abort_flag) + 1);  // [NB][8]: X, Y, Z, slot, v
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < NB; ++q) {
       ptx::mbar_init(&full[q], 2);  // the copies' arrive.expect_tx and the denominator table's arrive
       ptx::mbar_init(&empty[q], WARPS);
     }
@@ -167,17 +230,32 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
   __syncthreads();
 
-  if (warp == WARPS) {
-    // ---------------- producer warp ----------------
-    uint32_t ephase = 0u, pending = 0u, fphase = 0u;  // one bit per buffer
-    int b = 0;
-    bool ok = true;
+  if (warp >= WARPS) {
+    // ---------------- producer warps: buffer b = every NB-th item ----------------
+    const int b = warp - WARPS;
+    uint32_t ph = 0u;  // parity of the ring's current turn
+    int at = 0;        // buffer of the cursor's item
+    bool ok = true, issued = false;
     ItemCursor cur{0, 0, -1, -1};
     cursor_settle(P, cur);
-    for (; ok && cur.q < P.npieces; cur.bt += gridDim.x, cursor_settle(P, cur), b ^= 1) {
+    for (; ok && cur.q < P.npieces; cur.bt += gridDim.x, cursor_settle(P, cur), at = at + 1 == NB ? 0 : at + 1) {
+      if (at != b) continue;
+      const TcPiece& pc = P.pc[cur.q];
+      const EnergyCl& C = P.cl[pc.cl];
+      const int slot = cur.ls;
+      const int64_t bt = cur.bt;
+      const int64_t local = (int64_t)slot * C.nbt + bt;
+      int blk[3];
+      decode_bt(bt, blk);
+      // the loads that the item's table needs, before the wait for its buffer:
+      // the 24 virtual energies of the three blocks, one per lane
+      const Triple tr = P.triples[pc.t0 + slot];
+      const int lq = lane < 24 ? blk[lane >> 3] * TB + (lane & 7) : 0;
+      const double ev = (lane < 24 && lq < C.v) ? C.eps_v[lq] : 0.0;
+      const double eo = C.eps_o[tr.i] + C.eps_o[tr.j] + C.eps_o[tr.k];
       // buffer b free: all compute warps done with the item it held
       int good = 1;
-      if (lane == 0) good = ptx::mbar_wait(&empty[b], ((ephase >> b) & 1u) ^ 1u, P.wait_ns) ? 1 : 0;
+      if (lane == 0) good = ptx::mbar_wait(&empty[b], ph ^ 1u, P.wait_ns) ? 1 : 0;
       good = __shfl_sync(0xffffffffu, good, 0);
       if (!good || *abort_flag) {
         if (lane == 0 && !*abort_flag) {
@@ -190,15 +268,6 @@ __global__ void __launch_bounds__(THREADS, 1)
         ok = false;
         break;
       }
-      ephase ^= 1u << b;
-      const TcPiece& pc = P.pc[cur.q];
-      const EnergyCl& C = P.cl[pc.cl];
-      const int slot = cur.ls;
-      const int64_t bt = cur.bt;
-      const int64_t local = (int64_t)slot * C.nbt + bt;
-      int blk[3];
-      decode_bt(bt, blk);
-      const Triple tr = P.triples[pc.t0 + slot];
       unsigned char* base = smem + (size_t)b * L::buf;
       if (lane == 0) {
         meta[b * 8 + 0] = blk[0];
@@ -207,34 +276,28 @@ __global__ void __launch_bounds__(THREADS, 1)
         meta[b * 8 + 3] = pc.slot0 + slot;
         meta[b * 8 + 4] = C.v;
         ptx::mbar_arrive_expect_tx(&full[b], L::tx);  // first of the two arrivals
-        pending |= 1u << b;
       }
       __syncwarp();
       const CUtensorMap* map_ovs = &M.ovs[pc.cl];
       const CUtensorMap* map_t1 = &M.t1[pc.cl];
-      for (int q = lane; q < 28; q += 32) {
-        if (q == 0) {  // the item's 18 cubes, contiguous ([g][pid] as in shared memory)
-          ptx::bulk_load(base, pc.gbuf + local * (18 * TB * TB * TB * CW), 18 * L::cube_bytes, &full[b]);
-        } else if (q < 19) {
-          // ovs block (pair, sx, sy) with sx != sy: the only ones a permutation's Y reads
-          const int rr = q - 1, pair = rr / 6, od = rr % 6;
-          const int sx = od >> 1, sy = (od == 0) ? 1 : (od == 1) ? 2 : (od == 2) ? 0 : (od == 3) ? 2 : (od == 4) ? 0 : 1;
-          const int r = pair * 9 + sx * 3 + sy;
-          const int P1 = (pair == 1) ? tr.j : tr.i;
-          const int P2 = (pair == 0) ? tr.j : tr.k;
-          ptx::tma_load_4d(base + L::cubes + r * 256, map_ovs, &full[b], blk[sy] * TB, P2, blk[sx] * TB, P1);
-        } else {
-          const int r = q - 19, which = r / 3, s2 = r % 3;
-          const int occ = which == 0 ? tr.i : (which == 1 ? tr.j : tr.k);
-          ptx::tma_load_2d(base + L::cubes + L::ovs + r * 128, map_t1, &full[b], blk[s2] * TB, occ);
-        }
+      if (lane == 0) {  // the item's 18 cubes, contiguous ([g][pid] as in shared memory)
+        ptx::bulk_load(base, pc.gbuf + local * (18 * CUBE), 18 * L::cube_bytes, &full[b]);
+      } else if (lane < 19) {
+        // ovs block (pair, sx, sy) with sx != sy: the only ones a permutation's Y reads
+        const int rr = lane - 1, pair = rr / 6, od = rr % 6;
+        const int sx = od >> 1, sy = (od == 0) ? 1 : (od == 1) ? 2 : (od == 2) ? 0 : (od == 3) ? 2 : (od == 4) ? 0 : 1;
+        const int r = pair * 9 + sx * 3 + sy;
+        const int P1 = (pair == 1) ? tr.j : tr.i;
+        const int P2 = (pair == 0) ? tr.j : tr.k;
+        ptx::tma_load_4d(base + L::cubes + r * 256, map_ovs, &full[b], blk[sy] * TB, P2, blk[sx] * TB, P1);
+      } else if (lane < 28) {
+        const int r = lane - 19, which = r / 3, s2 = r % 3;
+        const int occ = which == 0 ? tr.i : (which == 1 ? tr.j : tr.k);
+        ptx::tma_load_2d(base + L::cubes + L::ovs + r * 128, map_t1, &full[b], blk[s2] * TB, occ);
       }
+      __syncwarp();
       {  // FP64 denominator pieces while the copies fly: dAB[la][lb] = e_i+e_j+e_k - e_a - e_b, epsC[lc] = e_c
-        // the 24 virtual energies of the three blocks, one load per lane, shared by shuffles
         double* dAB = reinterpret_cast<double*>(base + L::cubes + L::ovs + L::t1);
-        const int lq = lane < 24 ? blk[lane >> 3] * TB + (lane & 7) : 0;
-        const double ev = (lane < 24 && lq < C.v) ? C.eps_v[lq] : 0.0;
-        const double eo = C.eps_o[tr.i] + C.eps_o[tr.j] + C.eps_o[tr.k];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
           const int q = lane + 32 * r;  // every lane shuffles; lanes with q >= 72 store nothing
@@ -251,12 +314,11 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       __syncwarp();  // every lane's dAB stores are ordered before lane 0's release
       if (lane == 0) ptx::mbar_arrive(&full[b]);  // second arrival
-      fphase ^= 1u << b;
+      issued = true;
+      ph ^= 1u;
     }
-    // partials of the last items once their warps are done; copies in flight land
-    if (lane == 0)
-      for (int q = 0; q < 2; ++q)
-        if (((pending >> q) & 1u) && !ok) ptx::mbar_wait(&full[q], ((fphase >> q) & 1u) ^ 1u, P.wait_ns);
+    // copies in flight land before the block ends: on an abort the consumers no longer wait for them
+    if (lane == 0 && !ok && issued) ptx::mbar_wait(&full[b], ph ^ 1u, P.wait_ns);
   } else {
     // ---------------- compute warps ----------------
     // A thread takes the orbit (a,b,c) = its local point of the block triple.
@@ -267,7 +329,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     // memory first: 24 more stores and 18 more loads per thread, and two
     // block-wide barriers per item.)  The buffer goes back to the producer as
     // soon as the words are in registers.
-    uint32_t phase = 0u;  // one bit per buffer
+    uint32_t ph = 0u;
     int b = 0;
     const int la = (tid >> 6), lb = (tid >> 3) & 7, lc = tid & 7;
     int pos_off[6];
@@ -276,7 +338,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int u = n <= 1 ? la : (n <= 3 ? lb : lc);
       const int w = (n == 0 || n == 5) ? lb : ((n == 1 || n == 3) ? lc : la);
       const int z = (n == 0 || n == 2) ? lc : ((n == 1 || n == 4) ? lb : la);
-      pos_off[n] = n * 512 * CW + cube_off(u, w, z);
+      pos_off[n] = cube_off(u, w, z);
     }
     // this thread's float64 sum over its items of the current triple slot; the
     // warp's sum (fixed shuffle order) goes to the partials when the slot
@@ -292,9 +354,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     };
     ItemCursor cur{0, 0, -1, -1};
     cursor_settle(P, cur);
-    for (; cur.q < P.npieces; cur.bt += gridDim.x, cursor_settle(P, cur), b ^= 1) {
+    for (; cur.q < P.npieces; cur.bt += gridDim.x, cursor_settle(P, cur)) {
       int got = 0;
-      if (!*abort_flag) got = ptx::mbar_wait(&full[b], (phase >> b) & 1u, P.wait_ns) ? 1 : 0;
+      if (!*abort_flag) got = ptx::mbar_wait(&full[b], ph, P.wait_ns) ? 1 : 0;
       if (!__all_sync(0xffffffffu, got)) {
         if (lane == 0 && !*abort_flag) {
           *abort_flag = 1;
@@ -305,7 +367,6 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         break;
       }
-      phase ^= 1u << b;
       const int bx = meta[b * 8 + 0], by = meta[b * 8 + 1], bz = meta[b * 8 + 2], slot = meta[b * 8 + 3];
       const int vcl = meta[b * 8 + 4];
       if (slot != cur_slot) {
@@ -318,12 +379,22 @@ __global__ void __launch_bounds__(THREADS, 1)
       const float* ovsS = reinterpret_cast<const float*>(base + L::cubes);
       const float* t1S = reinterpret_cast<const float*>(base + L::cubes + L::ovs);
       const double* dAB = reinterpret_cast<const double*>(base + L::cubes + L::ovs + L::t1);
-      const double D = dAB[la * 8 + lb] - dAB[64 + lc];
-
       const int a = bx * TB + la, bb = by * TB + lb, c = bz * TB + lc;
       const bool valid = a < vcl && bb < vcl && c < vcl && !(bx == by && la < lb) && !(by == bz && lb < lc);
-      float wh[6], wl[6], y[6];
+      df w[6];
+      float y[6];
+      double D = 0.0;
       if (valid) {
+        D = dAB[la * 8 + lb] - dAB[64 + lc];
+        // plane word(s) of G block g at pid m
+        auto gv = [&](int g, int m) -> df {
+          const float* p = cube + (g * 6 + m) * CUBE;
+          if constexpr (FMT == G_PAIR) return {p[pos_off[m]], p[512 + pos_off[m]]};
+          if constexpr (FMT == G_MIXED)
+            return {p[pos_off[m]],
+                    __uint_as_float((uint32_t)reinterpret_cast<const unsigned short*>(p + 512)[pos_off[m]] << 16)};
+          return {p[pos_off[m]], 0.f};
+        };
         float t1v[3][3];  // [i, j, k][slot of the virtual]
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -340,18 +411,12 @@ __global__ void __launch_bounds__(THREADS, 1)
           const int s2 = 3 - s0 - s1;
           const int x = s0 == 0 ? la : (s0 == 1 ? lb : lc), yy = s1 == 0 ? la : (s1 == 1 ? lb : lc),
                     z = s2 == 0 ? la : (s2 == 1 ? lb : lc);
-          const float* g0 = cube + pos_off[n];
-          const float* g1 = cube + 6 * 512 * CW + pos_off[r1];
-          const float* g2 = cube + 12 * 512 * CW + pos_off[r2];
-          if constexpr (CW == 2) {
-            df wv = df_two_sum(g0[0], g1[0]);
-            wv = df_add(wv, df{g2[0], 0.f});
-            wv = df_norm(wv.h, __fadd_rn(wv.l, __fadd_rn(__fadd_rn(g0[512], g1[512]), g2[512])));
-            wh[n] = wv.h;
-            wl[n] = wv.l;
+          const df g0 = gv(0, n), g1 = gv(1, r1), g2 = gv(2, r2);
+          if constexpr (FMT == G_F32) {
+            w[n] = df{(g0.h + g1.h) + g2.h, 0.f};
           } else {
-            wh[n] = (g0[0] + g1[0]) + g2[0];
-            wl[n] = 0.f;
+            const df s = two_sum(g0.h, g1.h), s3 = two_sum(s.h, g2.h);
+            w[n] = df{s3.h, __fadd_rn(__fadd_rn(s.l, s3.l), __fadd_rn(__fadd_rn(g0.l, g1.l), g2.l))};
           }
           // Y at (x, y, z) = positions (s0, s1, s2):
           //   ovs(i,x,j,y) t1(k,z) + ovs(j,y,k,z) t1(i,x) + ovs(i,x,k,z) t1(j,y)
@@ -362,45 +427,47 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&empty[b]);  // this warp no longer reads buffer b
+      if (++b == NB) {
+        b = 0;
+        ph ^= 1u;
+      }
       if (valid) {
         // orbit weight A (Eq. E_corr_CCSD_T): 1, 1/2 or 1/6
         const bool all3 = (a == bb && bb == c), two = (a == bb || bb == c);
-        const double r0 = (double)__frcp_rn((float)D);
-        const double r1 = fma(r0, fma(-D, r0, 1.0), r0);  // 1/D to ~1e-14 (one Newton step)
-        if constexpr (CW == 2) {
-          df wd[5], vd[5];
-#pragma unroll
-          for (int n = 1; n < 6; ++n) {
-            df d = df_two_sum(wh[n], -wh[0]);
-            d = df_norm(d.h, __fadd_rn(d.l, __fsub_rn(wl[n], wl[0])));
-            wd[n - 1] = d;
-            vd[n - 1] = df_add(d, df{__fsub_rn(y[n], y[0]), 0.f});
+        const double r1 = recip(D);
+        if constexpr (FMT != G_F32) {
+          // differences of W~ within the even (0, 3, 4) and odd (1, 2, 5) positions, and even less odd
+          const df e1 = df_sub(w[0], w[3]), e2 = df_sub(w[3], w[4]);
+          const df o1 = df_sub(w[1], w[2]), o2 = df_sub(w[2], w[5]);
+          const df X = df_add(df_add(df_sub(w[0], w[1]), df_sub(w[3], w[2])), df_sub(w[4], w[5]));
+          // the same of V = W~ + Y
+          const df fe1 = df_addf(e1, __fsub_rn(y[0], y[3])), fe2 = df_addf(e2, __fsub_rn(y[3], y[4]));
+          const df fo1 = df_addf(o1, __fsub_rn(y[1], y[2])), fo2 = df_addf(o2, __fsub_rn(y[2], y[5]));
+          const df S = df_addf(df_addf(df_addf(X, __fsub_rn(y[0], y[1])), __fsub_rn(y[3], y[2])), __fsub_rn(y[4], y[5]));
+          df t{0.f, 0.f};
+          df_fma(t, X, df{2.f * S.h, 2.f * S.l});
+          df_fma(t, e1, df_2ab(fe1, fe2));
+          df_fma(t, e2, df_2ab(fe2, fe1));
+          df_fma(t, o1, df_2ab(fo1, fo2));
+          df_fma(t, o2, df_2ab(fo2, fo1));
+          df T = df_norm(t.h, t.l);
+          if (two) {
+            const float k = all3 ? 0.16666667f : 0.5f, kl = all3 ? -4.967054e-09f : 0.f;  // 1/6 as a float pair
+            const float p = __fmul_rn(T.h, k);
+            T = df_norm(p, fmaf(T.l, k, fmaf(T.h, kl, fmaf(T.h, k, -p))));
           }
-          const df w1 = wd[0], w2 = wd[1], w3 = wd[2], w4 = wd[3], w5 = wd[4];
-          const df v1 = vd[0], v2 = vd[1], v3 = vd[2], v4 = vd[3], v5 = vd[4];
-          const df Ae = df_add(w3, w4), Ao = df_add(df_add(w1, w2), w5);
-          const df Se = df_add(v3, v4), So = df_add(df_add(v1, v2), v5);
-          df dot = df_mul(w1, v1);
-          dot = df_add(dot, df_mul(w2, v2));
-          dot = df_add(dot, df_mul(w3, v3));
-          dot = df_add(dot, df_mul(w4, v4));
-          dot = df_add(dot, df_mul(w5, v5));
-          df T = df_add(df_scale(dot, 3.f), df_add(df_mul(Ae, Se), df_mul(Ao, So)));
-          T = df_add(T, df_scale(df_add(df_mul(Ae, So), df_mul(Ao, Se)), -2.f));
-          if (all3) T = df_mul(T, df{0.16666667f, -4.967054e-09f});  // 1/6 as a float pair
-          else if (two) T = df{T.h * 0.5f, T.l * 0.5f};
-          acc = fma((double)T.h, r1, acc);
-          acc = fma((double)T.l, r1, acc);
+          acc = fma(to_double(T.h), r1, acc);
+          acc = fma(to_double(T.l), r1, acc);
         } else {
-          float w[5], vv[5];
+          float d[5], vv[5];
 #pragma unroll
           for (int n = 1; n < 6; ++n) {
-            w[n - 1] = wh[n] - wh[0];
-            vv[n - 1] = w[n - 1] + (y[n] - y[0]);
+            d[n - 1] = w[n].h - w[0].h;
+            vv[n - 1] = d[n - 1] + (y[n] - y[0]);
           }
-          const float Ae = w[2] + w[3], Ao = w[0] + w[1] + w[4];
+          const float Ae = d[2] + d[3], Ao = d[0] + d[1] + d[4];
           const float Se = vv[2] + vv[3], So = vv[0] + vv[1] + vv[4];
-          const float dot = w[0] * vv[0] + w[1] * vv[1] + w[2] * vv[2] + w[3] * vv[3] + w[4] * vv[4];
+          const float dot = d[0] * vv[0] + d[1] * vv[1] + d[2] * vv[2] + d[3] * vv[3] + d[4] * vv[4];
           const float T = 3.f * dot + Ae * Se + Ao * So - 2.f * (Ae * So + Ao * Se);
           const double Tw = all3 ? (double)T * (1.0 / 6.0) : (double)(two ? 0.5f * T : T);
           acc = fma(Tw, r1, acc);
@@ -419,9 +486,13 @@ int64_t energy_tc_grid(int num_sms, int64_t items) {
   return std::max(1, num_sms);
 }
 
-size_t energy_tc_smem(int cw) {
-  const size_t buf = cw == 2 ? Layout<2>::buf : Layout<1>::buf;
-  return 2 * buf + 128 + 512;
+template <int FMT>
+static cudaError_t launch_fmt(const EnergyMaps& M, const EnergyParams& P, int64_t grid, cudaStream_t s) {
+  constexpr size_t smem = Layout<FMT>::smem;
+  const cudaError_t e = cudaFuncSetAttribute(k_energy_tc<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_energy_tc<FMT><<<(unsigned)grid, Layout<FMT>::threads, smem, s>>>(M, P);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s) {
@@ -442,19 +513,10 @@ cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s) {
   P.partials = e.partials;
   P.err = e.err;
   P.wait_ns = e.wait_ns;
-  const size_t smem = energy_tc_smem(e.cw);
   const int64_t grid = energy_tc_grid(e.num_sms, P.items);
-  cudaError_t err;
-  if (e.cw == 2) {
-    err = cudaFuncSetAttribute(k_energy_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_energy_tc<2><<<(unsigned)grid, THREADS, smem, s>>>(M, P);
-  } else {
-    err = cudaFuncSetAttribute(k_energy_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_energy_tc<1><<<(unsigned)grid, THREADS, smem, s>>>(M, P);
-  }
-  return cudaGetLastError();
+  if (e.fmt == G_MIXED) return launch_fmt<G_MIXED>(M, P, grid, s);
+  if (e.fmt == G_PAIR) return launch_fmt<G_PAIR>(M, P, grid, s);
+  return launch_fmt<G_F32>(M, P, grid, s);
 }
 
 // One block per slot: the partials of the blocks that took items of the triple

@@ -36,7 +36,7 @@ struct EnergyCl {
 };
 
 struct EnergyLaunch {
-  int ncl, npieces, cw, num_sms, nslots;  // nslots: G slots over all pieces
+  int ncl, npieces, fmt, num_sms, nslots;  // fmt: the G format; nslots: G slots over all pieces
   int64_t items;                          // sum over pieces of ns * nbt
   EnergyCl cl[TC_MAX_CL];
   TcPiece pc[TC_MAX_PIECES];
@@ -54,13 +54,21 @@ struct EnergyLaunch {
 cudaError_t launch_reduce_pieces(const double* partials, int grid, const Triple* triples,
                                  const TcPiece* pieces, int npieces, int nslots, cudaStream_t s);
 
+// Element formats of G.  G_F32: one FP32 plane of 512 per cube.  G_PAIR: an
+// FP32 hi plane, then an FP32 lo plane.  G_MIXED: an FP32 hi plane, then 512
+// BF16 lo values; the contraction holds lo in BF16 when it has one accumulator
+// set (|lo| <= ulp(hi) / 2, so the pair keeps 2^-33 of the value), and storing
+// it so loses nothing and cuts G's traffic by a quarter.
+enum GFormat { G_F32 = 1, G_PAIR = 2, G_MIXED = 3 };
+__host__ __device__ constexpr int g_cube_floats(int fmt) { return fmt == G_F32 ? 512 : (fmt == G_PAIR ? 1024 : 768); }
+
 // Layout of one 8x8x8 G cube (shared by the contraction epilogue that writes it
 // and the energy kernel that reads it): element (u, w, z) of a plane sits at
 //   u*64 + (w ^ (u & 3))*8 + (z ^ h),  h = (u & 3) | (((w ^ u) >> 2 & 1) << 2),
 // an XOR swizzle under which every access pattern of the energy kernel (one
 // of the three local indices fixed per warp, the other two spread over 4 x 8
-// threads) touches 32 distinct shared-memory banks.  A cube holds one plane
-// (FP32) or two (hi plane, then lo plane) of 512 floats.
+// threads) touches 32 distinct shared-memory banks (a BF16 plane: two lanes
+// to a bank at most).
 __host__ __device__ __forceinline__ int cube_row(int u, int w) { return u * 64 + (w ^ (u & 3)) * 8; }
 __host__ __device__ __forceinline__ int cube_zx(int u, int w) { return (u & 3) | ((((w ^ u) >> 2) & 1) << 2); }
 __host__ __device__ __forceinline__ int cube_off(int u, int w, int z) { return cube_row(u, w) + (z ^ cube_zx(u, w)); }
@@ -69,7 +77,7 @@ __host__ __device__ __forceinline__ int cube_off(int u, int w, int z) { return c
 // block triple S0 >= S1 >= S2 of 8-wide virtual blocks; it needs, for each of
 // the 3 G blocks g, the cubes at the 6 block orders
 //   pid: (S0,S1,S2) (S0,S2,S1) (S1,S0,S2) (S1,S2,S0) (S2,S0,S1) (S2,S1,S0).
-// They are stored contiguously as [slot][bt][g][pid][CW planes][512], so one
+// They are stored contiguously as [slot][bt][g][pid][cube], so one
 // bulk copy brings an item's 18 cubes.  A cube (X,Y,Z) whose indices repeat
 // serves several orders and is stored once per order.
 __host__ __device__ __forceinline__ int64_t block_triple_index(int s0, int s1, int s2) {
@@ -90,14 +98,13 @@ __host__ __device__ __forceinline__ void orbit_slots(int X, int Y, int Z, int64_
 }
 
 // floats of the G buffer per triple slot
-__host__ __device__ __forceinline__ int64_t g_slot_floats(int v, int cw) {
+__host__ __device__ __forceinline__ int64_t g_slot_floats(int v, int fmt) {
   const int64_t nb = (v + 7) / 8;
-  return nb * (nb + 1) * (nb + 2) / 6 * 18 * 512 * cw;
+  return nb * (nb + 1) * (nb + 2) / 6 * 18 * g_cube_floats(fmt);
 }
 
 constexpr int ENERGY_TC_WARPS = 16;
 int64_t energy_tc_grid(int num_sms, int64_t items);
-size_t energy_tc_smem(int cw);
 cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s);
 
 }  // namespace te

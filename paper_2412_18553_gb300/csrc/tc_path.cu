@@ -164,6 +164,20 @@ __device__ __forceinline__ void xor_permute8(float* v, int h) {
   }
 }
 
+// the same for eight 16-bit values, two per word
+__device__ __forceinline__ uint4 xor_permute8_packed(const uint32_t* v, int h) {
+  uint32_t a = v[0], b = v[1], c = v[2], d = v[3], t;
+  if (h & 1) {
+    a = __byte_perm(a, 0, 0x1032);
+    b = __byte_perm(b, 0, 0x1032);
+    c = __byte_perm(c, 0, 0x1032);
+    d = __byte_perm(d, 0, 0x1032);
+  }
+  if (h & 2) { t = a; a = b; b = t; t = c; c = d; d = t; }
+  if (h & 4) { t = a; a = c; c = t; t = b; b = d; d = t; }
+  return make_uint4(a, b, c, d);
+}
+
 __device__ __forceinline__ void store8(float* dst, const float* v) {
   float4* o4 = reinterpret_cast<float4*>(dst);
   o4[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -414,10 +428,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       const int x = c.x0 + row / C.TB;
       const int y = c.y0 + row % C.TB;
       const bool valid = x < C.v && y < C.v;
-      // orbit-major G: [slot][bt][g][pid][CW planes][512], swizzled rows (see
+      // orbit-major G: [slot][bt][g][pid][cube], swizzled rows (see
       // energy_tc.h); this row is (x, y) = (X*8 + xl, Y*8 + yl)
       const int nb = (C.v + 7) >> 3;
-      constexpr int CWF = is_ozaki(MODE) ? 2 : 1;
+      constexpr int CUBE = g_cube_floats(is_ozaki(MODE) ? G_PAIR : G_F32);  // with two accumulator sets
       float* const gslot = pc.gbuf + (int64_t)c.slot * C.slot_floats;
       const int roff = cube_row(x & 7, y & 7);
       const int zx = cube_zx(x & 7, y & 7);
@@ -477,21 +491,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     int64_t bt;
                     unsigned mask;
                     orbit_slots(x >> 3, y >> 3, Z, &bt, &mask);
-                    float l8[8];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                      const uint32_t w = lp[k][4 * h2 + q];
-                      l8[2 * q] = __uint_as_float(w << 16);
-                      l8[2 * q + 1] = __uint_as_float(w & 0xffff0000u);
-                    }
                     xor_permute8(hv[k] + 8 * h2, zx);
-                    xor_permute8(l8, zx);
-                    float* item = gslot + (bt * 18 + c.g * 6) * (512 * CWF);
+                    const uint4 l8 = xor_permute8_packed(lp[k] + 4 * h2, zx);
+                    constexpr int CUBE_M = g_cube_floats(G_MIXED);
+                    float* item = gslot + (bt * 18 + c.g * 6) * CUBE_M;
                     for (int pid = 0; pid < 6; ++pid) {
                       if (!((mask >> pid) & 1u)) continue;
-                      float* cube = item + pid * (512 * CWF);
+                      float* cube = item + pid * CUBE_M;
                       store8(cube + roff, hv[k] + 8 * h2);
-                      store8(cube + 512 + roff, l8);
+                      *reinterpret_cast<uint4*>(reinterpret_cast<unsigned short*>(cube + 512) + roff) = l8;
                     }
                   }
                 }
@@ -526,10 +534,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 orbit_slots(x >> 3, y >> 3, Z, &bt, &mask);
                 xor_permute8(hv + 8 * h2, zx);
                 xor_permute8(lv + 8 * h2, zx);
-                float* item = gslot + (bt * 18 + c.g * 6) * (512 * CWF);
+                float* item = gslot + (bt * 18 + c.g * 6) * CUBE;
                 for (int pid = 0; pid < 6; ++pid) {
                   if (!((mask >> pid) & 1u)) continue;
-                  float* cube = item + pid * (512 * CWF);
+                  float* cube = item + pid * CUBE;
                   store8(cube + roff, hv + 8 * h2);
                   store8(cube + 512 + roff, lv + 8 * h2);
                 }
@@ -609,7 +617,7 @@ static te_status get_encoder(TcState* st) {
 }
 
 struct TcPlan {
-  int mode, es, nparts, cw;
+  int mode, es, nparts, fmt;  // fmt: G format
   int vp, op, vq;
   int TA, TB, NT, n_mx, n_my, n_nt;
   int kw_chunks, ko_chunks, kw_elems, ko_elems, cbw, cbo;
@@ -630,7 +638,6 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   const bool oz = is_ozaki(mode);
   pl.es = (mode == TC_BF16X3 || oz) ? 2 : 4;
   pl.nparts = mode == TC_TF32 ? 1 : (mode == TC_OZAKI ? 4 : (mode == TC_OZAKI6 ? 5 : 2));
-  pl.cw = oz ? 2 : 1;
   const int nacc = oz ? 3 : 1;
   // TF32/BF16X3 (one accumulator) double-buffer at any N tile; the exact-slice
   // modes (three accumulators) take N tiles up to 160 single-buffered, and
@@ -668,6 +675,7 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   if (force_nnt > 0 && round_up((v + force_nnt - 1) / force_nnt, 16) <= (oz ? 160 : 256)) pl.n_nt = force_nnt;
   pl.NT = round_up((v + pl.n_nt - 1) / pl.n_nt, 16);
   pl.nbuf = (2 * nacc * pl.NT <= 512) ? 2 : 1;
+  pl.fmt = !oz ? G_F32 : (pl.nbuf == 1 ? G_MIXED : G_PAIR);  // as the kernel's epilogues store
   pl.cbw = oz ? 64 : 128;
   pl.kw_elems = pl.cbw / pl.es;
   pl.kw_chunks = (pl.vp + pl.kw_elems - 1) / pl.kw_elems;
@@ -687,7 +695,7 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   pl.ldz = round_up(v, 4);
   const int64_t tiles = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
   int64_t want = (4LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
-  const int64_t per_slot = g_slot_floats(v, pl.cw) * 4;
+  const int64_t per_slot = g_slot_floats(v, pl.fmt) * 4;
   const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(6LL << 30) / per_slot);
   want = std::max<int64_t>(want, 4);  // fewer launches per cluster
   want = std::min<int64_t>({want, mem_cap, 1024, std::max<int64_t>(1, ntri)});
@@ -1100,7 +1108,6 @@ static te_status gemm_params(const Handle* h, const std::vector<TcJob>& jobs, co
 static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float* pool, const TcPool& pq,
                             double* partials, cudaStream_t s) {
   const double nprod = (mode == TC_TF32) ? 1.0 : (mode == TC_OZAKI ? 10.0 : (mode == TC_OZAKI6 ? 15.0 : 3.0));
-  const int cw = is_ozaki(mode) ? 2 : 1;
   size_t j = 0;
   int64_t t = jobs.empty() ? 0 : jobs[0].t_begin;
   std::vector<TcPiece> pcs;
@@ -1192,7 +1199,7 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     std::memset(EL, 0, sizeof(*EL));
     EL->ncl = ncl;
     EL->npieces = (int)pcs.size();
-    EL->cw = cw;
+    EL->fmt = jobs[jl[0]].pl.fmt;  // one TMEM buffering per launch, so one format
     EL->num_sms = h->num_sms;
     EL->nslots = nslots;
     EL->items = items;
@@ -1249,7 +1256,7 @@ static te_status setup_job(Handle* h, TcState* st, const te_cluster* c, int mode
   J->t_begin = t_begin;
   J->t_end = t_end;
   J->nbt = energy_num_block_triples(J->v);
-  J->slot_floats = g_slot_floats(J->v, pl.cw);
+  J->slot_floats = g_slot_floats(J->v, pl.fmt);
   J->tiles_per_triple = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
   tc_carve_cluster(base, pl, J->o, J->v, num_unique_triples(J->o), &J->b);
   J->shares = J->b.etri;
@@ -1271,7 +1278,7 @@ static te_status check_k(int mode, int o, int v) {
 
 static TcPool single_pool(const TcPlan& pl, int v) {
   TcPool q;
-  q.pool_floats = (int64_t)pl.nslots * g_slot_floats(v, pl.cw);
+  q.pool_floats = (int64_t)pl.nslots * g_slot_floats(v, pl.fmt);
   q.max_slots = pl.nslots;
   q.par_slots = std::max<int64_t>(pl.nslots, TC_PAR_SLOTS);
   return q;
@@ -1447,7 +1454,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
     J.o = o;
     J.v = v;
     J.nbt = energy_num_block_triples(v);
-    J.slot_floats = g_slot_floats(v, pl.cw);
+    J.slot_floats = g_slot_floats(v, pl.fmt);
     J.tiles_per_triple = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
     const size_t cbytes = tc_carve_cluster(wbase, pl, o, v, nt, &J.b);
     cudaError_t e = cudaSuccess;
@@ -1548,12 +1555,10 @@ static constexpr int64_t BATCH_POOL_BYTES = int64_t(16) << 30;
 
 static TcPool batch_pool(Handle* h, const te_cluster* cs, int64_t n, int mode_p) {
   int64_t need = 0, biggest = 0;
-  int cw = 1;
   for (int64_t x = 0; x < n; ++x) {
     const int o = (int)cs[x].nocc, v = (int)cs[x].nvir;
     const int mode = tc_mode_of((te_precision)mode_p, o, v, h->ozaki_bits);
-    cw = is_ozaki(mode) ? 2 : 1;
-    const int64_t sf = g_slot_floats(v, cw);
+    const int64_t sf = g_slot_floats(v, make_plan(h, o, v, mode, num_unique_triples(o)).fmt);
     need += num_unique_triples(o) * sf;
     biggest = std::max(biggest, sf);
   }
