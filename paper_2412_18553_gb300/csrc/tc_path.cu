@@ -5,10 +5,26 @@
 // each one GEMM  D[(x,y), z] = sum_K A[(x,y), K] B[z, K]  with four K segments
 //   S1 ovvv[p,x,y,:] . t2[r,q,z,:]     S2 ovvv[q,y,x,:] . t2[r,p,z,:]
 //   S3 t2L[p,y,x,:] . nooT[q,r,z,:]    S4 t2L[q,x,y,:] . nooT[p,r,z,:]
-// run on tcgen05: TMA brings 128-row A tiles (TA values of x times TB of y)
-// and NT-row B tiles into swizzled shared memory; one thread issues
-// tcgen05.mma into FP32 accumulators in tensor memory; four epilogue warps
-// drain TMEM into the G buffer.
+// run on tcgen05 by pairs of CTAs (cta_group::2, the two SMs of a TPC): a pair
+// takes two 128-row A tiles (TA values of x times TB of y each) against one
+// B tile of NT rows, of which each CTA holds half.  TMA brings each CTA's part
+// into its swizzled shared memory; one thread of the pair's first CTA issues
+// the MMAs for both SMs into FP32 accumulators in tensor memory; eight epilogue
+// warps per CTA drain its TMEM into the G buffer.
+//
+// Why pairs, and who issues.  The ten slice products of a K step read their
+// operands from shared memory again each time; in a pair each SM reads its own
+// 128 A rows but only NT / 2 B rows, loads half of B, and four pipeline stages
+// fit instead of three.  That pays only once the issue keeps up: issued from a
+// single-thread branch, an MMA took 75 to 80 cycles whatever its N, because its
+// operands went to uniform registers one by one (see the issuer).  Main loop
+// plus stores of four triples at nvir = 320 (and the whole nocc=24 nvir=240
+// contraction): 3.10 ms (956 ms) lone CTAs and a single issuing thread; 3.10 ms
+// (931 ms) pairs alone; 3.15 ms (856 ms) uniform issue alone; 2.78 ms (711 ms)
+// both, 1.99 PFLOP/s of slice products at nvir = 320.  Tried on top and not
+// kept: a second place for the third accumulator where NT <= 128 leaves TMEM
+// for it (2% slower), sixteen epilogue warps (7% slower: spills), 128-byte
+// operand rows in two stages (7% slower).
 //
 // Operand forms, prepared once per call:
 //  * TF32, BF16X3, TF32X3: x = hi + lo, hi and lo the nearest 11-bit (TF32)
@@ -81,7 +97,7 @@ struct TcMapSet {
 struct TcCl {
   int o, v;
   int TA, TB, NT;
-  int n_mx, n_my, n_nt;
+  int n_my, n_mp, n_nt;    // M tiles along y; pairs of M tiles; N tiles
   int kw_chunks, ko_chunks;
   int kw_elems, ko_elems;  // elements per chunk
   int cbo;                 // chunk bytes of the o-segments (the v-segments use TcParams::cbw)
@@ -98,7 +114,7 @@ struct TcParams {
   uint32_t tmem_cols;
   int nbuf;                // TMEM accumulator sets (1 or 2)
   int nt_max;              // largest N tile: stride of the accumulator sets
-  int64_t total_tiles;
+  int64_t total_tiles;     // pair tiles
   const Triple* triples;
   unsigned int* err;
   unsigned long long wait_ns;
@@ -120,7 +136,16 @@ struct TileCoord {
   int cl, piece, slot, g, p, q, r, x0, y0, z0;
 };
 
-__device__ __forceinline__ TileCoord decode_tile(const TcParams& P, int64_t tt) {
+// the cluster of tile tt
+__device__ __forceinline__ int tile_cluster(const TcParams& P, int64_t tt) {
+  int q = 0;  // pieces are in tile order
+  while (q + 1 < P.npieces && P.pc[q + 1].tile0 <= tt) ++q;
+  return P.pc[q].cl;
+}
+
+// pair tile tt; x0 and y0 are those of CTA `rank`'s M tile (the second tile of an
+// odd last pair lies beyond x < v: its loads fill zeros, its rows are not stored)
+__device__ __forceinline__ TileCoord decode_tile(const TcParams& P, int64_t tt, int rank) {
   TileCoord c;
   int q = 0;  // pieces are in tile order
   while (q + 1 < P.npieces && P.pc[q + 1].tile0 <= tt) ++q;
@@ -129,10 +154,9 @@ __device__ __forceinline__ TileCoord decode_tile(const TcParams& P, int64_t tt) 
   int64_t rest = tt - pc.tile0;
   const int nt = (int)(rest % C.n_nt);
   rest /= C.n_nt;
-  const int my = (int)(rest % C.n_my);
-  rest /= C.n_my;
-  const int mx = (int)(rest % C.n_mx);
-  rest /= C.n_mx;
+  const int m = 2 * (int)(rest % C.n_mp) + rank;
+  rest /= C.n_mp;
+  const int mx = m / C.n_my, my = m - mx * C.n_my;
   c.g = (int)(rest % 3);
   c.slot = (int)(rest / 3);
   c.cl = pc.cl;
@@ -178,10 +202,11 @@ __device__ __forceinline__ uint4 xor_permute8_packed(const uint32_t* v, int h) {
   return make_uint4(a, b, c, d);
 }
 
+// one 32-byte sector in one store (dst 32-byte aligned)
 __device__ __forceinline__ void store8(float* dst, const float* v) {
-  float4* o4 = reinterpret_cast<float4*>(dst);
-  o4[0] = make_float4(v[0], v[1], v[2], v[3]);
-  o4[1] = make_float4(v[4], v[5], v[6], v[7]);
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
 }
 
 // Knuth's two-sum: s + e == a + b exactly
@@ -195,19 +220,17 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // epilogue: warp w drains TMEM lanes 32 (w % 4) .. +31 (the lane quarter its
 // warp index may access) and every (GEMM_EPI_WARPS / 4)-th 16-column chunk,
 // starting at chunk (w - 2) / 4.
-#ifndef TE_GEMM_EPI_WARPS
-#define TE_GEMM_EPI_WARPS 8
-#endif
-constexpr int GEMM_EPI_WARPS = TE_GEMM_EPI_WARPS;
+constexpr int GEMM_EPI_WARPS = 8;
 constexpr int GEMM_EPI_GROUPS = GEMM_EPI_WARPS / 4;
 constexpr int GEMM_THREADS = (2 + GEMM_EPI_WARPS) * 32;
 // 16-column chunks one epilogue warp holds in registers with a single
 // accumulator set (exact-slice N tiles of at most 160 columns)
 constexpr int EPI_CHUNKS = 5;
 constexpr int EPI_NT_MAX = 16 * GEMM_EPI_GROUPS * EPI_CHUNKS;
+constexpr int GEMM_PAIR = 2;  // CTAs per cluster
 
 template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+__global__ void __cluster_dims__(GEMM_PAIR, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
     k_gemm_tc(const __grid_constant__ TcMapSet maps, const __grid_constant__ TcParams P) {
   using MT = ModeTraits<MODE>;
   constexpr bool TF32 = MT::tf32;
@@ -229,6 +252,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  const int rank = (int)ptx::cluster_ctarank();  // rank 0 issues the pair's MMAs
+  const int64_t pair0 = blockIdx.x / GEMM_PAIR, npairs = gridDim.x / GEMM_PAIR;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < P.stages; ++s) {
@@ -237,7 +262,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       ptx::mbar_init(&tfull[a], 1);
-      ptx::mbar_init(&tempty[a], GEMM_EPI_WARPS);
+      ptx::mbar_init(&tempty[a], GEMM_PAIR * GEMM_EPI_WARPS);
     }
     ptx::mbar_init(drain, 1);
     *abort_flag = 0;
@@ -253,11 +278,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     ptx::tma_prefetch_desc(&m.b_noo);
   }
   if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, P.tmem_cols);
-    ptx::tmem_relinquish();
+    ptx::tmem_alloc_pair(tmem_slot, P.tmem_cols);
+    ptx::tmem_relinquish_pair();
   }
   ptx::tc_fence_before();
   __syncthreads();
+  ptx::cluster_sync();  // the barriers of both CTAs are initialised before either is signalled
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const uint32_t acc_stride = (uint32_t)(NACC * P.nt_max);  // TMEM columns between accumulator sets
@@ -269,8 +295,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       int pending[16];
       for (int s = 0; s < 16; ++s) pending[s] = -1;
       bool ok = true;
-      for (int64_t tt = blockIdx.x; ok && tt < P.total_tiles; tt += gridDim.x) {
-        const TileCoord c = decode_tile(P, tt);
+      for (int64_t tt = pair0; ok && tt < P.total_tiles; tt += npairs) {
+        const TileCoord c = decode_tile(P, tt, rank);
         const TcCl& C = P.cl[c.cl];
         const TcMaps& mp = maps.m[c.cl];
         for (int seg = 0; ok && seg < 4; ++seg) {
@@ -278,30 +304,32 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           const int nch = wide ? C.kw_chunks : C.ko_chunks;
           const int cb = wide ? P.cbw : C.cbo;
           const int ce = wide ? C.kw_elems : C.ko_elems;
-          const uint32_t bytes = (uint32_t)NPART * (128u * cb + (uint32_t)C.NT * cb);
+          const uint32_t bytes = (uint32_t)NPART * (2u * 128u * cb + (uint32_t)C.NT * cb);  // both CTAs'
           for (int ch = 0; ch < nch; ++ch) {
             if (*abort_flag || !ptx::mbar_wait(&empty[stage], phase ^ 1u, P.wait_ns)) {
               if (!*abort_flag) record_abort(P, abort_flag, 1);
               ok = false;
               break;
             }
-            ptx::mbar_arrive_expect_tx(&full[stage], bytes);
+            // the pair's bytes all count on rank 0's barrier, whose MMAs wait for them
+            if (rank == 0) ptx::mbar_arrive_expect_tx(&full[stage], bytes);
+            const uint32_t bar = ptx::mapa(&full[stage], 0);
             pending[stage] = (int)phase;
             unsigned char* sa = smem + (size_t)stage * P.stage_bytes;
             unsigned char* sb = sa + NPART * P.a_part_bytes;
-            const int kc = ch * ce;
+            const int kc = ch * ce, zr = c.z0 + rank * (C.NT / 2);
             if (seg == 0) {
-              ptx::tma_load_5d(sa, &mp.a_nat, &full[stage], kc, c.y0, c.x0, 0, c.p);
-              ptx::tma_load_5d(sb, &mp.b_t2, &full[stage], kc, c.z0, 0, c.q, c.r);
+              ptx::tma_load_5d_pair(sa, &mp.a_nat, bar, kc, c.y0, c.x0, 0, c.p);
+              ptx::tma_load_5d_pair(sb, &mp.b_t2, bar, kc, zr, 0, c.q, c.r);
             } else if (seg == 1) {
-              ptx::tma_load_5d(sa, &mp.a_tr, &full[stage], kc, c.y0, c.x0, 0, c.q);
-              ptx::tma_load_5d(sb, &mp.b_t2, &full[stage], kc, c.z0, 0, c.p, c.r);
+              ptx::tma_load_5d_pair(sa, &mp.a_tr, bar, kc, c.y0, c.x0, 0, c.q);
+              ptx::tma_load_5d_pair(sb, &mp.b_t2, bar, kc, zr, 0, c.p, c.r);
             } else if (seg == 2) {
-              ptx::tma_load_5d(sa, &mp.l_tr, &full[stage], kc, c.y0, c.x0, 0, c.p);
-              ptx::tma_load_5d(sb, &mp.b_noo, &full[stage], kc, c.z0, 0, c.r, c.q);
+              ptx::tma_load_5d_pair(sa, &mp.l_tr, bar, kc, c.y0, c.x0, 0, c.p);
+              ptx::tma_load_5d_pair(sb, &mp.b_noo, bar, kc, zr, 0, c.r, c.q);
             } else {
-              ptx::tma_load_5d(sa, &mp.l_nat, &full[stage], kc, c.y0, c.x0, 0, c.q);
-              ptx::tma_load_5d(sb, &mp.b_noo, &full[stage], kc, c.z0, 0, c.r, c.p);
+              ptx::tma_load_5d_pair(sa, &mp.l_nat, bar, kc, c.y0, c.x0, 0, c.q);
+              ptx::tma_load_5d_pair(sb, &mp.b_noo, bar, kc, zr, 0, c.r, c.p);
             }
             if (++stage == (uint32_t)P.stages) {
               stage = 0;
@@ -310,109 +338,120 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
         }
       }
-      // copies still in flight must land before the CTA exits
-      for (int s = 0; s < P.stages; ++s)
-        if (pending[s] >= 0) ptx::mbar_wait(&full[s], (uint32_t)pending[s], P.wait_ns);
+      // Before the pair exits: the MMAs have released every stage (their
+      // signals reach both CTAs), so every copy has landed too.  After an
+      // expired wait they may not come: rank 0 waits for the copies it
+      // expects, and both for longer than a copy takes.
+      for (int s = 0; s < P.stages; ++s) {
+        if (pending[s] < 0) continue;
+        if (ok && !*abort_flag) ptx::mbar_wait(&empty[s], (uint32_t)pending[s], P.wait_ns);
+        else if (rank == 0) ptx::mbar_wait(&full[s], (uint32_t)pending[s], P.wait_ns);
+      }
+      if (!ok || *abort_flag) ptx::pause_ns(200000);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t fmt = TF32 ? 2u : 1u;
-      uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
-      bool ok = true;
-      bool issued = false;
-      for (int64_t tt = blockIdx.x; ok && tt < P.total_tiles; tt += gridDim.x) {
-        const TileCoord c = decode_tile(P, tt);
-        const TcCl& C = P.cl[c.cl];
-        const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(C.NT >> 3) << 17) |
-                               ((uint32_t)(128 >> 4) << 24);
-        if (*abort_flag || !ptx::mbar_wait(&tempty[acc], acc_phase ^ 1u, P.wait_ns)) {
-          if (!*abort_flag) record_abort(P, abort_flag, 2);
-          break;
-        }
-        ptx::tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * acc_stride;
-        uint32_t first = 1;
-        for (int seg = 0; ok && seg < 4; ++seg) {
-          const bool wide = seg < 2;
-          const int nch = wide ? C.kw_chunks : C.ko_chunks;
-          const int cb = wide ? P.cbw : C.cbo;
-          const uint32_t lay = layout_code(cb);
-          const uint32_t sbo = 8u * (uint32_t)cb;
-          for (int ch = 0; ch < nch; ++ch) {
-            if (*abort_flag || !ptx::mbar_wait(&full[stage], phase, P.wait_ns)) {
-              if (!*abort_flag) record_abort(P, abort_flag, 3);
-              ok = false;
-              break;
-            }
-            ptx::tc_fence_after();
-            unsigned char* sa = smem + (size_t)stage * P.stage_bytes;
-            const uint32_t a0 = ptx::smem_u32(sa);
-            const uint32_t b0 = ptx::smem_u32(sa + NPART * P.a_part_bytes);
-            for (int ks = 0; ks < cb / 32; ++ks) {
-              uint64_t ad[NPART], bd[NPART];
+    // ---------------- MMA issuer (rank 0, for both SMs) ----------------
+    // The whole warp runs this loop, its branches decided by votes, and one
+    // elected lane issues: descriptors and addresses are then warp-uniform
+    // values in uniform registers, where tcgen05.mma takes its operands.  In a
+    // single-thread branch they were moved there one by one, 75 to 80 cycles
+    // per MMA whatever its N (64 cycles of tensor work at N = 128).
+    const uint32_t fmt = TF32 ? 2u : 1u;
+    uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
+    bool ok = true;
+    bool issued = false;
+    auto wait_all = [&](uint64_t* bar, uint32_t parity, unsigned site) -> bool {
+      const int got = (!*abort_flag && ptx::mbar_wait(bar, parity, P.wait_ns)) ? 1 : 0;
+      const bool all = __all_sync(0xffffffffu, got);
+      if (!all && lane == 0 && !*abort_flag) record_abort(P, abort_flag, site);
+      return all;
+    };
+    const uint32_t smem0 = ptx::smem_u32(smem);
+    for (int64_t tt = pair0; ok && rank == 0 && tt < P.total_tiles; tt += npairs) {
+      const TcCl& C = P.cl[tile_cluster(P, tt)];
+      const uint32_t NT = (uint32_t)C.NT;
+      const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((NT >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      if (!wait_all(&tempty[acc], acc_phase ^ 1u, 2)) break;
+      ptx::tc_fence_after();
+      const uint32_t d_tmem = tmem_base + acc * acc_stride;
+      uint32_t first = 1;
+      for (int seg = 0; ok && seg < 4; ++seg) {
+        const bool wide = seg < 2;
+        const int nch = wide ? C.kw_chunks : C.ko_chunks;
+        const uint32_t cb = wide ? (uint32_t)P.cbw : (uint32_t)C.cbo;
+        // one box per operand lands the slices back to back: 128 (A) or NT / 2 (B) rows of cb bytes each
+        const uint64_t desc0 = ptx::smem_desc(0, 8u * cb, layout_code((int)cb));
+        const uint32_t astep = (128u * cb) >> 4, bstep = (NT / 2 * cb) >> 4;  // slices, in descriptor units
+        for (int ch = 0; ch < nch; ++ch) {
+          if (!wait_all(&full[stage], phase, 3)) {
+            ok = false;
+            break;
+          }
+          ptx::tc_fence_after();
+          const uint32_t a0 = (smem0 + stage * P.stage_bytes) >> 4;
+          const uint32_t b0 = a0 + ((NPART * P.a_part_bytes) >> 4);
+          for (uint32_t ks = 0; ks < cb / 32; ++ks) {
+            uint64_t ad[NPART], bd[NPART];
 #pragma unroll
-              for (int k = 0; k < NPART; ++k) {
-                // one box per operand lands the slices back to back: 128 (A) or NT (B) rows of cb bytes each
-                ad[k] = ptx::smem_desc(a0 + k * (128u * (uint32_t)cb) + ks * 32, sbo, lay);
-                bd[k] = ptx::smem_desc(b0 + k * ((uint32_t)C.NT * (uint32_t)cb) + ks * 32, sbo, lay);
-              }
-              const uint32_t acc_in = first ? 0u : 1u;
+            for (int k = 0; k < NPART; ++k) {
+              ad[k] = desc0 + (a0 + k * astep + ks * 2);
+              bd[k] = desc0 + (b0 + k * bstep + ks * 2);
+            }
+            const uint32_t acc_in = first ? 0u : 1u;
+            if (ptx::elect_one()) {
               if constexpr (is_ozaki(MODE)) {
                 // slice products a_i b_j with i + j <= NPART - 1: level i + j = 0 and
                 // level 1 each in an exact accumulator, the higher levels in a third
-                const uint32_t d2 = d_tmem, d3 = d_tmem + C.NT, dr = d_tmem + 2 * C.NT;
-                ptx::mma<false>(d2, ad[0], bd[0], idesc, acc_in);
-                ptx::mma<false>(d3, ad[0], bd[1], idesc, acc_in);
-                ptx::mma<false>(d3, ad[1], bd[0], idesc, 1);
-                uint32_t rin = acc_in;
+                const uint32_t d2 = d_tmem, d3 = d_tmem + NT, dr = d_tmem + 2 * NT;
+                ptx::mma_pair<false>(d2, ad[0], bd[0], idesc, acc_in);
+                ptx::mma_pair<false>(d3, ad[0], bd[1], idesc, acc_in);
+                ptx::mma_acc_pair<false>(d3, ad[1], bd[0], idesc);
+                ptx::mma_pair<false>(dr, ad[0], bd[2], idesc, acc_in);
 #pragma unroll
                 for (int lev = 2; lev < NPART; ++lev)
 #pragma unroll
-                  for (int i = 0; i <= lev; ++i) {
-                    ptx::mma<false>(dr, ad[i], bd[lev - i], idesc, rin);
-                    rin = 1;
-                  }
+                  for (int i = lev == 2 ? 1 : 0; i <= lev; ++i) ptx::mma_acc_pair<false>(dr, ad[i], bd[lev - i], idesc);
               } else {
-                ptx::mma<TF32>(d_tmem, ad[0], bd[0], idesc, acc_in);
+                ptx::mma_pair<TF32>(d_tmem, ad[0], bd[0], idesc, acc_in);
                 if constexpr (NPART == 2) {
-                  ptx::mma<TF32>(d_tmem, ad[0], bd[1], idesc, 1);
-                  ptx::mma<TF32>(d_tmem, ad[1], bd[0], idesc, 1);
+                  ptx::mma_acc_pair<TF32>(d_tmem, ad[0], bd[1], idesc);
+                  ptx::mma_acc_pair<TF32>(d_tmem, ad[1], bd[0], idesc);
                 }
               }
-              first = 0;
             }
-            issued = true;
-            ptx::mma_commit(&empty[stage]);
-            if (++stage == (uint32_t)P.stages) {
-              stage = 0;
-              phase ^= 1u;
-            }
+            first = 0;
+          }
+          issued = true;
+          if (ptx::elect_one()) ptx::mma_commit_pair(&empty[stage]);
+          if (++stage == (uint32_t)P.stages) {
+            stage = 0;
+            phase ^= 1u;
           }
         }
-        if (!ok) break;
-        ptx::mma_commit(&tfull[acc]);
-        if (NBUF == 2) {
-          acc ^= 1u;
-          if (acc == 0) acc_phase ^= 1u;
-        } else {
-          acc_phase ^= 1u;
-        }
       }
-      // every issued MMA completes before TMEM is released
-      if (issued) {
-        ptx::mma_commit(drain);
-        ptx::mbar_wait(drain, 0, P.wait_ns);
+      if (!ok) break;
+      if (ptx::elect_one()) ptx::mma_commit_pair(&tfull[acc]);
+      if (NBUF == 2) {
+        acc ^= 1u;
+        if (acc == 0) acc_phase ^= 1u;
+      } else {
+        acc_phase ^= 1u;
       }
     }
+    // every issued MMA completes before TMEM is released
+    if (issued) {
+      if (ptx::elect_one()) ptx::mma_commit_pair_own(drain);
+      ptx::mbar_wait(drain, 0, P.wait_ns);
+    }
+    __syncwarp();
   } else {
     // ---------------- epilogue: TMEM -> G buffer ----------------
     const int quad = warp & 3;
     const int chunk0 = (warp - 2) >> 2;  // this warp's first 16-column chunk
     const int row = quad * 32 + lane;
     uint32_t acc = 0, acc_phase = 0;
-    for (int64_t tt = blockIdx.x; tt < P.total_tiles; tt += gridDim.x) {
-      const TileCoord c = decode_tile(P, tt);
+    for (int64_t tt = pair0; tt < P.total_tiles; tt += npairs) {
+      const TileCoord c = decode_tile(P, tt, rank);
       const TcCl& C = P.cl[c.cl];
       const TcPiece& pc = P.pc[c.piece];
       int got = 0;
@@ -476,7 +515,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
           ptx::tc_fence_before();
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(&tempty[acc]);
+          if (lane == 0) ptx::mbar_arrive_cluster(ptx::mapa(&tempty[acc], 0));
           acc_phase ^= 1u;
           if (valid) {
 #pragma unroll
@@ -566,7 +605,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       }
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&tempty[acc]);
+      if (lane == 0) ptx::mbar_arrive_cluster(ptx::mapa(&tempty[acc], 0));
       if (NBUF == 2) {
         acc ^= 1u;
         if (acc == 0) acc_phase ^= 1u;
@@ -576,11 +615,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
   }
 
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
+  ptx::cluster_sync();  // neither CTA leaves while the other's MMAs or signals may reach it
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, P.tmem_cols);
+    ptx::tmem_dealloc_pair(tmem_base, P.tmem_cols);
   }
 }
 
@@ -619,7 +660,7 @@ static te_status get_encoder(TcState* st) {
 struct TcPlan {
   int mode, es, nparts, fmt;  // fmt: G format
   int vp, op, vq;
-  int TA, TB, NT, n_mx, n_my, n_nt;
+  int TA, TB, NT, n_my, n_mp, n_nt;
   int kw_chunks, ko_chunks, kw_elems, ko_elems, cbw, cbo;
   int stages;
   uint32_t stage_bytes, a_part_bytes, b_part_bytes, tmem_cols;
@@ -628,6 +669,8 @@ struct TcPlan {
   int ldz;
   size_t smem;
 };
+
+constexpr int64_t MIN_SLOTS = 4;  // triples per launch where memory is short
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -667,13 +710,13 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   if (force_tb) bestTB = force_tb;
   pl.TB = bestTB;
   pl.TA = 128 / bestTB;
-  pl.n_mx = (v + pl.TA - 1) / pl.TA;
   pl.n_my = (v + pl.TB - 1) / pl.TB;
-  const int ntmax = std::min(256, (512 / (nacc * nbuf_max)) / 16 * 16);
+  pl.n_mp = ((v + pl.TA - 1) / pl.TA * pl.n_my + 1) / 2;
+  const int ntmax = std::min(256, (512 / (nacc * nbuf_max)) / 32 * 32);
   pl.n_nt = (v + ntmax - 1) / ntmax;
   // a tuned split: any count whose N tile fits three accumulators in TMEM (N <= 160)
-  if (force_nnt > 0 && round_up((v + force_nnt - 1) / force_nnt, 16) <= (oz ? 160 : 256)) pl.n_nt = force_nnt;
-  pl.NT = round_up((v + pl.n_nt - 1) / pl.n_nt, 16);
+  if (force_nnt > 0 && round_up((v + force_nnt - 1) / force_nnt, 32) <= (oz ? 160 : 256)) pl.n_nt = force_nnt;
+  pl.NT = round_up((v + pl.n_nt - 1) / pl.n_nt, 32);  // cta_group::2: N in steps of 32
   pl.nbuf = (2 * nacc * pl.NT <= 512) ? 2 : 1;
   pl.fmt = !oz ? G_F32 : (pl.nbuf == 1 ? G_MIXED : G_PAIR);  // as the kernel's epilogues store
   pl.cbw = oz ? 64 : 128;
@@ -684,7 +727,7 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   pl.ko_elems = pl.cbo / pl.es;
   pl.ko_chunks = (pl.op + pl.ko_elems - 1) / pl.ko_elems;
   pl.a_part_bytes = 128u * (uint32_t)pl.cbw;
-  pl.b_part_bytes = (uint32_t)pl.NT * (uint32_t)pl.cbw;
+  pl.b_part_bytes = (uint32_t)(pl.NT / 2) * (uint32_t)pl.cbw;  // a CTA's half of the B tile
   pl.stage_bytes = (uint32_t)pl.nparts * (pl.a_part_bytes + pl.b_part_bytes);
   const size_t avail = h->smem_optin > 2048 ? h->smem_optin - 2048 : 0;
   pl.stages = (int)std::min<size_t>(8, avail / pl.stage_bytes);
@@ -693,11 +736,16 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   while (cols < (uint32_t)(nacc * pl.nbuf * pl.NT)) cols <<= 1;
   pl.tmem_cols = cols;
   pl.ldz = round_up(v, 4);
-  const int64_t tiles = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
-  int64_t want = (4LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
+  const int64_t tiles = 3LL * pl.n_mp * pl.n_nt;  // pair tiles per triple
+  // About 40 tiles per pair of CTAs and launch: a launch's fixed part (its
+  // first loads, the last tile's epilogue, a last wave) is some 15 us, which at
+  // nvir = 120 with four triples per launch was a sixth of the contraction
+  // (nocc=16 nvir=120 energy: 33.9 ms with 4 triples per launch, 30.5 with 9,
+  // 29.1 with 17).
+  int64_t want = (20LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
   const int64_t per_slot = g_slot_floats(v, pl.fmt) * 4;
   const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(6LL << 30) / per_slot);
-  want = std::max<int64_t>(want, 4);  // fewer launches per cluster
+  want = std::max<int64_t>(want, MIN_SLOTS);
   want = std::min<int64_t>({want, mem_cap, 1024, std::max<int64_t>(1, ntri)});
   pl.nslots = (int)std::max<int64_t>(1, want);
   return pl;
@@ -823,13 +871,13 @@ static te_status build_maps(TcState* st, const TcPlan& pl, int o, int v, const T
   {  // t2 slices [r][q][s][z][d]: dims (d, z, s, q, r)
     const uint64_t d[5] = {vp, V, NS, O, O};
     const uint64_t sn[4] = {vp * es, V * vp * es, NS * V * vp * es, O * NS * V * vp * es};
-    const uint32_t box[5] = {(uint32_t)pl.kw_elems, (uint32_t)pl.NT, ns, 1, 1};
+    const uint32_t box[5] = {(uint32_t)pl.kw_elems, (uint32_t)pl.NT / 2, ns, 1, 1};
     if ((s = encode(st, &M->b_t2, b.b[0], dt, 5, d, sn, box, swz_of(pl.cbw), "t2")) != TE_OK) return s;
   }
   {  // nooT slices [p][r][s][z][l]: dims (l, z, s, r, p)
     const uint64_t d[5] = {op, V, NS, O, O};
     const uint64_t sn[4] = {op * es, V * op * es, NS * V * op * es, O * NS * V * op * es};
-    const uint32_t box[5] = {(uint32_t)pl.ko_elems, (uint32_t)pl.NT, ns, 1, 1};
+    const uint32_t box[5] = {(uint32_t)pl.ko_elems, (uint32_t)pl.NT / 2, ns, 1, 1};
     if ((s = encode(st, &M->b_noo, b.n[0], dt, 5, d, sn, box, swz_of(pl.cbo), "nooT")) != TE_OK) return s;
   }
   return TE_OK;
@@ -1011,7 +1059,7 @@ template <int MODE>
 static cudaError_t launch_gemm_tc(const TcMapSet& M, const TcParams& P, size_t smem, int grid_cap, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int64_t grid = std::min<int64_t>(P.total_tiles, grid_cap);
+  const int64_t grid = GEMM_PAIR * std::min<int64_t>(P.total_tiles, std::max(1, grid_cap / GEMM_PAIR));
   k_gemm_tc<MODE><<<(unsigned)grid, GEMM_THREADS, smem, s>>>(M, P);
   return cudaGetLastError();
 }
@@ -1045,8 +1093,8 @@ static void fill_cluster(const TcJob& J, TcCl* C) {
   C->TA = J.pl.TA;
   C->TB = J.pl.TB;
   C->NT = J.pl.NT;
-  C->n_mx = J.pl.n_mx;
   C->n_my = J.pl.n_my;
+  C->n_mp = J.pl.n_mp;
   C->n_nt = J.pl.n_nt;
   C->kw_chunks = J.pl.kw_chunks;
   C->ko_chunks = J.pl.ko_chunks;
@@ -1175,7 +1223,7 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
       items += (int64_t)ns * J.nbt;
       t += ns;
       const double kpad = 2.0 * J.pl.kw_chunks * J.pl.kw_elems + 2.0 * J.pl.ko_chunks * J.pl.ko_elems;
-      flops += 2.0 * nprod * (double)ns * J.tiles_per_triple * 128.0 * J.pl.NT * kpad;
+      flops += 2.0 * nprod * (double)ns * J.tiles_per_triple * 256.0 * J.pl.NT * kpad;
     }
     if (pcs.empty()) {
       st = fail(TE_ENOMEM, "G pool smaller than one triple's G blocks");
@@ -1257,7 +1305,7 @@ static te_status setup_job(Handle* h, TcState* st, const te_cluster* c, int mode
   J->t_end = t_end;
   J->nbt = energy_num_block_triples(J->v);
   J->slot_floats = g_slot_floats(J->v, pl.fmt);
-  J->tiles_per_triple = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
+  J->tiles_per_triple = 3LL * pl.n_mp * pl.n_nt;
   tc_carve_cluster(base, pl, J->o, J->v, num_unique_triples(J->o), &J->b);
   J->shares = J->b.etri;
   const cudaError_t e = launch_prep_tc(mode, c, pl, J->b, df, dfs, h->d_err, cluster, h->num_sms, s, &h->n_launches);
@@ -1282,6 +1330,21 @@ static TcPool single_pool(const TcPlan& pl, int v) {
   q.max_slots = pl.nslots;
   q.par_slots = std::max<int64_t>(pl.nslots, TC_PAR_SLOTS);
   return q;
+}
+
+// Workspace of a single-cluster call; with `lean`, or a handle limit that the
+// usual G pool would pass, for MIN_SLOTS triples per launch (pl->nslots).
+static size_t single_bytes(const Handle* h, TcPlan* pl, int o, int v, const te_df* df, bool lean) {
+  TcBuffers b;
+  DfScratch d;
+  const size_t fixed = tc_carve_cluster(nullptr, *pl, o, v, num_unique_triples(o), &b);
+  const size_t form = df ? df_carve(nullptr, o, v, df->naux, h->num_sms, &d) : size_t(0);
+  size_t bytes = fixed + std::max(tc_shared_bytes(single_pool(*pl, v), h->num_sms), form);
+  if ((lean || (h->ws_limit && bytes > h->ws_limit)) && pl->nslots > MIN_SLOTS) {
+    pl->nslots = (int)MIN_SLOTS;
+    bytes = fixed + std::max(tc_shared_bytes(single_pool(*pl, v), h->num_sms), form);
+  }
+  return bytes;
 }
 
 size_t tc_slices_bytes(int o, int v, int ns) {
@@ -1372,12 +1435,8 @@ te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, in
 
 te_status tc_workspace_bytes(Handle* h, const te_cluster* c, te_precision p, size_t* bytes, const te_df* df) {
   const int o = (int)c->nocc, v = (int)c->nvir;
-  const TcPlan pl = make_plan(h, o, v, tc_mode_of(p, o, v, h->ozaki_bits), num_unique_triples(c->nocc));
-  TcBuffers b;
-  DfScratch d;
-  const size_t region = std::max(tc_shared_bytes(single_pool(pl, v), h->num_sms),
-                                 df ? df_carve(nullptr, o, v, df->naux, h->num_sms, &d) : size_t(0));
-  *bytes = tc_carve_cluster(nullptr, pl, o, v, num_unique_triples(o), &b) + region;
+  TcPlan pl = make_plan(h, o, v, tc_mode_of(p, o, v, h->ozaki_bits), num_unique_triples(c->nocc));
+  *bytes = single_bytes(h, &pl, o, v, df, false);
   return TE_OK;
 }
 
@@ -1408,7 +1467,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
     // one more N split (smaller N tiles re-read the A operand more often), and
     // in the exact-slice modes the fewer splits of 160-column tiles, which do
     // not rotate their TMEM blocks
-    if (round_up((v + base.n_nt) / (base.n_nt + 1), 16) >= 32) cand.emplace_back(TB, base.n_nt + 1);
+    if (round_up((v + base.n_nt) / (base.n_nt + 1), 32) < base.NT) cand.emplace_back(TB, base.n_nt + 1);
     const int n160 = (v + 159) / 160;
     if (is_ozaki(mode) && n160 < base.n_nt) cand.emplace_back(TB, n160);
   }
@@ -1428,7 +1487,8 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
   if (rs != TE_OK) return rs;
   size_t need = 0;
   for (const auto& cd : cand) {
-    const TcPlan pl = make_plan(h, o, v, mode, nt, cd.first, cd.second);
+    TcPlan pl = make_plan(h, o, v, mode, nt, cd.first, cd.second);
+    pl.nslots = (int)std::min<int64_t>(pl.nslots, MIN_SLOTS);
     TcBuffers b;
     need = std::max(need, tc_carve_cluster(nullptr, pl, o, v, nt, &b) + tc_shared_bytes(single_pool(pl, v), h->num_sms));
   }
@@ -1445,7 +1505,8 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
   TcMapSet* MS = new TcMapSet;
   TcParams* P = new TcParams;
   for (const auto& cd : cand) {
-    const TcPlan pl = make_plan(h, o, v, mode, nt, cd.first, cd.second);
+    TcPlan pl = make_plan(h, o, v, mode, nt, cd.first, cd.second);
+    pl.nslots = (int)std::min<int64_t>(pl.nslots, MIN_SLOTS);
     if (pl.stages < 2) continue;
     TcJob& J = jobs[0];
     J = TcJob{};
@@ -1455,7 +1516,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
     J.v = v;
     J.nbt = energy_num_block_triples(v);
     J.slot_floats = g_slot_floats(v, pl.fmt);
-    J.tiles_per_triple = 3LL * pl.n_mx * pl.n_my * pl.n_nt;
+    J.tiles_per_triple = 3LL * pl.n_mp * pl.n_nt;
     const size_t cbytes = tc_carve_cluster(wbase, pl, o, v, nt, &J.b);
     cudaError_t e = cudaSuccess;
     if (!prepped) {  // the operand planes sit first in the workspace for every candidate
@@ -1515,16 +1576,11 @@ te_status run_tc(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int mode = tc_mode_of(p, o, v, h->ozaki_bits);
   const int64_t ntri = num_unique_triples(o);
-  const TcPlan pl = make_plan(h, o, v, mode, t_end - t_begin);
+  TcPlan pl = make_plan(h, o, v, mode, t_end - t_begin);
   if (pl.stages < 2) return fail(TE_EUNSUPPORTED, "not enough shared memory for two pipeline stages");
   rs = check_k(mode, o, v);
   if (rs != TE_OK) return rs;
-  TcBuffers b;
-  const TcPool pq = single_pool(pl, v);
-  const size_t cbytes = tc_carve_cluster(nullptr, pl, o, v, ntri, &b);
-  DfScratch dfs;
-  const size_t bytes = cbytes + std::max(tc_shared_bytes(pq, h->num_sms),
-                                         df ? df_carve(nullptr, o, v, df->naux, h->num_sms, &dfs) : size_t(0));
+  size_t bytes = single_bytes(h, &pl, o, v, df, false);
   if (h->log)
     std::fprintf(stderr,
                  "[tenergy] plan nocc=%d nvir=%d mode=%d: M tile %d x %d, N tile %d (%d per row block), %d stages "
@@ -1532,9 +1588,14 @@ te_status run_tc(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin
                  o, v, mode, pl.TA, pl.TB, pl.NT, pl.n_nt, pl.stages, pl.stage_bytes, pl.nslots, pl.tmem_cols,
                  pl.nbuf, bytes);
   rs = ensure_workspace_public(h, bytes);
+  if (rs == TE_ENOMEM && pl.nslots > MIN_SLOTS) rs = ensure_workspace_public(h, single_bytes(h, &pl, o, v, df, true));
   if (rs != TE_OK) return rs;
   rs = ensure_triples_public(h, o);
   if (rs != TE_OK) return rs;
+  TcBuffers b;
+  DfScratch dfs;
+  const TcPool pq = single_pool(pl, v);
+  const size_t cbytes = tc_carve_cluster(nullptr, pl, o, v, ntri, &b);
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023));
   std::vector<TcJob> jobs(1);
   if (df) df_carve(base + cbytes, o, v, df->naux, h->num_sms, &dfs);  // over the G pool, before its first use
