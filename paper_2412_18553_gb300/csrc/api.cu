@@ -646,7 +646,7 @@ te_status t_energy_vjp_batched(te_handle hh, const te_cluster* cs, int64_t n, te
   int64_t maxo = 1;
   for (int64_t x = 0; x < n; ++x) {
     need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(cs[x].nocc, cs[x].nvir)
-                                       : vjp_tc_bytes(cs[x].nocc, cs[x].nvir, h->num_sms));
+                                       : vjp_tc_bytes(h, cs[x].nocc, cs[x].nvir));
     maxo = std::max<int64_t>(maxo, cs[x].nocc);
   }
   te_status st = ensure_workspace(h, need);
@@ -739,8 +739,8 @@ te_status te_reserve(te_handle hh, const te_cluster* c, te_precision p, int what
     if (st != TE_OK) return st;
   }
   if (what & TE_RESERVE_VJP)
-    need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(c->nocc, c->nvir) : vjp_tc_bytes(c->nocc, c->nvir, h->num_sms));
-  if (what & TE_RESERVE_FRAG) need = std::max(need, frag_bytes(c->nocc, c->nvir, p, h->num_sms));
+    need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(c->nocc, c->nvir) : vjp_tc_bytes(h, c->nocc, c->nvir));
+  if (what & TE_RESERVE_FRAG) need = std::max(need, frag_bytes(h, c->nocc, c->nvir, p));
   te_status st = ensure_workspace(h, need);
   if (st != TE_OK) return st;
   return ensure_triples(h, (int)c->nocc);

@@ -27,6 +27,7 @@
 #include <cstring>
 
 #include "energy_tc.h"
+#include "fp_util.cuh"
 #include "ptx_sm100.cuh"
 
 namespace te {
@@ -114,41 +115,6 @@ __device__ __forceinline__ void df_fma(df& acc, df a, df b) {
 
 // 2 a + b and a + 2 b
 __device__ __forceinline__ df df_2ab(df a, df b) { return df_add(df{2.f * a.h, 2.f * a.l}, b); }
-
-// float64 conversions share the two float64 lanes with the arithmetic (64 issue
-// cycles of a scheduler each); the usual range is converted by integer
-// operations instead (same bits).  The rare conversions are volatile so that
-// the compiler does not issue them ahead of their branch.
-__device__ __forceinline__ double cvt_double(float f) {
-  double d;
-  asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
-  return d;
-}
-__device__ __forceinline__ float cvt_float(double d) {
-  float f;
-  asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(d));
-  return f;
-}
-__device__ __forceinline__ double to_double(float f) {
-  const uint32_t u = __float_as_uint(f), m = u & 0x7FFFFFFFu;
-  if (m - 0x00800000u < 0x7F000000u)  // normal
-    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(m << 29));
-  return cvt_double(f);
-}
-
-// 1/D to ~1e-14: FP32 seed of D rounded to nearest, one Newton step
-__device__ __forceinline__ double recip(double D) {
-  const uint32_t h = (uint32_t)__double2hiint(D), m = h & 0x7FFFFFFFu;
-  double r0;
-  if (m - ((1023u - 100u) << 20) < (200u << 20)) {  // 2^-100 <= |D| < 2^100
-    const unsigned long long b = (((unsigned long long)m << 32) | (uint32_t)__double2loint(D)) + (1ull << 28);
-    const float f = __frcp_rn(__uint_as_float((h & 0x80000000u) | ((uint32_t)(b >> 29) - (896u << 23))));
-    r0 = to_double(f);
-  } else {
-    r0 = cvt_double(__frcp_rn(cvt_float(D)));
-  }
-  return fma(r0, fma(-D, r0, 1.0), r0);
-}
 
 struct EnergyMaps {
   CUtensorMap ovs[TC_MAX_CL];  // per cluster: ovs32 [o][v][o][vq], 4D (b, j, a, i)
@@ -434,7 +400,7 @@ __global__ void __launch_bounds__(Layout<FMT>::threads, 1)
       if (valid) {
         // orbit weight A (Eq. E_corr_CCSD_T): 1, 1/2 or 1/6
         const bool all3 = (a == bb && bb == c), two = (a == bb || bb == c);
-        const double r1 = recip(D);
+        const double r1 = recip_newton(D, recip_seed(D));
         if constexpr (FMT != G_F32) {
           // differences of W~ within the even (0, 3, 4) and odd (1, 2, 5) positions, and even less odd
           const df e1 = df_sub(w[0], w[3]), e2 = df_sub(w[3], w[4]);

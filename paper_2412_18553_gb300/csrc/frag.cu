@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "adjoint_tc.cuh"
 #include "strided.h"
 #include "tc_path.h"
 #include "view_tc.h"
@@ -86,6 +87,10 @@ __global__ void __launch_bounds__(256) k_energy_proj(AdjArgs A, const double* __
   }
 }
 
+// ---------------------------------------------------------------------------
+// float64 form
+// ---------------------------------------------------------------------------
+
 struct FragWork {
   double *ovvvC, *t2C, *t2C2, *ooovC;      // C on occupied indices of the inputs
   double *t2L, *nooT, *ovs;                // float64 helper copies of the inputs
@@ -93,76 +98,70 @@ struct FragWork {
   double *G, *SG;                          // [3][v][v][v] each
   double *epart, *shares, *scratch;
   int64_t scratch_cap;
-  char* slices[3];                         // exact-slice planes (mixed precision only)
 };
 
-static size_t frag_layout(int64_t o, int64_t v, bool slices, int num_sms, char* base, FragWork* W);
+namespace {
 
-size_t frag_bytes(int64_t o, int64_t v, te_precision p, int num_sms) {
-  FragWork W;
-  return frag_layout(o, v, p != TE_FP64, num_sms, nullptr, &W);
-}
-
-// carve the workspace (base = nullptr: sizes only)
-static size_t frag_layout(int64_t o, int64_t v, bool slices, int num_sms, char* base, FragWork* W) {
-  const int64_t v3 = v * v * v, nt = num_unique_triples(o), nblk = (v3 + 255) / 256;
+struct Carve {
+  char* base;
   size_t off = 0;
-  auto take = [&](size_t bytes) {
+  char* take(size_t bytes) {
     off = (off + 1023) & ~size_t(1023);
     char* r = base ? base + off : nullptr;
     off += bytes;
     return r;
-  };
-  auto d = [&](int64_t n) { return reinterpret_cast<double*>(take((size_t)n * 8)); };
-  W->ovvvC = d(o * v3);
-  W->t2C = d(o * o * v * v);
-  W->t2C2 = d(o * o * v * v);
-  W->ooovC = d(o * o * o * v);
-  W->t2L = d(o * v * v * o);
-  W->nooT = d(o * o * v * o);
-  W->ovs = d(o * v * o * v);
-  W->t2LC = d(o * v * v * o);
-  W->nooTC = d(o * o * v * o);
-  W->ovs_unused = d(o * v * o * v);
-  W->G = d(3 * v3);
-  W->SG = d(3 * v3);
-  W->epart = d(nblk);
-  W->shares = d(std::max<int64_t>(1, nt));
-  W->scratch_cap = slices ? oz_scratch_cap(o, v, num_sms) : splitk_cap(o, v);
-  W->scratch = d(W->scratch_cap);
-  for (int k = 0; k < 3; ++k) W->slices[k] = slices ? take(tc_slices_bytes((int)o, (int)v) + 1024) : nullptr;
-  return off + 1024;
+  }
+  double* d(int64_t n) { return reinterpret_cast<double*>(take((size_t)n * 8)); }
+};
+
+// carve the workspace (base = nullptr: sizes only)
+size_t frag_layout(int64_t o, int64_t v, char* base, FragWork* W) {
+  const int64_t v3 = v * v * v, nt = num_unique_triples(o), nblk = (v3 + 255) / 256;
+  Carve c{base};
+  W->ovvvC = c.d(o * v3);
+  W->t2C = c.d(o * o * v * v);
+  W->t2C2 = c.d(o * o * v * v);
+  W->ooovC = c.d(o * o * o * v);
+  W->t2L = c.d(o * v * v * o);
+  W->nooT = c.d(o * o * v * o);
+  W->ovs = c.d(o * v * o * v);
+  W->t2LC = c.d(o * v * v * o);
+  W->nooTC = c.d(o * o * v * o);
+  W->ovs_unused = c.d(o * v * o * v);
+  W->G = c.d(3 * v3);
+  W->SG = c.d(3 * v3);
+  W->epart = c.d(nblk);
+  W->shares = c.d(std::max<int64_t>(1, nt));
+  W->scratch_cap = splitk_cap(o, v);
+  W->scratch = c.d(W->scratch_cap);
+  return c.off + 1024;
 }
 
-te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precision p, double* e_out,
-                   double* e_triples, cudaStream_t s) {
+// C on the occupied indices of the inputs
+cudaError_t transform_inputs(Handle* h, const te_cluster* c, const double* cf, double* ovvvC, double* t2C, double* t2C2,
+                             double* ooovC, cudaStream_t s) {
   const int o = (int)c->nocc, v = (int)c->nvir;
-  const int64_t v2 = (int64_t)v * v, v3 = v2 * v, nt = num_unique_triples(o), nblk = (v3 + 255) / 256;
-  const bool oz = p != TE_FP64;
-  te_status st = ensure_workspace_public(h, frag_bytes(o, v, p, h->num_sms));
-  if (st != TE_OK) return st;
-  st = ensure_triples_public(h, o);
-  if (st != TE_OK) return st;
-  FragWork W;
-  frag_layout(o, v, oz, h->num_sms,
-              reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023)), &W);
-
-  // C on the occupied indices of the inputs
+  const int64_t v2 = (int64_t)v * v, v3 = v2 * v;
   auto tr = [&](const double* in, int64_t outer, int64_t inner, double* out, int acc) {
     const int64_t n = outer * o * inner;
     k_occ_transform<<<(unsigned)std::min<int64_t>((n + 255) / 256, 8 * 1024), 256, 0, s>>>(in, cf, o, outer,
                                                                                            inner, out, acc);
     ++h->n_launches;
   };
-  tr(c->ovvv, 1, v3, W.ovvvC, 0);                           // ovvv[p,a,b,d]: first index
-  tr(c->t2, 1, (int64_t)o * v2, W.t2C, 0);                  // t2[r,q,a,b]: first index
-  tr(c->t2, o, v2, W.t2C, 1);                               //   plus second index
-  tr(c->t2, o, v2, W.t2C2, 0);                              // second index only
-  tr(c->ooov, 1, (int64_t)o * o * v, W.ooovC, 0);           // ooov[p,l,r,z]: first index
-  tr(c->ooov, (int64_t)o * o, v, W.ooovC, 1);               //   plus third index
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(TE_ECUDA, "transform launch: %s", cudaGetErrorString(e));
+  tr(c->ovvv, 1, v3, ovvvC, 0);                           // ovvv[p,a,b,d]: first index
+  tr(c->t2, 1, (int64_t)o * v2, t2C, 0);                  // t2[r,q,a,b]: first index
+  tr(c->t2, o, v2, t2C, 1);                               //   plus second index
+  tr(c->t2, o, v2, t2C2, 0);                              // second index only
+  tr(c->ooov, 1, (int64_t)o * o * v, ooovC, 0);           // ooov[p,l,r,z]: first index
+  tr(c->ooov, (int64_t)o * o, v, ooovC, 1);               //   plus third index
+  return cudaGetLastError();
+}
 
+te_status run_frag_fp64(Handle* h, const te_cluster* c, const double* cf, const FragWork& W, cudaStream_t s) {
+  const int o = (int)c->nocc, v = (int)c->nvir;
+  const int64_t v2 = (int64_t)v * v, v3 = v2 * v, nt = num_unique_triples(o), nblk = (v3 + 255) / 256;
+  cudaError_t e = transform_inputs(h, c, cf, W.ovvvC, W.t2C, W.t2C2, W.ooovC, s);
+  if (e != cudaSuccess) return fail(TE_ECUDA, "transform launch: %s", cudaGetErrorString(e));
   // float64 helper copies: t2L, nooT, ovs of the inputs; t2L of t2C2, nooT of ooovC
   Prepared P{};
   P.o = o; P.v = v; P.eps_o = c->eps_o; P.eps_v = c->eps_v; P.ovvv = c->ovvv; P.t2 = c->t2; P.t1 = c->t1;
@@ -176,80 +175,15 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
   if (e == cudaSuccess) e = launch_prep_fp64(&cx, &PX, s);
   h->n_launches += 6;
   if (e != cudaSuccess) return fail(TE_ECUDA, "prep: %s", cudaGetErrorString(e));
-
-  // exact-slice planes: the inputs; (ovvvC, t2C, ooovC) for ovvv, t2 and nooT;
-  // t2C2 for t2L
-  SliceSet S0{}, SA{}, SB{};
-  if (oz) {
-    te_cluster ca = *c, cb = *c;
-    ca.ovvv = W.ovvvC;
-    ca.t2 = W.t2C;
-    ca.ooov = W.ooovC;
-    cb.t2 = W.t2C2;
-    st = tc_prepare_slices(c, W.slices[0], &S0, h->num_sms, s, 4, h->d_err, 0, &h->n_launches);
-    if (st == TE_OK) st = tc_prepare_slices(&ca, W.slices[1], &SA, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
-    if (st == TE_OK) st = tc_prepare_slices(&cb, W.slices[2], &SB, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
-    if (st != TE_OK) return st;
-  }
-  // exact slices: the tcgen05 view GEMM (view_tc.cu) over the six segment
-  // views of each slice set, encoded once
-  VtBank bank;
-  bank.n = 0;
-  int m0[6], mA[6], mB[6];
-  const int NT = vt_ntile(v);
-  if (oz) {
-    if ((st = vt_slice_maps(&bank, S0, o, v, NT, m0)) != TE_OK) return st;
-    if ((st = vt_slice_maps(&bank, SA, o, v, NT, mA)) != TE_OK) return st;
-    if ((st = vt_slice_maps(&bank, SB, o, v, NT, mB)) != TE_OK) return st;
-  }
-
   std::vector<Triple> trip = unique_triples(o);
   const double third = 1.0 / 3.0;
   for (int64_t t = 0; t < nt && e == cudaSuccess; ++t) {
     const Triple T = trip[t];
-    if (oz) {
-      // per G block (p, q, r): the block itself (S1..S4 of the input slices)
-      // and its projection SG (two products per segment, one operand
-      // transformed), 1/3 for the average over the three occupied slots
-      VtBuild b;
-      vt_begin(&b, S0.ns);
-      for (int gi = 0; gi < 3; ++gi) {
-        int pp, qq, rr;
-        if (gi == 0) { pp = T.i; qq = T.j; rr = T.k; }
-        else if (gi == 1) { pp = T.j; qq = T.k; rr = T.i; }
-        else { pp = T.k; qq = T.i; rr = T.j; }
-        const int f_p[5] = {0, 0, 0, 0, pp}, f_q[5] = {0, 0, 0, 0, qq};
-        const int t_qr[5] = {0, 0, 0, qq, rr}, t_pr[5] = {0, 0, 0, pp, rr};
-        const int n_rq[5] = {0, 0, 0, rr, qq}, n_rp[5] = {0, 0, 0, rr, pp};
-        const int64_t rq = (int64_t)rr * o + qq, rp = (int64_t)rr * o + pp;
-        const int64_t nqr = (int64_t)qq * o + rr, npr = (int64_t)pp * o + rr;
-        auto u = [&](int m) { return vt_use(&b, bank, m); };
-        VtJob* J = vt_job(&b, v, v, v, 8, 16, NT, W.G + gi * v3, v2, v, 1, 1);
-        vt_seg(J, u(m0[0]), u(m0[4]), 1, v, f_p, t_qr, S0.e_ovvv + pp, S0.e_t2 + rq, 1.0);
-        vt_seg(J, u(m0[1]), u(m0[4]), 1, v, f_q, t_pr, S0.e_ovvv + qq, S0.e_t2 + rp, 1.0);
-        vt_seg(J, u(m0[3]), u(m0[5]), 1, o, f_p, n_rq, S0.e_t2L + pp, S0.e_nooT + nqr, 1.0);
-        vt_seg(J, u(m0[2]), u(m0[5]), 1, o, f_q, n_rp, S0.e_t2L + qq, S0.e_nooT + npr, 1.0);
-        VtJob* JS = vt_job(&b, v, v, v, 8, 16, NT, W.SG + gi * v3, v2, v, 1, 1);
-        JS->jalpha = third;
-        vt_seg(JS, u(mA[0]), u(m0[4]), 1, v, f_p, t_qr, SA.e_ovvv + pp, S0.e_t2 + rq, 1.0);  // ovvvC[p] t2[r,q]
-        vt_seg(JS, u(m0[0]), u(mA[4]), 1, v, f_p, t_qr, S0.e_ovvv + pp, SA.e_t2 + rq, 1.0);  // ovvv[p] t2C[r,q]
-        vt_seg(JS, u(mA[1]), u(m0[4]), 1, v, f_q, t_pr, SA.e_ovvv + qq, S0.e_t2 + rp, 1.0);  // ovvvC[q] t2[r,p]
-        vt_seg(JS, u(m0[1]), u(mA[4]), 1, v, f_q, t_pr, S0.e_ovvv + qq, SA.e_t2 + rp, 1.0);  // ovvv[q] t2C[r,p]
-        vt_seg(JS, u(mB[3]), u(m0[5]), 1, o, f_p, n_rq, SB.e_t2L + pp, S0.e_nooT + nqr, 1.0);  // t2LC[p] nooT[q][r]
-        vt_seg(JS, u(m0[3]), u(mA[5]), 1, o, f_p, n_rq, S0.e_t2L + pp, SA.e_nooT + nqr, 1.0);  // t2L[p] nooTC[q][r]
-        vt_seg(JS, u(mB[2]), u(m0[5]), 1, o, f_q, n_rp, SB.e_t2L + qq, S0.e_nooT + npr, 1.0);  // t2LC[q] nooT[p][r]
-        vt_seg(JS, u(m0[2]), u(mA[5]), 1, o, f_q, n_rp, S0.e_t2L + qq, SA.e_nooT + npr, 1.0);  // t2L[q] nooTC[p][r]
-      }
-      if ((st = vt_finish(&b, h->num_sms, nullptr, 0, nullptr)) != TE_OK) return st;
-      if ((st = vt_launch(h, &b, s)) != TE_OK) return st;
-    }
-    if (!oz) {
-      e = cudaMemsetAsync(W.SG, 0, sizeof(double) * 3 * v3, s);
-      if (e != cudaSuccess) break;
-      e = launch_gemm_fp64(&P, h->d_triples, t, 1, W.G, s);
-      ++h->n_launches;
-    }
-    for (int gi = 0; gi < 3 && e == cudaSuccess && !oz; ++gi) {
+    e = cudaMemsetAsync(W.SG, 0, sizeof(double) * 3 * v3, s);
+    if (e != cudaSuccess) break;
+    e = launch_gemm_fp64(&P, h->d_triples, t, 1, W.G, s);
+    ++h->n_launches;
+    for (int gi = 0; gi < 3 && e == cudaSuccess; ++gi) {
       int pp, qq, rr;
       if (gi == 0) { pp = T.i; qq = T.j; rr = T.k; }
       else if (gi == 1) { pp = T.j; qq = T.k; rr = T.i; }
@@ -281,11 +215,284 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
     e = launch_sum_share(W.epart, nblk, (double)T.m / 3.0, W.shares + t, s);
     h->n_launches += 2;
   }
-  if (e == cudaSuccess && e_triples && nt > 0)
-    e = cudaMemcpyAsync(e_triples, W.shares, sizeof(double) * nt, cudaMemcpyDeviceToDevice, s);
+  if (e != cudaSuccess) return fail(TE_ECUDA, "projected energy launch: %s", cudaGetErrorString(e));
+  return TE_OK;
+}
+
+// ---------------------------------------------------------------------------
+// exact-slice form: batches of triples, the epilogue in FP32 pairs
+// ---------------------------------------------------------------------------
+
+constexpr int FRAG_MAX_BATCH = 8;
+constexpr int64_t FRAG_BATCH_BYTES = int64_t(1) << 30;  // G and SG of a batch
+
+struct FragOz {
+  double *ovvvC, *t2C, *t2C2, *ooovC;
+  PairBuffers pb;
+  float2 *G, *SG;  // [slot][3][v^3]
+  int64_t stride;  // float2 between the slots of each
+  double *epart, *shares;
+  char* slices[3];
+};
+
+int frag_batch(int64_t o, int64_t v) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>({FRAG_MAX_BATCH, FRAG_BATCH_BYTES / (48 * v * v * v),
+                                                      std::max<int64_t>(1, num_unique_triples(o))}));
+}
+
+size_t frag_oz_layout(int64_t o, int64_t v, int B, char* base, FragOz* W) {
+  const int64_t v3 = v * v * v, nt = num_unique_triples(o);
+  Carve c{base};
+  W->ovvvC = c.d(o * v3);
+  W->t2C = c.d(o * o * v * v);
+  W->t2C2 = c.d(o * o * v * v);
+  W->ooovC = c.d(o * o * o * v);
+  W->pb.ovs = reinterpret_cast<pr*>(c.d(o * v * o * v));
+  W->pb.t1 = reinterpret_cast<pr*>(c.d(o * v));
+  W->pb.eps = reinterpret_cast<pr*>(c.d(o + v));
+  W->pb.hi = reinterpret_cast<unsigned int*>(c.take(64));
+  W->stride = (3 * v3 + 3) / 4 * 4;
+  W->G = reinterpret_cast<float2*>(c.d(B * W->stride));
+  W->SG = reinterpret_cast<float2*>(c.d(B * W->stride));
+  W->epart = c.d((int64_t)B * 8192);
+  W->shares = c.d(std::max<int64_t>(1, nt));
+  for (int k = 0; k < 3; ++k) W->slices[k] = c.take(tc_slices_bytes((int)o, (int)v) + 1024);
+  return c.off + 1024;
+}
+
+int frag_oz_batch(const Handle* h, int64_t o, int64_t v) {
+  FragOz W;
+  const int B = frag_batch(o, v);
+  return h->ws_limit && frag_oz_layout(o, v, B, nullptr, &W) > h->ws_limit ? 1 : B;
+}
+
+struct ProjArgs {
+  PairInputs in;
+  SliceExps x0, xa, xb;  // scales of the input slices, of (ovvvC, t2C, ., ooovC) and of t2C2's t2L
+  const float2 *G, *SG;
+  int64_t stride;
+  double* epart;   // [slot][gridDim.x]
+  double* shares;
+  int64_t t0;
+  int n;
+  Triple t[FRAG_MAX_BATCH];
+};
+
+// the projected block's scale: the largest of its eight products'
+__device__ __forceinline__ int sg_exp(const ProjArgs& A, int p, int q, int r) {
+  const int o = A.in.o, rq = r * o + q, rp = r * o + p, nqr = q * o + r, npr = p * o + r;
+  int e = max(A.xa.e_ovvv[p] + A.x0.e_t2[rq], A.x0.e_ovvv[p] + A.xa.e_t2[rq]);
+  e = max(e, max(A.xa.e_ovvv[q] + A.x0.e_t2[rp], A.x0.e_ovvv[q] + A.xa.e_t2[rp]));
+  e = max(e, max(A.xb.e_t2L[p] + A.x0.e_nooT[nqr], A.x0.e_t2L[p] + A.xa.e_nooT[nqr]));
+  return max(e, max(A.xb.e_t2L[q] + A.x0.e_nooT[npr], A.x0.e_t2L[q] + A.xa.e_nooT[npr]));
+}
+// scale of S W~, and of its three blocks relative to it
+__device__ __forceinline__ TripleScale proj_scale(const ProjArgs& A, Triple T) {
+  const int e0 = sg_exp(A, T.i, T.j, T.k), e1 = sg_exp(A, T.j, T.k, T.i), e2 = sg_exp(A, T.k, T.i, T.j);
+  TripleScale s;
+  s.E = max(e0, max(e1, e2));
+  s.f[0] = ldexpf(1.f, e0 - s.E);
+  s.f[1] = ldexpf(1.f, e1 - s.E);
+  s.f[2] = ldexpf(1.f, e2 - s.E);
+  s.fy = 0.f;
+  return s;
+}
+
+// per-block sums of (S W~) R[V] / D over the orbits of each slot
+__global__ void __launch_bounds__(256) k_proj_pairs(const __grid_constant__ ProjArgs A) {
+  __shared__ double red[8];
+  const int slot = blockIdx.y;
+  const Triple T = A.t[slot];
+  const TripleScale sc = triple_scale(A.in, A.x0, T), ss = proj_scale(A, T);
+  const int64_t v = A.in.v, norb = v * (v + 1) * (v + 2) / 6;
+  const float2 *G = A.G + slot * A.stride, *SG = A.SG + slot * A.stride;
+  const pr eo = occ_energy(A.in, T);
+  pr sum{0.f, 0.f};
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < norb; t += (int64_t)gridDim.x * blockDim.x) {
+    int a, b, c;
+    orbit_abc(t, &a, &b, &c);
+    pr W[6], Y[6], RV[6];
+    orbit_w(G, v, sc, a, b, c, W);
+    orbit_y(A.in, T, sc, a, b, c, Y);
+#pragma unroll
+    for (int n = 0; n < 6; ++n) Y[n] = pr_add(W[n], Y[n]);
+    r_orbit_pairs(Y, RV);
+    orbit_w(SG, v, ss, a, b, c, W);
+    const unsigned distinct = orbit_distinct(a, b, c);
+    pr x{0.f, 0.f};
+#pragma unroll
+    for (int n = 0; n < 6; ++n)
+      if (distinct >> n & 1u) pr_fma(x, W[n], RV[n]);
+    const pr r = pr_recip(pr_sub(pr_sub(pr_sub(eo, A.in.eps_v[a]), A.in.eps_v[b]), A.in.eps_v[c]));
+    pr_fma(sum, x, r);
+  }
+  double s = pr_double(sum);
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w];
+    A.epart[(int64_t)slot * gridDim.x + blockIdx.x] = t;
+  }
+}
+
+// the slots' shares: (m / 3) (1 / 3) 2^(E + E_S) times their block sums in a fixed order
+__global__ void __launch_bounds__(256) k_proj_shares(const __grid_constant__ ProjArgs A, int nblk) {
+  __shared__ double red[8];
+  const int slot = blockIdx.x;
+  const Triple T = A.t[slot];
+  double s = 0.0;
+  for (int e = threadIdx.x; e < nblk; e += 256) s += A.epart[(int64_t)slot * nblk + e];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w];
+    const int E = triple_scale(A.in, A.x0, T).E + proj_scale(A, T).E;
+    A.shares[A.t0 + slot] = ldexp(t * ((double)T.m / 9.0), E);
+  }
+}
+
+te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const FragOz& W, int B, cudaStream_t s) {
+  const int o = (int)c->nocc, v = (int)c->nvir;
+  const int64_t v2 = (int64_t)v * v, v3 = v2 * v, nt = num_unique_triples(o);
+  cudaError_t e = transform_inputs(h, c, cf, W.ovvvC, W.t2C, W.t2C2, W.ooovC, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(W.pb.hi, 0, 64, s);
+  if (e != cudaSuccess) return fail(TE_ECUDA, "transform launch: %s", cudaGetErrorString(e));
+  // exact-slice planes: the inputs; (ovvvC, t2C, ooovC) for ovvv, t2 and nooT;
+  // t2C2 for t2L
+  SliceSet S0{}, SA{}, SB{};
+  te_cluster ca = *c, cb = *c;
+  ca.ovvv = W.ovvvC;
+  ca.t2 = W.t2C;
+  ca.ooov = W.ooovC;
+  cb.t2 = W.t2C2;
+  te_status st = tc_prepare_slices(c, W.slices[0], &S0, h->num_sms, s, 4, h->d_err, 0, &h->n_launches, W.pb.hi);
+  if (st == TE_OK) st = tc_prepare_slices(&ca, W.slices[1], &SA, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
+  if (st == TE_OK) st = tc_prepare_slices(&cb, W.slices[2], &SB, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
+  if (st != TE_OK) return st;
+  e = launch_pair_inputs(c, W.pb, s);
+  ++h->n_launches;
+  if (e != cudaSuccess) return fail(TE_ECUDA, "pair launch: %s", cudaGetErrorString(e));
+  // the six segment views of each slice set, encoded once
+  VtBank bank;
+  bank.n = 0;
+  int m0[6], mA[6], mB[6];
+  const int NT = vt_ntile(v);
+  if ((st = vt_slice_maps(&bank, S0, o, v, NT, m0)) != TE_OK) return st;
+  if ((st = vt_slice_maps(&bank, SA, o, v, NT, mA)) != TE_OK) return st;
+  if ((st = vt_slice_maps(&bank, SB, o, v, NT, mB)) != TE_OK) return st;
+  const int grid = adjoint_grid(h->num_sms);
+  ProjArgs A;
+  A.in = pair_inputs(c, W.pb, o, v);
+  A.x0 = SliceExps{S0.e_ovvv, S0.e_t2, S0.e_t2L, S0.e_nooT};
+  A.xa = SliceExps{SA.e_ovvv, SA.e_t2, SA.e_t2L, SA.e_nooT};
+  A.xb = SliceExps{SB.e_ovvv, SB.e_t2, SB.e_t2L, SB.e_nooT};
+  A.G = W.G;
+  A.SG = W.SG;
+  A.stride = W.stride;
+  A.epart = W.epart;
+  A.shares = W.shares;
+  std::vector<Triple> trip = unique_triples(o);
+  VtBuild* bp = new VtBuild;
+  VtBuild& b = *bp;
+  struct Del {
+    VtBuild* b;
+    ~Del() { delete b; }
+  } del{bp};
+  for (int64_t t0 = 0; t0 < nt; t0 += B) {
+    A.n = (int)std::min<int64_t>(B, nt - t0);
+    A.t0 = t0;
+    // per G block (p, q, r): the block itself (S1..S4 of the input slices) and
+    // its projection SG (two products per segment, one operand transformed)
+    vt_begin(&b, S0.ns, true);
+    for (int x = 0; x < A.n; ++x) {
+      const Triple T = A.t[x] = trip[t0 + x];
+      for (int gi = 0; gi < 3; ++gi) {
+        int pp, qq, rr;
+        if (gi == 0) { pp = T.i; qq = T.j; rr = T.k; }
+        else if (gi == 1) { pp = T.j; qq = T.k; rr = T.i; }
+        else { pp = T.k; qq = T.i; rr = T.j; }
+        const int f_p[3] = {0, 0, pp}, f_q[3] = {0, 0, qq};
+        const int t_qr[3] = {0, qq, rr}, t_pr[3] = {0, pp, rr}, n_rq[3] = {0, rr, qq}, n_rp[3] = {0, rr, pp};
+        const int64_t rq = (int64_t)rr * o + qq, rp = (int64_t)rr * o + pp;
+        const int64_t nqr = (int64_t)qq * o + rr, npr = (int64_t)pp * o + rr;
+        auto seg = [&](int ma, int mb, int K, const int* fa, const int* fb, const int* ea, const int* eb) {
+          vt_seg(&b, vt_use(&b, bank, ma), vt_use(&b, bank, mb), 1, K, fa, fb, ea, eb, 1);
+        };
+        vt_job(&b, v, v, v, 8, 16, NT, W.G + x * W.stride + gi * v3, v2, v, 1, VT_PAIR);
+        seg(m0[0], m0[4], v, f_p, t_qr, S0.e_ovvv + pp, S0.e_t2 + rq);
+        seg(m0[1], m0[4], v, f_q, t_pr, S0.e_ovvv + qq, S0.e_t2 + rp);
+        seg(m0[3], m0[5], o, f_p, n_rq, S0.e_t2L + pp, S0.e_nooT + nqr);
+        seg(m0[2], m0[5], o, f_q, n_rp, S0.e_t2L + qq, S0.e_nooT + npr);
+        vt_job(&b, v, v, v, 8, 16, NT, W.SG + x * W.stride + gi * v3, v2, v, 1, VT_PAIR);
+        seg(mA[0], m0[4], v, f_p, t_qr, SA.e_ovvv + pp, S0.e_t2 + rq);   // ovvvC[p] t2[r,q]
+        seg(m0[0], mA[4], v, f_p, t_qr, S0.e_ovvv + pp, SA.e_t2 + rq);   // ovvv[p] t2C[r,q]
+        seg(mA[1], m0[4], v, f_q, t_pr, SA.e_ovvv + qq, S0.e_t2 + rp);   // ovvvC[q] t2[r,p]
+        seg(m0[1], mA[4], v, f_q, t_pr, S0.e_ovvv + qq, SA.e_t2 + rp);   // ovvv[q] t2C[r,p]
+        seg(mB[3], m0[5], o, f_p, n_rq, SB.e_t2L + pp, S0.e_nooT + nqr);  // t2LC[p] nooT[q][r]
+        seg(m0[3], mA[5], o, f_p, n_rq, S0.e_t2L + pp, SA.e_nooT + nqr);  // t2L[p] nooTC[q][r]
+        seg(mB[2], m0[5], o, f_q, n_rp, SB.e_t2L + qq, S0.e_nooT + npr);  // t2LC[q] nooT[p][r]
+        seg(m0[2], mA[5], o, f_q, n_rp, S0.e_t2L + qq, SA.e_nooT + npr);  // t2L[q] nooTC[p][r]
+      }
+    }
+    if ((st = vt_finish(&b, h->num_sms, nullptr, 0, nullptr)) != TE_OK) return st;
+    if ((st = vt_launch(h, &b, s)) != TE_OK) return st;
+    k_proj_pairs<<<dim3((unsigned)grid, (unsigned)A.n), 256, 0, s>>>(A);
+    k_proj_shares<<<(unsigned)A.n, 256, 0, s>>>(A, grid);
+    h->n_launches += 2;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return fail(TE_ECUDA, "projected energy launch: %s", cudaGetErrorString(e));
+  }
+  return TE_OK;
+}
+
+}  // namespace
+
+size_t frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p) {
+  if (p == TE_FP64) {
+    FragWork W;
+    return frag_layout(o, v, nullptr, &W);
+  }
+  FragOz W;
+  return frag_oz_layout(o, v, frag_oz_batch(h, o, v), nullptr, &W);
+}
+
+te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precision p, double* e_out,
+                   double* e_triples, cudaStream_t s) {
+  const int o = (int)c->nocc, v = (int)c->nvir;
+  const int64_t nt = num_unique_triples(o);
+  FragOz Z;
+  int B = p == TE_FP64 ? 1 : frag_oz_batch(h, o, v);
+  te_status st = ensure_workspace_public(h, frag_bytes(h, o, v, p));
+  if (st == TE_ENOMEM && B > 1) {
+    B = 1;
+    st = ensure_workspace_public(h, frag_oz_layout(o, v, B, nullptr, &Z));
+  }
+  if (st != TE_OK) return st;
+  st = ensure_triples_public(h, o);
+  if (st != TE_OK) return st;
+  char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023));
+  const double* shares;
+  if (p == TE_FP64) {
+    FragWork W;
+    frag_layout(o, v, base, &W);
+    shares = W.shares;
+    st = run_frag_fp64(h, c, cf, W, s);
+  } else {
+    frag_oz_layout(o, v, B, base, &Z);
+    shares = Z.shares;
+    st = run_frag_oz(h, c, cf, Z, B, s);
+  }
+  if (st != TE_OK) return st;
+  cudaError_t e = cudaSuccess;
+  if (e_triples && nt > 0)
+    e = cudaMemcpyAsync(e_triples, shares, sizeof(double) * nt, cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess && e_out) {
     if (nt > 0) {
-      e = launch_reduce_total(W.shares, nt, e_out, s);
+      e = launch_reduce_total(shares, nt, e_out, s);
       ++h->n_launches;
     } else {
       e = cudaMemsetAsync(e_out, 0, sizeof(double), s);
@@ -294,6 +501,5 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
   if (e != cudaSuccess) return fail(TE_ECUDA, "projected energy launch: %s", cudaGetErrorString(e));
   return TE_OK;
 }
-
 
 }  // namespace te

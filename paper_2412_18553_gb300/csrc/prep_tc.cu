@@ -6,6 +6,7 @@
 // largest magnitude is an integer maximum over the high words.
 #include <algorithm>
 
+#include "adjoint_tc.cuh"
 #include "prep_tc.h"
 #include "strided.h"
 
@@ -27,13 +28,6 @@ __device__ __forceinline__ double round_sig(double x) {
 
 __device__ __forceinline__ uint32_t bf16_bits(double x) {  // x exact in BF16
   return __float_as_uint((float)x) >> 16;
-}
-
-// d 2^-shift in BF16 for an integer |d| <= 128: exact, so the upper half of
-// the float is the value (the sum with 1.5 2^23 holds d in its low bits)
-__device__ __forceinline__ uint32_t digit_bits(int d, int shift) {
-  const float f = __fsub_rn(__uint_as_float(0x4B400000u + (uint32_t)d), 12582912.0f);
-  return __float_as_uint(__fmul_rn(f, __uint_as_float((uint32_t)(127 - shift) << 23))) >> 16;
 }
 
 // The slices m_k of t = x 2^-e, |t| < 1, by repeated rounding to nearest even:
@@ -85,12 +79,12 @@ __device__ __forceinline__ void split_value(double x, int e, uint32_t* w) {
     int m[NS];
     rint_digits<BETA, NS>(x, e, m);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) w[k] = digit_bits(m[k], BETA * (k + 1));
+    for (int k = 0; k < NS; ++k) w[k] = digit_bf16(m[k], BETA * (k + 1));
   } else if constexpr (MODE == TC_SLICE4 || MODE == TC_SLICE5) {
     int d[NS];
     slice_digits_int<NS>(x, e, d);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) w[k] = digit_bits(d[k], 7 * (k + 1));
+    for (int k = 0; k < NS; ++k) w[k] = digit_bf16(d[k], 7 * (k + 1));
   } else if constexpr (MODE == TC_BF16X3) {
     const double h = round_sig<8>(x);
     w[0] = bf16_bits(h);
@@ -102,12 +96,9 @@ __device__ __forceinline__ void split_value(double x, int e, uint32_t* w) {
   }
 }
 
-// e with 2^e > m, from the high word of m (0 for zero)
-__device__ __forceinline__ int exp_of_hi(unsigned int hi) { return hi == 0u ? 0 : (int)((hi >> 20) & 0x7FFu) - 1022; }
-
 // entries of the energy modes' scale table from max |ovvv|, |t2|, |ooov|
 __device__ __forceinline__ int energy_exp(const unsigned int* maxhi, int which) {
-  const int ev = exp_of_hi(maxhi[0]), et = exp_of_hi(maxhi[1]), eo = exp_of_hi(maxhi[2]);
+  const int ev = exp_of_high(maxhi[0]), et = exp_of_high(maxhi[1]), eo = exp_of_high(maxhi[2]);
   const int U = max(ev + et, et + eo);
   return which == 0 ? U - et : (which == 1 ? et : (which == 2 ? U - eo : (which == 3 ? eo : U)));
 }
@@ -122,7 +113,7 @@ constexpr int SPLIT_THREADS = 256;
 constexpr int SPLIT_CHUNKS = 4;  // chunks of four elements per thread (rows)
 
 __device__ __forceinline__ int row_exp(const SplitJob& J, const SplitScales& sc, uint32_t group) {
-  if (J.gexp) return exp_of_hi(sc.group_hi[(J.gexp - sc.group_exps) + group]);
+  if (J.gexp) return exp_of_high(sc.group_hi[(J.gexp - sc.group_exps) + group]);
   return sc.maxhi ? energy_exp(sc.maxhi, J.which) : 0;
 }
 
@@ -270,7 +261,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_split(const __grid_constant__
   const int64_t blk = (int64_t)blockIdx.x - J.block0;
   if (blockIdx.x == 0) {
     if (L.sc.maxhi && threadIdx.x < 5) L.sc.exps[threadIdx.x] = energy_exp(L.sc.maxhi, (int)threadIdx.x);
-    for (int g = threadIdx.x; g < L.sc.ngroups; g += SPLIT_THREADS) L.sc.group_exps[g] = exp_of_hi(L.sc.group_hi[g]);
+    for (int g = threadIdx.x; g < L.sc.ngroups; g += SPLIT_THREADS) L.sc.group_exps[g] = exp_of_high(L.sc.group_hi[g]);
   }
   if (J.kind == SPLIT_ROWS) split_rows<MODE>(J, L.sc, blk);
   else if (J.kind == SPLIT_COLS) split_cols<MODE>(J, L.sc, blk);
@@ -402,7 +393,7 @@ template <int NS>
 __global__ void __launch_bounds__(256) k_slice_planes(const double* __restrict__ x, int64_t n,
                                                       const unsigned int* __restrict__ xhi, int* __restrict__ e_out,
                                                       unsigned short* __restrict__ planes) {
-  const int e = exp_of_hi(*xhi);
+  const int e = exp_of_high(*xhi);
   if (blockIdx.x == 0 && threadIdx.x == 0) *e_out = e;
   const bool vec = (n & 3) == 0;
   for (int64_t i = 4 * (blockIdx.x * 256LL + threadIdx.x); i < n; i += 4 * 256LL * gridDim.x) {
@@ -412,7 +403,7 @@ __global__ void __launch_bounds__(256) k_slice_planes(const double* __restrict__
       int d[NS];
       rint_digits_wide<NS>(i + j < n ? __ldg(x + i + j) : 0.0, e, d);
 #pragma unroll
-      for (int k = 0; k < NS; ++k) w[j][k] = digit_bits(d[k], 7 * (k + 1));
+      for (int k = 0; k < NS; ++k) w[j][k] = digit_bf16(d[k], 7 * (k + 1));
     }
 #pragma unroll
     for (int k = 0; k < NS; ++k) {

@@ -23,7 +23,6 @@ struct AdjArgs {
   double* dY;           // [v^3]
   double* dD;           // [v^3]
   double* epart;        // per-block partial energies (unweighted by gE: m/3 e)
-  unsigned long long* dwmax;  // if set: max |dW~| (bit pattern of a non-negative double)
   double* dpart;        // per-block sums of dD (the orbital-energy gradient of the triple's occupied indices)
 };
 

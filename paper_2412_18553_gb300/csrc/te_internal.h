@@ -32,7 +32,7 @@ enum : unsigned int {
 // arrays, or with `groups` of ovvv[p], t2[r,q], ooov[p,:,r,:] and, for t2L,
 // t2[:,q].
 struct MaxOut {
-  unsigned int *ovvv, *t2, *ooov, *bov, *bvv, *t2L;
+  unsigned int *ovvv, *t2, *ooov, *bov, *bvv, *t2L, *ovov, *t1;
   bool groups;
 };
 // err null: the magnitudes only, no checks.
@@ -155,14 +155,18 @@ te_status run_vjp_fp64(Handle* h, const te_cluster* c, int64_t t_begin, int64_t 
                        double* e_out, te_cluster_grad* g, cudaStream_t s);
 // fragment-projected E(T) (vjp.cu): cf device [nocc][nocc]; precision TE_FP64 or
 // exact slices; per-triple shares to e_triples (nullable), total to e_out (nullable)
-size_t frag_bytes(int64_t o, int64_t v, te_precision p, int num_sms);
+size_t frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p);
 te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precision p, double* e_out,
                    double* e_triples, cudaStream_t s);
-// workspace bytes of the two adjoints (vjp.cu)
+// workspace bytes of the two adjoints (vjp.cu, adjoint_tc.cu)
 size_t vjp_fp64_bytes(int64_t o, int64_t v);
-size_t vjp_tc_bytes(int64_t o, int64_t v, int num_sms);
+size_t vjp_tc_bytes(const Handle* h, int64_t o, int64_t v);
+// threads of the adjoint epilogues stride over the orbits on this many blocks
+int adjoint_grid(int num_sms);
+// dovov[P1,x,P2,y] = (dOVS[P1,x,P2,y] + dOVS[P2,y,P1,x]) / 2
+cudaError_t launch_dovov(int o, int v, const double* dOVS, double* dovov, cudaStream_t s);
 // the same with the contractions on the tensor cores in exact BF16 slices
-// (vjp.cu); makes the value checks, which the float64 adjoint leaves to its caller
+// (adjoint_tc.cu); makes the value checks, which the float64 adjoint leaves to its caller
 te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_end, double gE,
                      double* e_out, te_cluster_grad* g, cudaStream_t s, int64_t cluster);
 

@@ -1,17 +1,24 @@
 // Exact-slice contractions on tcgen05 over tensor-map views (see view_tc.h).
 //
 // Warp roles of the persistent kernel: warp 0 issues the TMA copies (one
-// five-dimensional box per operand slice and stage), one thread of warp 1
-// issues tcgen05.mma into three FP32 accumulators in tensor memory, warps 2..9
-// (two per TMEM lane quarter, half of the N tile each) drain every
-// accumulation block into a double-float (FP32 pair) sum held in registers and
-// release the accumulators at once, so the next block's MMAs overlap the rest
-// of the epilogue.  A unit's sum goes to float64 once, at its end: GB300's
-// float64 rate is a small fraction of its FP32 rate, and a float64 update per
-// block and element cost more than the MMAs at short K.
+// five-dimensional box per operand and stage, all slices in it), warp 1 issues
+// tcgen05.mma into three FP32 accumulators in tensor memory (the whole warp in
+// step, one elected lane: the operands then sit in uniform registers; issued
+// from a single-thread branch an MMA took 75 to 80 cycles whatever its size),
+// warps 2..9 (two per TMEM lane quarter, half of the N tile each) drain every
+// accumulation block into a double-float (FP32 pair) sum held in registers, two
+// columns per packed instruction, and release the accumulators at once, so the
+// next block's MMAs overlap the rest of the epilogue.  A unit's sum leaves once,
+// at its end: GB300's float64 rate is a small fraction of its FP32 rate, and a
+// float64 update per block and element cost more than the MMAs at short K.
+//
+// Pairs of CTAs share a B tile (cta_group::2): each loads its 128 A rows and half
+// of B, rank 0 issues the MMAs of both SMs, and all bytes of the pair count on
+// rank 0's barriers; the release of a stage and of the accumulators goes to both
+// CTAs.
 // Shared memory per stage: the A slices (128 rows of 64 bytes each, 64-byte
-// swizzle, K-major) then the B slices (NT rows each).  Every wait is bounded;
-// on expiry the kernel records the error word and unwinds.
+// swizzle, K-major) then this CTA's B rows of every slice.  Every wait is
+// bounded; on expiry the kernel records the error word and unwinds.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -19,6 +26,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "fp_util.cuh"
 #include "ptx_sm100.cuh"
 #include "tc_path.h"
 #include "view_tc.h"
@@ -35,57 +43,75 @@ constexpr uint32_t VT_ROW_BYTES = VT_KC * 2;         // 64
 constexpr uint32_t VT_A_SLICE = 128u * VT_ROW_BYTES;  // 8 KB
 
 struct VtUnit {
-  int job, split, m1_0, m2_0, n0;
+  int job, split, m, n0;
   int64_t b_begin, b_end;
 };
 
-__device__ __forceinline__ VtUnit vt_decode(const VtParams& P, int64_t u) {
+// unit u; m: the m tile of CTA `rank` (PAIR: of the unit's two)
+template <bool PAIR>
+__device__ __forceinline__ VtUnit vt_decode(const VtParams& P, int64_t u, int rank) {
   VtUnit U;
-  int j = 0;
-  while (j + 1 < P.njobs && P.job[j + 1].unit0 <= u) ++j;
+  int j = 0, top = P.njobs;  // the last job with unit0 <= u
+  while (top - j > 1) {
+    const int mid = (j + top) >> 1;
+    if (P.job[mid].unit0 <= u) j = mid;
+    else top = mid;
+  }
   const VtJob& J = P.job[j];
-  int64_t l = u - J.unit0;
+  uint32_t l = (uint32_t)(u - J.unit0);
   U.job = j;
-  U.split = (int)(l % J.nsplit);
-  l /= J.nsplit;
-  const int nt = (int)(l % J.nn);
-  l /= J.nn;
-  const int m2t = (int)(l % J.nm2);
-  const int m1t = (int)(l / J.nm2);
-  U.m1_0 = m1t * J.TA;
-  U.m2_0 = m2t * J.TB;
-  U.n0 = nt * J.NT;
+  U.split = (int)(l % (uint32_t)J.nsplit);
+  l /= (uint32_t)J.nsplit;
+  const uint32_t mu = l / (uint32_t)J.nn;
+  U.n0 = (int)(l - mu * (uint32_t)J.nn) * J.NT;
+  U.m = PAIR ? 2 * (int)mu + rank : (int)mu;
   U.b_begin = J.nblocks * U.split / J.nsplit;
   U.b_end = J.nblocks * (U.split + 1) / J.nsplit;
   return U;
 }
 
-// segment and chunk range [c0, c1) of the job's accumulation block b
-__device__ __forceinline__ int vt_block(const VtJob& J, int64_t b, int* c0, int* c1) {
-  int s = 0;
-  while (s + 1 < J.nseg && b >= J.seg[s].nblk) {
-    b -= J.seg[s].nblk;
+// accumulation blocks of a unit, in order
+struct VtBlock {
+  int seg, c0, c1;  // segment (in VtParams::seg) and its chunk range
+};
+__device__ __forceinline__ VtBlock vt_first(const VtParams& P, const VtJob& J, int64_t b) {
+  int s = J.seg0;
+  for (;;) {
+    const int nblk = (P.seg[s].nchunks + J.bchunks - 1) / J.bchunks;
+    if (b < nblk) break;
+    b -= nblk;
     ++s;
   }
-  *c0 = (int)b * J.seg[s].bchunks;
-  *c1 = min(*c0 + J.seg[s].bchunks, J.seg[s].nchunks);
-  return s;
+  const int c0 = (int)b * J.bchunks;
+  return VtBlock{s, c0, min(c0 + J.bchunks, P.seg[s].nchunks)};
+}
+__device__ __forceinline__ void vt_next(const VtParams& P, const VtJob& J, VtBlock& B) {
+  if (B.c1 < P.seg[B.seg].nchunks) {
+    B.c0 = B.c1;
+  } else {
+    ++B.seg;
+    B.c0 = 0;
+    if (B.seg >= J.seg0 + J.nseg) return;  // past the last block
+  }
+  B.c1 = min(B.c0 + J.bchunks, P.seg[B.seg].nchunks);
 }
 
-__device__ __forceinline__ void vt_load(void* dst, const CUtensorMap* map, const VtRoles& R, const int* fix, int kc,
-                                        int r2, int r1, int k1, int sl, uint64_t* bar) {
+template <bool PAIR>
+__device__ __forceinline__ void vt_load(void* dst, const CUtensorMap* map, const VtRoles& R, const int16_t* fix,
+                                        int kc, int r2, int r1, int k1, uint64_t* own, uint32_t bar) {
   int c[5];
 #pragma unroll
   for (int d = 0; d < 5; ++d) {
-    int x = fix[d];
+    int x = d >= 2 ? fix[d - 2] : 0;
     if (d == R.k2) x = kc;
     if (d == R.r2) x = r2;
     if (d == R.r1) x = r1;
     if (d == R.k1) x = k1;
-    if (d == R.s) x = sl;
+    if (d == R.s) x = 0;
     c[d] = x;
   }
-  ptx::tma_load_5d(dst, map, bar, c[0], c[1], c[2], c[3], c[4]);
+  if (PAIR) ptx::tma_load_5d_pair(dst, map, bar, c[0], c[1], c[2], c[3], c[4]);
+  else ptx::tma_load_5d(dst, map, own, c[0], c[1], c[2], c[3], c[4]);
 }
 
 __device__ __forceinline__ void vt_abort(const VtParams& P, volatile int* abort_flag, unsigned site) {
@@ -96,9 +122,25 @@ __device__ __forceinline__ void vt_abort(const VtParams& P, volatile int* abort_
   }
 }
 
-template <int NS>
-__global__ void __launch_bounds__(VT_THREADS, 1)
-    k_view_tc(const __grid_constant__ VtMaps maps, const __grid_constant__ VtParams P) {
+template <bool PAIR>
+__device__ __forceinline__ void vt_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  if (PAIR) ptx::mma_pair<false>(d, a, b, idesc, acc);
+  else ptx::mma<false>(d, a, b, idesc, acc);
+}
+template <bool PAIR>
+__device__ __forceinline__ void vt_mma_acc(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+  if (PAIR) ptx::mma_acc_pair<false>(d, a, b, idesc);
+  else ptx::mma_acc<false>(d, a, b, idesc);
+}
+template <bool PAIR>
+__device__ __forceinline__ void vt_commit(uint64_t* bar) {
+  if (PAIR) ptx::mma_commit_pair(bar);
+  else ptx::mma_commit(bar);
+}
+
+// FOLD: every job of the launch is VT_STORE (view_tc.h says how they sum).
+template <int NS, bool PAIR, bool FOLD>
+__device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams& P) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                          ~uintptr_t(1023));
@@ -112,23 +154,32 @@ __global__ void __launch_bounds__(VT_THREADS, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  constexpr int W = PAIR ? 2 : 1;  // CTAs per unit
+  const int rank = PAIR ? (int)ptx::cluster_ctarank() : 0;
+  const int64_t u0 = blockIdx.x / W, ustep = gridDim.x / W;
   if (threadIdx.x == 0) {
     for (int s = 0; s < P.stages; ++s) {
       ptx::mbar_init(&full[s], 1);
       ptx::mbar_init(&empty[s], 1);
     }
     ptx::mbar_init(tfull, 1);
-    ptx::mbar_init(tempty, VT_EPI_WARPS);
+    ptx::mbar_init(tempty, W * VT_EPI_WARPS);
     ptx::mbar_init(drain, 1);
     *abort_flag = 0;
     ptx::fence_barrier_init();
   }
   if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, P.tmem_cols);
-    ptx::tmem_relinquish();
+    if (PAIR) {
+      ptx::tmem_alloc_pair(tmem_slot, P.tmem_cols);
+      ptx::tmem_relinquish_pair();
+    } else {
+      ptx::tmem_alloc(tmem_slot, P.tmem_cols);
+      ptx::tmem_relinquish();
+    }
   }
   ptx::tc_fence_before();
   __syncthreads();
+  if (PAIR) ptx::cluster_sync();  // the barriers of both CTAs are initialised before either is signalled
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -139,146 +190,164 @@ __global__ void __launch_bounds__(VT_THREADS, 1)
       int pending[8];
       for (int s = 0; s < 8; ++s) pending[s] = -1;
       bool ok = true;
-      for (int64_t u = blockIdx.x; ok && u < P.total_units; u += gridDim.x) {
-        const VtUnit U = vt_decode(P, u);
+      for (int64_t u = u0; ok && u < P.total_units; u += ustep) {
+        const VtUnit U = vt_decode<PAIR>(P, u, rank);
         const VtJob& J = P.job[U.job];
-        const uint32_t bytes = (uint32_t)NS * (VT_A_SLICE + (uint32_t)J.NT * VT_ROW_BYTES);
+        // the second tile of an odd last pair lies beyond the rows: its loads fill zeros
+        const int m1t = U.m / J.nm2, m1_0 = m1t * J.TA, m2_0 = (U.m - m1t * J.nm2) * J.TB;
+        const int br = PAIR ? U.n0 + rank * (J.NT / 2) : U.n0;
+        const uint32_t bytes = (uint32_t)NS * (W * VT_A_SLICE + (uint32_t)J.NT * VT_ROW_BYTES);
+        VtBlock B = vt_first(P, J, U.b_begin);
         for (int64_t b = U.b_begin; ok && b < U.b_end; ++b) {
-          int c0, c1;
-          const VtSeg& S = J.seg[vt_block(J, b, &c0, &c1)];
+          const VtSeg& S = P.seg[B.seg];
           const VtRoles& RA = P.roles[S.amap];
           const VtRoles& RB = P.roles[S.bmap];
-          for (int c = c0; c < c1; ++c) {
+          int k1 = B.c0 / S.nk2c, k2c = B.c0 - k1 * S.nk2c;
+          for (int c = B.c0; c < B.c1; ++c) {
             if (*abort_flag || !ptx::mbar_wait(&empty[stage], phase ^ 1u, P.wait_ns)) {
               if (!*abort_flag) vt_abort(P, abort_flag, 21);
               ok = false;
               break;
             }
-            ptx::mbar_arrive_expect_tx(&full[stage], bytes);
+            if (rank == 0) ptx::mbar_arrive_expect_tx(&full[stage], bytes);
+            const uint32_t bar = PAIR ? ptx::mapa(&full[stage], 0) : 0u;
             pending[stage] = (int)phase;
             unsigned char* sa = smem + (size_t)stage * P.stage_bytes;
             unsigned char* sb = sa + NS * VT_A_SLICE;
-            const int k1 = c / S.nk2c;
-            const int kc = (c - k1 * S.nk2c) * VT_KC;
-#pragma unroll
-            for (int sl = 0; sl < NS; ++sl) {
-              vt_load(sa + sl * VT_A_SLICE, &maps.m[S.amap], RA, S.afix, kc, U.m2_0, U.m1_0, k1, sl, &full[stage]);
-              vt_load(sb + sl * (uint32_t)J.NT * VT_ROW_BYTES, &maps.m[S.bmap], RB, S.bfix, kc, U.n0, 0, k1, sl,
-                      &full[stage]);
+            vt_load<PAIR>(sa, &maps.m[S.amap], RA, S.afix, k2c * VT_KC, m2_0, m1_0, k1, &full[stage], bar);
+            vt_load<PAIR>(sb, &maps.m[S.bmap], RB, S.bfix, k2c * VT_KC, br, 0, k1, &full[stage], bar);
+            if (++k2c == S.nk2c) {
+              k2c = 0;
+              ++k1;
             }
             if (++stage == (uint32_t)P.stages) {
               stage = 0;
               phase ^= 1u;
             }
           }
+          vt_next(P, J, B);
         }
       }
-      // copies still in flight land before the CTA exits
-      for (int s = 0; s < P.stages; ++s)
-        if (pending[s] >= 0) ptx::mbar_wait(&full[s], (uint32_t)pending[s], P.wait_ns);
+      // Before the CTA (or pair) exits: the MMAs have released every stage, so
+      // every copy has landed too.  After an expired wait they may not come:
+      // rank 0 waits for the copies it expects, and both for longer than a
+      // copy takes.
+      for (int s = 0; s < P.stages; ++s) {
+        if (pending[s] < 0) continue;
+        if (ok && !*abort_flag) ptx::mbar_wait(&empty[s], (uint32_t)pending[s], P.wait_ns);
+        else if (rank == 0) ptx::mbar_wait(&full[s], (uint32_t)pending[s], P.wait_ns);
+      }
+      if (!ok || *abort_flag) ptx::pause_ns(200000);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, acc_phase = 0;
-      bool ok = true, issued = false;
-      const uint32_t sbo = 8u * VT_ROW_BYTES;  // 8 rows of the 64-byte swizzle
-      for (int64_t u = blockIdx.x; ok && u < P.total_units; u += gridDim.x) {
-        const VtUnit U = vt_decode(P, u);
-        const VtJob& J = P.job[U.job];
-        // kind::f16, BF16 A and B (K-major), FP32 accumulation, M = 128, N = NT
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(J.NT >> 3) << 17) |
-                               ((uint32_t)(128 >> 4) << 24);
-        const uint32_t d0 = tmem_base, d1 = tmem_base + (uint32_t)J.NT, dr = tmem_base + 2u * (uint32_t)J.NT;
-        for (int64_t b = U.b_begin; ok && b < U.b_end; ++b) {
-          int c0, c1;
-          vt_block(J, b, &c0, &c1);
-          if (*abort_flag || !ptx::mbar_wait(tempty, acc_phase ^ 1u, P.wait_ns)) {
-            if (!*abort_flag) vt_abort(P, abort_flag, 22);
+    // ---------------- MMA issuer (rank 0) ----------------
+    uint32_t stage = 0, phase = 0, acc_phase = 0;
+    bool ok = true, issued = false;
+    auto wait_all = [&](uint64_t* bar, uint32_t parity, unsigned site) -> bool {
+      const int got = (!*abort_flag && ptx::mbar_wait(bar, parity, P.wait_ns)) ? 1 : 0;
+      const bool all = __all_sync(0xffffffffu, got);
+      if (!all && lane == 0 && !*abort_flag) vt_abort(P, abort_flag, site);
+      return all;
+    };
+    const uint32_t smem0 = ptx::smem_u32(smem);
+    const uint64_t desc0 = ptx::smem_desc(0, 8u * VT_ROW_BYTES, 4u);  // 8 rows of the 64-byte swizzle
+    for (int64_t u = u0; ok && rank == 0 && u < P.total_units; u += ustep) {
+      const VtUnit U = vt_decode<PAIR>(P, u, 0);
+      const VtJob& J = P.job[U.job];
+      const uint32_t NT = (uint32_t)J.NT;
+      // kind::f16, BF16 A and B (K-major), FP32 accumulation, M = 128 or 256, N = NT
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((NT >> 3) << 17) |
+                             ((uint32_t)(W * 128 >> 4) << 24);
+      const uint32_t d0 = tmem_base, d1 = tmem_base + NT, dr = tmem_base + 2u * NT;
+      const uint32_t bstep = (NT / W) * VT_ROW_BYTES >> 4;
+      VtBlock B = vt_first(P, J, U.b_begin);
+      for (int64_t b = U.b_begin; ok && b < U.b_end; ++b) {
+        if (!wait_all(tempty, acc_phase ^ 1u, 22)) {
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+        uint32_t first = 1;
+        for (int c = B.c0; c < B.c1; ++c) {
+          if (!wait_all(&full[stage], phase, 23)) {
             ok = false;
             break;
           }
           ptx::tc_fence_after();
-          uint32_t first = 1;
-          for (int c = c0; c < c1; ++c) {
-            if (*abort_flag || !ptx::mbar_wait(&full[stage], phase, P.wait_ns)) {
-              if (!*abort_flag) vt_abort(P, abort_flag, 23);
-              ok = false;
-              break;
+          const uint32_t a0 = (smem0 + stage * P.stage_bytes) >> 4;
+          const uint32_t b0 = a0 + (NS * VT_A_SLICE >> 4);
+#pragma unroll
+          for (int ks = 0; ks < VT_KC / 16; ++ks) {
+            uint64_t ad[NS], bd[NS];
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+              ad[k] = desc0 + (a0 + k * (VT_A_SLICE >> 4) + ks * 2);
+              bd[k] = desc0 + (b0 + k * bstep + ks * 2);
             }
-            ptx::tc_fence_after();
-            unsigned char* sa = smem + (size_t)stage * P.stage_bytes;
-            const uint32_t a0 = ptx::smem_u32(sa);
-            const uint32_t b0 = ptx::smem_u32(sa + NS * VT_A_SLICE);
-#pragma unroll
-            for (int ks = 0; ks < VT_KC / 16; ++ks) {
-              uint64_t ad[NS], bd[NS];
-#pragma unroll
-              for (int k = 0; k < NS; ++k) {
-                ad[k] = ptx::smem_desc(a0 + k * VT_A_SLICE + ks * 32, sbo, 4u);
-                bd[k] = ptx::smem_desc(b0 + k * (uint32_t)J.NT * VT_ROW_BYTES + ks * 32, sbo, 4u);
-              }
-              // slice products a_i b_j, i + j <= NS - 1: level 0 and level 1 in
-              // their own (exact) accumulators, the higher levels in a third
-              const uint32_t acc_in = first ? 0u : 1u;
-              ptx::mma<false>(d0, ad[0], bd[0], idesc, acc_in);
-              ptx::mma<false>(d1, ad[0], bd[1], idesc, acc_in);
-              ptx::mma<false>(d1, ad[1], bd[0], idesc, 1);
-              uint32_t rin = acc_in;
+            // slice products a_i b_j, i + j <= NS - 1: level 0 and level 1 in
+            // their own (exact) accumulators, the higher levels in a third
+            const uint32_t acc_in = first ? 0u : 1u;
+            if (ptx::elect_one()) {
+              vt_mma<PAIR>(d0, ad[0], bd[0], idesc, acc_in);
+              vt_mma<PAIR>(d1, ad[0], bd[1], idesc, acc_in);
+              vt_mma_acc<PAIR>(d1, ad[1], bd[0], idesc);
+              vt_mma<PAIR>(dr, ad[0], bd[2], idesc, acc_in);
 #pragma unroll
               for (int lev = 2; lev < NS; ++lev)
 #pragma unroll
-                for (int i = 0; i <= lev; ++i) {
-                  ptx::mma<false>(dr, ad[i], bd[lev - i], idesc, rin);
-                  rin = 1;
-                }
-              first = 0;
+                for (int i = lev == 2 ? 1 : 0; i <= lev; ++i) vt_mma_acc<PAIR>(dr, ad[i], bd[lev - i], idesc);
             }
-            issued = true;
-            ptx::mma_commit(&empty[stage]);
-            if (++stage == (uint32_t)P.stages) {
-              stage = 0;
-              phase ^= 1u;
-            }
+            first = 0;
           }
-          if (!ok) break;
-          ptx::mma_commit(tfull);
-          acc_phase ^= 1u;
+          issued = true;
+          if (ptx::elect_one()) vt_commit<PAIR>(&empty[stage]);
+          if (++stage == (uint32_t)P.stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
-      }
-      // every issued MMA completes before TMEM is released
-      if (issued) {
-        ptx::mma_commit(drain);
-        ptx::mbar_wait(drain, 0, P.wait_ns);
+        if (!ok) break;
+        if (ptx::elect_one()) vt_commit<PAIR>(tfull);
+        acc_phase ^= 1u;
+        vt_next(P, J, B);
       }
     }
+    // every issued MMA completes before TMEM is released
+    if (issued) {
+      if (ptx::elect_one()) {
+        if (PAIR) ptx::mma_commit_pair_own(drain);
+        else ptx::mma_commit(drain);
+      }
+      ptx::mbar_wait(drain, 0, P.wait_ns);
+    }
+    __syncwarp();
   } else {
-    // ---------------- epilogue: TMEM -> double-float -> float64 ----------------
+    // ---------------- epilogue: TMEM -> double-float -> output ----------------
     const int quad = warp & 3;               // the lane quarter this warp may read
     const int half = (warp - 2) >> 2;        // which half of the N tile
     const int row = quad * 32 + lane;
     const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16);
     uint32_t acc_phase = 0;
     bool ok = true;
-    for (int64_t u = blockIdx.x; ok && u < P.total_units; u += gridDim.x) {
-      const VtUnit U = vt_decode(P, u);
+    for (int64_t u = u0; ok && u < P.total_units; u += ustep) {
+      const VtUnit U = vt_decode<PAIR>(P, u, rank);
       const VtJob& J = P.job[U.job];
-      const int m1 = U.m1_0 + row / J.TB, m2 = U.m2_0 + row % J.TB;
+      const int m1t = U.m / J.nm2;
+      const int m1 = m1t * J.TA + row / J.TB, m2 = (U.m - m1t * J.nm2) * J.TB + row % J.TB;
       const bool valid = m1 < J.M1 && m2 < J.M2;
       const int ncol = J.NT >> 1, c_lo = half * ncol;
       // the unit's sum is kept relative to 2^eref, the largest scale of the
       // job's segments: every block's weight 2^(e - eref) <= 1 is exact in FP32
       int eref = -100000;
-      for (int q = 0; q < J.nseg; ++q) eref = max(eref, *J.seg[q].ea + *J.seg[q].eb);
-      float hi[VT_HALF], lo[VT_HALF];
+      for (int q = lane; q < J.nseg; q += 32) eref = max(eref, *P.seg[J.seg0 + q].ea + *P.seg[J.seg0 + q].eb);
+      eref = __reduce_max_sync(0xffffffffu, eref);
+      f2 hi[VT_HALF / 2], lo[VT_HALF / 2];
 #pragma unroll
-      for (int q = 0; q < VT_HALF; ++q) {
-        hi[q] = 0.f;
-        lo[q] = 0.f;
-      }
+      for (int q = 0; q < VT_HALF / 2; ++q) hi[q] = lo[q] = f2{0ull};
+      VtBlock B = vt_first(P, J, U.b_begin);
       for (int64_t b = U.b_begin; b < U.b_end; ++b) {
-        int c0, c1;
-        const VtSeg& S = J.seg[vt_block(J, b, &c0, &c1)];
+        const VtSeg& S = P.seg[B.seg];
+        const float wk1 = ldexpf(S.sign < 0 ? -1.f : 1.f, *S.ea + *S.eb - eref);
         int got = 0;
         if (!*abort_flag) got = ptx::mbar_wait(tfull, acc_phase, P.wait_ns) ? 1 : 0;
         // warp-uniform: tcgen05.ld below is .sync.aligned
@@ -288,7 +357,7 @@ __global__ void __launch_bounds__(VT_THREADS, 1)
           break;
         }
         ptx::tc_fence_after();
-        const float wk = ldexpf(S.alpha < 0.0 ? -1.f : 1.f, *S.ea + *S.eb - eref);
+        const f2 wk = f2_make(wk1, wk1);
 #pragma unroll
         for (int q = 0; q < VT_HALF / 8; ++q) {
           if (8 * q < ncol) {
@@ -296,61 +365,132 @@ __global__ void __launch_bounds__(VT_THREADS, 1)
             float a0[8], a1[8], a2[8];
             ptx::tmem_ld8x3(tbase + cc, tbase + (uint32_t)J.NT + cc, tbase + 2u * (uint32_t)J.NT + cc, a0, a1, a2);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < 4; ++j) {
+              f2& H = hi[4 * q + j];
+              f2& L = lo[4 * q + j];
               // level 0 + level 1 exactly (both exact FP32 sums), the rest rounded
-              const float s0 = __fadd_rn(a0[j], a1[j]);
-              const float bb = __fsub_rn(s0, a0[j]);
-              const float e0 = __fadd_rn(__fsub_rn(a0[j], __fsub_rn(s0, bb)), __fsub_rn(a1[j], bb));
-              const float x = __fmul_rn(s0, wk), y = __fmul_rn(__fadd_rn(e0, a2[j]), wk);
-              // (hi, lo) += (x, y)
-              const float t = __fadd_rn(hi[8 * q + j], x);
-              const float tb = __fsub_rn(t, hi[8 * q + j]);
-              const float te = __fadd_rn(__fsub_rn(hi[8 * q + j], __fsub_rn(t, tb)), __fsub_rn(x, tb));
-              const float l = __fadd_rn(te, __fadd_rn(lo[8 * q + j], y));
-              hi[8 * q + j] = __fadd_rn(t, l);
-              lo[8 * q + j] = __fsub_rn(l, __fsub_rn(hi[8 * q + j], t));
+              f2 s0, e0, t, te;
+              f2_two_sum(f2_make(a0[2 * j], a0[2 * j + 1]), f2_make(a1[2 * j], a1[2 * j + 1]), s0, e0);
+              const f2 x = f2_mul(s0, wk), y = f2_mul(f2_add(e0, f2_make(a2[2 * j], a2[2 * j + 1])), wk);
+              f2_two_sum(H, x, t, te);
+              f2 l;
+              if constexpr (FOLD) {
+                l = f2_add(te, f2_add(L, y));
+              } else {  // y can be 2^-14 of the operands' scale, far above the last bits of lo
+                f2 t2, te2;
+                f2_two_sum(t, y, t2, te2);
+                l = f2_add(L, f2_add(te, te2));
+                t = t2;
+              }
+              H = f2_add(t, l);
+              L = f2_sub(l, f2_sub(H, t));
             }
           }
         }
         ptx::tc_fence_before();
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(tempty);
+        if (lane == 0) {
+          if (PAIR) ptx::mbar_arrive_cluster(ptx::mapa(tempty, 0));
+          else ptx::mbar_arrive(tempty);
+        }
         acc_phase ^= 1u;
+        vt_next(P, J, B);
       }
       if (!ok || !valid) continue;
+      if (J.out == VT_PAIR) {
+        float2* dst = static_cast<float2*>(J.C) + (int64_t)m1 * J.c_m1 + (int64_t)m2 * J.c_m2 + U.n0 + c_lo;
+#pragma unroll
+        for (int q = 0; q < VT_HALF / 4; ++q) {
+          if (4 * q < ncol && U.n0 + c_lo + 4 * q < J.N) {
+            float h[4], l[4];
+            f2_get(hi[2 * q], h[0], h[1]);
+            f2_get(hi[2 * q + 1], h[2], h[3]);
+            f2_get(lo[2 * q], l[0], l[1]);
+            f2_get(lo[2 * q + 1], l[2], l[3]);
+            if (J.vec) {
+              asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + 4 * q), "f"(h[0]), "f"(l[0]),
+                           "f"(h[1]), "f"(l[1]), "f"(h[2]), "f"(l[2]), "f"(h[3]), "f"(l[3])
+                           : "memory");
+            } else {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (U.n0 + c_lo + 4 * q + j < J.N) dst[4 * q + j] = make_float2(h[j], l[j]);
+            }
+          }
+        }
+        continue;
+      }
       const double scale = ldexp(J.jalpha, eref);
       double* dst;
       int64_t dn;
-      const bool store = J.nsplit > 1 || J.overwrite;
+      const bool store = J.nsplit > 1 || J.out == VT_STORE;
       if (J.nsplit > 1) {
         dst = J.part + ((int64_t)U.split * ((int64_t)J.M1 * J.M2) + (int64_t)m1 * J.M2 + m2) * J.N;
         dn = 1;
       } else {
-        dst = J.C + (int64_t)m1 * J.c_m1 + (int64_t)m2 * J.c_m2;
+        dst = static_cast<double*>(J.C) + (int64_t)m1 * J.c_m1 + (int64_t)m2 * J.c_m2;
         dn = J.c_n;
       }
+      dst += (int64_t)(U.n0 + c_lo) * dn;
 #pragma unroll
-      for (int q = 0; q < VT_HALF / 8; ++q) {
-        if (8 * q < ncol) {
-          const int n0 = U.n0 + c_lo + 8 * q;
-          double old[8];
+      for (int q = 0; q < VT_HALF / 4; ++q) {
+        const int left = J.N - (U.n0 + c_lo + 4 * q);
+        if (4 * q < ncol && left > 0) {
+          double* d = dst + 4 * q * dn;
+          double old[4];
+          if (store) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) old[j] = (!store && n0 + j < J.N) ? dst[(int64_t)(n0 + j) * dn] : 0.0;
+            for (int j = 0; j < 4; ++j) old[j] = 0.0;
+          } else if (J.vec) {
+            asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+                         : "=d"(old[0]), "=d"(old[1]), "=d"(old[2]), "=d"(old[3])
+                         : "l"(d)
+                         : "memory");
+          } else {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (n0 + j < J.N)
-              dst[(int64_t)(n0 + j) * dn] = fma(scale, (double)hi[8 * q + j] + (double)lo[8 * q + j], old[j]);
+            for (int j = 0; j < 4; ++j) old[j] = j < left ? d[j * dn] : 0.0;
+          }
+          float h[4], l[4];
+          f2_get(hi[2 * q], h[0], h[1]);
+          f2_get(hi[2 * q + 1], h[2], h[3]);
+          f2_get(lo[2 * q], l[0], l[1]);
+          f2_get(lo[2 * q + 1], l[2], l[3]);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) old[j] = fma(scale, to_double(h[j]) + to_double(l[j]), old[j]);
+          if (J.vec) {
+            asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(d), "d"(old[0]), "d"(old[1]), "d"(old[2]),
+                         "d"(old[3])
+                         : "memory");
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (j < left) d[j * dn] = old[j];
+          }
         }
       }
     }
   }
 
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
+  if (PAIR) ptx::cluster_sync();  // neither CTA leaves while the other's MMAs or signals may reach it
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, P.tmem_cols);
+    if (PAIR) ptx::tmem_dealloc_pair(tmem_base, P.tmem_cols);
+    else ptx::tmem_dealloc(tmem_base, P.tmem_cols);
   }
+}
+
+template <int NS>
+__global__ void __launch_bounds__(VT_THREADS, 1)
+    k_view_tc(const __grid_constant__ VtMaps maps, const __grid_constant__ VtParams P) {
+  view_tc_body<NS, false, false>(maps, P);
+}
+template <int NS, bool FOLD>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(VT_THREADS, 1)
+    k_view_tc_pair(const __grid_constant__ VtMaps maps, const __grid_constant__ VtParams P) {
+  view_tc_body<NS, true, FOLD>(maps, P);
 }
 
 // C[(m1, m2), n] += sum_z part[z][(m1, m2)][n], z in order, for every split job
@@ -367,7 +507,7 @@ __global__ void __launch_bounds__(256) k_vt_reduce(const __grid_constant__ VtPar
     for (int z = 0; z < J.nsplit; ++z) s += J.part[z * total + x];
     const int64_t m = x / J.N;
     const int n = (int)(x - m * J.N);
-    double* cp = J.C + (m / J.M2) * J.c_m1 + (m % J.M2) * J.c_m2 + (int64_t)n * J.c_n;
+    double* cp = static_cast<double*>(J.C) + (m / J.M2) * J.c_m1 + (m % J.M2) * J.c_m2 + (int64_t)n * J.c_n;
     *cp += s;
   }
 }
@@ -427,16 +567,20 @@ PFN_cuTensorMapEncodeTiled_v12000 vt_encoder() {
 
 }  // namespace
 
-void vt_begin(VtBuild* b, int ns) {
-  std::memset(b, 0, sizeof(*b));
+void vt_begin(VtBuild* b, int ns, bool pair) {
+  // the tables' entries are written whole when they are taken
+  b->P.njobs = b->P.nsegs = 0;
   b->P.ns = ns;
+  b->nmaps = 0;
+  b->pair = pair;
+  b->full = false;
   for (int q = 0; q < VT_BANK_MAX; ++q) b->slot[q] = -1;
 }
 
 te_status vt_bank_add(VtBank* k, const VtView& v, int rows_r2, int rows_r1, int* idx) {
   if (k->n >= VT_BANK_MAX) return fail(TE_EINVAL, "view GEMM: more than %d tensor maps", VT_BANK_MAX);
   const VtRoles& R = v.roles;
-  if (R.k2 != 0 || v.stride[0] != 1 || R.r2 <= 0 || R.s <= 0 || (R.r1 >= 0 && R.r1 < R.r2))
+  if (R.k2 != 0 || v.stride[0] != 1 || R.r2 <= 0 || R.s < R.r2 || R.s < R.r1 || (R.r1 >= 0 && R.r1 < R.r2))
     return fail(TE_EINVAL, "view GEMM: bad view roles");
   if ((reinterpret_cast<uintptr_t>(v.base) & 15) != 0) return fail(TE_EINVAL, "view GEMM: base not 16-byte aligned");
   if (rows_r2 < 1 || rows_r2 > 256 || rows_r1 < 1 || rows_r1 > 256) return fail(TE_EINVAL, "view GEMM: box rows");
@@ -460,12 +604,14 @@ te_status vt_bank_add(VtBank* k, const VtView& v, int rows_r2, int rows_r1, int*
   box[R.k2] = VT_KC;
   box[R.r2] = (cuuint32_t)rows_r2;
   if (R.r1 >= 0) box[R.r1] = (cuuint32_t)rows_r1;
+  box[R.s] = (cuuint32_t)v.dims[R.s];  // every slice in one copy
   CUtensorMap* m = &k->m[k->n];
   CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(v.base), gd, gs, box, e1,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(TE_ECUDA, "view GEMM: tensor map encoding failed (CUresult %d)", (int)r);
   k->r[k->n] = R;
+  k->r[k->n].rows = (int16_t)(rows_r2 * rows_r1);
   *idx = k->n++;
   return TE_OK;
 }
@@ -485,85 +631,94 @@ int64_t vt_seg_blocks(int K1, int K2, int bchunks) {
   return (nchunks + bchunks - 1) / bchunks;
 }
 
-VtJob* vt_job(VtBuild* b, int M1, int M2, int N, int TA, int TB, int NT, double* C, int64_t c_m1, int64_t c_m2,
-              int64_t c_n, int overwrite) {
-  if (b->P.njobs >= VT_MAX_JOBS) return nullptr;
+VtJob* vt_job(VtBuild* b, int M1, int M2, int N, int TA, int TB, int NT, void* C, int64_t c_m1, int64_t c_m2,
+              int64_t c_n, VtOut out) {
+  if (b->P.njobs >= VT_MAX_JOBS) {
+    b->full = true;
+    return nullptr;
+  }
   VtJob* j = &b->P.job[b->P.njobs++];
-  std::memset(j, 0, sizeof(*j));
+  *j = VtJob{};
   j->M1 = M1;
   j->M2 = M2;
   j->N = N;
-  j->TA = TA;
-  j->TB = TB;
-  j->NT = NT;
-  j->nm1 = (M1 + TA - 1) / TA;
+  j->TA = (int16_t)TA;
+  j->TB = (int16_t)TB;
+  j->NT = (int16_t)NT;
   j->nm2 = (M2 + TB - 1) / TB;
+  const int nm = (M1 + TA - 1) / TA * j->nm2;
+  j->nmu = b->pair ? (nm + 1) / 2 : nm;
   j->nn = (N + NT - 1) / NT;
   j->nsplit = 1;
+  j->seg0 = (int16_t)b->P.nsegs;
+  j->bchunks = VT_BLOCK_CHUNKS;
   j->C = C;
   j->c_m1 = c_m1;
   j->c_m2 = c_m2;
   j->c_n = c_n;
-  j->overwrite = overwrite;
+  j->out = (int16_t)out;
   j->jalpha = 1.0;
   return j;
 }
 
-void vt_seg(VtJob* j, int amap, int bmap, int K1, int K2, const int* afix, const int* bfix, const int* ea,
-            const int* eb, double alpha) {
-  if (j->nseg >= VT_MAX_SEGS) {  // vt_finish reports it
-    j->seg[0].amap = -1;
+void vt_seg(VtBuild* b, int amap, int bmap, int K1, int K2, const int* afix, const int* bfix, const int* ea,
+            const int* eb, int sign) {
+  if (b->P.nsegs >= VT_MAX_SEGS || b->P.njobs == 0 || amap < 0 || bmap < 0) {  // vt_finish reports it
+    b->full = true;
     return;
   }
-  VtSeg& s = j->seg[j->nseg++];
+  VtJob& j = b->P.job[b->P.njobs - 1];
+  ++j.nseg;
+  VtSeg& s = b->P.seg[b->P.nsegs++];
   s.amap = (int8_t)amap;
   s.bmap = (int8_t)bmap;
-  s.K1 = K1;
-  s.K2 = K2;
   s.nk2c = (K2 + VT_KC - 1) / VT_KC;
   s.nchunks = K1 * s.nk2c;
-  s.bchunks = VT_BLOCK_CHUNKS;
-  s.nblk = (int)vt_seg_blocks(K1, K2);
-  for (int d = 0; d < 5; ++d) {
-    s.afix[d] = afix ? afix[d] : 0;
-    s.bfix[d] = bfix ? bfix[d] : 0;
+  for (int d = 0; d < 3; ++d) {
+    s.afix[d] = (int16_t)(afix ? afix[d] : 0);
+    s.bfix[d] = (int16_t)(bfix ? bfix[d] : 0);
   }
   s.ea = ea;
   s.eb = eb;
-  s.alpha = alpha;
-  j->nblocks += s.nblk;
+  s.sign = (int16_t)sign;
+  j.nblocks += (s.nchunks + VT_BLOCK_CHUNKS - 1) / VT_BLOCK_CHUNKS;
 }
 
-int64_t vt_splits(int64_t tiles, int64_t nblocks, int num_sms) {
+int64_t vt_splits(int64_t tiles, int64_t nblocks, int units_at_once) {
   // jobs with long K only (the partials cost a reduction pass): enough units
   // for about four waves over the SMs, and at most 64 blocks per unit
   if (nblocks < 8) return 1;
-  const int64_t want = std::max<int64_t>((nblocks + 63) / 64, (4LL * num_sms + tiles - 1) / tiles);
+  const int64_t want = std::max<int64_t>((nblocks + 63) / 64, (4LL * units_at_once + tiles - 1) / tiles);
   return std::max<int64_t>(1, std::min<int64_t>(nblocks, want));
 }
 
 te_status vt_finish(VtBuild* b, int num_sms, double* part_scratch, int64_t scratch_cap, int64_t* used) {
-  int64_t units = 0, off = 0, red = 0;
+  if (b->full) return fail(TE_EINVAL, "view GEMM: launch tables full, or a segment without a tensor map");
+  const int at_once = std::max(1, b->pair ? num_sms / 2 : num_sms);
+  int64_t units = 0, off = 0, red = 0, launch_tiles = 0;
+  for (int q = 0; q < b->P.njobs; ++q) launch_tiles += (int64_t)b->P.job[q].nmu * b->P.job[q].nn;
   for (int q = 0; q < b->P.njobs; ++q) {
     VtJob& J = b->P.job[q];
     if (J.nseg == 0) return fail(TE_EINVAL, "view GEMM: job without segments");
-    for (int g = 0; g < J.nseg; ++g) {
-      if (J.seg[g].amap < 0 || J.seg[g].bmap < 0 || J.seg[g].amap >= b->nmaps || J.seg[g].bmap >= b->nmaps)
-        return fail(TE_EINVAL, "view GEMM: segment without a tensor map");
-      if (J.seg[g].alpha != 1.0 && J.seg[g].alpha != -1.0)
-        return fail(TE_EINVAL, "view GEMM: segment factor other than +-1");
+    if ((J.out == VT_STORE) != (b->pair && b->P.job[0].out == VT_STORE))
+      return fail(TE_EINVAL, "view GEMM: VT_STORE jobs go in a pair launch of their own");
+    int kblocks = 0;
+    for (int g = J.seg0; g < J.seg0 + J.nseg; ++g) {
+      const VtSeg& S = b->P.seg[g];
+      if (S.sign != 1 && S.sign != -1) return fail(TE_EINVAL, "view GEMM: segment factor other than +-1");
+      if (b->P.roles[S.amap].rows != 128 || b->P.roles[S.bmap].rows != (b->pair ? J.NT / 2 : J.NT))
+        return fail(TE_EINVAL, "view GEMM: box rows do not fit the tile");
+      kblocks += (S.nchunks + VT_SPLIT_CHUNKS - 1) / VT_SPLIT_CHUNKS;
     }
-    const int64_t tiles = (int64_t)J.nm1 * J.nm2 * J.nn;
-    if (!J.overwrite && part_scratch && tiles < num_sms && J.nblocks * VT_BLOCK_CHUNKS >= 8 * VT_SPLIT_CHUNKS) {
-      J.nblocks = 0;
-      for (int g = 0; g < J.nseg; ++g) {
-        J.seg[g].bchunks = VT_SPLIT_CHUNKS;
-        J.seg[g].nblk = (int)vt_seg_blocks(J.seg[g].K1, J.seg[g].K2, VT_SPLIT_CHUNKS);
-        J.nblocks += J.seg[g].nblk;
-      }
-    }
+    // the other jobs of the launch share the SMs: a job alone gets its part of them
+    const int64_t tiles = (int64_t)J.nmu * J.nn;
+    const int64_t share = std::max<int64_t>(1, at_once * tiles / std::max<int64_t>(1, launch_tiles));
     int64_t ns = 1;
-    if (!J.overwrite && part_scratch) ns = vt_splits(tiles, J.nblocks, num_sms);
+    if (J.out == VT_ADD && part_scratch && launch_tiles < at_once && J.nblocks * VT_BLOCK_CHUNKS >= 8 * VT_SPLIT_CHUNKS) {
+      J.bchunks = VT_SPLIT_CHUNKS;
+      J.nblocks = kblocks;
+    }
+    if (J.out == VT_ADD && part_scratch) ns = vt_splits(tiles, J.nblocks, (int)share);
     const int64_t mn = (int64_t)J.M1 * J.M2 * J.N;
     while (ns > 1 && off + ns * mn > scratch_cap) ns = std::max<int64_t>(1, ns / 2);
     J.nsplit = (int)ns;
@@ -571,10 +726,17 @@ te_status vt_finish(VtBuild* b, int num_sms, double* part_scratch, int64_t scrat
     J.red0 = 0;
     if (ns > 1) {
       J.part = part_scratch + off;
-      off += ns * mn;
+      off += (ns * mn + 3) / 4 * 4;
       J.red0 = red;
       red += mn;
     }
+    // four columns per access: contiguous, whole groups of four, 32-byte aligned
+    const int64_t es = 8;
+    if (ns > 1) J.vec = J.N % 4 == 0 ? 1 : 0;
+    else
+      J.vec = J.c_n == 1 && J.N % 4 == 0 && J.c_m1 % 4 == 0 && J.c_m2 % 4 == 0 &&
+              (reinterpret_cast<uintptr_t>(J.C) % (4 * es)) == 0;
+    if (ns > 1 && (reinterpret_cast<uintptr_t>(J.part) % (4 * es)) != 0) J.vec = 0;
     J.unit0 = units;
     units += tiles * ns;
   }
@@ -584,16 +746,17 @@ te_status vt_finish(VtBuild* b, int num_sms, double* part_scratch, int64_t scrat
   return TE_OK;
 }
 
-int64_t vt_split_doubles(int64_t tiles, int64_t nblocks, int64_t mn, int num_sms) {
-  const int64_t ns = vt_splits(tiles, nblocks, num_sms);
+int64_t vt_split_doubles(int64_t tiles, int64_t nblocks, int64_t mn, int units_at_once) {
+  const int64_t ns = vt_splits(tiles, nblocks, units_at_once);
   return ns > 1 ? ns * mn : 0;
 }
 
 template <int NS>
 static cudaError_t vt_launch_ns(const VtBuild* b, int grid, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_view_tc<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto* k = !b->pair ? k_view_tc<NS> : (b->P.job[0].out == VT_STORE ? k_view_tc_pair<NS, true> : k_view_tc_pair<NS, false>);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_view_tc<NS><<<(unsigned)grid, VT_THREADS, smem, s>>>(b->maps, b->P);
+  k<<<(unsigned)grid, VT_THREADS, smem, s>>>(b->maps, b->P);
   return cudaGetLastError();
 }
 
@@ -603,14 +766,14 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s) {
   int nt_max = 16;
   for (int q = 0; q < P.njobs; ++q) {
     const VtJob& J = P.job[q];
-    if (J.NT % 16 != 0 || J.NT < 16 || J.NT > VT_NT_MAX || J.TA * J.TB != 128)
+    if (J.NT % 32 != 0 || J.NT < 32 || J.NT > VT_NT_MAX || J.TA * J.TB != 128)
       return fail(TE_EINVAL, "view GEMM: tile %d x %d x %d", J.TA, J.TB, J.NT);
-    nt_max = std::max(nt_max, J.NT);
+    nt_max = std::max<int>(nt_max, J.NT);
   }
   P.nt_max = nt_max;
-  P.stage_bytes = (uint32_t)P.ns * (VT_A_SLICE + (uint32_t)nt_max * VT_ROW_BYTES);
+  P.stage_bytes = (uint32_t)P.ns * (VT_A_SLICE + (uint32_t)(b->pair ? nt_max / 2 : nt_max) * VT_ROW_BYTES);
   const size_t avail = h->smem_optin > 2048 ? h->smem_optin - 2048 : 0;
-  P.stages = (int)std::min<size_t>(4, avail / P.stage_bytes);
+  P.stages = (int)std::min<size_t>(8, avail / P.stage_bytes);
   if (P.stages < 2) return fail(TE_EUNSUPPORTED, "view GEMM: not enough shared memory for two stages");
   uint32_t cols = 32;
   while (cols < 3u * (uint32_t)nt_max) cols <<= 1;
@@ -618,7 +781,8 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s) {
   P.err = h->d_err;
   P.wait_ns = h->wait_limit_ns;
   const size_t smem = (size_t)P.stages * P.stage_bytes + 1024 + 256;
-  const int grid = (int)std::min<int64_t>(P.total_units, std::max(1, h->num_sms));
+  const int grid = b->pair ? 2 * (int)std::min<int64_t>(P.total_units, std::max(1, h->num_sms / 2))
+                           : (int)std::min<int64_t>(P.total_units, std::max(1, h->num_sms));
   cudaError_t e = P.ns == 5 ? vt_launch_ns<5>(b, grid, smem, s) : vt_launch_ns<4>(b, grid, smem, s);
   if (e != cudaSuccess) return fail(TE_ECUDA, "view GEMM launch: %s", cudaGetErrorString(e));
   ++h->n_launches;
@@ -633,7 +797,7 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s) {
 
 int vt_ntile(int64_t n) {
   const int64_t t = (n + VT_NT_MAX - 1) / VT_NT_MAX;
-  return (int)(((n + t - 1) / t + 15) / 16 * 16);
+  return (int)(((n + t - 1) / t + 31) / 32 * 32);
 }
 
 te_status vt_slice_maps(VtBank* k, const SliceSet& S, int o, int v, int nt, int* idx) {
@@ -649,9 +813,9 @@ te_status vt_slice_maps(VtBank* k, const SliceSet& S, int o, int v, int nt, int*
       {S.ovvv, {V, V, V, NS, O}, {1, V * vp, vp, (uint64_t)S.ovvv_plane, (uint64_t)S.ovvv_p}, XY, 16, 8},
       {S.t2L, {O, V, V, NS, O}, {1, op, V * op, (uint64_t)S.t2L_plane, (uint64_t)S.t2L_q}, XY, 16, 8},
       {S.t2L, {O, V, V, NS, O}, {1, V * op, op, (uint64_t)S.t2L_plane, (uint64_t)S.t2L_q}, XY, 16, 8},
-      {S.t2, {V, V, NS, O, O}, {1, vp, (uint64_t)S.t2_plane, (uint64_t)S.t2_rq, O * (uint64_t)S.t2_rq}, ROW, nt, 1},
+      {S.t2, {V, V, NS, O, O}, {1, vp, (uint64_t)S.t2_plane, (uint64_t)S.t2_rq, O * (uint64_t)S.t2_rq}, ROW, nt / 2, 1},
       {S.nooT, {O, V, NS, O, O}, {1, op, (uint64_t)S.nooT_plane, (uint64_t)S.nooT_pr, O * (uint64_t)S.nooT_pr}, ROW,
-       nt, 1},
+       nt / 2, 1},
   };
   for (int q = 0; q < 6; ++q) {
     VtView w;

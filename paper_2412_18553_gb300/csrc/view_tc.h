@@ -12,10 +12,15 @@
 // blocks in double-float (FP32 pairs, 2^-48 relative) and its total to C (or
 // to a split-K partial) in float64.
 //
-// Work unit: (job, m tile, n tile, K split).  A unit owns its output tile (or
-// its split's partial tile) for the whole launch, so no two units write the
-// same element and the result has a fixed summation order.  Jobs of one
-// launch must write disjoint outputs.
+// Work unit: (job, m tile or pair of m tiles, n tile, K split).  A unit owns its
+// output tile (or its split's partial tile) for the whole launch, so no two
+// units write the same element and the result has a fixed summation order.
+// Jobs of one launch must write disjoint outputs.
+//
+// A launch runs on pairs of CTAs (cta_group::2: two m tiles against one B tile of
+// which each CTA holds half) or on lone CTAs, for jobs whose rows fill one
+// tile only.  The B maps of a pair launch have boxes of NT / 2 rows, those of a
+// lone launch NT rows.
 #pragma once
 #include <cuda.h>
 
@@ -25,46 +30,55 @@
 
 namespace te {
 
-constexpr int VT_MAX_MAPS = 16;
-constexpr int VT_MAX_SEGS = 8;
-constexpr int VT_MAX_JOBS = 12;
+constexpr int VT_MAX_MAPS = 20;
+constexpr int VT_MAX_SEGS = 288;     // per launch: the tables travel as kernel parameters (32 KB)
+constexpr int VT_MAX_JOBS = 96;
 constexpr int VT_KC = 32;            // K elements per pipeline stage: 64-byte rows, 64-byte swizzle
 constexpr int VT_BLOCK_CHUNKS = 32;  // stages per exact accumulation block: K <= 1024
 constexpr int VT_NT_MAX = 128;       // N tile: three accumulators; an epilogue thread holds NT/2 column sums
 
 // Which of a tensor map's five dimensions holds each index of the view; -1 when
 // the view has no such index (r1 for single-index rows, k1 when K = k2 alone).
-// k2 is always dimension 0 (contiguous); rows r2 come before r1.
+// k2 is always dimension 0 (contiguous); rows r2 come before r1 and before the
+// slices s, which one copy brings together.  rows: the box's row count.
 struct VtRoles {
   int8_t k2, r2, r1, k1, s;
+  int16_t rows;
 };
 
 struct VtSeg {
   int8_t amap, bmap;
-  int K1, K2;
-  int nk2c;         // stages along k2: ceil(K2 / VT_KC)
-  int nchunks;      // K1 * nk2c
-  int bchunks;      // stages per accumulation block (at most VT_BLOCK_CHUNKS)
-  int nblk;         // accumulation blocks: ceil(nchunks / bchunks)
-  int afix[5], bfix[5];  // coordinates of the dimensions with no role (group indices)
-  const int* ea;    // scale exponents (device)
+  int16_t sign;              // +1 or -1 (a job's common factor is VtJob::jalpha)
+  int16_t afix[3], bfix[3];  // coordinates of dimensions 2, 3, 4 where they have no role (group indices)
+  int nk2c;                  // stages along k2: ceil(K2 / VT_KC)
+  int nchunks;               // K1 * nk2c
+  const int* ea;             // scale exponents (device)
   const int* eb;
-  double alpha;     // +1 or -1 (a job's common factor is VtJob::jalpha)
 };
+
+// float64 +=, float64 =, or the unit's FP32 pair (hi, lo) as it is: relative to
+// 2^(the largest scale of the job's segments), jalpha not applied
+enum VtOut { VT_ADD = 0, VT_STORE = 1, VT_PAIR = 2 };
+// How a block joins a unit's sum.  VT_ADD and VT_PAIR sum without error beyond
+// the pair's own 2^-48; VT_STORE rounds the higher levels' part to FP32 against
+// the low word first (2^-38 of the operands' scale, with few blocks per unit): the
+// adjoint's G, whose last bits decide how dW~ is cut.
 
 struct VtJob {
   int M1, M2, N;
-  int TA, TB, NT;   // row tile TA values of m1 x TB values of m2 (TA TB = 128); NT columns
-  int nm1, nm2, nn, nsplit, nseg;
-  int overwrite;    // the first block of a unit stores (nsplit == 1 only)
-  double jalpha;    // factor of the whole job (1 unless set)
-  int64_t unit0;    // first unit of the job in the launch
-  int64_t nblocks;  // accumulation blocks over all segments
-  double* C;        // element (m1, m2, n) at m1 c_m1 + m2 c_m2 + n c_n
+  int16_t TA, TB, NT;  // row tile TA values of m1 x TB values of m2 (TA TB = 128); NT columns
+  int16_t out;         // VtOut; VT_STORE and VT_PAIR run unsplit
+  int16_t seg0, nseg;  // segments in VtParams::seg
+  int16_t bchunks;     // stages per accumulation block
+  int16_t vec;         // four columns per access (contiguous, 32-byte aligned)
+  int nm2, nmu, nn, nsplit;  // m tiles along m2, units along m, N tiles
+  double jalpha;       // factor of the whole job (1 unless set)
+  int64_t unit0;       // first unit of the job in the launch
+  int64_t nblocks;     // accumulation blocks over all segments
+  void* C;             // element (m1, m2, n) at m1 c_m1 + m2 c_m2 + n c_n
   int64_t c_m1, c_m2, c_n;
-  double* part;     // nsplit > 1: [nsplit][M1 M2][N], added into C by vt_launch
-  int64_t red0;     // first element of the job in the launch's split-reduction index space
-  VtSeg seg[VT_MAX_SEGS];
+  double* part;        // nsplit > 1: [nsplit][M1 M2][N], added into C by vt_launch
+  int64_t red0;        // first element of the job in the launch's split-reduction index space
 };
 
 struct VtMaps {
@@ -72,7 +86,7 @@ struct VtMaps {
 };
 
 struct VtParams {
-  int njobs, ns;
+  int njobs, ns, nsegs;
   int stages;
   uint32_t stage_bytes;  // A part (ns x 128 rows x 64 B) then B part (ns x nt_max rows x 64 B)
   uint32_t tmem_cols;
@@ -83,7 +97,9 @@ struct VtParams {
   unsigned long long wait_ns;
   VtRoles roles[VT_MAX_MAPS];
   VtJob job[VT_MAX_JOBS];
+  VtSeg seg[VT_MAX_SEGS];
 };
+static_assert(sizeof(VtMaps) + sizeof(VtParams) <= 32764, "kernel parameters");
 
 // A BF16 slice array seen through a five-dimensional tensor map: dims and
 // strides in elements (stride[0] = 1), the roles of the dimensions, and the
@@ -103,8 +119,8 @@ struct VtBank {
   int n;
 };
 // Encode a view (rows per box: rows_r2 x rows_r1, rows_r1 = 1 for
-// single-index rows) as bank entry *idx; fails if a stride or the base breaks
-// the tensor-map rules.
+// single-index rows; all ns slices) as bank entry *idx; fails if a stride or the
+// base breaks the tensor-map rules.
 te_status vt_bank_add(VtBank* k, const VtView& v, int rows_r2, int rows_r1, int* idx);
 
 // Host-side launch under construction.
@@ -113,25 +129,29 @@ struct VtBuild {
   VtParams P;
   int nmaps;
   int8_t slot[VT_BANK_MAX];  // launch-local map index of each bank entry, -1 if unused
+  bool pair, full;           // full: a table overflowed
 };
 
-void vt_begin(VtBuild* b, int ns);
+// pair: run on CTA pairs
+void vt_begin(VtBuild* b, int ns, bool pair);
 // launch-local map index of bank entry idx (copied on first use); -1 when the
 // launch holds VT_MAX_MAPS maps already
 int vt_use(VtBuild* b, const VtBank& k, int idx);
-// Append a job; segments are filled by the caller through the returned pointer.
-VtJob* vt_job(VtBuild* b, int M1, int M2, int N, int TA, int TB, int NT, double* C, int64_t c_m1, int64_t c_m2,
-              int64_t c_n, int overwrite);
-void vt_seg(VtJob* j, int amap, int bmap, int K1, int K2, const int* afix, const int* bfix, const int* ea,
-            const int* eb, double alpha);
+// Append a job (null when the launch is full; vt_finish reports it); its
+// segments follow by vt_seg before the next job.
+VtJob* vt_job(VtBuild* b, int M1, int M2, int N, int TA, int TB, int NT, void* C, int64_t c_m1, int64_t c_m2,
+              int64_t c_n, VtOut out);
+// afix, bfix: coordinates of dimensions 2, 3, 4
+void vt_seg(VtBuild* b, int amap, int bmap, int K1, int K2, const int* afix, const int* bfix, const int* ea,
+            const int* eb, int sign);
 // Choose split counts (jobs that overwrite, or all jobs when part_scratch is
 // null, keep one split) and unit offsets; part_scratch holds the partials,
 // consecutively per split job.  The doubles of scratch used go to *used.
 te_status vt_finish(VtBuild* b, int num_sms, double* part_scratch, int64_t scratch_cap, int64_t* used);
 // Split count and partial doubles vt_finish chooses for a job of `tiles`
 // output tiles, `nblocks` accumulation blocks and mn outputs.
-int64_t vt_splits(int64_t tiles, int64_t nblocks, int num_sms);
-int64_t vt_split_doubles(int64_t tiles, int64_t nblocks, int64_t mn, int num_sms);
+int64_t vt_splits(int64_t tiles, int64_t nblocks, int units_at_once);
+int64_t vt_split_doubles(int64_t tiles, int64_t nblocks, int64_t mn, int units_at_once);
 // Accumulation blocks of one segment over K = K1 x K2 with bchunks stages per
 // block.
 int64_t vt_seg_blocks(int K1, int K2, int bchunks = VT_BLOCK_CHUNKS);
@@ -142,13 +162,13 @@ constexpr int VT_SPLIT_CHUNKS = 8;
 // every job into C in split order.
 te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s);
 
-// N tile for an output of n columns: at most VT_NT_MAX, a multiple of 16.
+// N tile for an output of n columns: at most VT_NT_MAX, a multiple of 32.
 int vt_ntile(int64_t n);
 
 struct SliceSet;
 // The six views of an exact-slice operand set (tc_prepare_slices) that the
 // four K segments of a G block read, rows (x, y) in tiles of 8 x 16 and z in
-// tiles of nt: idx[0..5] = ovvv rows (x, y), ovvv rows (y, x), t2L rows
+// tiles of nt (pair launches): idx[0..5] = ovvv rows (x, y), ovvv rows (y, x), t2L rows
 // (x, y), t2L rows (y, x), t2 rows z, nooT rows z.  Group coordinates: ovvv
 // and t2L take their occupied index at dimension 4; t2[r][q] takes q at 3 and
 // r at 4; nooT[p][r] takes r at 3 and p at 4.
