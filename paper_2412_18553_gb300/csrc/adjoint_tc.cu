@@ -86,16 +86,17 @@ __global__ void __launch_bounds__(256) k_adjoint_batch(const __grid_constant__ A
   a.j = T.j;
   a.k = T.k;
   const double w = B.w[slot];
-  const int64_t v = a.v, norb = v * (v + 1) * (v + 2) / 6;
+  const int64_t v = a.v, steps = orbit_steps(a.v);
+  const OrbitTile tile = orbit_tile();
   double* dW = A.dW + slot * A.w_stride;
   float2* dY = A.dY + slot * A.d_stride;
   float2* dD = A.dD + slot * A.d_stride;
   const double eo = a.eps_o[T.i] + a.eps_o[T.j] + a.eps_o[T.k];
   pr contrib{0.f, 0.f}, dsum{0.f, 0.f};
   double wmax = 0.0;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < norb; t += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t t = blockIdx.x; t < steps; t += gridDim.x) {
     int x, y, z;
-    orbit_abc(t, &x, &y, &z);
+    if (!orbit_at(tile, t, (int)v, &x, &y, &z)) continue;
     double W[6], Y[6], RW[6], RY[6];
     int64_t idx[6];
     orbit_values(a, x, y, z, W, Y);
@@ -162,8 +163,15 @@ struct YParts {
   int64_t stride;  // doubles between slots
 };
 
-// One block per plane a of a slot.  Rows: warp per b, lanes along c; columns:
-// thread per c, b in order.
+// sum over the warp, in lane 0
+__device__ __forceinline__ void warp_sum(pr& s) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+    s = pr_add(s, pr{__shfl_down_sync(0xffffffffu, s.h, off), __shfl_down_sync(0xffffffffu, s.l, off)});
+}
+
+// One block per plane a of a slot: its rows (warp per b, lanes along c), then its
+// columns (lanes along c, warps along b).  The plane is read twice, from L2.
 __global__ void __launch_bounds__(256) k_y_planes(const __grid_constant__ AdjEpi A, const __grid_constant__ AdjBatch B,
                                                   const __grid_constant__ YParts Yp) {
   __shared__ double red[2][8];
@@ -185,38 +193,69 @@ __global__ void __launch_bounds__(256) k_y_planes(const __grid_constant__ AdjEpi
   pr all{0.f, 0.f}, alld{0.f, 0.f};
   for (int b = warp; b < v; b += 8) {
     const pr* ovs_jk = ovs(T.j, b, T.k);
+    const float2 *yr = dY + (int64_t)b * V, *dr = dD + (int64_t)b * V;
     pr s0{0.f, 0.f}, s2{0.f, 0.f}, sd{0.f, 0.f};
-    for (int c = lane; c < v; c += 32) {
-      const pr y = pr_load(dY + (int64_t)b * V + c), d = pr_load(dD + (int64_t)b * V + c);
-      pr_fma(s0, y, t1k[c]);
-      pr_fma(s2, y, ovs_ik[c]);
-      pr_fma(all, y, ovs_jk[c]);
-      sd = pr_add(sd, d);
+    for (int c0 = lane; c0 < v; c0 += 128) {  // four elements in flight
+      pr y[4], d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool in = c0 + 32 * u < v;
+        y[u] = in ? pr_load(yr + c0 + 32 * u) : pr{0.f, 0.f};
+        d[u] = in ? pr_load(dr + c0 + 32 * u) : pr{0.f, 0.f};
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = min(c0 + 32 * u, v - 1);
+        pr_fma(s0, y[u], t1k[c]);
+        pr_fma(s2, y[u], ovs_ik[c]);
+        pr_fma(all, y[u], ovs_jk[c]);
+        sd = pr_add(sd, d[u]);
+      }
     }
     alld = pr_add(alld, sd);
-    double x0 = pr_double(s0), x2 = pr_double(s2), xd = pr_double(sd);
-    for (int off = 16; off > 0; off >>= 1) {
-      x0 += __shfl_down_sync(0xffffffffu, x0, off);
-      x2 += __shfl_down_sync(0xffffffffu, x2, off);
-      xd += __shfl_down_sync(0xffffffffu, xd, off);
-    }
+    warp_sum(s0);
+    warp_sum(s2);
+    warp_sum(sd);
     if (lane == 0) {
-      Yp.s[0][so + a * V + b] = x0 * ft;
-      Yp.p[1][so + a * V + b] = x2 * fo;
-      Yp.p[2][so + a * V + b] = xd * fd;
+      Yp.s[0][so + a * V + b] = pr_double(s0) * ft;
+      Yp.p[1][so + a * V + b] = pr_double(s2) * fo;
+      Yp.p[2][so + a * V + b] = pr_double(sd) * fd;
     }
   }
-  for (int c = threadIdx.x; c < v; c += 256) {
+  // columns: 32 at a time, warp w takes the rows b = w, w + 8, ...
+  __shared__ float2 col[3][8][33];
+  for (int c0 = 0; c0 < v; c0 += 32) {
+    const int c = c0 + lane;
+    const bool in = c < v;
     pr s2{0.f, 0.f}, p0{0.f, 0.f}, sd{0.f, 0.f};
-    for (int b = 0; b < v; ++b) {
-      const pr y = pr_load(dY + (int64_t)b * V + c), d = pr_load(dD + (int64_t)b * V + c);
-      pr_fma(s2, y, t1j[b]);
-      pr_fma(p0, y, ovs_ij[b]);
-      sd = pr_add(sd, d);
+    for (int b0 = warp; b0 < v; b0 += 32) {
+      pr y[4], d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool ok = in && b0 + 8 * u < v;
+        y[u] = ok ? pr_load(dY + (int64_t)(b0 + 8 * u) * V + c) : pr{0.f, 0.f};
+        d[u] = ok ? pr_load(dD + (int64_t)(b0 + 8 * u) * V + c) : pr{0.f, 0.f};
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int b = min(b0 + 8 * u, v - 1);
+        pr_fma(s2, y[u], t1j[b]);
+        pr_fma(p0, y[u], ovs_ij[b]);
+        sd = pr_add(sd, d[u]);
+      }
     }
-    Yp.s[2][so + a * V + c] = pr_double(s2) * ft;
-    Yp.p[0][so + a * V + c] = pr_double(p0) * fo;
-    Yp.p[3][so + a * V + c] = pr_double(sd) * fd;
+    col[0][warp][lane] = make_float2(s2.h, s2.l);
+    col[1][warp][lane] = make_float2(p0.h, p0.l);
+    col[2][warp][lane] = make_float2(sd.h, sd.l);
+    __syncthreads();
+    if (warp < 3 && in) {
+      pr t{0.f, 0.f};
+#pragma unroll
+      for (int w = 0; w < 8; ++w) t = pr_add(t, pr{col[warp][w][lane].x, col[warp][w][lane].y});
+      double* out = warp == 0 ? Yp.s[2] : (warp == 1 ? Yp.p[0] : Yp.p[3]);
+      out[so + a * V + c] = pr_double(t) * (warp == 0 ? ft : (warp == 1 ? fo : fd));
+    }
+    __syncthreads();
   }
   double x = pr_double(all), xd = pr_double(alld);
   for (int off = 16; off > 0; off >>= 1) {
@@ -248,7 +287,7 @@ __global__ void __launch_bounds__(256) k_y_sum_a(const __grid_constant__ AdjEpi 
   const float2* dY = A.dY + slot * A.d_stride + bc;
   const pr* t1i = A.in.t1 + (int64_t)B.t[slot].i * v;
   pr s{0.f, 0.f};
-#pragma unroll 4
+#pragma unroll 8
   for (int a = 0; a < v; ++a) pr_fma(s, pr_load(dY + a * v2), t1i[a]);
   Yp.s[1][slot * Yp.stride + bc] = pr_double(s) * ldexp(1.0, A.eslot[slot] + B.we[slot] + *A.in.e_t1);
 }
@@ -349,70 +388,66 @@ __global__ void __launch_bounds__(256) k_y_small(const __grid_constant__ AdjEpi 
 // permutation q holding the slices of dW~[pi_q(x, y, z)]:
 //   0, 1, 2: pi = (x,y,z), (z,x,y), (y,z,x);  3, 4, 5: (z,y,x), (x,z,y), (y,x,z).
 // With 2^e > max |dW~| (e written to e_out) the digits are slice_digits' (integer
-// operations on the bits of dW~).  A block handles a 32 x 64 tile of the (c, z) plane at one value of
-// the third index, c being the index along which dW~ is contiguous for this
-// permutation (or y when that is z), so both the reads and the writes (two
-// elements per 32-bit store) are coalesced.
+// operations on the bits of dW~).  A block takes a 16 x 16 x 16 cube of dW~: each
+// value is read and cut once, and every layout is written from shared memory in
+// rows of 16 elements (32 bytes).  HBM bounds it: 8 bytes read and 2 NS written per
+// value and layout.
 template <int NS>
 __global__ void __launch_bounds__(256) k_dw_slices(const double* __restrict__ dWs, int64_t w_stride, int v, int vp,
                                                    int perm0, const unsigned long long* __restrict__ dwmax,
                                                    int* __restrict__ e_out, bf* __restrict__ out, int64_t lay_elems,
                                                    int64_t slot_elems, int nperm) {
-  __shared__ double tile[32][65];
-  const int slot = blockIdx.z / nperm, buf = blockIdx.z - slot * nperm, perm = perm0 + buf;
+  // [slice][i][j][k], rows of 16 elements on 18 and planes of 16 rows on 290: the
+  // transposed reads below then spread over the banks
+  constexpr int RS = 18, PS = 16 * RS + 2;
+  __shared__ unsigned short cube[NS][16 * PS];
+  const int slot = blockIdx.z;
   const double* dW = dWs + slot * w_stride;
   const double mx = __longlong_as_double((long long)dwmax[slot]);
   int ex = 0;
   if (mx > 0.0) frexp(mx, &ex);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && buf == 0 && threadIdx.x == 0) e_out[slot] = ex;
-  const int64_t V = v, V2 = V * V, plane = V2 * vp;
-  int64_t sx, sy, sz;  // source strides of the output indices (x, y, z)
-  switch (perm) {
-    case 0: sx = V2; sy = V; sz = 1; break;
-    case 1: sx = V; sy = 1; sz = V2; break;
-    case 2: sx = 1; sy = V2; sz = V; break;
-    case 3: sx = 1; sy = V; sz = V2; break;
-    case 4: sx = V2; sy = 1; sz = V; break;
-    default: sx = V; sy = V2; sz = 1; break;
-  }
-  // c: the tile's other index (0 = x, 1 = y); w: the block's fixed index
-  const int cidx = (sx == 1) ? 0 : 1;
-  const int64_t sc_ = cidx == 0 ? sx : sy, sw = cidx == 0 ? sy : sx;
-  const int ntz = (v + 63) / 64;
-  const int c0 = (int)(blockIdx.x / ntz) * 32, z0 = (int)(blockIdx.x % ntz) * 64;
-  const int w = blockIdx.y;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  if (sz == 1) {  // threads along z
-    for (int i = ty; i < 32; i += 8)
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) e_out[slot] = ex;
+  const int nt = (v + 15) / 16;
+  const int a0 = blockIdx.y * 16, b0 = (int)(blockIdx.x / nt) * 16, c0 = (int)(blockIdx.x % nt) * 16;
+  const int64_t V = v, plane = V * V * vp;
+  const int k = threadIdx.x & 15, j0 = threadIdx.x >> 4;
+#pragma unroll 4
+  for (int i = 0; i < 16; ++i) {
+    const bool in = a0 + i < v && b0 + j0 < v && c0 + k < v;
+    int d[NS];
+    slice_digits_int<NS>(in ? dW[((int64_t)(a0 + i) * V + b0 + j0) * V + c0 + k] : 0.0, ex, d);
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int cc = c0 + i, zz = z0 + tx + 32 * q;
-        if (cc < v && zz < v) tile[i][tx + 32 * q] = dW[w * sw + cc * sc_ + zz];
-      }
-  } else {  // threads along c, where dW~ is contiguous
-    for (int i = ty; i < 64; i += 8) {
-      const int cc = c0 + tx, zz = z0 + i;
-      if (cc < v && zz < v) tile[tx][i] = dW[w * sw + cc * sc_ + zz * sz];
-    }
+    for (int s = 0; s < NS; ++s) cube[s][i * PS + j0 * RS + k] = (unsigned short)digit_bf16(d[s], 7 * (s + 1));
   }
   __syncthreads();
-  bf* o = out + slot * slot_elems + buf * lay_elems;
-  for (int i = ty; i < 32; i += 8) {
-    const int cc = c0 + i, zz = z0 + 2 * tx;
-    if (cc >= v || zz >= v) continue;
-    uint32_t wd[2][NS];
+  // Output rows: (x, y) fixed, z along the row; thread = (row, half of 8 elements).
+  // In terms of the cube's (i, j, k) = offsets of dW~'s (first, second, third) index
+  const int half = threadIdx.x & 1, r0 = threadIdx.x >> 1;
+  for (int q = 0; q < nperm; ++q) {
+    const int perm = perm0 + q;
+    // which of dW~'s indices (0, 1, 2) are x, y and z
+    const int px = perm == 0 ? 0 : perm == 1 ? 1 : perm == 2 ? 2 : perm == 3 ? 2 : perm == 4 ? 0 : 1;
+    const int py = perm == 0 ? 1 : perm == 1 ? 2 : perm == 2 ? 0 : perm == 3 ? 1 : perm == 4 ? 2 : 0;
+    const int pz = 3 - px - py;
+    auto org = [&](int p) { return p == 0 ? a0 : (p == 1 ? b0 : c0); };
+    auto stp = [&](int p) { return p == 0 ? PS : (p == 1 ? RS : 1); };
+    const int x0 = org(px), y0 = org(py), z0 = org(pz), sx = stp(px), sy = stp(py), sz = stp(pz);
+    bf* o = out + slot * slot_elems + q * lay_elems;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      int d[NS];
-      slice_digits_int<NS>(zz + q < v ? tile[i][2 * tx + q] : 0.0, ex, d);
+    for (int rr = 0; rr < 2; ++rr) {
+      const int r = r0 + 128 * rr, x = r >> 4, y = r & 15, zz = 8 * half;
+      if (x0 + x >= v || y0 + y >= v || z0 + zz >= vp) continue;
+      const int at = x * sx + y * sy + zz * sz;
+      bf* dst = o + ((int64_t)(x0 + x) * V + y0 + y) * vp + z0 + zz;  // vp and z0 + zz are multiples of 8
 #pragma unroll
-      for (int s = 0; s < NS; ++s) wd[q][s] = digit_bf16(d[s], 7 * (s + 1));
+      for (int s = 0; s < NS; ++s) {
+        uint32_t w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          w[u] = (uint32_t)cube[s][at + 2 * u * sz] | ((uint32_t)cube[s][at + (2 * u + 1) * sz] << 16);
+        *reinterpret_cast<uint4*>(dst + s * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
     }
-    const int64_t xi = cidx == 0 ? cc : w, yi = cidx == 0 ? w : cc;
-    const int64_t at = (xi * V + yi) * vp + zz;  // even: vp and zz are
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-      *reinterpret_cast<uint32_t*>(o + s * plane + at) = __byte_perm(wd[0][s], wd[1][s], 0x5410);
   }
 }
 
@@ -798,7 +833,8 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
     k_y_small<<<1 + (v + 255) / 256, 256, 0, s>>>(A, Bt, Yp, AdjOut{g->eps_o, g->eps_v, g->t1, dOVS, shares, t0}, agrid);
     ++h->n_launches;
     auto slices = [&](int perm0, int nperm) {
-      const dim3 grid((unsigned)((v + 31) / 32 * ((v + 63) / 64)), (unsigned)v, (unsigned)(Bt.n * nperm));
+      const unsigned n16 = (unsigned)((v + 15) / 16);
+      const dim3 grid(n16 * n16, n16, (unsigned)Bt.n);
       bf* out = reinterpret_cast<bf*>(region);
       if (ns == 5)
         k_dw_slices<5><<<grid, 256, 0, s>>>(dW, A.w_stride, v, (int)vp, perm0, dwmax, dwexp, out, lay_stride, ls, nperm);

@@ -142,6 +142,32 @@ __device__ __forceinline__ void orbit_abc(int64_t t, int* pa, int* pb, int* pc) 
   *pc = (int)(rem - (int64_t)b * (b + 1) / 2);
 }
 
+// The epilogues' orbits go by block triples of 8 x 8 x 8 (X >= Y >= Z), half of one
+// per block of 256 threads and step.  A warp covers 2 x 4 x 4 of (a, b, c), so
+// that of the six positions' accesses (8 bytes each, contiguous in the last
+// index) those ending in b or c use whole 32-byte sectors and those ending in a
+// half of them; 32 consecutive c used a quarter in four positions of six.
+struct OrbitTile {
+  int la, lb, lc;
+};
+__device__ __forceinline__ OrbitTile orbit_tile() {
+  const int t = threadIdx.x;
+  return {((t >> 4) & 1) | ((t >> 6) & 2), ((t >> 2) & 3) | ((t >> 4) & 4), (t & 3) | ((t >> 3) & 4)};
+}
+__device__ __forceinline__ int64_t orbit_steps(int v) {
+  const int64_t nb = (v + 7) / 8;
+  return nb * (nb + 1) * (nb + 2) / 3;  // two per block triple
+}
+// this thread's orbit in step t; false where it is none (a >= b >= c, a < v)
+__device__ __forceinline__ bool orbit_at(const OrbitTile& o, int64_t t, int v, int* a, int* b, int* c) {
+  int X, Y, Z;
+  orbit_abc(t >> 1, &X, &Y, &Z);
+  *a = X * 8 + (int)(t & 1) * 4 + o.la;
+  *b = Y * 8 + o.lb;
+  *c = Z * 8 + o.lc;
+  return *a < v && *a >= *b && *b >= *c;
+}
+
 // Positions abc, acb, bac, bca, cab, cba.  G_g at the six permutations of
 // (a, b, c) is read once; W~ at position n is G_0 there, G_1 at the cyclic
 // successor and G_2 at the one after.

@@ -304,13 +304,14 @@ __global__ void __launch_bounds__(256) k_proj_pairs(const __grid_constant__ Proj
   const int slot = blockIdx.y;
   const Triple T = A.t[slot];
   const TripleScale sc = triple_scale(A.in, A.x0, T), ss = proj_scale(A, T);
-  const int64_t v = A.in.v, norb = v * (v + 1) * (v + 2) / 6;
+  const int64_t v = A.in.v, steps = orbit_steps(A.in.v);
+  const OrbitTile tile = orbit_tile();
   const float2 *G = A.G + slot * A.stride, *SG = A.SG + slot * A.stride;
   const pr eo = occ_energy(A.in, T);
   pr sum{0.f, 0.f};
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < norb; t += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t t = blockIdx.x; t < steps; t += gridDim.x) {
     int a, b, c;
-    orbit_abc(t, &a, &b, &c);
+    if (!orbit_at(tile, t, (int)v, &a, &b, &c)) continue;
     pr W[6], Y[6], RV[6];
     orbit_w(G, v, sc, a, b, c, W);
     orbit_y(A.in, T, sc, a, b, c, Y);
