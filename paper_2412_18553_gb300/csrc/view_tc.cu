@@ -6,9 +6,9 @@
 // step, one elected lane: the operands then sit in uniform registers; issued
 // from a single-thread branch an MMA took 75 to 80 cycles whatever its size),
 // warps 2..9 (two per TMEM lane quarter, half of the N tile each) drain every
-// accumulation block into a double-float (FP32 pair) sum held in registers, two
-// columns per packed instruction, and release the accumulators at once, so the
-// next block's MMAs overlap the rest of the epilogue.  A unit's sum leaves once,
+// accumulation block into an FP32 pair sum held in registers and release the
+// accumulators at once, so the next block's MMAs overlap the rest of the
+// epilogue.  A unit's sum leaves once,
 // at its end: GB300's float64 rate is a small fraction of its FP32 rate, and a
 // float64 update per block and element cost more than the MMAs at short K.
 //
@@ -138,8 +138,32 @@ __device__ __forceinline__ void vt_commit(uint64_t* bar) {
   else ptx::mma_commit(bar);
 }
 
-// FOLD: every job of the launch is VT_STORE (view_tc.h says how they sum).
-template <int NS, bool PAIR, bool FOLD>
+// How a block joins the unit's sum (view_tc.h), two columns per packed
+// instruction: a0 and a1, the exact FP32 sums of levels 0 and 1, a2 the rest, w a
+// power of two.  These instructions sit between two blocks' MMAs, so each output
+// kind pays for the precision it needs: VT_STORE 20, VT_PAIR 17, VT_ADD 23.
+template <int SUM>
+__device__ __forceinline__ void join(f2& H, f2& L, f2 a0, f2 a1, f2 a2, f2 w) {
+  f2 s0, e0, t, te;
+  f2_two_sum(a0, a1, s0, e0);
+  const f2 x = f2_mul(s0, w), y = f2_mul(f2_add(e0, a2), w);
+  f2_two_sum(H, x, t, te);
+  if constexpr (SUM == VT_STORE) {
+    const f2 l = f2_add(te, f2_add(L, y));
+    H = f2_add(t, l);
+    L = f2_sub(l, f2_sub(H, t));
+  } else if constexpr (SUM == VT_PAIR) {
+    H = t;
+    L = f2_add(L, f2_add(te, y));
+  } else {  // y can be 2^-14 of the operands' scale, far above the last bits of L: added without error
+    f2 ye;
+    f2_two_sum(t, y, H, ye);
+    L = f2_add(L, f2_add(te, ye));
+  }
+}
+
+// SUM: the output kind of every job of the launch.
+template <int NS, bool PAIR, int SUM>
 __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams& P) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -348,6 +372,7 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
       for (int64_t b = U.b_begin; b < U.b_end; ++b) {
         const VtSeg& S = P.seg[B.seg];
         const float wk1 = ldexpf(S.sign < 0 ? -1.f : 1.f, *S.ea + *S.eb - eref);
+        const f2 wk = f2_make(wk1, wk1);
         int got = 0;
         if (!*abort_flag) got = ptx::mbar_wait(tfull, acc_phase, P.wait_ns) ? 1 : 0;
         // warp-uniform: tcgen05.ld below is .sync.aligned
@@ -357,7 +382,6 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
           break;
         }
         ptx::tc_fence_after();
-        const f2 wk = f2_make(wk1, wk1);
 #pragma unroll
         for (int q = 0; q < VT_HALF / 8; ++q) {
           if (8 * q < ncol) {
@@ -365,26 +389,9 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
             float a0[8], a1[8], a2[8];
             ptx::tmem_ld8x3(tbase + cc, tbase + (uint32_t)J.NT + cc, tbase + 2u * (uint32_t)J.NT + cc, a0, a1, a2);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              f2& H = hi[4 * q + j];
-              f2& L = lo[4 * q + j];
-              // level 0 + level 1 exactly (both exact FP32 sums), the rest rounded
-              f2 s0, e0, t, te;
-              f2_two_sum(f2_make(a0[2 * j], a0[2 * j + 1]), f2_make(a1[2 * j], a1[2 * j + 1]), s0, e0);
-              const f2 x = f2_mul(s0, wk), y = f2_mul(f2_add(e0, f2_make(a2[2 * j], a2[2 * j + 1])), wk);
-              f2_two_sum(H, x, t, te);
-              f2 l;
-              if constexpr (FOLD) {
-                l = f2_add(te, f2_add(L, y));
-              } else {  // y can be 2^-14 of the operands' scale, far above the last bits of lo
-                f2 t2, te2;
-                f2_two_sum(t, y, t2, te2);
-                l = f2_add(L, f2_add(te, te2));
-                t = t2;
-              }
-              H = f2_add(t, l);
-              L = f2_sub(l, f2_sub(H, t));
-            }
+            for (int j = 0; j < 4; ++j)
+              join<SUM>(hi[4 * q + j], lo[4 * q + j], f2_make(a0[2 * j], a0[2 * j + 1]), f2_make(a1[2 * j], a1[2 * j + 1]),
+                        f2_make(a2[2 * j], a2[2 * j + 1]), wk);
           }
         }
         ptx::tc_fence_before();
@@ -397,7 +404,7 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
         vt_next(P, J, B);
       }
       if (!ok || !valid) continue;
-      if (J.out == VT_PAIR) {
+      if constexpr (SUM == VT_PAIR) {
         float2* dst = static_cast<float2*>(J.C) + (int64_t)m1 * J.c_m1 + (int64_t)m2 * J.c_m2 + U.n0 + c_lo;
 #pragma unroll
         for (int q = 0; q < VT_HALF / 4; ++q) {
@@ -485,12 +492,12 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
 template <int NS>
 __global__ void __launch_bounds__(VT_THREADS, 1)
     k_view_tc(const __grid_constant__ VtMaps maps, const __grid_constant__ VtParams P) {
-  view_tc_body<NS, false, false>(maps, P);
+  view_tc_body<NS, false, VT_ADD>(maps, P);
 }
-template <int NS, bool FOLD>
+template <int NS, int SUM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(VT_THREADS, 1)
     k_view_tc_pair(const __grid_constant__ VtMaps maps, const __grid_constant__ VtParams P) {
-  view_tc_body<NS, true, FOLD>(maps, P);
+  view_tc_body<NS, true, SUM>(maps, P);
 }
 
 // C[(m1, m2), n] += sum_z part[z][(m1, m2)][n], z in order, for every split job
@@ -700,8 +707,8 @@ te_status vt_finish(VtBuild* b, int num_sms, double* part_scratch, int64_t scrat
   for (int q = 0; q < b->P.njobs; ++q) {
     VtJob& J = b->P.job[q];
     if (J.nseg == 0) return fail(TE_EINVAL, "view GEMM: job without segments");
-    if ((J.out == VT_STORE) != (b->pair && b->P.job[0].out == VT_STORE))
-      return fail(TE_EINVAL, "view GEMM: VT_STORE jobs go in a pair launch of their own");
+    if (J.out != b->P.job[0].out || (J.out != VT_ADD && !b->pair))
+      return fail(TE_EINVAL, "view GEMM: one output kind per launch; VT_STORE and VT_PAIR on CTA pairs");
     int kblocks = 0;
     for (int g = J.seg0; g < J.seg0 + J.nseg; ++g) {
       const VtSeg& S = b->P.seg[g];
@@ -753,7 +760,11 @@ int64_t vt_split_doubles(int64_t tiles, int64_t nblocks, int64_t mn, int units_a
 
 template <int NS>
 static cudaError_t vt_launch_ns(const VtBuild* b, int grid, size_t smem, cudaStream_t s) {
-  auto* k = !b->pair ? k_view_tc<NS> : (b->P.job[0].out == VT_STORE ? k_view_tc_pair<NS, true> : k_view_tc_pair<NS, false>);
+  auto* k = k_view_tc<NS>;
+  if (b->pair) {
+    const int out = b->P.job[0].out;
+    k = out == VT_STORE ? k_view_tc_pair<NS, VT_STORE> : (out == VT_PAIR ? k_view_tc_pair<NS, VT_PAIR> : k_view_tc_pair<NS, VT_ADD>);
+  }
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k<<<(unsigned)grid, VT_THREADS, smem, s>>>(b->maps, b->P);

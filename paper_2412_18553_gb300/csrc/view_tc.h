@@ -57,12 +57,12 @@ struct VtSeg {
 };
 
 // float64 +=, float64 =, or the unit's FP32 pair (hi, lo) as it is: relative to
-// 2^(the largest scale of the job's segments), jalpha not applied
-enum VtOut { VT_ADD = 0, VT_STORE = 1, VT_PAIR = 2 };
-// How a block joins a unit's sum.  VT_ADD and VT_PAIR sum without error beyond
-// the pair's own 2^-48; VT_STORE rounds the higher levels' part to FP32 against
-// the low word first (2^-38 of the operands' scale, with few blocks per unit): the
+// 2^(the largest scale of the job's segments), jalpha not applied.  One kind per
+// launch; VT_STORE and VT_PAIR on CTA pairs.  VT_ADD sums a unit's blocks to 2^-48 of the sum;
+// VT_STORE and VT_PAIR round the higher levels' part to FP32 against the low
+// word first (2^-38 of the operands' scale; few blocks per unit).  VT_STORE is the
 // adjoint's G, whose last bits decide how dW~ is cut.
+enum VtOut { VT_ADD = 0, VT_STORE = 1, VT_PAIR = 2 };
 
 struct VtJob {
   int M1, M2, N;
