@@ -18,10 +18,11 @@
 // swapped), both density blocks are single contractions against T~:
 //   gamma_vv[a,b] = 2 sum_{(ij),c} t[ij,a,c] T~[ij,b,c]
 //   gamma_oo[i,j] = 2 delta_ij - 2 sum_{k,(ab)} t[i,k,ab] T~[j,k,ab]
-// The eigenvalues come from the cyclic Jacobi method in the parallel
-// (round-robin) ordering, one block per matrix, float64 throughout, with the
-// matrix in shared memory up to order 168; one launch takes the matrices of
-// up to 32 clusters, whose density blocks stay in the workspace until then.
+// The eigenvalues come from a Householder reduction to tridiagonal form (one
+// block per matrix, in shared memory up to order 167) and bisection with Sturm
+// counts (one thread per eigenvalue), float64 throughout; two launches take the
+// matrices of up to 32 clusters, whose density blocks stay in the workspace until
+// then.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -68,145 +69,199 @@ __global__ void k_two_identity(double* __restrict__ g, int o) {
 }
 
 // One symmetric matrix for the eigensolver: the source (n x n), the output
-// eigenvalues (n, ascending), the padded order m (n rounded up to even; the
-// padding row and column are zero and never rotate) and a global working copy
-// (m x m) for an order too large for shared memory (null otherwise).
+// eigenvalues (n, ascending), n doubles each for the tridiagonal form and a
+// global working copy (n x n) for an order too large for shared memory (null
+// otherwise).
 struct EigJob {
   double* a;
   const double* src;
   double* out;
-  int n, m;
+  double *d, *e;  // diagonal; squares of the off-diagonal; both of the matrix times 2^-e[n - 1]
+  int n;
 };
 
-// Orders up to this one keep their working copy in shared memory:
-// 168^2 doubles plus 84 pairs' rotations fit the 227 KB of one block.
-constexpr int kJacobiSmemM = 168;
+// Orders up to this one keep their working copy in shared memory: 167^2
+// doubles, two vectors and the partial sums fit the 227 KB of one block.
+constexpr int kEigSmemN = 167;
+constexpr int EIG_THREADS = 512;
 
 struct EigJobs {
   int count;
   EigJob j[64];
 };
 
-// Shared memory of one job: rotations of its m / 2 pairs, then its working
-// copy unless it has a global one.
-__host__ __device__ inline size_t jacobi_rot_bytes(int m) { return ((size_t)(m / 2) * 20 + 15) & ~size_t(15); }
-__host__ __device__ inline size_t jacobi_smem_bytes(const EigJob& j) {
-  return jacobi_rot_bytes(j.m) + (j.a ? 0 : (size_t)j.m * j.m * 8);
+// Shared memory of one job: the vectors v and w, the partial sums, then its
+// working copy unless it has a global one.
+__host__ __device__ inline size_t eig_vec_doubles(int n) { return 2 * (size_t)n + (n > EIG_THREADS ? n : EIG_THREADS); }
+__host__ __device__ inline size_t eig_smem_bytes(const EigJob& j) {
+  return 8 * (eig_vec_doubles(j.n) + (j.a ? 0 : (size_t)j.n * j.n));
 }
 
-// Parallel-order cyclic Jacobi: in step s of a sweep the index at position 0
-// stays and the others rotate; pair k is (label(k), label(m-1-k)) with
-// label(0) = 0, label(x) = 1 + (x - 1 + s) mod (m - 1).  The m/2 rotations of a
-// step act on disjoint index pairs, so they are applied at once: rows p, q of
-// every pair, then columns p, q.  The matrix taken is the symmetric part of the
-// block ((A + A^T) / 2): a density computed in exact slices is symmetric only
-// to about 1e-9 of its scale, and an orthogonal similarity cannot remove an
-// antisymmetric part.  Sweeps repeat until the off-diagonal mass is below
-// 1e-30 of the matrix's, stops decreasing (rounding floor), or 60 sweeps have
-// run.  Then the diagonal is sorted.  Dynamic shared memory: the rotations
-// (cosines, sines, then the p and q indices, m / 2 each), then the working
-// copy when the job has no global one.
-__global__ void __launch_bounds__(512, 1) k_jacobi(const __grid_constant__ EigJobs J) {
+__device__ __forceinline__ double warp_sum(double x) {
+  for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+  return x;
+}
+
+// Householder reduction of the symmetric part (A + A^T) / 2 (a density computed
+// in exact slices is symmetric only to about 1e-9 of its scale), scaled by a
+// power of two to entries below 1: step k takes x = A[k+1.., k], v = x + sign(x_0)
+// |x| e_0, beta = 1 / (|x|^2 + |x_0| |x|), p = beta A v, w = p - (beta / 2) (v . p)
+// v, and A <- A - v w^T - w v^T on the trailing block; the subdiagonal entry is
+// -sign(x_0) |x|.
+// About n^3 float64 operations on two lanes per cycle of one SM: 1 ms at n = 160.
+// (A parallel-order cyclic Jacobi solver, 24 ms for the sixteen matrices of the
+// clusters nocc 8 .. 20, nvir = 8 nocc, was bound by the same two lanes with
+// six sweeps of 4 n^3; this and the bisection take 3.0 ms (1.8 and 1.2).)
+__global__ void __launch_bounds__(EIG_THREADS, 1) k_tridiag(const __grid_constant__ EigJobs J) {
   const EigJob& jb = J.j[blockIdx.x];
-  const int n = jb.n, m = jb.m;
-  extern __shared__ __align__(16) unsigned char jac_smem[];
-  double* cs = reinterpret_cast<double*>(jac_smem);
-  double* sn = cs + m / 2;
-  unsigned short* pp = reinterpret_cast<unsigned short*>(sn + m / 2);
-  unsigned short* qq = pp + m / 2;
-  double* A = jb.a ? jb.a : reinterpret_cast<double*>(jac_smem + jacobi_rot_bytes(m));
-  __shared__ double red[32];
-  __shared__ int done;
-  __shared__ double prev_off;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) prev_off = -1.0;
-  for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
-    const int r = (int)(e / m), c = (int)(e % m);
-    A[e] = (r < n && c < n) ? 0.5 * (jb.src[(int64_t)r * n + c] + jb.src[(int64_t)c * n + r]) : 0.0;
-  }
+  const int n = jb.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  extern __shared__ __align__(16) unsigned char eig_smem[];
+  double* v = reinterpret_cast<double*>(eig_smem);
+  double* w = v + n;
+  double* part = w + n;
+  double* A = jb.a ? jb.a : v + eig_vec_doubles(n);
+  __shared__ double sh[2];
+  __shared__ unsigned int top;
+  if (tid == 0) top = 0u;
   __syncthreads();
-  const int half = m / 2;
-  for (int sweep = 0; sweep < 60; ++sweep) {
-    // convergence test: off-diagonal and total squared mass
-    double off = 0.0, tot = 0.0;
-    for (int64_t e = tid; e < (int64_t)m * m; e += nt) {
-      const double x = A[e];
-      tot += x * x;
-      if (e / m != e % m) off += x * x;
-    }
-    for (int d = 16; d > 0; d >>= 1) {
-      off += __shfl_down_sync(0xffffffffu, off, d);
-      tot += __shfl_down_sync(0xffffffffu, tot, d);
-    }
-    if ((tid & 31) == 0) {
-      red[tid >> 5] = off;
-      if (tid == 0) done = 0;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double so = 0.0;
-      for (int w = 0; w < (nt >> 5); ++w) so += red[w];
-      red[0] = so;
-    }
-    __syncthreads();
-    const double off_all = red[0];
-    __syncthreads();
-    if ((tid & 31) == 0) red[tid >> 5] = tot;
-    __syncthreads();
-    if (tid == 0) {
-      double st = 0.0;
-      for (int w = 0; w < (nt >> 5); ++w) st += red[w];
-      done = (off_all <= 1e-30 * st || (prev_off >= 0.0 && off_all >= prev_off)) ? 1 : 0;
-      prev_off = off_all;
-    }
-    __syncthreads();
-    if (done) break;
-    for (int s = 0; s < m - 1; ++s) {
-      for (int k = tid; k < half; k += nt) {
-        auto label = [&](int x) { return x == 0 ? 0 : 1 + (x - 1 + s) % (m - 1); };
-        const int p = label(k), q = label(m - 1 - k);
-        const double apq = A[(int64_t)p * m + q];
-        double c = 1.0, t = 0.0;
-        if (apq != 0.0) {
-          const double theta = (A[(int64_t)q * m + q] - A[(int64_t)p * m + p]) / (2.0 * apq);
-          const double at = fabs(theta);
-          t = at > 1e150 ? 0.5 / theta : copysign(1.0, theta) / (at + sqrt(at * at + 1.0));
-          c = 1.0 / sqrt(t * t + 1.0);
-        }
-        pp[k] = (unsigned short)p;
-        qq[k] = (unsigned short)q;
-        cs[k] = c;
-        sn[k] = t * c;
-      }
-      __syncthreads();
-      for (int64_t e = tid; e < (int64_t)half * m; e += nt) {  // rows p, q of every pair
-        const int k = (int)(e / m), col = (int)(e % m);
-        const int64_t rp = (int64_t)pp[k] * m + col, rq = (int64_t)qq[k] * m + col;
-        const double ap = A[rp], aq = A[rq], c = cs[k], s_ = sn[k];
-        A[rp] = c * ap - s_ * aq;
-        A[rq] = s_ * ap + c * aq;
-      }
-      __syncthreads();
-      for (int64_t e = tid; e < (int64_t)half * m; e += nt) {  // columns p, q of every pair
-        const int k = (int)(e % half), row = (int)(e / half);
-        const int64_t cp = (int64_t)row * m + pp[k], cq = (int64_t)row * m + qq[k];
-        const double ap = A[cp], aq = A[cq], c = cs[k], s_ = sn[k];
-        A[cp] = c * ap - s_ * aq;
-        A[cq] = s_ * ap + c * aq;
-      }
-      __syncthreads();
-    }
+  unsigned int m = 0;
+  for (int64_t e = tid; e < (int64_t)n * n; e += EIG_THREADS) {
+    const int r = (int)(e / n), c = (int)(e % n);
+    const double x = 0.5 * jb.src[e] + 0.5 * jb.src[(int64_t)c * n + r];
+    A[e] = x;
+    m = max(m, (unsigned int)__double2hiint(x) & 0x7FFFFFFFu);
   }
-  // eigenvalues ascending: each by its rank (ties by index)
-  for (int i = tid; i < n; i += nt) {
-    const double di = A[(int64_t)i * m + i];
-    int rank = 0;
-    for (int j2 = 0; j2 < n; ++j2) {
-      const double dj = A[(int64_t)j2 * m + j2];
-      rank += (dj < di || (dj == di && j2 < i)) ? 1 : 0;
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) atomicMax(&top, m);
+  __syncthreads();
+  const int ex = top == 0u ? 0 : (int)(top >> 20) - 1022;  // 2^ex > max |a|
+  const double sc = ldexp(1.0, -ex);
+  for (int64_t e = tid; e < (int64_t)n * n; e += EIG_THREADS) A[e] *= sc;
+  __syncthreads();
+  for (int k = 0; k + 1 < n; ++k) {
+    const int na = n - k - 1;  // order of the trailing block
+    const double* row = A + (int64_t)k * n + k + 1;
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = lane; i < na; i += 32) s = fma(row[i], row[i], s);
+      s = warp_sum(s);
+      const double x0 = row[0], nx = sqrt(s);
+      // a block of one entry is tridiagonal already; so is a column below 1e-100
+      const double beta = na > 1 && s > 1e-200 ? 1.0 / (s + fabs(x0) * nx) : 0.0;
+      const double alpha = na > 1 ? copysign(nx, -x0) : x0;
+      for (int i = lane; i < na; i += 32) v[i] = i == 0 ? x0 - alpha : row[i];
+      if (lane == 0) {
+        sh[0] = beta;
+        jb.d[k] = A[(int64_t)k * n + k];
+        jb.e[k] = alpha * alpha;
+      }
     }
-    jb.out[rank] = di;
+    __syncthreads();
+    const double beta = sh[0];
+    if (beta == 0.0) {
+      __syncthreads();
+      continue;
+    }
+    double* T = A + (int64_t)(k + 1) * n + k + 1;  // trailing block, row stride n
+    // p = A v: rows split into as many parts as there are threads for
+    const int parts = na < EIG_THREADS ? EIG_THREADS / na : 1;
+    for (int t = tid; t < parts * na; t += EIG_THREADS) {
+      const int q = t / na, i = t - q * na, j0 = na * q / parts, j1 = na * (q + 1) / parts;
+      double s0 = 0.0, s1 = 0.0;
+      int j = j0;
+      for (; j + 1 < j1; j += 2) {  // A is symmetric: its rows read along i
+        s0 = fma(T[(int64_t)j * n + i], v[j], s0);
+        s1 = fma(T[(int64_t)(j + 1) * n + i], v[j + 1], s1);
+      }
+      if (j < j1) s0 = fma(T[(int64_t)j * n + i], v[j], s0);
+      part[t] = s0 + s1;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = lane; i < na; i += 32) {
+        double p = part[i];
+        for (int q = 1; q < parts; ++q) p += part[q * na + i];
+        p *= beta;
+        w[i] = p;
+        s = fma(p, v[i], s);
+      }
+      s = 0.5 * beta * warp_sum(s);
+      for (int i = lane; i < na; i += 32) w[i] = fma(-s, v[i], w[i]);
+    }
+    __syncthreads();
+    for (int i = warp; i < na; i += EIG_THREADS / 32) {
+      const double vi = -v[i], wi = -w[i];
+      for (int j = lane; j < na; j += 32) T[(int64_t)i * n + j] = fma(vi, w[j], fma(wi, v[j], T[(int64_t)i * n + j]));
+    }
+    __syncthreads();
   }
+  if (tid == 0) {
+    jb.d[n - 1] = A[(int64_t)n * n - 1];
+    jb.e[n - 1] = (double)ex;
+  }
+}
+
+// Eigenvalue number m (ascending) of a job's tridiagonal matrix by bisection: a
+// thread per eigenvalue, a warp per block (a warp alone on its SM has both
+// float64 lanes).  The count of eigenvalues below x is that of the sign changes
+// of the leading minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (three float64
+// operations a step; the quotients' form takes six with a reciprocal: 2.97
+// against 1.20 ms at n = 160).  A minor below 2^-90 of the last one counts as
+// -2^-90 of it; pairs are rescaled by a power of two.  All threads start from one interval and
+// take the same branch at the same x, so the results ascend.
+__global__ void __launch_bounds__(32) k_bisect(const __grid_constant__ EigJobs J) {
+  const EigJob& jb = J.j[blockIdx.y];
+  const int n = jb.n, lane = threadIdx.x, m = blockIdx.x * 32 + lane;
+  if (blockIdx.x * 32 >= n) return;
+  extern __shared__ __align__(16) unsigned char eig_smem[];
+  double* d = reinterpret_cast<double*>(eig_smem);
+  double* e2 = d + n;
+  double lo = 1e300, hi = -1e300;
+  for (int i = lane; i < n; i += 32) {
+    d[i] = jb.d[i];
+    e2[i] = i + 1 < n ? jb.e[i] : 0.0;
+  }
+  __syncwarp();
+  for (int i = lane; i < n; i += 32) {  // Gershgorin discs
+    const double r = (i > 0 ? sqrt(e2[i - 1]) : 0.0) + sqrt(e2[i]);
+    lo = fmin(lo, d[i] - r);
+    hi = fmax(hi, d[i] + r);
+  }
+  for (int k = 16; k > 0; k >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, k));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, k));
+  }
+  const double pad = 1e-15 * fmax(fabs(lo), fabs(hi)) + 1e-300;
+  lo -= pad;
+  hi += pad;
+  // 2^-58 of the first interval, itself at most a few times the largest entry
+  for (int it = 0; it < 58; ++it) {
+    const double x = 0.5 * (lo + hi);
+    int below = 0;
+    double p1 = 1.0, p0 = 1.0, e = 0.0;
+    for (int i = 0; i < n; ++i) {
+      double p = fma(d[i] - x, p1, -(e * p0));
+      int h = __double2hiint(p);
+      const int h1 = __double2hiint(p1);
+      if ((h & 0x7FF00000) + (90 << 20) < (h1 & 0x7FF00000)) {
+        h = (int)(((unsigned int)h1 ^ 0x80000000u) - (90u << 20));
+        p = __hiloint2double(h, __double2loint(p1));
+      }
+      below += (h ^ h1) < 0 ? 1 : 0;
+      p0 = p1;
+      p1 = p;
+      const int ex = ((h >> 20) & 0x7FF) - 1023;
+      if (ex > 300 || ex < -300) {
+        p1 = __hiloint2double(h - ex * (1 << 20), __double2loint(p1));
+        p0 = __hiloint2double(h1 - ex * (1 << 20), __double2loint(p0));
+      }
+      e = e2[i];
+    }
+    if (below > m) hi = x;
+    else lo = x;
+  }
+  if (m < n) jb.out[m] = ldexp(0.5 * (lo + hi), (int)jb.e[n - 1]);
 }
 
 }  // namespace
@@ -236,25 +291,32 @@ static size_t mp2_bytes(int64_t o, int64_t v, int64_t naux, bool oz, int num_sms
 }
 
 // Bytes one cluster keeps until its group's eigensolver launch: the gamma
-// blocks (when the caller did not ask for them) and global working copies for
-// orders above kJacobiSmemM.
+// blocks (when the caller did not ask for them), the tridiagonal forms and
+// global working copies for orders above kEigSmemN.
 static size_t mp2_keep_bytes(int64_t o, int64_t v) {
-  const int64_t mo = (o + 1) / 2 * 2, mv = (v + 1) / 2 * 2;
-  size_t b = al256((size_t)o * o * 8) + al256((size_t)v * v * 8);
-  if (mo > kJacobiSmemM) b += al256((size_t)mo * mo * 8);
-  if (mv > kJacobiSmemM) b += al256((size_t)mv * mv * 8);
+  size_t b = al256((size_t)o * o * 8) + al256((size_t)v * v * 8) + al256((size_t)o * 16) + al256((size_t)v * 16);
+  if (o > kEigSmemN) b += al256((size_t)o * o * 8);
+  if (v > kEigSmemN) b += al256((size_t)v * v * 8);
   return b;
 }
 
 // Clusters per eigensolver launch: two matrices each, 64 jobs.
 constexpr int64_t kMp2Group = 32;
 
-static cudaError_t launch_jacobi(EigJobs* jobs, cudaStream_t s) {
+static cudaError_t launch_eig(EigJobs* jobs, cudaStream_t s) {
   size_t bytes = 16;
-  for (int k = 0; k < jobs->count; ++k) bytes = std::max(bytes, jacobi_smem_bytes(jobs->j[k]));
-  cudaError_t e = cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  int nmax = 1;
+  for (int k = 0; k < jobs->count; ++k) {
+    bytes = std::max(bytes, eig_smem_bytes(jobs->j[k]));
+    nmax = std::max(nmax, jobs->j[k].n);
+  }
+  cudaError_t e = cudaFuncSetAttribute(k_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  k_jacobi<<<jobs->count, 512, bytes, s>>>(*jobs);
+  k_tridiag<<<jobs->count, EIG_THREADS, bytes, s>>>(*jobs);
+  const size_t b2 = (size_t)nmax * 16;
+  e = cudaFuncSetAttribute(k_bisect, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b2);
+  if (e != cudaSuccess) return e;
+  k_bisect<<<dim3((unsigned)((nmax + 31) / 32), (unsigned)jobs->count), 32, b2, s>>>(*jobs);
   jobs->count = 0;
   return cudaGetLastError();
 }
@@ -329,9 +391,10 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     double* tt = reinterpret_cast<double*>(take((size_t)t2n * 8));
     double* goo = reinterpret_cast<double*>(take_from(keep, (size_t)o * o * 8));
     double* gvv = reinterpret_cast<double*>(take_from(keep, (size_t)v * v * 8));
-    const int mo = (int)((o + 1) / 2 * 2), mv = (int)((v + 1) / 2 * 2);
-    double* eo_work = mo > kJacobiSmemM ? reinterpret_cast<double*>(take_from(keep, (size_t)mo * mo * 8)) : nullptr;
-    double* ev_work = mv > kJacobiSmemM ? reinterpret_cast<double*>(take_from(keep, (size_t)mv * mv * 8)) : nullptr;
+    double* eo_tri = reinterpret_cast<double*>(take_from(keep, (size_t)o * 16));
+    double* ev_tri = reinterpret_cast<double*>(take_from(keep, (size_t)v * 16));
+    double* eo_work = o > kEigSmemN ? reinterpret_cast<double*>(take_from(keep, (size_t)o * o * 8)) : nullptr;
+    double* ev_work = v > kEigSmemN ? reinterpret_cast<double*>(take_from(keep, (size_t)v * v * 8)) : nullptr;
     const int64_t cap = mp2_scratch(o, v, P, oz, h->num_sms);
     const int64_t cap64 = std::min(cap, mp2_scratch(o, v, P, false, h->num_sms));
     double* scratch = reinterpret_cast<double*>(take((size_t)cap * 8));
@@ -383,14 +446,13 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
             GemmView{t2, tt, goo, o, 1, o, o, v * v, o * v * v, 0, v * v, 1, v * v, 1, o * v * v, o, 0, 1, -2.0},
             h->num_sms, scratch, cap64, s, &h->n_launches);
     }
-    // populations: one eigensolver block per requested matrix, launched
-    // once per group of clusters (their blocks stay in the kept region)
+    // populations: the eigensolver's two launches once per group of clusters (their blocks stay in the kept region)
     if (e == cudaSuccess) {
-      if (q.pop_o) jobs->j[jobs->count++] = EigJob{eo_work, goo, q.pop_o, (int)o, mo};
-      if (q.pop_v) jobs->j[jobs->count++] = EigJob{ev_work, gvv, q.pop_v, (int)v, mv};
+      if (q.pop_o) jobs->j[jobs->count++] = EigJob{eo_work, goo, q.pop_o, eo_tri, eo_tri + o, (int)o};
+      if (q.pop_v) jobs->j[jobs->count++] = EigJob{ev_work, gvv, q.pop_v, ev_tri, ev_tri + v, (int)v};
       if (jobs->count > 0 && ((x + 1) % kMp2Group == 0 || x + 1 == n)) {
-        e = launch_jacobi(jobs, s);
-        ++h->n_launches;
+        e = launch_eig(jobs, s);
+        h->n_launches += 2;
       }
     }
   }
