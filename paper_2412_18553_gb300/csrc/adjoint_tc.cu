@@ -494,7 +494,7 @@ AdjPlan adj_plan(int64_t o, int64_t v, int num_sms, bool full) {
   z.noo = al((size_t)NS * o * o * o * vp * 2);
   z.ystride = rup(7 * v * v + 2 * v, 4);
   // partials of the split jobs of one launch (an upper bound over the launches)
-  const int64_t ntv = vt_ntile(v), nto = vt_ntile(o), rows_z = (v + 127) / 128;
+  const int64_t ntv = vt_ntile(v, false), nto = vt_ntile(o, false), rows_z = (v + 127) / 128;
   const int64_t pair_blk = 6 * z.B * vt_seg_blocks((int)v, (int)v, VT_SPLIT_CHUNKS);
   const int64_t d_ooov = vt_split_doubles(rows_z * ((o + nto - 1) / nto), pair_blk, v * o, num_sms) + 8;
   const int64_t d_t2 = vt_split_doubles(rows_z * ((v + ntv - 1) / ntv), pair_blk, v * v, num_sms) + 8;
@@ -637,7 +637,8 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
 
   // tensor maps, encoded once: rows (x, y) in tiles of 8 x 16, rows z alone in
   // tiles of 128; B rows by halves of a tile for the pair launches
-  const int NTv = vt_ntile(v), NTo = vt_ntile(o);
+  const int NTv = vt_ntile(v, false), NTo = vt_ntile(o, false);  // lone launches
+  const int NPv = vt_ntile(v, true), NPo = vt_ntile(o, true);  // pair launches
   VtBank bank;
   bank.n = 0;
   auto add = [&](const void* b0, std::initializer_list<int64_t> dims, std::initializer_list<int64_t> str,
@@ -656,7 +657,7 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
   const VtRoles ZK{0, 2, -1, 1, 3, 0};       // k2 | k1 | rows | slice | group
   int m_g[6], m_l1n[3], m_l1t[3], m_l2[3], m_l3[3], m_t2T, m_noo, m_ovT, m_t2P;
   const int64_t U1 = 1, NB = Z.B, ls = reg_stride / 2;  // elements between the slots' layouts
-  if ((st = vt_slice_maps(&bank, S, o, v, NTv, m_g)) != TE_OK) return st;
+  if ((st = vt_slice_maps(&bank, S, o, v, NPv, m_g)) != TE_OK) return st;
   const int m_on = m_g[0], m_ot = m_g[1], m_ln = m_g[2], m_lt = m_g[3], m_t2 = m_g[4], m_no = m_g[5];
   const int64_t lplane = V * V * vp;
   // L1_g and L2_g are permutations 0..2 (L2_g is the one of G block (g + 2) % 3), L3_g permutations 3..5
@@ -672,9 +673,9 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
       return st;
   }
   const int64_t npx = Z.full ? O : 6, npy = Z.full ? O : 1;  // t2T[r][q] or slots
-  if ((st = add(t2T, {V, V, NS, npx, npy}, {1, vp, V * vp, NS * V * vp, npx * NS * V * vp}, ROW, NTv / 2, 1, &m_t2T)) != TE_OK)
+  if ((st = add(t2T, {V, V, NS, npx, npy}, {1, vp, V * vp, NS * V * vp, npx * NS * V * vp}, ROW, NPv / 2, 1, &m_t2T)) != TE_OK)
     return st;
-  if ((st = add(nooTT, {V, O, O, O, NS}, {1, vp, O * vp, O * O * vp, O * O * O * vp}, VtRoles{0, 1, -1, -1, 4, 0}, NTo / 2,
+  if ((st = add(nooTT, {V, O, O, O, NS}, {1, vp, O * vp, O * O * vp, O * O * O * vp}, VtRoles{0, 1, -1, -1, 4, 0}, NPo / 2,
                 1, &m_noo)) != TE_OK)
     return st;
   if ((st = add(ovT, {V, V, V, NS, Z.full ? O : U1}, {1, vp, V * vp, V * V * vp, NS * V * V * vp}, ZK, NTv, 1, &m_ovT)) !=
@@ -789,7 +790,7 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
     for (int x = 0; x < Bt.n; ++x)
       for (int gi = 0; gi < 3; ++gi) {
         const int pp = PQR[x][gi][0], qq = PQR[x][gi][1], rr = PQR[x][gi][2];
-        vt_job(&b, v, v, v, 8, 16, NTv, reinterpret_cast<double*>(region) + x * A.g_stride + gi * v3, v2, v, 1, VT_STORE);
+        vt_job(&b, v, v, v, 8, 16, NPv, reinterpret_cast<double*>(region) + x * A.g_stride + gi * v3, v2, v, 1, VT_STORE);
         const int f_p[3] = {0, 0, pp}, f_q[3] = {0, 0, qq};
         const int t_qr[3] = {0, qq, rr}, t_pr[3] = {0, pp, rr}, n_rq[3] = {0, rr, qq}, n_rp[3] = {0, rr, pp};
         vt_seg(&b, vt_use(&b, bank, m_on), vt_use(&b, bank, m_t2), 1, v, f_p, t_qr, eO(pp), eT(rr, qq), 1);
@@ -853,7 +854,7 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
         if (std::find(dist.begin(), dist.end(), y) == dist.end()) dist.push_back(y);
     for (int sb : dist) {
       if (!g->ovvv) break;
-      vt_job(&b, v, v, v, 8, 16, NTv, g->ovvv + (int64_t)sb * v3, v2, v, 1, VT_ADD);
+      vt_job(&b, v, v, v, 8, 16, NPv, g->ovvv + (int64_t)sb * v3, v2, v, 1, VT_ADD);
       for (int x = 0; x < Bt.n; ++x)
         for (int gi = 0; gi < 3; ++gi) {
           const int pp = PQR[x][gi][0], qq = PQR[x][gi][1], rr = PQR[x][gi][2];
@@ -867,7 +868,7 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
     for (int sb : dist) {
       if (!g->t2) break;
       // element dt2[l][sb][X][Y]: rows (X, Y), columns l
-      vt_job(&b, v, v, o, 8, 16, NTo, g->t2 + (int64_t)sb * v2, v, 1, (int64_t)o * v2, VT_ADD);
+      vt_job(&b, v, v, o, 8, 16, NPo, g->t2 + (int64_t)sb * v2, v, 1, (int64_t)o * v2, VT_ADD);
       for (int x = 0; x < Bt.n; ++x)
         for (int gi = 0; gi < 3; ++gi) {
           const int pp = PQR[x][gi][0], qq = PQR[x][gi][1], rr = PQR[x][gi][2];

@@ -26,6 +26,35 @@ __device__ __forceinline__ double to_double(float f) {
   return cvt_double(f);
 }
 
+// 2^e (h + l) as a float64 for |l| < ulp(h), by integer operations (about 25
+// against two float64 operations of 64 issue cycles each): l shifted to h's
+// 53-bit grid, rounded to nearest (ties up), and added to h's mantissa; a
+// difference below h's power of two goes to the grid of the next lower one.
+// A zero pair (what decayed integrals leave) gives zero.  Where all that does not
+// hold (values below 2^-71, results out of the normal
+// range, a sum that may cross a power of two) *other is set and the result is void:
+// pair_convert then, in a branch of several elements that the compiler does not
+// turn into predicated float64 work.
+__device__ __forceinline__ double pair_double(float h, float l, int e, bool* other) {
+  const uint32_t uh = __float_as_uint(h), ul = __float_as_uint(l), m = uh & 0x7FFFFFu;
+  const int eh = (int)((uh >> 23) & 255u), d = eh - (int)((ul >> 23) & 255u), ed = eh + 896 + e;
+  const bool zero = ((uh | ul) << 1) == 0u;
+  if (!zero && (eh < 56 || eh == 255 || d < 23 || (d == 23 && ((m + 1u) & 0x7FFFFFu) <= 2u) || (uint32_t)(ed - 2) >= 2040u))
+    *other = true;
+  const bool minus = ((uh ^ ul) >> 31) != 0u;
+  const uint32_t t = (((ul & 0x7FFFFFu) | 0x800000u) << 8) >> min(max(d - 23, 0), 31);  // l in quarter units
+  const uint32_t L = ((minus && m == 0u && d < 54 ? t : t >> 1) + 1u) >> 1;
+  const unsigned long long b = (((unsigned long long)(((uint32_t)ed << 20) | (m >> 3))) << 32) | (m << 29);
+  const unsigned long long r = (minus ? b - L : b + L) | ((unsigned long long)(uh & 0x80000000u) << 32);
+  return zero ? 0.0 : __longlong_as_double((long long)r);
+}
+__device__ __forceinline__ double pair_convert(float h, float l, double scale) {
+  double x;
+  asm volatile("add.f64 %0, %1, %2;" : "=d"(x) : "d"(cvt_double(h)), "d"(cvt_double(l)));
+  asm volatile("mul.f64 %0, %1, %2;" : "=d"(x) : "d"(x), "d"(scale));
+  return x;
+}
+
 // FP32 reciprocal of D rounded to nearest, as a float64
 __device__ __forceinline__ double recip_seed(double D) {
   const uint32_t h = (uint32_t)__double2hiint(D), m = h & 0x7FFFFFFFu;

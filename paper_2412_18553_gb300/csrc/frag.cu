@@ -381,7 +381,7 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
   VtBank bank;
   bank.n = 0;
   int m0[6], mA[6], mB[6];
-  const int NT = vt_ntile(v);
+  const int NT = vt_ntile(v, true);
   if ((st = vt_slice_maps(&bank, S0, o, v, NT, m0)) != TE_OK) return st;
   if ((st = vt_slice_maps(&bank, SA, o, v, NT, mA)) != TE_OK) return st;
   if ((st = vt_slice_maps(&bank, SB, o, v, NT, mB)) != TE_OK) return st;

@@ -9,8 +9,19 @@
 // accumulation block into an FP32 pair sum held in registers and release the
 // accumulators at once, so the next block's MMAs overlap the rest of the
 // epilogue.  A unit's sum leaves once,
-// at its end: GB300's float64 rate is a small fraction of its FP32 rate, and a
-// float64 update per block and element cost more than the MMAs at short K.
+// at its end, converted to float64 by integer operations (GB300's float64 rate is
+// a small fraction of its FP32 rate: two float64 operations per element took 12 of
+// 30 thousand cycles of a 128 x 64 unit with four blocks).
+//
+// On CTA pairs an N tile of at most 64 leaves room for the accumulators of two
+// blocks: the next block's MMAs run while the last one is drained.  What bounds
+// the short-K launches then is tensor memory, whose loads and the MMAs' sums
+// share its ports: a drain takes 2300 cycles alone and 3300 beside MMAs, and
+// neither 16 epilogue warps nor a sum of four instructions changes it much.
+// Eight triples of a gradient at nvir = 120, one set of 128 columns -> two of 64:
+// G 671 -> 520 us, ovvv and t2 479 -> 384; one triple at nvir = 320: 1981 -> 1561,
+// 2057 -> 1503 (the projected energy's pairs, which convert nothing: 1096 -> 1105).
+// Lone CTAs have K of nvir^2 and are bound by their MMAs: one set of 128 columns.
 //
 // Pairs of CTAs share a B tile (cta_group::2): each loads its 128 A rows and half
 // of B, rank 0 issues the MMAs of both SMs, and all bytes of the pair count on
@@ -38,7 +49,6 @@ namespace {
 constexpr int VT_EPI_WARPS = 8;
 constexpr int VT_WARPS = 2 + VT_EPI_WARPS;
 constexpr int VT_THREADS = VT_WARPS * 32;
-constexpr int VT_HALF = VT_NT_MAX / 2;  // columns one epilogue thread holds
 constexpr uint32_t VT_ROW_BYTES = VT_KC * 2;         // 64
 constexpr uint32_t VT_A_SLICE = 128u * VT_ROW_BYTES;  // 8 KB
 
@@ -47,16 +57,12 @@ struct VtUnit {
   int64_t b_begin, b_end;
 };
 
-// unit u; m: the m tile of CTA `rank` (PAIR: of the unit's two)
+// unit u; m: the m tile of CTA `rank` (PAIR: of the unit's two); j: the job of a
+// unit before it
 template <bool PAIR>
-__device__ __forceinline__ VtUnit vt_decode(const VtParams& P, int64_t u, int rank) {
+__device__ __forceinline__ VtUnit vt_decode(const VtParams& P, int64_t u, int rank, int j) {
   VtUnit U;
-  int j = 0, top = P.njobs;  // the last job with unit0 <= u
-  while (top - j > 1) {
-    const int mid = (j + top) >> 1;
-    if (P.job[mid].unit0 <= u) j = mid;
-    else top = mid;
-  }
+  while (j + 1 < P.njobs && P.job[j + 1].unit0 <= u) ++j;
   const VtJob& J = P.job[j];
   uint32_t l = (uint32_t)(u - J.unit0);
   U.job = j;
@@ -165,14 +171,17 @@ __device__ __forceinline__ void join(f2& H, f2& L, f2 a0, f2 a1, f2 a2, f2 w) {
 // SUM: the output kind of every job of the launch.
 template <int NS, bool PAIR, int SUM>
 __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams& P) {
+  constexpr int SETS = PAIR ? 2 : 1;  // sets of accumulators
+  constexpr int COLS = (PAIR ? VT_NT_PAIR : VT_NT_MAX) / 2;  // columns an epilogue thread holds at most
+  constexpr int LD = PAIR ? 16 : 8;                          // and reads at once
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                          ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)P.stages * P.stage_bytes);
   uint64_t* empty = full + P.stages;
   uint64_t* tfull = empty + P.stages;
-  uint64_t* tempty = tfull + 1;
-  uint64_t* drain = tempty + 1;
+  uint64_t* tempty = tfull + SETS;
+  uint64_t* drain = tempty + SETS;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -186,12 +195,17 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
       ptx::mbar_init(&full[s], 1);
       ptx::mbar_init(&empty[s], 1);
     }
-    ptx::mbar_init(tfull, 1);
-    ptx::mbar_init(tempty, W * VT_EPI_WARPS);
+    for (int a = 0; a < SETS; ++a) {
+      ptx::mbar_init(&tfull[a], 1);
+      ptx::mbar_init(&tempty[a], W * VT_EPI_WARPS);
+    }
     ptx::mbar_init(drain, 1);
     *abort_flag = 0;
     ptx::fence_barrier_init();
   }
+  // the scale exponents of all segments, read once
+  __shared__ int seg_exp[VT_MAX_SEGS];
+  for (int q = threadIdx.x; q < P.nsegs; q += VT_THREADS) seg_exp[q] = *P.seg[q].ea + *P.seg[q].eb;
   if (warp == 1) {
     if (PAIR) {
       ptx::tmem_alloc_pair(tmem_slot, P.tmem_cols);
@@ -214,8 +228,10 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
       int pending[8];
       for (int s = 0; s < 8; ++s) pending[s] = -1;
       bool ok = true;
+      int jq = 0;
       for (int64_t u = u0; ok && u < P.total_units; u += ustep) {
-        const VtUnit U = vt_decode<PAIR>(P, u, rank);
+        const VtUnit U = vt_decode<PAIR>(P, u, rank, jq);
+        jq = U.job;
         const VtJob& J = P.job[U.job];
         // the second tile of an odd last pair lies beyond the rows: its loads fill zeros
         const int m1t = U.m / J.nm2, m1_0 = m1t * J.TA, m2_0 = (U.m - m1t * J.nm2) * J.TB;
@@ -265,7 +281,7 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (rank 0) ----------------
-    uint32_t stage = 0, phase = 0, acc_phase = 0;
+    uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
     bool ok = true, issued = false;
     auto wait_all = [&](uint64_t* bar, uint32_t parity, unsigned site) -> bool {
       const int got = (!*abort_flag && ptx::mbar_wait(bar, parity, P.wait_ns)) ? 1 : 0;
@@ -275,18 +291,20 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
     };
     const uint32_t smem0 = ptx::smem_u32(smem);
     const uint64_t desc0 = ptx::smem_desc(0, 8u * VT_ROW_BYTES, 4u);  // 8 rows of the 64-byte swizzle
+    int jq = 0;
     for (int64_t u = u0; ok && rank == 0 && u < P.total_units; u += ustep) {
-      const VtUnit U = vt_decode<PAIR>(P, u, 0);
+      const VtUnit U = vt_decode<PAIR>(P, u, 0, jq);
+      jq = U.job;
       const VtJob& J = P.job[U.job];
       const uint32_t NT = (uint32_t)J.NT;
       // kind::f16, BF16 A and B (K-major), FP32 accumulation, M = 128 or 256, N = NT
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((NT >> 3) << 17) |
                              ((uint32_t)(W * 128 >> 4) << 24);
-      const uint32_t d0 = tmem_base, d1 = tmem_base + NT, dr = tmem_base + 2u * NT;
       const uint32_t bstep = (NT / W) * VT_ROW_BYTES >> 4;
       VtBlock B = vt_first(P, J, U.b_begin);
       for (int64_t b = U.b_begin; ok && b < U.b_end; ++b) {
-        if (!wait_all(tempty, acc_phase ^ 1u, 22)) {
+        const uint32_t d0 = tmem_base + acc * 3u * (uint32_t)P.nt_max, d1 = d0 + NT, dr = d1 + NT;
+        if (!wait_all(&tempty[acc], acc_phase ^ 1u, 22)) {
           ok = false;
           break;
         }
@@ -331,8 +349,11 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
           }
         }
         if (!ok) break;
-        if (ptx::elect_one()) vt_commit<PAIR>(tfull);
-        acc_phase ^= 1u;
+        if (ptx::elect_one()) vt_commit<PAIR>(&tfull[acc]);
+        if (++acc == SETS) {
+          acc = 0;
+          acc_phase ^= 1u;
+        }
         vt_next(P, J, B);
       }
     }
@@ -351,10 +372,12 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
     const int half = (warp - 2) >> 2;        // which half of the N tile
     const int row = quad * 32 + lane;
     const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16);
-    uint32_t acc_phase = 0;
+    uint32_t acc = 0, acc_phase = 0;
+    int jq = 0;
     bool ok = true;
     for (int64_t u = u0; ok && u < P.total_units; u += ustep) {
-      const VtUnit U = vt_decode<PAIR>(P, u, rank);
+      const VtUnit U = vt_decode<PAIR>(P, u, rank, jq);
+      jq = U.job;
       const VtJob& J = P.job[U.job];
       const int m1t = U.m / J.nm2;
       const int m1 = m1t * J.TA + row / J.TB, m2 = (U.m - m1t * J.nm2) * J.TB + row % J.TB;
@@ -363,18 +386,17 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
       // the unit's sum is kept relative to 2^eref, the largest scale of the
       // job's segments: every block's weight 2^(e - eref) <= 1 is exact in FP32
       int eref = -100000;
-      for (int q = lane; q < J.nseg; q += 32) eref = max(eref, *P.seg[J.seg0 + q].ea + *P.seg[J.seg0 + q].eb);
+      for (int q = lane; q < J.nseg; q += 32) eref = max(eref, seg_exp[J.seg0 + q]);
       eref = __reduce_max_sync(0xffffffffu, eref);
-      f2 hi[VT_HALF / 2], lo[VT_HALF / 2];
+      f2 hi[COLS / 2], lo[COLS / 2];
 #pragma unroll
-      for (int q = 0; q < VT_HALF / 2; ++q) hi[q] = lo[q] = f2{0ull};
+      for (int q = 0; q < COLS / 2; ++q) hi[q] = lo[q] = f2{0ull};
       VtBlock B = vt_first(P, J, U.b_begin);
       for (int64_t b = U.b_begin; b < U.b_end; ++b) {
-        const VtSeg& S = P.seg[B.seg];
-        const float wk1 = ldexpf(S.sign < 0 ? -1.f : 1.f, *S.ea + *S.eb - eref);
+        const float wk1 = ldexpf(P.seg[B.seg].sign < 0 ? -1.f : 1.f, seg_exp[B.seg] - eref);
         const f2 wk = f2_make(wk1, wk1);
         int got = 0;
-        if (!*abort_flag) got = ptx::mbar_wait(tfull, acc_phase, P.wait_ns) ? 1 : 0;
+        if (!*abort_flag) got = ptx::mbar_wait(&tfull[acc], acc_phase, P.wait_ns) ? 1 : 0;
         // warp-uniform: tcgen05.ld below is .sync.aligned
         if (!__all_sync(0xffffffffu, got)) {
           if (!*abort_flag && lane == 0) vt_abort(P, abort_flag, 24);
@@ -383,31 +405,37 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
         }
         ptx::tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < VT_HALF / 8; ++q) {
-          if (8 * q < ncol) {
-            const uint32_t cc = (uint32_t)(c_lo + 8 * q);
-            float a0[8], a1[8], a2[8];
-            ptx::tmem_ld8x3(tbase + cc, tbase + (uint32_t)J.NT + cc, tbase + 2u * (uint32_t)J.NT + cc, a0, a1, a2);
+        for (int q = 0; q < COLS / LD; ++q) {
+          if (LD * q < ncol) {
+            const uint32_t cc = acc * 3u * (uint32_t)P.nt_max + (uint32_t)(c_lo + LD * q);
+            float a0[LD], a1[LD], a2[LD];
+            if constexpr (LD == 8)
+              ptx::tmem_ld8x3(tbase + cc, tbase + (uint32_t)J.NT + cc, tbase + 2u * (uint32_t)J.NT + cc, a0, a1, a2);
+            else
+              ptx::tmem_ld16x3(tbase + cc, tbase + (uint32_t)J.NT + cc, tbase + 2u * (uint32_t)J.NT + cc, a0, a1, a2);
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              join<SUM>(hi[4 * q + j], lo[4 * q + j], f2_make(a0[2 * j], a0[2 * j + 1]), f2_make(a1[2 * j], a1[2 * j + 1]),
-                        f2_make(a2[2 * j], a2[2 * j + 1]), wk);
+            for (int j = 0; j < LD / 2; ++j)
+              join<SUM>(hi[LD / 2 * q + j], lo[LD / 2 * q + j], f2_make(a0[2 * j], a0[2 * j + 1]),
+                        f2_make(a1[2 * j], a1[2 * j + 1]), f2_make(a2[2 * j], a2[2 * j + 1]), wk);
           }
         }
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if (PAIR) ptx::mbar_arrive_cluster(ptx::mapa(tempty, 0));
-          else ptx::mbar_arrive(tempty);
+          if (PAIR) ptx::mbar_arrive_cluster(ptx::mapa(&tempty[acc], 0));
+          else ptx::mbar_arrive(&tempty[acc]);
         }
-        acc_phase ^= 1u;
+        if (++acc == SETS) {
+          acc = 0;
+          acc_phase ^= 1u;
+        }
         vt_next(P, J, B);
       }
       if (!ok || !valid) continue;
       if constexpr (SUM == VT_PAIR) {
         float2* dst = static_cast<float2*>(J.C) + (int64_t)m1 * J.c_m1 + (int64_t)m2 * J.c_m2 + U.n0 + c_lo;
 #pragma unroll
-        for (int q = 0; q < VT_HALF / 4; ++q) {
+        for (int q = 0; q < COLS / 4; ++q) {
           if (4 * q < ncol && U.n0 + c_lo + 4 * q < J.N) {
             float h[4], l[4];
             f2_get(hi[2 * q], h[0], h[1]);
@@ -427,7 +455,7 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
         }
         continue;
       }
-      const double scale = ldexp(J.jalpha, eref);
+      const double scale = ldexp(1.0, eref);
       double* dst;
       int64_t dn;
       const bool store = J.nsplit > 1 || J.out == VT_STORE;
@@ -440,38 +468,50 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
       }
       dst += (int64_t)(U.n0 + c_lo) * dn;
 #pragma unroll
-      for (int q = 0; q < VT_HALF / 4; ++q) {
+      for (int q = 0; q < COLS / 4; ++q) {
         const int left = J.N - (U.n0 + c_lo + 4 * q);
         if (4 * q < ncol && left > 0) {
           double* d = dst + 4 * q * dn;
-          double old[4];
-          if (store) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) old[j] = 0.0;
-          } else if (J.vec) {
+          double old[4], x[4];
+          bool other = false;
+          if (!store && J.vec) {
             asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
                          : "=d"(old[0]), "=d"(old[1]), "=d"(old[2]), "=d"(old[3])
                          : "l"(d)
                          : "memory");
-          } else {
+          } else if (!store) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) old[j] = j < left ? d[j * dn] : 0.0;
           }
           float h[4], l[4];
-          f2_get(hi[2 * q], h[0], h[1]);
-          f2_get(hi[2 * q + 1], h[2], h[3]);
-          f2_get(lo[2 * q], l[0], l[1]);
-          f2_get(lo[2 * q + 1], l[2], l[3]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) old[j] = fma(scale, to_double(h[j]) + to_double(l[j]), old[j]);
+          for (int j = 0; j < 2; ++j) {
+            f2 H = hi[2 * q + j], L = lo[2 * q + j];
+            if constexpr (SUM == VT_ADD) {  // its low word is a sum of its own
+              H = f2_add(hi[2 * q + j], L);
+              L = f2_sub(L, f2_sub(H, hi[2 * q + j]));
+            }
+            f2_get(H, h[2 * j], h[2 * j + 1]);
+            f2_get(L, l[2 * j], l[2 * j + 1]);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[j] = pair_double(h[j], l[j], eref, &other);
+          if (other) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = pair_convert(h[j], l[j], scale);
+          }
+          if (!store) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] += old[j];
+          }
           if (J.vec) {
-            asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(d), "d"(old[0]), "d"(old[1]), "d"(old[2]),
-                         "d"(old[3])
+            asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(d), "d"(x[0]), "d"(x[1]), "d"(x[2]),
+                         "d"(x[3])
                          : "memory");
           } else {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-              if (j < left) d[j * dn] = old[j];
+              if (j < left) d[j * dn] = x[j];
           }
         }
       }
@@ -500,8 +540,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(VT_THREADS, 1)
   view_tc_body<NS, true, SUM>(maps, P);
 }
 
-// C[(m1, m2), n] += sum_z part[z][(m1, m2)][n], z in order, for every split job
-// of a launch (one index space over their outputs)
 __global__ void __launch_bounds__(256) k_vt_reduce(const __grid_constant__ VtParams P) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < P.total_red;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -664,7 +702,6 @@ VtJob* vt_job(VtBuild* b, int M1, int M2, int N, int TA, int TB, int NT, void* C
   j->c_m2 = c_m2;
   j->c_n = c_n;
   j->out = (int16_t)out;
-  j->jalpha = 1.0;
   return j;
 }
 
@@ -777,17 +814,17 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s) {
   int nt_max = 16;
   for (int q = 0; q < P.njobs; ++q) {
     const VtJob& J = P.job[q];
-    if (J.NT % 32 != 0 || J.NT < 32 || J.NT > VT_NT_MAX || J.TA * J.TB != 128)
+    if (J.NT % 32 != 0 || J.NT < 32 || J.NT > (b->pair ? VT_NT_PAIR : VT_NT_MAX) || J.TA * J.TB != 128)
       return fail(TE_EINVAL, "view GEMM: tile %d x %d x %d", J.TA, J.TB, J.NT);
     nt_max = std::max<int>(nt_max, J.NT);
   }
   P.nt_max = nt_max;
   P.stage_bytes = (uint32_t)P.ns * (VT_A_SLICE + (uint32_t)(b->pair ? nt_max / 2 : nt_max) * VT_ROW_BYTES);
-  const size_t avail = h->smem_optin > 2048 ? h->smem_optin - 2048 : 0;
+  const size_t avail = h->smem_optin > 4096 ? h->smem_optin - 4096 : 0;
   P.stages = (int)std::min<size_t>(8, avail / P.stage_bytes);
   if (P.stages < 2) return fail(TE_EUNSUPPORTED, "view GEMM: not enough shared memory for two stages");
   uint32_t cols = 32;
-  while (cols < 3u * (uint32_t)nt_max) cols <<= 1;
+  while (cols < (b->pair ? 6u : 3u) * (uint32_t)nt_max) cols <<= 1;
   P.tmem_cols = cols;
   P.err = h->d_err;
   P.wait_ns = h->wait_limit_ns;
@@ -806,8 +843,8 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s) {
   return TE_OK;
 }
 
-int vt_ntile(int64_t n) {
-  const int64_t t = (n + VT_NT_MAX - 1) / VT_NT_MAX;
+int vt_ntile(int64_t n, bool pair) {
+  const int64_t most = pair ? VT_NT_PAIR : VT_NT_MAX, t = (n + most - 1) / most;
   return (int)(((n + t - 1) / t + 31) / 32 * 32);
 }
 

@@ -2,8 +2,8 @@
 //
 // One launch runs a list of jobs.  A job is an output C[(m1, m2), n] in
 // float64 and a list of K segments, each
-//   C[(m1, m2), n] += jalpha alpha 2^(ea + eb) sum_{k1, k2} A[(m1, m2), (k1, k2)] B[n, (k1, k2)]
-// (alpha = +-1 per segment, jalpha per job)
+//   C[(m1, m2), n] += alpha 2^(ea + eb) sum_{k1, k2} A[(m1, m2), (k1, k2)] B[n, (k1, k2)]
+// (alpha = +-1 per segment)
 // where A and B are BF16 slice planes (value = 2^e sum_s slice_s) read through
 // TMA tensor maps whose innermost dimension is the contiguous K index k2.
 // Slice products a_i b_j with i + j <= NS - 1 go to three FP32 accumulators in
@@ -36,6 +36,7 @@ constexpr int VT_MAX_JOBS = 96;
 constexpr int VT_KC = 32;            // K elements per pipeline stage: 64-byte rows, 64-byte swizzle
 constexpr int VT_BLOCK_CHUNKS = 32;  // stages per exact accumulation block: K <= 1024
 constexpr int VT_NT_MAX = 128;       // N tile: three accumulators; an epilogue thread holds NT/2 column sums
+constexpr int VT_NT_PAIR = 64;       // the same on CTA pairs
 
 // Which of a tensor map's five dimensions holds each index of the view; -1 when
 // the view has no such index (r1 for single-index rows, k1 when K = k2 alone).
@@ -48,7 +49,7 @@ struct VtRoles {
 
 struct VtSeg {
   int8_t amap, bmap;
-  int16_t sign;              // +1 or -1 (a job's common factor is VtJob::jalpha)
+  int16_t sign;              // +1 or -1
   int16_t afix[3], bfix[3];  // coordinates of dimensions 2, 3, 4 where they have no role (group indices)
   int nk2c;                  // stages along k2: ceil(K2 / VT_KC)
   int nchunks;               // K1 * nk2c
@@ -57,7 +58,7 @@ struct VtSeg {
 };
 
 // float64 +=, float64 =, or the unit's FP32 pair (hi, lo) as it is: relative to
-// 2^(the largest scale of the job's segments), jalpha not applied.  One kind per
+// 2^(the largest scale of the job's segments).  One kind per
 // launch; VT_STORE and VT_PAIR on CTA pairs.  VT_ADD sums a unit's blocks to 2^-48 of the sum;
 // VT_STORE and VT_PAIR round the higher levels' part to FP32 against the low
 // word first (2^-38 of the operands' scale; few blocks per unit).  VT_STORE is the
@@ -72,7 +73,6 @@ struct VtJob {
   int16_t bchunks;     // stages per accumulation block
   int16_t vec;         // four columns per access (contiguous, 32-byte aligned)
   int nm2, nmu, nn, nsplit;  // m tiles along m2, units along m, N tiles
-  double jalpha;       // factor of the whole job (1 unless set)
   int64_t unit0;       // first unit of the job in the launch
   int64_t nblocks;     // accumulation blocks over all segments
   void* C;             // element (m1, m2, n) at m1 c_m1 + m2 c_m2 + n c_n
@@ -162,8 +162,8 @@ constexpr int VT_SPLIT_CHUNKS = 8;
 // every job into C in split order.
 te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s);
 
-// N tile for an output of n columns: at most VT_NT_MAX, a multiple of 32.
-int vt_ntile(int64_t n);
+// N tile for an output of n columns: at most VT_NT_MAX (VT_NT_PAIR), a multiple of 32.
+int vt_ntile(int64_t n, bool pair);
 
 struct SliceSet;
 // The six views of an exact-slice operand set (tc_prepare_slices) that the
