@@ -31,6 +31,7 @@
 
 #include "strided.h"
 #include "te_internal.h"
+#include "view_tc.h"
 
 namespace te {
 
@@ -267,26 +268,22 @@ __global__ void __launch_bounds__(32) k_bisect(const __grid_constant__ EigJobs J
 }  // namespace
 
 
-// Doubles of split-K partial tiles for the three contractions.  The
-// exact-slice GEMM splits K into blocks of at most 1024 (exactness) and, for
-// outputs with few tiles, into about two blocks per SM; the float64 GEMM fits
-// its split count to the capacity it is given.
-static int64_t mp2_scratch(int64_t o, int64_t v, int64_t naux, bool oz, int num_sms) {
-  const int64_t ov = o * v;
-  const int64_t f64 = std::max<int64_t>(splitk_cap(o, v), 80LL * std::max(o * o, v * v));
-  if (!oz) return f64;
-  return std::max({gemm_oz_scratch(ov, ov, naux, num_sms), f64, (int64_t)1});  // (ia|jb) split K
+// Doubles of split-K partial tiles for the float64 contractions, which fit their
+// split counts to what they are given.
+static int64_t mp2_scratch(int64_t o, int64_t v) {
+  return std::max<int64_t>(splitk_cap(o, v), 80LL * std::max(o * o, v * v));
 }
+static int64_t mp2_pitch(int64_t naux) { return (naux + 7) / 8 * 8; }  // rows of the slices: steps of 16 bytes
 
 static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Bytes of workspace one cluster uses while its contractions run (the largest
 // is allocated; the next cluster reuses it).
-static size_t mp2_bytes(int64_t o, int64_t v, int64_t naux, bool oz, int num_sms) {
+static size_t mp2_bytes(int64_t o, int64_t v, int64_t naux, bool oz) {
   const size_t ovov = (size_t)o * v * o * v, t2n = (size_t)o * o * v * v;
   size_t b = al256(ovov * 8) + 2 * al256(t2n * 8);                       // ovov, t2 (own copy), T~
-  b += al256((size_t)mp2_scratch(o, v, naux, oz, num_sms) * 8);          // split-K partial tiles
-  if (oz) b += al256((size_t)naux * o * v * 8) + al256(64);              // slices of Bov (4 x 2 B per element), scale
+  b += al256((size_t)mp2_scratch(o, v) * 8);                             // split-K partial tiles
+  if (oz) b += al256((size_t)mp2_pitch(naux) * o * v * 8) + al256(64);   // slices of Bov (4 x 2 B per element), scale
   return b;
 }
 
@@ -350,7 +347,7 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     const te_mp2_out& q = outs[x];
     if (!q.t2 && !q.gamma_oo && !q.gamma_vv && !q.pop_o && !q.pop_v)
       return fail(TE_EINVAL, "cluster %lld: no output requested", (long long)x);
-    need_tr = std::max(need_tr, mp2_bytes(c.nocc, c.nvir, c.naux, oz, h->num_sms));
+    need_tr = std::max(need_tr, mp2_bytes(c.nocc, c.nvir, c.naux, oz));
     if (x % kMp2Group == 0) group_keep = 0;
     group_keep += mp2_keep_bytes(c.nocc, c.nvir);
     need_keep = std::max(need_keep, group_keep);
@@ -395,33 +392,33 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     double* ev_tri = reinterpret_cast<double*>(take_from(keep, (size_t)v * 16));
     double* eo_work = o > kEigSmemN ? reinterpret_cast<double*>(take_from(keep, (size_t)o * o * 8)) : nullptr;
     double* ev_work = v > kEigSmemN ? reinterpret_cast<double*>(take_from(keep, (size_t)v * v * 8)) : nullptr;
-    const int64_t cap = mp2_scratch(o, v, P, oz, h->num_sms);
-    const int64_t cap64 = std::min(cap, mp2_scratch(o, v, P, false, h->num_sms));
+    const int64_t cap = mp2_scratch(o, v);
     double* scratch = reinterpret_cast<double*>(take((size_t)cap * 8));
     if (q.t2) t2 = q.t2;
     if (q.gamma_oo) goo = q.gamma_oo;
     if (q.gamma_vv) gvv = q.gamma_vv;
     // input values: finite, max eps_o < min eps_v (reported by te_sync); the
     // same pass finds max |Bov|, the scale of its slices
-    __nv_bfloat16* bs = oz ? reinterpret_cast<__nv_bfloat16*>(take((size_t)P * ov * 8)) : nullptr;
+    __nv_bfloat16* bs = oz ? reinterpret_cast<__nv_bfloat16*>(take((size_t)mp2_pitch(P) * ov * 8)) : nullptr;
     unsigned int* mx = oz ? reinterpret_cast<unsigned int*>(take(64)) : nullptr;
     if (oz) e = cudaMemsetAsync(mx, 0, 4, s);
     if (e == cudaSuccess)
       e = launch_check_mp2(c.eps_o, o, c.eps_v, v, c.Bov, P * ov, x, h->d_err, h->num_sms, s, mx);
     ++h->n_launches;
     // (ia|jb) = sum_P B[P,i,a] B[P,j,b]: rows (i,a), columns (j,b), K = P
-    if (e == cudaSuccess) e = cudaMemsetAsync(ovov, 0, (size_t)ov * ov * 8, s);
     if (!oz) {
+      if (e == cudaSuccess) e = cudaMemsetAsync(ovov, 0, (size_t)ov * ov * 8, s);
       if (e == cudaSuccess)
         e = gemm_strided(GemmView{c.Bov, c.Bov, ovov, o, v, ov, P, 1, v, 1, ov, 0, ov, 0, 1, v * ov, ov, 1, 1.0, true},
                          h->num_sms, scratch, cap, s, &h->n_launches);
     } else {
       int* ex = reinterpret_cast<int*>(mx + 3);
-      if (e == cudaSuccess) e = slice_planes(c.Bov, P * ov, 4, mx, ex, bs, s, &h->n_launches);
-      if (e == cudaSuccess)
-        e = gemm_oz(OzView{bs, bs, P * ov, P * ov, ovov, o, v, ov, P, 1, v, 1, ov, 0, ov, 0, 1, v * ov, ov, 1, 1.0,
-                           ex, ex, 0},
-                    h->num_sms, scratch, cap, s, &h->n_launches);
+      const int64_t Pp = mp2_pitch(P);
+      if (e == cudaSuccess) e = slice_rows(c.Bov, ov, P, Pp, 4, mx, ex, bs, s, &h->n_launches);
+      if (e == cudaSuccess) {
+        const te_status st = vt_product(h, bs, ov * Pp, ov, bs, ov * Pp, ov, P, Pp, 4, ex, ex, ovov, s);
+        if (st != TE_OK) return st;
+      }
     }
     // amplitudes, then the two density contractions in float64 in both modes:
     // their K (o^2 v and o v^2 terms) spans the amplitudes' whole dynamic
@@ -435,7 +432,7 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
       if (e == cudaSuccess) e = cudaMemsetAsync(gvv, 0, (size_t)v * v * 8, s);
       if (e == cudaSuccess)
         e = gemm_strided(GemmView{t2, tt, gvv, v, 1, v, o * o, v, v, 0, v * v, 1, v * v, 1, v, v, 0, 1, 2.0},
-                         h->num_sms, scratch, cap64, s, &h->n_launches);
+                         h->num_sms, scratch, cap, s, &h->n_launches);
       if (e == cudaSuccess) {
         k_two_identity<<<grid_of(o * o), 256, 0, s>>>(goo, (int)o);
         ++h->n_launches;
@@ -444,7 +441,7 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
       if (e == cudaSuccess)
         e = gemm_strided(
             GemmView{t2, tt, goo, o, 1, o, o, v * v, o * v * v, 0, v * v, 1, v * v, 1, o * v * v, o, 0, 1, -2.0},
-            h->num_sms, scratch, cap64, s, &h->n_launches);
+            h->num_sms, scratch, cap, s, &h->n_launches);
     }
     // populations: the eigensolver's two launches once per group of clusters (their blocks stay in the kept region)
     if (e == cudaSuccess) {

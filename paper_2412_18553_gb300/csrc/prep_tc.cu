@@ -388,46 +388,44 @@ __device__ __forceinline__ void rint_digits_wide(double x, int e, int* m) {
   }
 }
 
-// slice s at planes + s n; four elements per thread where the planes allow
+// x [P][n] to rows of K: slice s of x[p][i] at planes[(s n + i) Pp + p], the
+// K-contiguous rows that a tensor map reads.  A block takes 64 p x 32 i: x is read
+// along i, the planes are written along p (128 bytes per row and slice).
+constexpr int SP_P = 64, SP_I = 32;
 template <int NS>
-__global__ void __launch_bounds__(256) k_slice_planes(const double* __restrict__ x, int64_t n,
-                                                      const unsigned int* __restrict__ xhi, int* __restrict__ e_out,
-                                                      unsigned short* __restrict__ planes) {
-  const int e = exp_of_high(*xhi);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *e_out = e;
-  const bool vec = (n & 3) == 0;
-  for (int64_t i = 4 * (blockIdx.x * 256LL + threadIdx.x); i < n; i += 4 * 256LL * gridDim.x) {
-    uint32_t w[4][NS];
+__global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ x, int64_t n, int64_t P, int64_t Pp,
+                                                    const unsigned int* __restrict__ xhi, int* __restrict__ e_out,
+                                                    unsigned short* __restrict__ planes) {
+  __shared__ unsigned short t[NS][SP_I][SP_P + 2];
+  const int e = exp_of_high(*xhi), tid = threadIdx.x;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *e_out = e;
+  const int64_t i0 = (int64_t)blockIdx.x * SP_I, p0 = (int64_t)blockIdx.y * SP_P;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int d[NS];
-      rint_digits_wide<NS>(i + j < n ? __ldg(x + i + j) : 0.0, e, d);
+  for (int q = tid; q < SP_P * SP_I; q += 256) {
+    const int i = q % SP_I, p = q / SP_I;
+    int d[NS];
+    rint_digits_wide<NS>(i0 + i < n && p0 + p < P ? __ldg(x + (p0 + p) * n + i0 + i) : 0.0, e, d);
 #pragma unroll
-      for (int k = 0; k < NS; ++k) w[j][k] = digit_bf16(d[k], 7 * (k + 1));
-    }
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      unsigned short* p = planes + k * n + i;
-      if (vec) {
-        *reinterpret_cast<uint2*>(p) = make_uint2(__byte_perm(w[0][k], w[1][k], 0x5410), __byte_perm(w[2][k], w[3][k], 0x5410));
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (i + j < n) p[j] = (unsigned short)w[j][k];
-      }
-    }
+    for (int k = 0; k < NS; ++k) t[k][i][p] = (unsigned short)digit_bf16(d[k], 7 * (k + 1));
+  }
+  __syncthreads();
+  for (int q = tid; q < NS * SP_I * (SP_P / 2); q += 256) {
+    const int p = 2 * (q % (SP_P / 2)), r = q / (SP_P / 2), i = r % SP_I, k = r / SP_I;
+    if (i0 + i < n && p0 + p < Pp)  // Pp is even
+      *reinterpret_cast<uint32_t*>(planes + ((int64_t)k * n + i0 + i) * Pp + p0 + p) =
+          *reinterpret_cast<const uint32_t*>(&t[k][i][p]);
   }
 }
 
 }  // namespace
 
-cudaError_t slice_planes(const double* x, int64_t n, int ns, const unsigned int* xhi, int* ex, __nv_bfloat16* planes,
-                         cudaStream_t s, int64_t* launches) {
-  if (ns != 4 && ns != 5) return cudaErrorInvalidValue;
-  const int grid = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 1023) / 1024), 1 << 20);
+cudaError_t slice_rows(const double* x, int64_t n, int64_t P, int64_t Pp, int ns, const unsigned int* xhi, int* ex,
+                       __nv_bfloat16* planes, cudaStream_t s, int64_t* launches) {
+  if ((ns != 4 && ns != 5) || P > 65535LL * SP_P || n > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)((n + SP_I - 1) / SP_I), (unsigned)((P + SP_P - 1) / SP_P));
   unsigned short* p = reinterpret_cast<unsigned short*>(planes);
-  if (ns == 5) k_slice_planes<5><<<grid, 256, 0, s>>>(x, n, xhi, ex, p);
-  else k_slice_planes<4><<<grid, 256, 0, s>>>(x, n, xhi, ex, p);
+  if (ns == 5) k_slice_rows<5><<<grid, 256, 0, s>>>(x, n, P, Pp, xhi, ex, p);
+  else k_slice_rows<4><<<grid, 256, 0, s>>>(x, n, P, Pp, xhi, ex, p);
   ++*launches;
   return cudaGetLastError();
 }

@@ -1,6 +1,5 @@
-// Strided-view contractions shared by the adjoint (vjp.cu) and the
-// fragment-projected energy (frag.cu): a float64 DFMA GEMM and an exact-slice
-// BF16 tensor-core GEMM over two-index row and K views, and the per-element
+// Shared by the adjoint, the fragment-projected energy and the MP2 step: a float64
+// DFMA GEMM over two-index row and K views, exact slices, and the per-element
 // assembly of W~ and Y from a triple's three natural-layout G blocks.
 #pragma once
 #include <cuda_bf16.h>
@@ -101,13 +100,6 @@ __device__ __forceinline__ void slice_digits_int(double x, int e, int* d) {
   }
   d[0] = (int)N;
 }
-template <int NS>
-__device__ __forceinline__ void slice_digits(double x, int e, float* d) {
-  int n[NS];
-  slice_digits_int<NS>(x, e, n);
-#pragma unroll
-  for (int k = 0; k < NS; ++k) d[k] = (float)n[k];
-}
 
 // C[m,n] += alpha sum_k A[m,k] B[k,n], m = (m1, m2) and k = (k1, k2) with a
 // stride per index (float64, DFMA; deterministic split-K)
@@ -123,39 +115,16 @@ struct GemmView {
   bool symmetric = false;  // A and B are the same view and C[m,n] and C[n,m] two elements: half the tiles
 };
 
-// the same over NS BF16 slice planes per operand (slice s at base + s *
-// plane; NS = ns, 4 when 0), C (+)= alpha 2^(ea + eb) sum_k A B (exact-slice
-// products on mma.sync)
-struct OzView {
-  const __nv_bfloat16* A;
-  const __nv_bfloat16* B;
-  int64_t a_ps, b_ps;  // slice plane strides (elements)
-  double* C;
-  int64_t M1, M2, N, K1, K2;
-  int64_t a_m1, a_m2, a_k1, a_k2;
-  int64_t b_k1, b_k2, b_n;
-  int64_t c_m1, c_m2, c_n;
-  double alpha;
-  const int* ea;  // device scale exponents of A's and B's slices
-  const int* eb;
-  int overwrite;  // store instead of accumulate (single K split only)
-  int ns;         // slices per operand: 4 (also when 0) or 5
-};
-
 cudaError_t gemm_strided(const GemmView& g, int num_sms, double* scratch, int64_t scratch_cap, cudaStream_t s,
                          int64_t* launches);
-cudaError_t gemm_oz(const OzView& g, int num_sms, double* scratch, int64_t scratch_cap, cudaStream_t s,
-                    int64_t* launches);
-// NS (4 or 5) 7-bit slice planes of x[0..n) with one power-of-two scale: x =
-// 2^e sum_s m_s 2^-7(s+1) + r, |r| <= 2^(e - 7 NS - 1), 2^e > max |x|, whose
-// high word is *xhi (launch_absmax); e goes to *ex, slice s to planes + s n.
-cudaError_t slice_planes(const double* x, int64_t n, int ns, const unsigned int* xhi, int* ex,
-                         __nv_bfloat16* planes, cudaStream_t s, int64_t* launches);
-// doubles of split-K scratch gemm_oz needs for an M x N output over K
-int64_t gemm_oz_scratch(int64_t M, int64_t N, int64_t K, int num_sms);
-// doubles of split-K scratch the two GEMMs need for a cluster's contractions
+// NS (4 or 5) 7-bit slices of x [P][n] with one power-of-two scale: x = 2^e sum_s
+// m_s 2^-7(s+1) + r, |r| <= 2^(e - 7 NS - 1), 2^e > max |x|, whose high word is
+// *xhi (launch_absmax); e goes to *ex, slice s of x[p][i] to planes[(s n + i) Pp + p]
+// (Pp a multiple of 8, at least P).
+cudaError_t slice_rows(const double* x, int64_t n, int64_t P, int64_t Pp, int ns, const unsigned int* xhi, int* ex,
+                       __nv_bfloat16* planes, cudaStream_t s, int64_t* launches);
+// doubles of split-K scratch the GEMM needs for a cluster's contractions
 int64_t splitk_cap(int64_t o, int64_t v);
-int64_t oz_scratch_cap(int64_t o, int64_t v, int num_sms);
 // out = scale * (fixed-order sum of part[0..n))
 cudaError_t launch_sum_share(const double* part, int64_t n, double scale, double* out, cudaStream_t s);
 

@@ -53,6 +53,7 @@
 #include "ptx_sm100.cuh"
 #include "strided.h"
 #include "tc_path.h"
+#include "view_tc.h"
 
 namespace te {
 
@@ -914,28 +915,27 @@ static te_status build_energy_maps(TcState* st, const TcPlan& pl, int o, int v, 
 // ---------------------------------------------------------------------------
 // ovvv from density-fitting factors (t_energy_df):
 //   ovvv[p,x,y,d] = sum_P Bov[P,p,x] Bvv[P,y,d]
-// formed nst slabs at a time by the exact-slice strided GEMM (five 7-bit
-// slices per factor, K blocks of at most 1024 accumulated in float64) into a
-// float64 staging block, then cut into the contraction's operand form.
+// formed nst slabs at a time by the exact-slice view GEMM (five 7-bit slices
+// per factor, K in exact blocks of at most 1024) into a float64 staging block,
+// then cut into the contraction's operand form.
 // ---------------------------------------------------------------------------
 
 constexpr int DF_NS = 5;                                  // slices per factor
 constexpr size_t DF_STAGE_BYTES = size_t(2) << 30;        // staging block limit
-constexpr int64_t DF_KBLOCK = 1024;                       // exact level-0/1 sums
 
 // Scratch of the formation.  It shares the region of the G pool, which the
 // contraction only writes after every operand is ready (stream order).
 struct DfScratch {
-  __nv_bfloat16 *bov = nullptr, *bvv = nullptr;  // DF_NS planes each
+  __nv_bfloat16 *bov = nullptr, *bvv = nullptr;  // DF_NS planes each, [p, x][Pp] and [y, d][Pp]
   unsigned int* mx = nullptr;                    // max |Bov|, max |Bvv| (high words)
   int* ex = nullptr;                             // their scale exponents
   double* stage = nullptr;                       // nst slabs of v^3
-  double* part = nullptr;                        // split-K partial tiles
-  int64_t part_cap = 0;
   int nst = 0;
 };
 
-static size_t df_carve(char* base, int o, int v, int64_t naux, int num_sms, DfScratch* d) {
+static int64_t df_pitch(int64_t naux) { return (naux + 7) / 8 * 8; }  // tensor-map rows in steps of 16 bytes
+
+static size_t df_carve(char* base, int o, int v, int64_t naux, DfScratch* d) {
   size_t off = 0;
   auto take = [&](size_t bytes) -> char* {
     off = (off + 1023) & ~size_t(1023);
@@ -945,40 +945,19 @@ static size_t df_carve(char* base, int o, int v, int64_t naux, int num_sms, DfSc
   };
   const size_t v3 = (size_t)v * v * v;
   d->nst = (int)std::max<size_t>(1, std::min<size_t>((size_t)o, DF_STAGE_BYTES / (v3 * 8)));
-  d->bov = reinterpret_cast<__nv_bfloat16*>(take((size_t)DF_NS * naux * o * v * 2));
-  d->bvv = reinterpret_cast<__nv_bfloat16*>(take((size_t)DF_NS * naux * v * v * 2));
+  d->bov = reinterpret_cast<__nv_bfloat16*>(take((size_t)DF_NS * df_pitch(naux) * o * v * 2));
+  d->bvv = reinterpret_cast<__nv_bfloat16*>(take((size_t)DF_NS * df_pitch(naux) * v * v * 2));
   d->mx = reinterpret_cast<unsigned int*>(take(16));
   d->ex = reinterpret_cast<int*>(take(8));
   d->stage = reinterpret_cast<double*>(take((size_t)d->nst * v3 * 8));
-  // the largest split-K scratch over the slab counts and K blocks that occur
-  int64_t cap = 0;
-  const int64_t kcs[2] = {std::min<int64_t>(naux, DF_KBLOCK), naux % DF_KBLOCK};
-  const int nes[2] = {d->nst, o % d->nst};
-  for (int64_t kc : kcs)
-    for (int ne : nes)
-      if (kc > 0 && ne > 0) cap = std::max(cap, gemm_oz_scratch((int64_t)ne * v, (int64_t)v * v, kc, num_sms));
-  d->part_cap = cap;
-  d->part = reinterpret_cast<double*>(take((size_t)std::max<int64_t>(cap, 1) * 8));
   return (off + 1023) & ~size_t(1023);
 }
 
 // slabs p0 .. p0+ne-1 of ovvv into the staging block ([p - p0][x][y][d])
-static cudaError_t df_form(const te_df* df, int o, int v, int p0, int ne, const DfScratch& d, int num_sms,
-                           cudaStream_t s, int64_t* launches) {
-  const int64_t P = df->naux, ov = (int64_t)o * v, vv = (int64_t)v * v;
-  for (int64_t k0 = 0; k0 < P; k0 += DF_KBLOCK) {
-    const int64_t kc = std::min<int64_t>(DF_KBLOCK, P - k0);
-    // rows m = (p, x) contiguous in Bov[P][o][v]; columns n = (y, d) contiguous in Bvv[P][v][v]
-    const OzView g{d.bov + k0 * ov + (int64_t)p0 * v, d.bvv + k0 * vv, P * ov, P * vv, d.stage,
-                   (int64_t)ne * v, 1, vv, kc, 1,
-                   1, 0, ov, 0,
-                   vv, 0, 1,
-                   vv, 0, 1,
-                   1.0, d.ex, d.ex + 1, k0 == 0 ? 1 : 0, DF_NS};
-    const cudaError_t e = gemm_oz(g, num_sms, d.part, d.part_cap, s, launches);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+static te_status df_form(Handle* h, const te_df* df, int o, int v, int p0, int ne, const DfScratch& d, cudaStream_t s) {
+  const int64_t Pp = df_pitch(df->naux), ov = (int64_t)o * v, vv = (int64_t)v * v;
+  return vt_product(h, d.bov + (int64_t)p0 * v * Pp, ov * Pp, (int64_t)ne * v, d.bvv, vv * Pp, vv, df->naux, Pp, DF_NS, d.ex,
+                    d.ex + 1, d.stage, s);
 }
 
 // Operand planes of one cluster: one pass over the inputs for the value
@@ -986,9 +965,12 @@ static cudaError_t df_form(const te_df* df, int o, int v, int p0, int ne, const 
 // operand.  With df, ovvv comes from the factors (the slabs are formed once
 // for the maximum in the exact-slice modes, once for the slices: the same bits
 // both times); else from c->ovvv.
-static cudaError_t launch_prep_tc(int mode, const te_cluster* c, const TcPlan& pl, const TcBuffers& b,
+static te_status launch_prep_tc(Handle* h, int mode, const te_cluster* c, const TcPlan& pl, const TcBuffers& b,
                                   const te_df* df, const DfScratch* dfs, unsigned int* err, int64_t cluster,
-                                  int num_sms, cudaStream_t s, int64_t* launches) {
+                                  cudaStream_t s) {
+  auto bad = [](cudaError_t e) { return fail(TE_ECUDA, "operand split launch: %s", cudaGetErrorString(e)); };
+  const int num_sms = h->num_sms;
+  int64_t* const launches = &h->n_launches;
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int64_t v2 = (int64_t)v * v, v3 = v2 * v;
   const bool oz = is_ozaki(mode);
@@ -999,28 +981,30 @@ static cudaError_t launch_prep_tc(int mode, const te_cluster* c, const TcPlan& p
       mo.ovvv = df ? nullptr : b.maxhi;
       mo.t2 = b.maxhi + 1;
       mo.ooov = b.maxhi + 2;
-      if ((e = cudaMemsetAsync(b.maxhi, 0, 4 * 4, s)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(b.maxhi, 0, 4 * 4, s)) != cudaSuccess) return bad(e);
     }
     if (df) {
       mo.bov = dfs->mx;
       mo.bvv = dfs->mx + 1;
-      if ((e = cudaMemsetAsync(dfs->mx, 0, 2 * 4, s)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(dfs->mx, 0, 2 * 4, s)) != cudaSuccess) return bad(e);
     }
     e = launch_check_inputs(c, cluster, err, num_sms, s, df, &mo);
     ++*launches;
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return bad(e);
   }
   if (df) {
-    e = slice_planes(df->Bov, df->naux * o * v, DF_NS, dfs->mx, dfs->ex, dfs->bov, s, launches);
-    if (e == cudaSuccess) e = slice_planes(df->Bvv, df->naux * v2, DF_NS, dfs->mx + 1, dfs->ex + 1, dfs->bvv, s, launches);
+    const int64_t P = df->naux, Pp = df_pitch(P);
+    e = slice_rows(df->Bov, (int64_t)o * v, P, Pp, DF_NS, dfs->mx, dfs->ex, dfs->bov, s, launches);
+    if (e == cudaSuccess) e = slice_rows(df->Bvv, v2, P, Pp, DF_NS, dfs->mx + 1, dfs->ex + 1, dfs->bvv, s, launches);
     for (int p0 = 0; oz && p0 < o && e == cudaSuccess; p0 += dfs->nst) {
       const int ne = std::min(dfs->nst, o - p0);
-      e = df_form(df, o, v, p0, ne, *dfs, num_sms, s, launches);
+      const te_status st = df_form(h, df, o, v, p0, ne, *dfs, s);
+      if (st != TE_OK) return st;
       const MaxArray a{dfs->stage, 1, (int64_t)ne * v3, 0, b.maxhi, nullptr, 0, 0u};
-      if (e == cudaSuccess) e = launch_absmax(&a, 1, nullptr, 0, nullptr, 0, 0, nullptr, num_sms, s);
+      e = launch_absmax(&a, 1, nullptr, 0, nullptr, 0, 0, nullptr, num_sms, s);
       ++*launches;
     }
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return bad(e);
   }
   SplitScales sc{};
   if (oz) {
@@ -1044,15 +1028,15 @@ static cudaError_t launch_prep_tc(int mode, const te_cluster* c, const TcPlan& p
   const size_t group = (size_t)pl.nparts * v2 * pl.vp * pl.es;
   for (int p0 = 0; df && p0 < o && e == cudaSuccess; p0 += dfs->nst) {
     const int ne = std::min(dfs->nst, o - p0);
-    e = df_form(df, o, v, p0, ne, *dfs, num_sms, s, launches);
-    if (e != cudaSuccess) break;
+    const te_status st = df_form(h, df, o, v, p0, ne, *dfs, s);
+    if (st != TE_OK) return st;
     Parts Ap{};
     for (int k = 0; k < MAX_PARTS; ++k) Ap.p[k] = b.a[k] ? static_cast<char*>(b.a[k]) + (size_t)p0 * group : nullptr;
     const SplitJob slab{SPLIT_ROWS, dfs->stage, Ap, nullptr, v, pl.vp, ne * v2, 1, 0, 0, v2, 1, 0, nullptr, 0};
     e = launch_split(mode, &slab, 1, sc, s);
     ++*launches;
   }
-  return e;
+  return e == cudaSuccess ? TE_OK : bad(e);
 }
 
 template <int MODE>
@@ -1308,9 +1292,9 @@ static te_status setup_job(Handle* h, TcState* st, const te_cluster* c, int mode
   J->tiles_per_triple = 3LL * pl.n_mp * pl.n_nt;
   tc_carve_cluster(base, pl, J->o, J->v, num_unique_triples(J->o), &J->b);
   J->shares = J->b.etri;
-  const cudaError_t e = launch_prep_tc(mode, c, pl, J->b, df, dfs, h->d_err, cluster, h->num_sms, s, &h->n_launches);
-  if (e != cudaSuccess) return fail(TE_ECUDA, "operand split launch: %s", cudaGetErrorString(e));
-  te_status rs = build_maps(st, pl, J->o, J->v, J->b, &J->maps);
+  te_status rs = launch_prep_tc(h, mode, c, pl, J->b, df, dfs, h->d_err, cluster, s);
+  if (rs != TE_OK) return rs;
+  rs = build_maps(st, pl, J->o, J->v, J->b, &J->maps);
   if (rs != TE_OK) return rs;
   return build_energy_maps(st, pl, J->o, J->v, J->b, &J->em);
 }
@@ -1338,7 +1322,7 @@ static size_t single_bytes(const Handle* h, TcPlan* pl, int o, int v, const te_d
   TcBuffers b;
   DfScratch d;
   const size_t fixed = tc_carve_cluster(nullptr, *pl, o, v, num_unique_triples(o), &b);
-  const size_t form = df ? df_carve(nullptr, o, v, df->naux, h->num_sms, &d) : size_t(0);
+  const size_t form = df ? df_carve(nullptr, o, v, df->naux, &d) : size_t(0);
   size_t bytes = fixed + std::max(tc_shared_bytes(single_pool(*pl, v), h->num_sms), form);
   if ((lean || (h->ws_limit && bytes > h->ws_limit)) && pl->nslots > MIN_SLOTS) {
     pl->nslots = (int)MIN_SLOTS;
@@ -1525,7 +1509,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
     const size_t cbytes = tc_carve_cluster(wbase, pl, o, v, nt, &J.b);
     cudaError_t e = cudaSuccess;
     if (!prepped) {  // the operand planes sit first in the workspace for every candidate
-      e = launch_prep_tc(mode, c, pl, J.b, nullptr, nullptr, nullptr, 0, h->num_sms, s, &h->n_launches);
+      if (launch_prep_tc(h, mode, c, pl, J.b, nullptr, nullptr, nullptr, 0, s) != TE_OK) e = cudaErrorUnknown;
       prepped = true;
     }
     if (e != cudaSuccess || build_maps(st, pl, o, v, J.b, &J.maps) != TE_OK) continue;
@@ -1603,7 +1587,7 @@ te_status run_tc(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin
   const size_t cbytes = tc_carve_cluster(nullptr, pl, o, v, ntri, &b);
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023));
   std::vector<TcJob> jobs(1);
-  if (df) df_carve(base + cbytes, o, v, df->naux, h->num_sms, &dfs);  // over the G pool, before its first use
+  if (df) df_carve(base + cbytes, o, v, df->naux, &dfs);  // over the G pool, before its first use
   rs = setup_job(h, st, c, mode, t_begin, t_end, pl, base, &jobs[0], 0, s, df, df ? &dfs : nullptr);
   if (rs != TE_OK) return rs;
   if (e_tri_out) jobs[0].shares = e_tri_out;  // shares[t - t_begin]

@@ -36,6 +36,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 
 #include "fp_util.cuh"
 #include "ptx_sm100.cuh"
@@ -744,8 +745,8 @@ te_status vt_finish(VtBuild* b, int num_sms, double* part_scratch, int64_t scrat
   for (int q = 0; q < b->P.njobs; ++q) {
     VtJob& J = b->P.job[q];
     if (J.nseg == 0) return fail(TE_EINVAL, "view GEMM: job without segments");
-    if (J.out != b->P.job[0].out || (J.out != VT_ADD && !b->pair))
-      return fail(TE_EINVAL, "view GEMM: one output kind per launch; VT_STORE and VT_PAIR on CTA pairs");
+    if (J.out != b->P.job[0].out || (J.out == VT_PAIR && !b->pair))
+      return fail(TE_EINVAL, "view GEMM: one output kind per launch; VT_PAIR on CTA pairs");
     int kblocks = 0;
     for (int g = J.seg0; g < J.seg0 + J.nseg; ++g) {
       const VtSeg& S = b->P.seg[g];
@@ -846,6 +847,28 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s) {
 int vt_ntile(int64_t n, bool pair) {
   const int64_t most = pair ? VT_NT_PAIR : VT_NT_MAX, t = (n + most - 1) / most;
   return (int)(((n + t - 1) / t + 31) / 32 * 32);
+}
+
+te_status vt_product(Handle* h, const void* a, int64_t a_plane, int64_t m, const void* b, int64_t b_plane, int64_t n,
+                     int64_t K, int64_t Kp, int ns, const int* ea, const int* eb, double* C, cudaStream_t s) {
+  const VtRoles ROW{0, 1, -1, -1, 2, 0};
+  const int NT = vt_ntile(n, false);
+  VtBank bank;
+  bank.n = 0;
+  int ma = 0, mb = 0;
+  const uint64_t NS = (uint64_t)ns;
+  const VtView va{a, {(uint64_t)K, (uint64_t)m, NS, 1, 1}, {1, (uint64_t)Kp, (uint64_t)a_plane, 0, 0}, ROW};
+  const VtView vb{b, {(uint64_t)K, (uint64_t)n, NS, 1, 1}, {1, (uint64_t)Kp, (uint64_t)b_plane, 0, 0}, ROW};
+  te_status st = vt_bank_add(&bank, va, 128, 1, &ma);
+  if (st == TE_OK) st = vt_bank_add(&bank, vb, NT, 1, &mb);
+  if (st != TE_OK) return st;
+  std::unique_ptr<VtBuild> B(new VtBuild);
+  vt_begin(B.get(), ns, false);
+  const int none[3] = {0, 0, 0};
+  vt_job(B.get(), 1, (int)m, (int)n, 1, 128, NT, C, 0, n, 1, VT_STORE);
+  vt_seg(B.get(), vt_use(B.get(), bank, ma), vt_use(B.get(), bank, mb), 1, (int)K, none, none, ea, eb, 1);
+  st = vt_finish(B.get(), h->num_sms, nullptr, 0, nullptr);
+  return st == TE_OK ? vt_launch(h, B.get(), s) : st;
 }
 
 te_status vt_slice_maps(VtBank* k, const SliceSet& S, int o, int v, int nt, int* idx) {

@@ -59,8 +59,8 @@ struct VtSeg {
 
 // float64 +=, float64 =, or the unit's FP32 pair (hi, lo) as it is: relative to
 // 2^(the largest scale of the job's segments).  One kind per
-// launch; VT_STORE and VT_PAIR on CTA pairs.  VT_ADD sums a unit's blocks to 2^-48 of the sum;
-// VT_STORE and VT_PAIR round the higher levels' part to FP32 against the low
+// launch; VT_PAIR on CTA pairs only.  VT_ADD (and VT_STORE on lone CTAs) sums a unit's blocks to 2^-48 of the sum;
+// VT_STORE on pairs and VT_PAIR round the higher levels' part to FP32 against the low
 // word first (2^-38 of the operands' scale; few blocks per unit).  VT_STORE is the
 // adjoint's G, whose last bits decide how dW~ is cut.
 enum VtOut { VT_ADD = 0, VT_STORE = 1, VT_PAIR = 2 };
@@ -164,6 +164,15 @@ te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s);
 
 // N tile for an output of n columns: at most VT_NT_MAX (VT_NT_PAIR), a multiple of 32.
 int vt_ntile(int64_t n, bool pair);
+
+// C[i][j] = 2^(ea + eb) sum_k A[i][k] B[j][k] (i < m, j < n; C has rows of n) over ns
+// slice planes with rows of Kp elements (Kp a multiple of 8, planes 16-byte aligned),
+// on lone CTAs: K of hundreds or more, bound by the MMAs.  The ovvv of nocc=16
+// nvir=160 from 704 auxiliary functions (five slices): 1.17 ms, 3.40 ms with mma.sync on
+// row-contiguous factors; batches of MP2 steps gain by as much (eight clusters of
+// nocc 8 .. 20, nvir = 8 nocc, exact slices: 18.0 ms a call).
+te_status vt_product(Handle* h, const void* a, int64_t a_plane, int64_t m, const void* b, int64_t b_plane, int64_t n,
+                     int64_t K, int64_t Kp, int ns, const int* ea, const int* eb, double* C, cudaStream_t s);
 
 struct SliceSet;
 // The six views of an exact-slice operand set (tc_prepare_slices) that the

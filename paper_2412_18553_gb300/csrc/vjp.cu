@@ -16,9 +16,6 @@
 // + ovs(jb,kc) t1(ia) + ovs(ia,kc) t1(jb) with ovs = (ovov + ovov^T)/2 gives the
 // ovov and t1 parts.  Triples are processed one after another on the stream
 // and every accumulation has a fixed order, so the gradient is deterministic.
-#include <atomic>
-#include <cuda_bf16.h>
-
 #include <algorithm>
 #include <initializer_list>
 #include <vector>
@@ -231,368 +228,6 @@ cudaError_t gemm_strided(const GemmView& g, int num_sms, double* scratch, int64_
   if (nsplit > 1) {
     const int64_t MN = M * g.N;
     k_splitk_add<<<(unsigned)std::min<int64_t>((MN + 255) / 256, 4096), 256, 0, s>>>(g, nsplit, scratch);
-    ++*launches;
-  }
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// exact-slice strided GEMM on the tensor cores (mma.sync, BF16 -> FP32):
-//   C[m,n] (+)= alpha 2^(ea + eb) sum_k A[m,k] B[k,n]
-// A and B are NS BF16 slice planes each (slice s at base + s * plane; NS = 4,
-// or 5 for 35-bit operands), read through the same two-index strided views as
-// the float64 kernel.  The slice products a_i b_j with i + j <= NS - 1 (ten,
-// or fifteen) go to three FP32 accumulators:
-// level 0 and level 1 exactly (K <= 1024 per block keeps their partial sums
-// integer multiples of the level's unit below 2^24), the higher levels
-// approximately; each block's sums go to float64 once, at its end.
-// ---------------------------------------------------------------------------
-
-
-constexpr int OZ_BM = 64, OZ_BN = 64, OZ_BK = 32, OZ_KMAX = 1024;
-constexpr int OZ_THREADS = 256;  // eight warps, each 32 x 16 outputs
-constexpr int OZ_LD = OZ_BK + 8;  // padded row (bf16): conflict-free fragment loads
-
-__device__ __forceinline__ void mma_bf16_16816(float* d, const uint32_t* a, const uint32_t* b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// Tiles of 64 x 64 outputs, 32 k per stage, two stages in flight (cp.async).
-// Each operand tile sits in shared memory k-major ([row][k]) when its view is
-// contiguous along k, else row-major ([k][row]) when contiguous along its rows
-// (columns); 16-byte chunks of eight BF16 values are copied asynchronously
-// where the view allows, element by element otherwise.
-template <bool AK, bool BK, int NS>
-struct OzTile {
-  static constexpr int A = AK ? OZ_BM * OZ_LD : OZ_BK * (OZ_BM + 8);
-  static constexpr int B = BK ? OZ_BN * OZ_LD : OZ_BK * (OZ_BN + 8);
-  static constexpr int STAGE = NS * (A + B);  // elements
-  static constexpr size_t BYTES = 2 * STAGE * sizeof(__nv_bfloat16);
-};
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-
-// four 8 x 8 BF16 matrices from shared memory, as stored / transposed
-__device__ __forceinline__ void ldsm_x4(uint32_t* r, const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t* r, const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-
-// Eight elements (rows r + e step_r, k + e step_k) of every slice, element by
-// element, zero outside the view: ragged edges and views without a
-// contiguous index.  Rolled loops, so the pipelined loop stays small enough
-// for the instruction cache.
-__device__ __forceinline__ void oz_fill_slow(const __nv_bfloat16* __restrict__ src, int64_t ps, __nv_bfloat16* dst,
-                                          int dps, int ns, int r, int k, int step_r, int step_k, int R, int ke,
-                                          int R2, int64_t r1s, int64_t r2s, int K2, int64_t k1s, int64_t k2s) {
-#pragma unroll 1
-  for (int e = 0; e < 8; ++e) {
-    const int rr = r + e * step_r, kk = k + e * step_k;
-    const bool ok = rr < R && kk < ke;
-    const int64_t off =
-        ok ? (int64_t)(rr / R2) * r1s + (int64_t)(rr % R2) * r2s + (int64_t)(kk / K2) * k1s + (int64_t)(kk % K2) * k2s
-           : 0;
-#pragma unroll 1
-    for (int sl = 0; sl < ns; ++sl) dst[sl * dps + e] = ok ? src[off + sl * ps] : __float2bfloat16_rn(0.f);
-  }
-}
-
-template <bool AK, bool BK, int NS>
-__global__ void __launch_bounds__(OZ_THREADS, 2) k_gemm_oz2(OzView g, int kchunk, double* __restrict__ part,
-                                                            int a_vec, int b_vec) {
-  using T = OzTile<AK, BK, NS>;
-  extern __shared__ __align__(16) unsigned char oz_smem[];
-  __nv_bfloat16* smem = reinterpret_cast<__nv_bfloat16*>(oz_smem);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int M = (int)(g.M1 * g.M2), N = (int)g.N, K2 = (int)g.K2;
-  const int m0 = blockIdx.x * OZ_BM, n0 = blockIdx.y * OZ_BN;
-  const int kb = blockIdx.z * kchunk, ke = min((int)(g.K1 * g.K2), kb + kchunk);
-  const int nst = (ke - kb + OZ_BK - 1) / OZ_BK;
-
-  auto a_row = [&](int m) { return (int64_t)(m / (int)g.M2) * g.a_m1 + (int64_t)(m % (int)g.M2) * g.a_m2; };
-  auto a_kof = [&](int k) { return (int64_t)(k / K2) * g.a_k1 + (int64_t)(k % K2) * g.a_k2; };
-  auto b_kof = [&](int k) { return (int64_t)(k / K2) * g.b_k1 + (int64_t)(k % K2) * g.b_k2; };
-  // 256 chunks of 8 elements per slice and operand, OZ_CH per thread; the row
-  // (column) part of a chunk's offset is the same at every stage
-  constexpr int OZ_CH = 256 / OZ_THREADS;
-  int64_t a_roff[OZ_CH];
-#pragma unroll
-  for (int c2 = 0; c2 < OZ_CH; ++c2) {
-    const int c = tid + OZ_THREADS * c2;
-    const int m = AK ? m0 + (c >> 2) : m0 + (c & 7) * 8;
-    a_roff[c2] = m < M ? a_row(m) : 0;
-  }
-
-  // one 8-element chunk: elements e = 0..7 along the tile's contiguous direction
-  auto load_stage = [&](int buf, int k0) {
-    __nv_bfloat16* As = smem + buf * T::STAGE;
-    __nv_bfloat16* Bs = As + NS * T::A;
-#pragma unroll
-    for (int c2 = 0; c2 < OZ_CH; ++c2) {
-      const int c = tid + OZ_THREADS * c2;
-      // ---- A ----
-      {
-        int m, k, step_m, step_k;  // first element and the step between the 8
-        __nv_bfloat16* dst0;
-        if (AK) {
-          m = m0 + (c >> 2);
-          k = k0 + (c & 3) * 8;
-          step_m = 0;
-          step_k = 1;
-          dst0 = As + (c >> 2) * OZ_LD + (c & 3) * 8;
-        } else {
-          k = k0 + (c >> 3);
-          m = m0 + (c & 7) * 8;
-          step_m = 1;
-          step_k = 0;
-          dst0 = As + (c >> 3) * (OZ_BM + 8) + (c & 7) * 8;
-        }
-        const bool full = a_vec && (AK ? (m < M && k + 8 <= ke) : (k < ke && m + 8 <= M));
-        if (full) {
-          const __nv_bfloat16* src = g.A + a_roff[c2] + a_kof(k);
-#pragma unroll
-          for (int sl = 0; sl < NS; ++sl) cp_async16(dst0 + sl * T::A, src + sl * g.a_ps);
-        } else {
-          oz_fill_slow(g.A, g.a_ps, dst0, T::A, NS, m, k, step_m, step_k, M, ke, (int)g.M2, g.a_m1, g.a_m2, K2,
-                       g.a_k1, g.a_k2);
-        }
-      }
-      // ---- B ----
-      {
-        int n, k, step_n, step_k;
-        __nv_bfloat16* dst0;
-        if (BK) {
-          n = n0 + (c >> 2);
-          k = k0 + (c & 3) * 8;
-          step_n = 0;
-          step_k = 1;
-          dst0 = Bs + (c >> 2) * OZ_LD + (c & 3) * 8;
-        } else {
-          k = k0 + (c >> 3);
-          n = n0 + (c & 7) * 8;
-          step_n = 1;
-          step_k = 0;
-          dst0 = Bs + (c >> 3) * (OZ_BN + 8) + (c & 7) * 8;
-        }
-        const bool full = b_vec && (BK ? (n < N && k + 8 <= ke) : (k < ke && n + 8 <= N));
-        if (full) {
-          const __nv_bfloat16* src = g.B + (int64_t)n * g.b_n + b_kof(k);
-#pragma unroll
-          for (int sl = 0; sl < NS; ++sl) cp_async16(dst0 + sl * T::B, src + sl * g.b_ps);
-        } else {
-          oz_fill_slow(g.B, g.b_ps, dst0, T::B, NS, n, k, step_n, step_k, N, ke, 1, g.b_n, 0, K2, g.b_k1, g.b_k2);
-        }
-      }
-    }
-  };
-
-  const int wm = (warp & 1) * 32, wn = (warp >> 1) * 16;
-  const int gq = lane >> 2, tq = lane & 3;
-  float acc[3][2][2][4];
-#pragma unroll
-  for (int l = 0; l < 3; ++l)
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[l][i][j][q] = 0.f;
-
-  if (nst > 0) load_stage(0, kb);
-  cp_async_commit();
-  for (int st = 0; st < nst; ++st) {
-    if (st + 1 < nst) load_stage((st + 1) & 1, kb + (st + 1) * OZ_BK);
-    cp_async_commit();
-    cp_async_wait1();  // every group but the newest: this stage's copies have landed
-    __syncthreads();
-    const __nv_bfloat16* As = smem + (st & 1) * T::STAGE;
-    const __nv_bfloat16* Bs = As + NS * T::A;
-#pragma unroll
-    for (int kk = 0; kk < OZ_BK; kk += 16) {
-      // ldmatrix: lane l addresses row (l & 7) of 8 x 8 matrix (l >> 3)
-      const int lr = lane & 7, lm = lane >> 3;
-      uint32_t bf[NS][2][2];
-#pragma unroll
-      for (int sl = 0; sl < NS; ++sl) {
-        // matrices: (cols 0-7, k kk), (cols 0-7, k kk+8), (cols 8-15, k kk), (cols 8-15, k kk+8)
-        const __nv_bfloat16* b = Bs + sl * T::B;
-        uint32_t t[4];
-        const int cb = wn + (lm >> 1) * 8;
-        if (BK) ldsm_x4(t, b + (cb + lr) * OZ_LD + kk + (lm & 1) * 8);
-        else ldsm_x4_t(t, b + (kk + lr + (lm & 1) * 8) * (OZ_BN + 8) + cb);
-        bf[sl][0][0] = t[0];
-        bf[sl][0][1] = t[1];
-        bf[sl][1][0] = t[2];
-        bf[sl][1][1] = t[3];
-      }
-#pragma unroll
-      for (int sa = 0; sa < NS; ++sa) {
-        uint32_t af[2][4];  // A slice sa, loaded when its products are due
-        const __nv_bfloat16* a = As + sa * T::A;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int r = wm + i * 16;
-          // matrices: (rows r, k kk), (rows r+8, k kk), (rows r, k kk+8), (rows r+8, k kk+8)
-          if (AK) ldsm_x4(af[i], a + (r + lr + (lm & 1) * 8) * OZ_LD + kk + (lm >> 1) * 8);
-          else ldsm_x4_t(af[i], a + (kk + lr + (lm >> 1) * 8) * (OZ_BM + 8) + r + (lm & 1) * 8);
-        }
-#pragma unroll
-        for (int sb = 0; sb < NS - sa; ++sb) {
-          const int lev = sa + sb == 0 ? 0 : (sa + sb == 1 ? 1 : 2);
-#pragma unroll
-          for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) mma_bf16_16816(acc[lev][i][j], af[i], bf[sb][j]);
-        }
-      }
-    }
-    __syncthreads();  // the buffer is refilled two stages on
-  }
-  const double scale = ldexp(g.alpha, *g.ea + *g.eb);
-  // this thread's four output rows (i, half h) and their offsets in C
-  int64_t crow[2][2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {
-      const int m = m0 + wm + i * 16 + gq + hh * 8;
-      crow[i][hh] = m < M ? (int64_t)(m / (int)g.M2) * g.c_m1 + (int64_t)(m % (int)g.M2) * g.c_m2 : 0;
-    }
-  // Per 16-row half: every old value of C is loaded before any store, so the
-  // loads overlap (a store could otherwise alias the next load).
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    double val[2][4], old[2][4];
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int m = m0 + wm + i * 16 + gq + (q >> 1) * 8;
-        const int n = n0 + wn + j * 8 + 2 * tq + (q & 1);
-        val[j][q] = scale * (((double)acc[0][i][j][q] + (double)acc[1][i][j][q]) + (double)acc[2][i][j][q]);
-        old[j][q] = (!part && !g.overwrite && m < M && n < N) ? g.C[crow[i][q >> 1] + n * g.c_n] : 0.0;
-      }
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int m = m0 + wm + i * 16 + gq + (q >> 1) * 8;
-        const int n = n0 + wn + j * 8 + 2 * tq + (q & 1);
-        if (m >= M || n >= N) continue;
-        if (part) part[((int64_t)blockIdx.z * M + m) * N + n] = val[j][q];
-        else g.C[crow[i][q >> 1] + n * g.c_n] = old[j][q] + val[j][q];
-      }
-  }
-}
-
-// C[m,n] += sum_z part[z][m][n], z in order (alpha is already applied)
-__global__ void k_splitk_add_oz(OzView g, int nsplit, const double* __restrict__ part) {
-  const int M = (int)(g.M1 * g.M2);
-  const int64_t MN = (int64_t)M * g.N;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < MN; e += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;  // in split order; unrolled so that many loads are in flight
-#pragma unroll 16
-    for (int z = 0; z < nsplit; ++z) s += part[z * MN + e];
-    const int m = (int)(e / g.N), n = (int)(e % g.N);
-    double* cp = g.C + (int64_t)(m / (int)g.M2) * g.c_m1 + (int64_t)(m % (int)g.M2) * g.c_m2 + n * g.c_n;
-    *cp = g.overwrite ? s : *cp + s;
-  }
-}
-
-template <bool AK, bool BK, int NS>
-static cudaError_t launch_oz2(const OzView& g, dim3 grid, int kchunk, double* part, int av, int bv, cudaStream_t s) {
-  const size_t bytes = OzTile<AK, BK, NS>::BYTES;
-  static std::atomic<unsigned long long> opted{0};  // devices this instantiation may use `bytes` on
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (!(opted.load() & bit)) {
-    e = cudaFuncSetAttribute(k_gemm_oz2<AK, BK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
-    opted.fetch_or(bit);
-  }
-  k_gemm_oz2<AK, BK, NS><<<grid, OZ_THREADS, bytes, s>>>(g, kchunk, part, av, bv);
-  return cudaGetLastError();
-}
-
-// K in splits of at most OZ_KMAX (exactness), more when the output has few
-// tiles: the K chunk per split (a multiple of OZ_BK)
-static int oz_kchunk(int64_t M, int64_t N, int64_t K, int num_sms) {
-  const int64_t tm = (M + OZ_BM - 1) / OZ_BM, tn = (N + OZ_BN - 1) / OZ_BN;
-  const int64_t steps = (K + OZ_BK - 1) / OZ_BK;
-  int64_t ns = std::max<int64_t>((K + OZ_KMAX - 1) / OZ_KMAX, (2LL * num_sms + tm * tn - 1) / (tm * tn));
-  ns = std::min<int64_t>(ns, std::max<int64_t>(1, steps / 4));
-  ns = std::max<int64_t>(ns, (K + OZ_KMAX - 1) / OZ_KMAX);
-  return (int)(((steps + ns - 1) / ns) * OZ_BK);
-}
-
-int64_t gemm_oz_scratch(int64_t M, int64_t N, int64_t K, int num_sms) {
-  const int kchunk = oz_kchunk(M, N, K, num_sms);
-  const int64_t nsplit = (K + kchunk - 1) / kchunk;
-  return nsplit > 1 ? nsplit * M * N : 0;
-}
-
-cudaError_t gemm_oz(const OzView& g, int num_sms, double* scratch, int64_t scratch_cap, cudaStream_t s,
-                           int64_t* launches) {
-  const int64_t M = g.M1 * g.M2, K = g.K1 * g.K2;
-  const int64_t tm = (M + OZ_BM - 1) / OZ_BM, tn = (g.N + OZ_BN - 1) / OZ_BN;
-  const int kchunk = oz_kchunk(M, g.N, K, num_sms);
-  const int nsplit = (int)((K + kchunk - 1) / kchunk);
-  if (nsplit > 1 && (int64_t)nsplit * M * g.N > scratch_cap) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)tm, (unsigned)tn, (unsigned)nsplit);
-  // tile orientation per operand: k-major if the view is contiguous along k,
-  // else row-major if contiguous along its rows (columns), else k-major
-  // element by element
-  auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const bool a_k = g.a_ps % 8 == 0 && al16(g.A) &&
-                   ((g.K2 == 1 && g.a_k1 == 1) || (g.K2 % 8 == 0 && g.a_k2 == 1 && g.a_k1 % 8 == 0)) &&
-                   (g.a_m1 % 8 == 0 || g.M1 == 1) && (g.a_m2 % 8 == 0 || g.M2 == 1);
-  const bool a_m = !a_k && g.a_ps % 8 == 0 && al16(g.A) &&
-                   ((g.M2 == 1 && g.a_m1 == 1) || (g.M2 % 8 == 0 && g.a_m2 == 1 && g.a_m1 % 8 == 0)) &&
-                   g.a_k1 % 8 == 0 && (g.K2 == 1 || g.a_k2 % 8 == 0);
-  const bool b_k = g.b_ps % 8 == 0 && al16(g.B) &&
-                   ((g.K2 == 1 && g.b_k1 == 1) || (g.K2 % 8 == 0 && g.b_k2 == 1 && g.b_k1 % 8 == 0)) && g.b_n % 8 == 0;
-  const bool b_n = !b_k && g.b_ps % 8 == 0 && al16(g.B) && g.b_n == 1 && g.b_k1 % 8 == 0 &&
-                   (g.K2 == 1 || g.b_k2 % 8 == 0);
-  double* pp = nsplit > 1 ? scratch : nullptr;
-  const bool AK = !a_m, BK = !b_n;
-  const int av = (a_k || a_m) ? 1 : 0, bv = (b_k || b_n) ? 1 : 0;
-  cudaError_t err;
-  if (g.ns == 5) {
-    if (AK && BK) err = launch_oz2<true, true, 5>(g, grid, kchunk, pp, av, bv, s);
-    else if (AK) err = launch_oz2<true, false, 5>(g, grid, kchunk, pp, av, bv, s);
-    else if (BK) err = launch_oz2<false, true, 5>(g, grid, kchunk, pp, av, bv, s);
-    else err = launch_oz2<false, false, 5>(g, grid, kchunk, pp, av, bv, s);
-  } else if (g.ns == 0 || g.ns == 4) {
-    if (AK && BK) err = launch_oz2<true, true, 4>(g, grid, kchunk, pp, av, bv, s);
-    else if (AK) err = launch_oz2<true, false, 4>(g, grid, kchunk, pp, av, bv, s);
-    else if (BK) err = launch_oz2<false, true, 4>(g, grid, kchunk, pp, av, bv, s);
-    else err = launch_oz2<false, false, 4>(g, grid, kchunk, pp, av, bv, s);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  if (err != cudaSuccess) return err;
-  ++*launches;
-  if (nsplit > 1) {
-    const int64_t MN = M * g.N;
-    k_splitk_add_oz<<<(unsigned)std::min<int64_t>((MN + 255) / 256, 4096), 256, 0, s>>>(g, nsplit, scratch);
     ++*launches;
   }
   return cudaGetLastError();
