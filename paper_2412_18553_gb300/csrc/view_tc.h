@@ -162,7 +162,8 @@ constexpr int VT_SPLIT_CHUNKS = 8;
 // every job into C in split order.
 te_status vt_launch(Handle* h, VtBuild* b, cudaStream_t s);
 
-// N tile for an output of n columns: at most VT_NT_MAX (VT_NT_PAIR), a multiple of 32.
+// N tile for an output of n columns: at most VT_NT_MAX in steps of 16, on CTA pairs
+// VT_NT_PAIR in steps of 32.
 int vt_ntile(int64_t n, bool pair);
 
 // C[i][j] = 2^(ea + eb) sum_k A[i][k] B[j][k] (i < m, j < n; C has rows of n) over ns
