@@ -63,8 +63,8 @@
  *              are kept as FP32 pairs.  Meets 1e-7 Ha where FP32
  *              accumulation does not.
  *   In every mode D, 1/D, the products with 1/D and all sums are float64;
- *   the tensor-core modes form the orbit sum of R from deviations
- *   W_n - W_0 (no cancellation of the part of W~ that R annihilates).
+ *   the tensor-core modes form the orbit sum of R from differences of W~ in
+ *   FP32 pairs (no cancellation of the part of W~ that R annihilates).
  */
 #ifndef TENERGY_H
 #define TENERGY_H
@@ -159,7 +159,8 @@ te_status t_energy_batched(te_handle h, const te_cluster* cs, int64_t n,
  * receives E(T) (one device double).  TE_FP64 runs every contraction in
  * float64; the other modes run them on the tcgen05 tensor cores in exact
  * 7-bit BF16 slices (the TE_OZAKI scheme; gradients to ~1e-7 of each tensor's
- * largest entry), with the epilogue and all sums in float64.  Deterministic. */
+ * largest entry), with W~, its adjoint and their slices from float64 and what
+ * only enters sums in FP32 pairs.  Deterministic. */
 te_status t_energy_vjp(te_handle h, const te_cluster* c, te_precision p,
                        double gE, double* e_out, te_cluster_grad* g,
                        te_stream_t s);
@@ -290,16 +291,15 @@ typedef struct {
 } te_mp2_out;
 
 /* The MP2 step for n clusters (HOST arrays cs and outs of n entries each).
- * p = TE_FP64 (every contraction on the DFMA units) or TE_OZAKI (the three
+ * p = TE_FP64 (every contraction on the DFMA units) or TE_OZAKI (the
  * (ia|jb) contraction in exact BF16 slices on the tensor cores, the density
  * contractions in float64; outputs within about 2e-8 of their largest entry,
  * so populations far below the largest are better taken from TE_FP64).  The
- * eigenvalues come from a float64 Jacobi solver in
+ * eigenvalues come from a Householder reduction and bisection in float64 in
  * either mode (nvir <= 4094).  Input values are checked on the device
  * (finite, max eps_o < min eps_v; te_sync reports TE_EINVAL naming the
  * array and the cluster).  Workspace: about 8 (4 o^2 v^2) bytes for the
- * largest member in TE_FP64, plus its exact-slice copies and split-K partial
- * tiles in TE_OZAKI.  Deterministic. */
+ * largest member in TE_FP64, plus its exact-slice copies in TE_OZAKI.  Deterministic. */
 te_status t_mp2_bno_batched(te_handle h, const te_mp2_cluster* cs, const te_mp2_out* outs, int64_t n,
                             te_precision p, te_stream_t s);
 

@@ -1,5 +1,5 @@
 // The exact-slice adjoint of E(T) (see vjp.cu for the formulas): contractions on
-// tcgen05 (view_tc.cu), the epilogue in pairs of FP32.
+// tcgen05 (view_tc.cu), what only enters sums in pairs of FP32.
 //
 // Triples go in batches of consecutive canonical triples (up to eight, as many
 // as about a gigabyte of G, dW~ and layouts holds), and each stage is one launch
@@ -15,6 +15,13 @@
 // instructions.  To keep FP32's range out of the picture the pairs are held
 // relative to a power of two: W~ and Y to 2^E, E the largest scale of the
 // triple's segments and of Y, and the gradients' factors carry the rest.
+//
+// What bounds the kernels around the contractions, one triple at nvir = 320: the
+// epilogue (1.06 ms; 1.85 with a warp along one orbit index, whose G reads touch 32
+// lines; 4 v^3 float64 values moved would take 0.16) its float64 operations; the dW~
+// slices (0.82 ms for all six layouts, cut once; 1.01 when cut for three at a time) and
+// the Y and denominator planes (0.39; 0.75 with one load in flight per thread)
+// memory.  The view GEMM launches take 5.6 of the 9.1 ms (view_tc.cu).
 //
 // Where the operand transposes of all occupied indices would take too much
 // memory (a large cluster: full = false) a triple goes alone, the transposes are

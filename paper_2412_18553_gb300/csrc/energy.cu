@@ -182,11 +182,6 @@ cudaError_t launch_energy_f64(const Prepared* P, const Triple* d_triples, int64_
   return launch_energy<double>(P, d_triples, t0, nslots, gbuf, P->v, P->ovs, P->t1, partials, nbt, s);
 }
 
-cudaError_t launch_energy_f32(const Prepared* P, const Triple* d_triples, int64_t t0, int nslots,
-                              const float* gbuf, int ldz, double* partials, int64_t nbt, cudaStream_t s) {
-  return launch_energy<float>(P, d_triples, t0, nslots, gbuf, ldz, P->ovs32, P->t1_32, partials, nbt, s);
-}
-
 // ---------------------------------------------------------------------------
 // Deterministic compensated sums
 // ---------------------------------------------------------------------------

@@ -110,7 +110,7 @@ __device__ __forceinline__ double warp_sum(double x) {
 // v, and A <- A - v w^T - w v^T on the trailing block; the subdiagonal entry is
 // -sign(x_0) |x|.
 // About n^3 float64 operations on two lanes per cycle of one SM: 1 ms at n = 160.
-// (A parallel-order cyclic Jacobi solver, 24 ms for the sixteen matrices of the
+// (A parallel-order cyclic Jacobi solver, 24 ms for the sixteen matrices of eight
 // clusters nocc 8 .. 20, nvir = 8 nocc, was bound by the same two lanes with
 // six sweeps of 4 n^3; this and the bisection take 3.0 ms (1.8 and 1.2).)
 __global__ void __launch_bounds__(EIG_THREADS, 1) k_tridiag(const __grid_constant__ EigJobs J) {

@@ -136,12 +136,9 @@ int64_t gemm_fp64_tiles(int64_t v);
 cudaError_t launch_gemm_fp64(const Prepared* P, const Triple* d_triples, int64_t t0,
                              int nslots, double* gbuf, cudaStream_t s);
 
-// energy over G buffers: T = float (mixed) or double (fp64)
+// energy over G buffers in float64
 cudaError_t launch_energy_f64(const Prepared* P, const Triple* d_triples, int64_t t0,
                               int nslots, const double* gbuf, double* partials,
-                              int64_t nbt, cudaStream_t s);
-cudaError_t launch_energy_f32(const Prepared* P, const Triple* d_triples, int64_t t0,
-                              int nslots, const float* gbuf, int ldz, double* partials,
                               int64_t nbt, cudaStream_t s);
 // writes e_out[slot] = (m/3) * sum of the slot's partials, for triples t0 .. t0+nslots-1
 cudaError_t launch_reduce_triples(const double* partials, int64_t nbt, const Triple* d_triples,

@@ -21,7 +21,8 @@
 // Eight triples of a gradient at nvir = 120, one set of 128 columns -> two of 64:
 // G 671 -> 520 us, ovvv and t2 479 -> 384; one triple at nvir = 320: 1981 -> 1561,
 // 2057 -> 1503 (the projected energy's pairs, which convert nothing: 1096 -> 1105).
-// Lone CTAs have K of nvir^2 and are bound by their MMAs: one set of 128 columns.
+// Lone CTAs have K of nvir^2: few drains, so one set of 128 columns, whose operands
+// from L2 bound them (tensor pipe 49% active at nvir = 320).
 //
 // Pairs of CTAs share a B tile (cta_group::2): each loads its 128 A rows and half
 // of B, rank 0 issues the MMAs of both SMs, and all bytes of the pair count on

@@ -168,7 +168,7 @@ int vt_ntile(int64_t n, bool pair);
 
 // C[i][j] = 2^(ea + eb) sum_k A[i][k] B[j][k] (i < m, j < n; C has rows of n) over ns
 // slice planes with rows of Kp elements (Kp a multiple of 8, planes 16-byte aligned),
-// on lone CTAs: K of hundreds or more, bound by the MMAs.  The ovvv of nocc=16
+// on lone CTAs: K of hundreds or more, so few drains.  The ovvv of nocc=16
 // nvir=160 from 704 auxiliary functions (five slices): 1.17 ms, 3.40 ms with mma.sync on
 // row-contiguous factors; batches of MP2 steps gain by as much (eight clusters of
 // nocc 8 .. 20, nvir = 8 nocc, exact slices: 18.0 ms a call).
