@@ -19,9 +19,9 @@
 // What bounds the kernels around the contractions, one triple at nvir = 320: the
 // epilogue (1.06 ms; 1.85 with a warp along one orbit index, whose G reads touch 32
 // lines; 4 v^3 float64 values moved would take 0.16) its float64 operations; the dW~
-// slices (0.82 ms for all six layouts, cut once; 1.01 when cut for three at a time) and
+// slices (0.55 ms for all six layouts, cut once; 1.01 when cut for three at a time) and
 // the Y and denominator planes (0.39; 0.75 with one load in flight per thread)
-// memory.  The view GEMM launches take 5.6 of the 9.1 ms (view_tc.cu).
+// memory.  The view GEMM launches take 5.6 of the 8.8 ms (view_tc.cu).
 //
 // Where the operand transposes of all occupied indices would take too much
 // memory (a large cluster: full = false) a triple goes alone, the transposes are
@@ -394,11 +394,13 @@ __global__ void __launch_bounds__(256) k_y_small(const __grid_constant__ AdjEpi 
 // Slices of index permutations of dW~ into layouts L[x][y][z] (z padded to vp),
 // permutation q holding the slices of dW~[pi_q(x, y, z)]:
 //   0, 1, 2: pi = (x,y,z), (z,x,y), (y,z,x);  3, 4, 5: (z,y,x), (x,z,y), (y,x,z).
-// With 2^e > max |dW~| (e written to e_out) the digits are slice_digits' (integer
+// With 2^e > max |dW~| (e written to e_out) the digits are slice_digits_int's (integer
 // operations on the bits of dW~).  A block takes a 16 x 16 x 16 cube of dW~: each
 // value is read and cut once, and every layout is written from shared memory in
-// rows of 16 elements (32 bytes).  HBM bounds it: 8 bytes read and 2 NS written per
-// value and layout.
+// rows of 16 elements (32 bytes); 64 consecutive blocks take a cube of 64^3, so that
+// the pieces of a 128-byte line meet in L2 in every layout.  HBM bounds it: 8 bytes
+// read and 2 NS written per value and layout; one triple at nvir = 320: 0.55 ms (0.82 with
+// the blocks in row order, whose pieces of the transposed layouts lie 400 blocks apart).
 template <int NS>
 __global__ void __launch_bounds__(256) k_dw_slices(const double* __restrict__ dWs, int64_t w_stride, int v, int vp,
                                                    int perm0, const unsigned long long* __restrict__ dwmax,
@@ -413,9 +415,11 @@ __global__ void __launch_bounds__(256) k_dw_slices(const double* __restrict__ dW
   const double mx = __longlong_as_double((long long)dwmax[slot]);
   int ex = 0;
   if (mx > 0.0) frexp(mx, &ex);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) e_out[slot] = ex;
-  const int nt = (v + 15) / 16;
-  const int a0 = blockIdx.y * 16, b0 = (int)(blockIdx.x / nt) * 16, c0 = (int)(blockIdx.x % nt) * 16;
+  if (blockIdx.x == 0 && threadIdx.x == 0) e_out[slot] = ex;
+  const int n4 = (v + 63) / 64, sub = blockIdx.x & 63, sup = blockIdx.x >> 6;
+  const int a0 = sup / (n4 * n4) * 64 + (sub >> 4) * 16, b0 = sup / n4 % n4 * 64 + (sub >> 2 & 3) * 16,
+            c0 = sup % n4 * 64 + (sub & 3) * 16;
+  if (a0 >= v || b0 >= v || c0 >= v) return;
   const int64_t V = v, plane = V * V * vp;
   const int k = threadIdx.x & 15, j0 = threadIdx.x >> 4;
 #pragma unroll 4
@@ -841,8 +845,8 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
     k_y_small<<<1 + (v + 255) / 256, 256, 0, s>>>(A, Bt, Yp, AdjOut{g->eps_o, g->eps_v, g->t1, dOVS, shares, t0}, agrid);
     ++h->n_launches;
     auto slices = [&](int perm0, int nperm) {
-      const unsigned n16 = (unsigned)((v + 15) / 16);
-      const dim3 grid(n16 * n16, n16, (unsigned)Bt.n);
+      const unsigned n4 = (unsigned)((v + 63) / 64);
+      const dim3 grid(64 * n4 * n4 * n4, 1, (unsigned)Bt.n);
       bf* out = reinterpret_cast<bf*>(region);
       if (ns == 5)
         k_dw_slices<5><<<grid, 256, 0, s>>>(dW, A.w_stride, v, (int)vp, perm0, dwmax, dwexp, out, lay_stride, ls, nperm);
