@@ -32,6 +32,7 @@
 #include <cmath>
 #include <initializer_list>
 #include <map>
+#include <new>
 #include <vector>
 
 #include "adjoint_tc.cuh"
@@ -728,7 +729,8 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
   Yp.stride = Z.ystride;
 
   std::vector<Triple> trip = unique_triples(o);
-  VtBuild* bp = new VtBuild;
+  VtBuild* bp = new (std::nothrow) VtBuild;
+  if (!bp) return fail(TE_ENOMEM, "view GEMM tables");
   VtBuild& b = *bp;
   struct Del {
     VtBuild* b;

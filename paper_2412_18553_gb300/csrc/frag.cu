@@ -3,6 +3,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "adjoint_tc.cuh"
@@ -399,7 +400,8 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
   A.epart = W.epart;
   A.shares = W.shares;
   std::vector<Triple> trip = unique_triples(o);
-  VtBuild* bp = new VtBuild;
+  VtBuild* bp = new (std::nothrow) VtBuild;
+  if (!bp) return fail(TE_ENOMEM, "view GEMM tables");
   VtBuild& b = *bp;
   struct Del {
     VtBuild* b;

@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <cstring>
 #include <memory>
+#include <new>
 
 #include "fp_util.cuh"
 #include "ptx_sm100.cuh"
@@ -865,7 +866,8 @@ te_status vt_product(Handle* h, const void* a, int64_t a_plane, int64_t m, const
   te_status st = vt_bank_add(&bank, va, 128, 1, &ma);
   if (st == TE_OK) st = vt_bank_add(&bank, vb, NT, 1, &mb);
   if (st != TE_OK) return st;
-  std::unique_ptr<VtBuild> B(new VtBuild);
+  std::unique_ptr<VtBuild> B(new (std::nothrow) VtBuild);
+  if (!B) return fail(TE_ENOMEM, "view GEMM tables");
   vt_begin(B.get(), ns, false);
   const int none[3] = {0, 0, 0};
   vt_job(B.get(), 1, (int)m, (int)n, 1, 128, NT, C, 0, n, 1, VT_STORE);
