@@ -283,8 +283,10 @@ __global__ void __launch_bounds__(Layout<FMT>::threads, 1)
       issued = true;
       ph ^= 1u;
     }
-    // copies in flight land before the block ends: on an abort the consumers no longer wait for them
-    if (lane == 0 && !ok && issued) ptx::mbar_wait(&full[b], ph ^ 1u, P.wait_ns);
+    // The copies of this buffer's last item land before the block ends.  The
+    // consumers wait for them only as long as none of their waits has expired,
+    // which this warp's own loop need not have seen.
+    if (lane == 0 && issued) ptx::mbar_wait(&full[b], ph ^ 1u, P.wait_ns);
   } else {
     // ---------------- compute warps ----------------
     // A thread takes the orbit (a,b,c) = its local point of the block triple.
