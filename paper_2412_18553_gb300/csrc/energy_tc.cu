@@ -71,9 +71,12 @@ __device__ __forceinline__ void decode_bt(int64_t bt, int* blk) {
 }
 
 // ---- pairs of FP32 (value h + l): error-free transformations ----
-// Knuth two-sum, FMA two-product; the rn intrinsics forbid contraction.  The
-// pairs are not renormalised: l stays a small correction of what was summed
-// into h, and a difference whose h cancels keeps its l.
+// Knuth two-sum, FMA two-product; the rn intrinsics forbid contraction.  W~
+// and its differences are renormalised, |l| <= ulp(h) / 2, after every
+// operation: where R annihilates most of W~ the high parts cancel, and a low
+// part left as large as what remains of them would cut the products that
+// follow to 24 + 8 bits (W~ 2^15 times its differences: 4e-13 of a share
+// against 1e-15).  Sums of products and of FP32 terms stay as they come.
 struct df {
   float h, l;
 };
@@ -84,9 +87,14 @@ __device__ __forceinline__ df two_sum(float a, float b) {
   return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
 }
 
+__device__ __forceinline__ df df_norm(float h, float l) {
+  const float s = __fadd_rn(h, l);
+  return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+
 __device__ __forceinline__ df df_add(df a, df b) {
   const df s = two_sum(a.h, b.h);
-  return {s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+  return df_norm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
 }
 
 __device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df{-b.h, -b.l}); }
@@ -94,11 +102,6 @@ __device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df{-b.h, -b.
 __device__ __forceinline__ df df_addf(df a, float b) {
   const df s = two_sum(a.h, b);
   return {s.h, __fadd_rn(s.l, a.l)};
-}
-
-__device__ __forceinline__ df df_norm(float h, float l) {
-  const float s = __fadd_rn(h, l);
-  return {s, __fsub_rn(l, __fsub_rn(s, h))};
 }
 
 // acc += a b
@@ -113,8 +116,11 @@ __device__ __forceinline__ void df_fma(df& acc, df a, df b) {
   acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
 }
 
-// 2 a + b and a + 2 b
-__device__ __forceinline__ df df_2ab(df a, df b) { return df_add(df{2.f * a.h, 2.f * a.l}, b); }
+// 2 a + b
+__device__ __forceinline__ df df_2ab(df a, df b) {
+  const df s = two_sum(2.f * a.h, b.h);
+  return {s.h, __fadd_rn(s.l, __fadd_rn(2.f * a.l, b.l))};
+}
 
 struct EnergyMaps {
   CUtensorMap ovs[TC_MAX_CL];  // per cluster: ovs32 [o][v][o][vq], 4D (b, j, a, i)
@@ -384,7 +390,7 @@ __global__ void __launch_bounds__(Layout<FMT>::threads, 1)
             w[n] = df{(g0.h + g1.h) + g2.h, 0.f};
           } else {
             const df s = two_sum(g0.h, g1.h), s3 = two_sum(s.h, g2.h);
-            w[n] = df{s3.h, __fadd_rn(__fadd_rn(s.l, s3.l), __fadd_rn(__fadd_rn(g0.l, g1.l), g2.l))};
+            w[n] = df_norm(s3.h, __fadd_rn(__fadd_rn(s.l, s3.l), __fadd_rn(__fadd_rn(g0.l, g1.l), g2.l)));
           }
           // Y at (x, y, z) = positions (s0, s1, s2):
           //   ovs(i,x,j,y) t1(k,z) + ovs(j,y,k,z) t1(i,x) + ovs(i,x,k,z) t1(j,y)

@@ -1,0 +1,72 @@
+"""What the exact-slice modes hold beside the operands' slices.
+
+Inputs that are integers of at most 14 bits fill two 7-bit slices: every slice
+product and every sum of them below 2^24 units of its level is exact, so the
+contraction is exact and what separates a result from the exact one is the word
+length of what is kept afterwards."""
+import numpy as np
+import pytest
+import torch
+
+import tegen
+from gpu_common import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+P6 = (((0, 1, 2), (0, 1, 2)), ((1, 2, 0), (2, 0, 1)), ((2, 0, 1), (1, 2, 0)),
+      ((0, 2, 1), (0, 2, 1)), ((2, 1, 0), (2, 1, 0)), ((1, 0, 2), (1, 0, 2)))
+
+
+@pytest.fixture(scope="module")
+def te():
+    return need_gpu()
+
+
+def dev(arrs):
+    return {n: torch.as_tensor(np.ascontiguousarray(x)).cuda() for n, x in arrs.items()}
+
+
+def integers(o, v, seed):
+    """Integrals and amplitudes +-(8000 + (-8 .. 8)): W~ is a 36-bit integer, nearly
+    the same in all permutations of an orbit; R leaves 2^-15 of it.  No Y."""
+    rng = np.random.default_rng(seed)
+    n = lambda *shape: 8000.0 + rng.integers(-8, 9, shape)  # noqa: E731
+    t2 = n(o, o, v, v)
+    lower = np.arange(o)[:, None] > np.arange(o)
+    t2[lower] = np.swapaxes(np.swapaxes(t2, 0, 1), 2, 3)[lower]
+    base = tegen.make_cluster(o, v, 4 * (o + v), seed).arrays()
+    return dict(eps_o=base["eps_o"], eps_v=base["eps_v"], ovvv=n(o, v, v, v), ooov=-n(o, o, o, v),
+                ovov=np.zeros((o, v, o, v)), t1=np.zeros((o, v)), t2=t2)
+
+
+def exact_shares(a):
+    """Integer W~ and R, extended precision for the rest; sum R = 0 over an orbit,
+    so W~ less a constant serves."""
+    I = {k: a[k].astype(np.int64) for k in ("ovvv", "ooov", "t2")}  # noqa: E741
+    eo, ev = a["eps_o"].astype(np.longdouble), a["eps_v"].astype(np.longdouble)
+    out = []
+    for t in [(i, j, k) for i in range(len(eo)) for j in range(i + 1) for k in range(j + 1) if not i == j == k]:
+        W = 0
+        for occ, vir in P6:
+            p, q, r = (t[n] for n in occ)
+            W = W + (np.einsum("abd,cd->abc", I["ovvv"][p], I["t2"][r, q])
+                     - np.einsum("la,lbc->abc", I["ooov"][q, :, p], I["t2"][:, r])).transpose(vir)
+        R = (4 * W + W.transpose(1, 2, 0) + W.transpose(2, 0, 1)
+             - 2 * (W.transpose(2, 1, 0) + W.transpose(0, 2, 1) + W.transpose(1, 0, 2)))
+        D = eo[list(t)].sum() - ev[:, None, None] - ev[None, :, None] - ev[None, None, :]
+        m = (W - W[0, 0, 0]).astype(np.longdouble)
+        out.append((m * R.astype(np.longdouble) / D).sum() * (1 if len(set(t)) == 2 else 2))
+    return np.array(out)
+
+
+# The differences of W~ and their products are integers that pairs hold exactly; 1/D
+# comes from one Newton step on an FP32 seed, (2^-24)^2 = 4e-15, the float64 sums add 1e-15.
+BAR = 2e-14
+
+
+@pytest.mark.parametrize("v", [9, 33, 48, 64])
+def test_energy_epilogue_where_most_of_w_cancels(te, v):
+    a = integers(3, v, v)
+    e = te.t_energy_triples(dev(a), precision="ozaki").cpu().numpy()
+    ref = exact_shares(a)
+    assert float(np.abs((e - ref) / ref).max()) <= BAR
