@@ -57,8 +57,9 @@ cudaError_t launch_reduce_pieces(const double* partials, int grid, const Triple*
 // Element formats of G.  G_F32: one FP32 plane of 512 per cube.  G_PAIR: an
 // FP32 hi plane, then an FP32 lo plane.  G_MIXED: an FP32 hi plane, then 512
 // BF16 lo values; the contraction holds lo in BF16 when it has one accumulator
-// set (|lo| <= ulp(hi) / 2, so the pair keeps 2^-33 of the value), and storing
-// it so loses nothing and cuts G's traffic by a quarter.
+// set and an N tile of more than 80 columns (|lo| <= ulp(hi) / 2, so the pair
+// keeps 2^-33 of the value), and storing it so loses nothing and cuts G's
+// traffic by a quarter.
 enum GFormat { G_F32 = 1, G_PAIR = 2, G_MIXED = 3 };
 __host__ __device__ constexpr int g_cube_floats(int fmt) { return fmt == G_F32 ? 512 : (fmt == G_PAIR ? 1024 : 768); }
 

@@ -114,6 +114,7 @@ struct TcParams {
   uint32_t a_part_bytes;   // 128 rows x cbw
   uint32_t tmem_cols;
   int nbuf;                // TMEM accumulator sets (1 or 2)
+  int fmt;                 // G format
   int nt_max;              // largest N tile: stride of the accumulator sets
   int64_t total_tiles;     // pair tiles
   const Triple* triples;
@@ -228,9 +229,12 @@ constexpr int GEMM_THREADS = (2 + GEMM_EPI_WARPS) * 32;
 // accumulator set (exact-slice N tiles of at most 160 columns)
 constexpr int EPI_CHUNKS = 5;
 constexpr int EPI_NT_MAX = 16 * GEMM_EPI_GROUPS * EPI_CHUNKS;
+constexpr int EPI_NT_LO32 = 96;  // the widest such tile whose low words stay FP32
 constexpr int GEMM_PAIR = 2;  // CTAs per cluster
 
-template <int MODE>
+// LO32: G's low words are FP32 (G_PAIR), else BF16 where they are held in
+// registers (G_MIXED); the exact-slice modes only
+template <int MODE, bool LO32>
 __global__ void __cluster_dims__(GEMM_PAIR, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
     k_gemm_tc(const __grid_constant__ TcMapSet maps, const __grid_constant__ TcParams P) {
   using MT = ModeTraits<MODE>;
@@ -480,15 +484,18 @@ __global__ void __cluster_dims__(GEMM_PAIR, 1, 1) __launch_bounds__(GEMM_THREADS
         if (NBUF == 1) {
           // One accumulator set: copy it to registers as (hi, lo) pairs and
           // release it before the stores, so that the next tile's MMAs run
-          // while this tile's G is written.  A warp holds at most
-          // EPI_CHUNKS 16-column chunks (N tiles <= 160, checked on the
-          // host).  lo is held rounded to BF16 (two per register): |lo| <=
-          // ulp(hi) / 2, so the pair keeps 2^-33 of the value, far below the
-          // 2^-28 of the exact-slice operands.
-          float hv[EPI_CHUNKS][16];
-          uint32_t lp[EPI_CHUNKS][8];
+          // while this tile's G is written.  With N tiles of at most EPI_NT_LO32
+          // columns lo stays FP32 (at most three 16-column chunks per warp);
+          // a wider tile (at most EPI_CHUNKS chunks, checked on the host)
+          // holds lo rounded to BF16, two per register: |lo| <= ulp(hi) / 2, so
+          // the pair keeps 2^-33 of the value, far below the 2^-28 of the
+          // exact-slice operands.
+          constexpr int CH = LO32 ? EPI_NT_LO32 / (16 * GEMM_EPI_GROUPS) : EPI_CHUNKS, LW = LO32 ? 16 : 8;
+          constexpr int CUBE1 = g_cube_floats(LO32 ? G_PAIR : G_MIXED);
+          float hv[CH][16];
+          uint32_t lp[CH][LW];
 #pragma unroll
-          for (int k = 0; k < EPI_CHUNKS; ++k) {
+          for (int k = 0; k < CH; ++k) {
             const int c0 = 16 * chunk0 + 32 * k;
             if (c0 < C.NT) {
 #pragma unroll
@@ -508,8 +515,13 @@ __global__ void __cluster_dims__(GEMM_PAIR, 1, 1) __launch_bounds__(GEMM_THREADS
                     hv[k][8 * half + j + q] = hi * gscale;
                     l2[q] = __fsub_rn(lo, __fsub_rn(hi, s)) * gscale;
                   }
-                  const __nv_bfloat162 b = __floats2bfloat162_rn(l2[0], l2[1]);
-                  lp[k][4 * half + (j >> 1)] = *reinterpret_cast<const uint32_t*>(&b);
+                  if constexpr (LO32) {
+                    lp[k][8 * half + j] = __float_as_uint(l2[0]);
+                    lp[k][8 * half + j + 1] = __float_as_uint(l2[1]);
+                  } else {
+                    const __nv_bfloat162 b = __floats2bfloat162_rn(l2[0], l2[1]);
+                    lp[k][4 * half + (j >> 1)] = *reinterpret_cast<const uint32_t*>(&b);
+                  }
                 }
               }
             }
@@ -518,29 +530,36 @@ __global__ void __cluster_dims__(GEMM_PAIR, 1, 1) __launch_bounds__(GEMM_THREADS
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive_cluster(ptx::mapa(&tempty[acc], 0));
           acc_phase ^= 1u;
-          if (valid) {
+          if (!valid) continue;
 #pragma unroll
-            for (int k = 0; k < EPI_CHUNKS; ++k) {
-              const int c0 = 16 * chunk0 + 32 * k;
-              if (c0 < C.NT) {
-                const int z = c.z0 + c0;  // multiple of 16: two whole Z blocks
+          for (int k = 0; k < CH; ++k) {
+            const int c0 = 16 * chunk0 + 32 * k;
+            if (c0 < C.NT) {
+              const int z = c.z0 + c0;  // multiple of 16: two whole Z blocks
 #pragma unroll
-                for (int h2 = 0; h2 < 2; ++h2) {
-                  const int Z = (z >> 3) + h2;
-                  if (Z < nb) {
-                    int64_t bt;
-                    unsigned mask;
-                    orbit_slots(x >> 3, y >> 3, Z, &bt, &mask);
-                    xor_permute8(hv[k] + 8 * h2, zx);
-                    const uint4 l8 = xor_permute8_packed(lp[k] + 4 * h2, zx);
-                    constexpr int CUBE_M = g_cube_floats(G_MIXED);
-                    float* item = gslot + (bt * 18 + c.g * 6) * CUBE_M;
-                    for (int pid = 0; pid < 6; ++pid) {
-                      if (!((mask >> pid) & 1u)) continue;
-                      float* cube = item + pid * CUBE_M;
-                      store8(cube + roff, hv[k] + 8 * h2);
-                      *reinterpret_cast<uint4*>(reinterpret_cast<unsigned short*>(cube + 512) + roff) = l8;
-                    }
+              for (int h2 = 0; h2 < 2; ++h2) {
+                const int Z = (z >> 3) + h2;
+                if (Z < nb) {
+                  int64_t bt;
+                  unsigned mask;
+                  orbit_slots(x >> 3, y >> 3, Z, &bt, &mask);
+                  xor_permute8(hv[k] + 8 * h2, zx);
+                  float lv[LO32 ? 8 : 1];
+                  uint4 l8 = make_uint4(0u, 0u, 0u, 0u);
+                  if constexpr (LO32) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) lv[j] = __uint_as_float(lp[k][8 * h2 + j]);
+                    xor_permute8(lv, zx);
+                  } else {
+                    l8 = xor_permute8_packed(lp[k] + 4 * h2, zx);
+                  }
+                  float* item = gslot + (bt * 18 + c.g * 6) * CUBE1;
+                  for (int pid = 0; pid < 6; ++pid) {
+                    if (!((mask >> pid) & 1u)) continue;
+                    float* cube = item + pid * CUBE1;
+                    store8(cube + roff, hv[k] + 8 * h2);
+                    if constexpr (LO32) store8(cube + 512 + roff, lv);
+                    else *reinterpret_cast<uint4*>(reinterpret_cast<unsigned short*>(cube + 512) + roff) = l8;
                   }
                 }
               }
@@ -685,7 +704,7 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   const int nacc = oz ? 3 : 1;
   // TF32/BF16X3 (one accumulator) double-buffer at any N tile; the exact-slice
   // modes (three accumulators) take N tiles up to 160 single-buffered, and
-  // double-buffer when 2 x 3 x NT <= 512 columns (NT <= 80)
+  // double-buffer when 2 x 3 x NT <= 512 columns (NT <= 64, in steps of 32)
   const int nbuf_max = oz ? 1 : 2;
   pl.vp = round_up(v, 16);
   pl.op = round_up(o, 16);
@@ -719,7 +738,10 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   if (force_nnt > 0 && round_up((v + force_nnt - 1) / force_nnt, 32) <= (oz ? 160 : 256)) pl.n_nt = force_nnt;
   pl.NT = round_up((v + pl.n_nt - 1) / pl.n_nt, 32);  // cta_group::2: N in steps of 32
   pl.nbuf = (2 * nacc * pl.NT <= 512) ? 2 : 1;
-  pl.fmt = !oz ? G_F32 : (pl.nbuf == 1 ? G_MIXED : G_PAIR);  // as the kernel's epilogues store
+  // G's low words stay FP32 in tiles of at most 80 columns (two accumulator sets
+  // up to 64, one set and three chunks per epilogue warp above), also where the
+  // step of 32 pads the tile to 96; wider tiles round them to BF16.
+  pl.fmt = !oz ? G_F32 : ((v + pl.n_nt - 1) / pl.n_nt <= 80 ? G_PAIR : G_MIXED);
   pl.cbw = oz ? 64 : 128;
   pl.kw_elems = pl.cbw / pl.es;
   pl.kw_chunks = (pl.vp + pl.kw_elems - 1) / pl.kw_elems;
@@ -1039,12 +1061,12 @@ static te_status launch_prep_tc(Handle* h, int mode, const te_cluster* c, const 
   return e == cudaSuccess ? TE_OK : bad(e);
 }
 
-template <int MODE>
+template <int MODE, bool LO32 = false>
 static cudaError_t launch_gemm_tc(const TcMapSet& M, const TcParams& P, size_t smem, int grid_cap, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<MODE, LO32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t grid = GEMM_PAIR * std::min<int64_t>(P.total_tiles, std::max(1, grid_cap / GEMM_PAIR));
-  k_gemm_tc<MODE><<<(unsigned)grid, GEMM_THREADS, smem, s>>>(M, P);
+  k_gemm_tc<MODE, LO32><<<(unsigned)grid, GEMM_THREADS, smem, s>>>(M, P);
   return cudaGetLastError();
 }
 
@@ -1053,8 +1075,10 @@ static cudaError_t launch_gemm_any(int mode, const TcMapSet& M, const TcParams& 
   if (mode == TC_BF16X3) return launch_gemm_tc<TC_BF16X3>(M, P, smem, grid_cap, s);
   if (mode == TC_TF32X3) return launch_gemm_tc<TC_TF32X3>(M, P, smem, grid_cap, s);
   if (mode == TC_TF32) return launch_gemm_tc<TC_TF32>(M, P, smem, grid_cap, s);
-  if (mode == TC_OZAKI) return launch_gemm_tc<TC_OZAKI>(M, P, smem, grid_cap, s);
-  return launch_gemm_tc<TC_OZAKI6>(M, P, smem, grid_cap, s);
+  const bool lo32 = P.fmt == G_PAIR;
+  if (mode == TC_OZAKI)
+    return lo32 ? launch_gemm_tc<TC_OZAKI, true>(M, P, smem, grid_cap, s) : launch_gemm_tc<TC_OZAKI>(M, P, smem, grid_cap, s);
+  return lo32 ? launch_gemm_tc<TC_OZAKI6, true>(M, P, smem, grid_cap, s) : launch_gemm_tc<TC_OZAKI6>(M, P, smem, grid_cap, s);
 }
 
 // One cluster of a run: its plan, buffers, tensor maps and triple range.
@@ -1116,9 +1140,11 @@ static te_status gemm_params(const Handle* h, const std::vector<TcJob>& jobs, co
   P->stages = (int)std::min<size_t>(8, avail / stage_max);
   if (P->stages < 2) return fail(TE_EUNSUPPORTED, "not enough shared memory for two pipeline stages");
   P->nbuf = p0.nbuf;
+  P->fmt = p0.fmt;
   P->nt_max = nt_max;
-  if (is_ozaki(mode) && P->nbuf == 1 && nt_max > EPI_NT_MAX)
-    return fail(TE_EUNSUPPORTED, "N tile %d above the epilogue's %d columns", nt_max, EPI_NT_MAX);
+  const int nt_held = P->fmt == G_PAIR ? EPI_NT_LO32 : EPI_NT_MAX;
+  if (is_ozaki(mode) && P->nbuf == 1 && nt_max > nt_held)
+    return fail(TE_EUNSUPPORTED, "N tile %d above the epilogue's %d columns", nt_max, nt_held);
   uint32_t cols = 32;
   while (cols < (uint32_t)(nacc * P->nbuf * nt_max)) cols <<= 1;
   P->tmem_cols = cols;
@@ -1132,7 +1158,7 @@ static te_status gemm_params(const Handle* h, const std::vector<TcJob>& jobs, co
 }
 
 // Runs the jobs' triples in rounds: each round fills the G pool with pieces
-// (up to TC_MAX_CL clusters, TC_MAX_PIECES pieces, one TMEM buffering), then
+// (up to TC_MAX_CL clusters, TC_MAX_PIECES pieces, one TMEM buffering and G format), then
 // launches the contraction and the energy epilogue once.  The shares are
 // reduced when the partials of par_slots triples or TC_MAX_PIECES runs of
 // triples have come together, and at the end; then each job's total.  Pieces
@@ -1165,7 +1191,7 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     }
     if (j >= jobs.size()) break;
     int jl[TC_MAX_CL];
-    int ncl = 0, nbuf = -1, nslots = 0;
+    int ncl = 0, nbuf = -1, fmt = 0, nslots = 0;
     int64_t used = 0, tiles = 0, items = 0;
     double flops = 0.0;
     pcs.clear();
@@ -1180,14 +1206,15 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
       for (int q = 0; q < ncl; ++q)
         if (jl[q] == (int)j) cl = q;
       if (cl < 0) {
-        if (ncl == TC_MAX_CL || (nbuf >= 0 && J.pl.nbuf != nbuf)) break;
+        if (ncl == TC_MAX_CL || (nbuf >= 0 && (J.pl.nbuf != nbuf || J.pl.fmt != fmt))) break;
         cl = ncl;
       }
       const int64_t fit = std::min((pq.pool_floats - used) / J.slot_floats, pq.max_slots - nslots);
       if (fit <= 0) break;
       if (cl == ncl) {
         jl[ncl++] = (int)j;
-        nbuf = J.pl.nbuf;  // one TMEM buffering per launch
+        nbuf = J.pl.nbuf;  // one TMEM buffering and one G format per launch
+        fmt = J.pl.fmt;
       }
       const int ns = (int)std::min<int64_t>(fit, J.t_end - t);
       TcPiece pc{};
@@ -1231,7 +1258,7 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     std::memset(EL, 0, sizeof(*EL));
     EL->ncl = ncl;
     EL->npieces = (int)pcs.size();
-    EL->fmt = jobs[jl[0]].pl.fmt;  // one TMEM buffering per launch, so one format
+    EL->fmt = jobs[jl[0]].pl.fmt;
     EL->num_sms = h->num_sms;
     EL->nslots = nslots;
     EL->items = items;

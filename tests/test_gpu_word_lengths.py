@@ -70,3 +70,21 @@ def test_energy_epilogue_where_most_of_w_cancels(te, v):
     e = te.t_energy_triples(dev(a), precision="ozaki").cpu().numpy()
     ref = exact_shares(a)
     assert float(np.abs((e - ref) / ref).max()) <= BAR
+
+
+@pytest.mark.parametrize("v", [65, 72, 79, 80])
+def test_g_keeps_an_fp32_low_word_up_to_80_columns(te, v):
+    """The low word of G has 10 bits here: BF16 would cut it to units of 2 to 4."""
+    a = integers(3, v, v)
+    e = te.t_energy_triples(dev(a), precision="ozaki").cpu().numpy()
+    ref = exact_shares(a)
+    assert float(np.abs((e - ref) / ref).max()) <= BAR
+
+
+def test_g_formats_in_one_batch(te):
+    """Members whose tiles, accumulator sets and low words differ: the shares of a
+    member do not depend on the others, nor on the order of its triples."""
+    a = [dev(integers(2, v, v)) for v in (96, 64, 81, 72, 65, 80, 33)]
+    e = te.t_energy_batched(a, "ozaki")
+    one = torch.stack([te.t_energy(x, "ozaki") for x in a])
+    assert float(((e - one) / one).abs().max()) <= BAR
