@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "adjoint_tc.cuh"
+#include "fp_util.cuh"
 #include "strided.h"
 #include "tc_path.h"
 #include "view_tc.h"
@@ -221,15 +222,14 @@ te_status run_frag_fp64(Handle* h, const te_cluster* c, const double* cf, const 
 }
 
 // ---------------------------------------------------------------------------
-// exact-slice form: batches of triples, the epilogue in FP32 pairs
+// exact-slice form: batches of triples
 // ---------------------------------------------------------------------------
 
 constexpr int FRAG_MAX_BATCH = 8;
 constexpr int64_t FRAG_BATCH_BYTES = int64_t(1) << 30;  // G and SG of a batch
 
 struct FragOz {
-  double *ovvvC, *t2C, *t2C2, *ooovC;
-  PairBuffers pb;
+  double *ovvvC, *t2C, *t2C2, *ooovC, *ovs;
   float2 *G, *SG;  // [slot][3][v^3]
   int64_t stride;  // float2 between the slots of each
   double *epart, *shares;
@@ -241,21 +241,18 @@ int frag_batch(int64_t o, int64_t v) {
                                                       std::max<int64_t>(1, num_unique_triples(o))}));
 }
 
-size_t frag_oz_layout(int64_t o, int64_t v, int B, char* base, FragOz* W) {
+size_t frag_oz_layout(const Handle* h, int64_t o, int64_t v, int B, char* base, FragOz* W) {
   const int64_t v3 = v * v * v, nt = num_unique_triples(o);
   Carve c{base};
   W->ovvvC = c.d(o * v3);
   W->t2C = c.d(o * o * v * v);
   W->t2C2 = c.d(o * o * v * v);
   W->ooovC = c.d(o * o * o * v);
-  W->pb.ovs = reinterpret_cast<pr*>(c.d(o * v * o * v));
-  W->pb.t1 = reinterpret_cast<pr*>(c.d(o * v));
-  W->pb.eps = reinterpret_cast<pr*>(c.d(o + v));
-  W->pb.hi = reinterpret_cast<unsigned int*>(c.take(64));
+  W->ovs = c.d(o * v * o * v);
   W->stride = (3 * v3 + 3) / 4 * 4;
   W->G = reinterpret_cast<float2*>(c.d(B * W->stride));
   W->SG = reinterpret_cast<float2*>(c.d(B * W->stride));
-  W->epart = c.d((int64_t)B * 8192);
+  W->epart = c.d((int64_t)B * adjoint_grid(h->num_sms));
   W->shares = c.d(std::max<int64_t>(1, nt));
   for (int k = 0; k < 3; ++k) W->slices[k] = c.take(tc_slices_bytes((int)o, (int)v) + 1024);
   return c.off + 1024;
@@ -264,15 +261,15 @@ size_t frag_oz_layout(int64_t o, int64_t v, int B, char* base, FragOz* W) {
 int frag_oz_batch(const Handle* h, int64_t o, int64_t v) {
   FragOz W;
   const int B = frag_batch(o, v);
-  return h->ws_limit && frag_oz_layout(o, v, B, nullptr, &W) > h->ws_limit ? 1 : B;
+  return h->ws_limit && frag_oz_layout(h, o, v, B, nullptr, &W) > h->ws_limit ? 1 : B;
 }
 
 struct ProjArgs {
-  PairInputs in;
-  SliceExps x0, xa, xb;  // scales of the input slices, of (ovvvC, t2C, ., ooovC) and of t2C2's t2L
-  const float2 *G, *SG;
+  AdjArgs a;              // inputs
+  SliceExps x0, xa, xb;   // scales of the input slices, of (ovvvC, t2C, ., ooovC) and of t2C2's t2L
+  const float2 *G, *SG;   // pairs relative to the largest scale of their products
   int64_t stride;
-  double* epart;   // [slot][gridDim.x]
+  double* epart;          // [slot][gridDim.x]
   double* shares;
   int64_t t0;
   int n;
@@ -281,58 +278,95 @@ struct ProjArgs {
 
 // the projected block's scale: the largest of its eight products'
 __device__ __forceinline__ int sg_exp(const ProjArgs& A, int p, int q, int r) {
-  const int o = A.in.o, rq = r * o + q, rp = r * o + p, nqr = q * o + r, npr = p * o + r;
+  const int o = A.a.o, rq = r * o + q, rp = r * o + p, nqr = q * o + r, npr = p * o + r;
   int e = max(A.xa.e_ovvv[p] + A.x0.e_t2[rq], A.x0.e_ovvv[p] + A.xa.e_t2[rq]);
   e = max(e, max(A.xa.e_ovvv[q] + A.x0.e_t2[rp], A.x0.e_ovvv[q] + A.xa.e_t2[rp]));
   e = max(e, max(A.xb.e_t2L[p] + A.x0.e_nooT[nqr], A.x0.e_t2L[p] + A.xa.e_nooT[nqr]));
   return max(e, max(A.xb.e_t2L[q] + A.x0.e_nooT[npr], A.x0.e_t2L[q] + A.xa.e_nooT[npr]));
 }
-// scale of S W~, and of its three blocks relative to it
-__device__ __forceinline__ TripleScale proj_scale(const ProjArgs& A, Triple T) {
-  const int e0 = sg_exp(A, T.i, T.j, T.k), e1 = sg_exp(A, T.j, T.k, T.i), e2 = sg_exp(A, T.k, T.i, T.j);
-  TripleScale s;
-  s.E = max(e0, max(e1, e2));
-  s.f[0] = ldexpf(1.f, e0 - s.E);
-  s.f[1] = ldexpf(1.f, e1 - s.E);
-  s.f[2] = ldexpf(1.f, e2 - s.E);
-  s.fy = 0.f;
-  return s;
+
+// A block at the six positions of an orbit, as float64: the pairs are exact in it.
+// The conversions are integer operations (pair_double): as float64 ones they would
+// be 36 of 120 per orbit.
+__device__ __forceinline__ void orbit_block(const float2* __restrict__ G, const int64_t* at, int e, double* g) {
+  float2 x[6];
+  bool other = false;
+#pragma unroll
+  for (int n = 0; n < 6; ++n) x[n] = __ldg(G + at[n]);
+#pragma unroll
+  for (int n = 0; n < 6; ++n) g[n] = pair_double(x[n].x, x[n].y, e, &other);
+  if (other) {
+    const double scale = ldexp(1.0, e);
+#pragma unroll
+    for (int n = 0; n < 6; ++n) g[n] = pair_convert(x[n].x, x[n].y, scale);
+  }
+}
+// W~ (or S W~): G_0 at a position, G_1 at its cyclic successor, G_2 at the one after
+__device__ __forceinline__ void orbit_w(const float2* G, int64_t v3, const int* e, const int64_t* at, double* W) {
+  constexpr int r1[6] = {3, 5, 1, 4, 0, 2}, r2[6] = {4, 2, 5, 0, 3, 1};
+  double g[6];
+  orbit_block(G, at, e[0], W);
+  orbit_block(G + v3, at, e[1], g);
+#pragma unroll
+  for (int n = 0; n < 6; ++n) W[n] += g[r1[n]];
+  orbit_block(G + 2 * v3, at, e[2], g);
+#pragma unroll
+  for (int n = 0; n < 6; ++n) W[n] += g[r2[n]];
 }
 
-// per-block sums of (S W~) R[V] / D over the orbits of each slot, in FP32 pairs: in
-// float64 (k_energy_proj) two lanes per SM and cycle bound it, 102 of the 320 ms of
-// nocc=16 nvir=120 once; now 30 of 143
-__global__ void __launch_bounds__(256) k_proj_pairs(const __grid_constant__ ProjArgs A) {
+// per-block sums of (S W~) R[V] / D over the orbits of each slot, in float64 from
+// the pairs on.  Its two lanes per SM and cycle bound it, some 70 operations per
+// orbit, 30 of the 47 ms it takes at nocc=16 nvir=120 (161 ms in all; with W~, D and
+// the sums in FP32 pairs 30 and 143, at 48 bits; one thread per element of v^3, a
+// sixth of them an orbit, 102 of 320).  Four blocks per SM: 47 ms, two 52.
+__global__ void __launch_bounds__(256, 4) k_proj_batch(const __grid_constant__ ProjArgs A) {
   __shared__ double red[8];
   const int slot = blockIdx.y;
   const Triple T = A.t[slot];
-  const TripleScale sc = triple_scale(A.in, A.x0, T), ss = proj_scale(A, T);
-  const int64_t v = A.in.v, steps = orbit_steps(A.in.v);
-  const OrbitTile tile = orbit_tile();
+  const AdjArgs& a = A.a;
+  const int eg[3] = {g_exp(A.x0, a.o, T.i, T.j, T.k), g_exp(A.x0, a.o, T.j, T.k, T.i), g_exp(A.x0, a.o, T.k, T.i, T.j)};
+  const int es[3] = {sg_exp(A, T.i, T.j, T.k), sg_exp(A, T.j, T.k, T.i), sg_exp(A, T.k, T.i, T.j)};
   const float2 *G = A.G + slot * A.stride, *SG = A.SG + slot * A.stride;
-  const pr eo = occ_energy(A.in, T);
-  pr sum{0.f, 0.f};
+  const int64_t v = a.v, v3 = v * v * v, steps = orbit_steps(a.v);
+  const OrbitTile tile = orbit_tile();
+  const int64_t ox = (int64_t)a.o * v;  // doubles between the rows of ovs
+  const double *ovs_ij = a.ovs + T.i * v * ox + T.j * v, *ovs_jk = a.ovs + T.j * v * ox + T.k * v,
+               *ovs_ik = a.ovs + T.i * v * ox + T.k * v;
+  const double *t1i = a.t1 + T.i * v, *t1j = a.t1 + T.j * v, *t1k = a.t1 + T.k * v;
+  const double eo = a.eps_o[T.i] + a.eps_o[T.j] + a.eps_o[T.k];
+  double sum = 0.0;
   for (int64_t t = blockIdx.x; t < steps; t += gridDim.x) {
-    int a, b, c;
-    if (!orbit_at(tile, t, (int)v, &a, &b, &c)) continue;
-    pr W[6], Y[6], RV[6];
-    orbit_w(G, v, sc, a, b, c, W);
-    orbit_y(A.in, T, sc, a, b, c, Y);
+    int x, y, z;
+    if (!orbit_at(tile, t, a.v, &x, &y, &z)) continue;
+    double V[6], S[6], RV[6];
+    int64_t at[6];
+    orbit_index(v, x, y, z, at);
+    orbit_w(G, v3, eg, at, V);
+    const int p[6][3] = {{x, y, z}, {x, z, y}, {y, x, z}, {y, z, x}, {z, x, y}, {z, y, x}};
 #pragma unroll
-    for (int n = 0; n < 6; ++n) Y[n] = pr_add(W[n], Y[n]);
-    r_orbit_pairs(Y, RV);
-    orbit_w(SG, v, ss, a, b, c, W);
-    const unsigned distinct = orbit_distinct(a, b, c);
-    pr x{0.f, 0.f};
+    for (int n = 0; n < 6; ++n) {  // V = W~ + Y
+      const int q0 = p[n][0], q1 = p[n][1], q2 = p[n][2];
+      V[n] = fma(ovs_ij[(int64_t)q0 * ox + q1], t1k[q2], V[n]);
+      V[n] = fma(ovs_jk[(int64_t)q1 * ox + q2], t1i[q0], V[n]);
+      V[n] = fma(ovs_ik[(int64_t)q0 * ox + q2], t1j[q1], V[n]);
+    }
+    {  // r_orbit with the class sums combined first
+      const double se = (V[0] + V[3]) + V[4], so = (V[1] + V[2]) + V[5];
+      const double ue = fma(-2.0, so, se), uo = fma(-2.0, se, so);
+#pragma unroll
+      for (int n = 0; n < 6; ++n) RV[n] = fma(3.0, V[n], n == 0 || n == 3 || n == 4 ? ue : uo);
+    }
+    orbit_w(SG, v3, es, at, S);
+    const unsigned distinct = orbit_distinct(x, y, z);
+    double e = 0.0;
 #pragma unroll
     for (int n = 0; n < 6; ++n)
-      if (distinct >> n & 1u) pr_fma(x, W[n], RV[n]);
-    const pr r = pr_recip(pr_sub(pr_sub(pr_sub(eo, A.in.eps_v[a]), A.in.eps_v[b]), A.in.eps_v[c]));
-    pr_fma(sum, x, r);
+      if (distinct >> n & 1u) e = fma(S[n], RV[n], e);
+    const double D = eo - a.eps_v[x] - a.eps_v[y] - a.eps_v[z];
+    sum = fma(e, recip_newton(D, recip_newton(D, recip_seed(D))), sum);
   }
-  double s = pr_double(sum);
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
@@ -341,11 +375,10 @@ __global__ void __launch_bounds__(256) k_proj_pairs(const __grid_constant__ Proj
   }
 }
 
-// the slots' shares: (m / 3) (1 / 3) 2^(E + E_S) times their block sums in a fixed order
+// the slots' shares: (m / 3) (1 / 3) times their block sums in a fixed order
 __global__ void __launch_bounds__(256) k_proj_shares(const __grid_constant__ ProjArgs A, int nblk) {
   __shared__ double red[8];
   const int slot = blockIdx.x;
-  const Triple T = A.t[slot];
   double s = 0.0;
   for (int e = threadIdx.x; e < nblk; e += 256) s += A.epart[(int64_t)slot * nblk + e];
   for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
@@ -354,8 +387,7 @@ __global__ void __launch_bounds__(256) k_proj_shares(const __grid_constant__ Pro
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < 8; ++w) t += red[w];
-    const int E = triple_scale(A.in, A.x0, T).E + proj_scale(A, T).E;
-    A.shares[A.t0 + slot] = ldexp(t * ((double)T.m / 9.0), E);
+    A.shares[A.t0 + slot] = t * ((double)A.t[slot].m / 9.0);
   }
 }
 
@@ -363,7 +395,6 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int64_t v2 = (int64_t)v * v, v3 = v2 * v, nt = num_unique_triples(o);
   cudaError_t e = transform_inputs(h, c, cf, W.ovvvC, W.t2C, W.t2C2, W.ooovC, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(W.pb.hi, 0, 64, s);
   if (e != cudaSuccess) return fail(TE_ECUDA, "transform launch: %s", cudaGetErrorString(e));
   // exact-slice planes: the inputs; (ovvvC, t2C, ooovC) for ovvv, t2 and nooT;
   // t2C2 for t2L
@@ -373,13 +404,15 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
   ca.t2 = W.t2C;
   ca.ooov = W.ooovC;
   cb.t2 = W.t2C2;
-  te_status st = tc_prepare_slices(c, W.slices[0], &S0, h->num_sms, s, 4, h->d_err, 0, &h->n_launches, W.pb.hi);
+  te_status st = tc_prepare_slices(c, W.slices[0], &S0, h->num_sms, s, 4, h->d_err, 0, &h->n_launches);
   if (st == TE_OK) st = tc_prepare_slices(&ca, W.slices[1], &SA, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
   if (st == TE_OK) st = tc_prepare_slices(&cb, W.slices[2], &SB, h->num_sms, s, 4, nullptr, 0, &h->n_launches);
   if (st != TE_OK) return st;
-  e = launch_pair_inputs(c, W.pb, s);
+  Prepared P{};
+  P.ovs = W.ovs;
+  e = launch_prep_fp64(c, &P, s);
   ++h->n_launches;
-  if (e != cudaSuccess) return fail(TE_ECUDA, "pair launch: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return fail(TE_ECUDA, "prep: %s", cudaGetErrorString(e));
   // the six segment views of each slice set, encoded once
   VtBank bank;
   bank.n = 0;
@@ -389,8 +422,13 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
   if ((st = vt_slice_maps(&bank, SA, o, v, NT, mA)) != TE_OK) return st;
   if ((st = vt_slice_maps(&bank, SB, o, v, NT, mB)) != TE_OK) return st;
   const int grid = adjoint_grid(h->num_sms);
-  ProjArgs A;
-  A.in = pair_inputs(c, W.pb, o, v);
+  ProjArgs A{};
+  A.a.o = o;
+  A.a.v = v;
+  A.a.ovs = W.ovs;
+  A.a.t1 = c->t1;
+  A.a.eps_o = c->eps_o;
+  A.a.eps_v = c->eps_v;
   A.x0 = SliceExps{S0.e_ovvv, S0.e_t2, S0.e_t2L, S0.e_nooT};
   A.xa = SliceExps{SA.e_ovvv, SA.e_t2, SA.e_t2L, SA.e_nooT};
   A.xb = SliceExps{SB.e_ovvv, SB.e_t2, SB.e_t2L, SB.e_nooT};
@@ -445,7 +483,7 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
     }
     if ((st = vt_finish(&b, h->num_sms, nullptr, 0, nullptr)) != TE_OK) return st;
     if ((st = vt_launch(h, &b, s)) != TE_OK) return st;
-    k_proj_pairs<<<dim3((unsigned)grid, (unsigned)A.n), 256, 0, s>>>(A);
+    k_proj_batch<<<dim3((unsigned)grid, (unsigned)A.n), 256, 0, s>>>(A);
     k_proj_shares<<<(unsigned)A.n, 256, 0, s>>>(A, grid);
     h->n_launches += 2;
     e = cudaGetLastError();
@@ -462,7 +500,7 @@ size_t frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p) {
     return frag_layout(o, v, nullptr, &W);
   }
   FragOz W;
-  return frag_oz_layout(o, v, frag_oz_batch(h, o, v), nullptr, &W);
+  return frag_oz_layout(h, o, v, frag_oz_batch(h, o, v), nullptr, &W);
 }
 
 te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precision p, double* e_out,
@@ -474,7 +512,7 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
   te_status st = ensure_workspace_public(h, frag_bytes(h, o, v, p));
   if (st == TE_ENOMEM && B > 1) {
     B = 1;
-    st = ensure_workspace_public(h, frag_oz_layout(o, v, B, nullptr, &Z));
+    st = ensure_workspace_public(h, frag_oz_layout(h, o, v, B, nullptr, &Z));
   }
   if (st != TE_OK) return st;
   st = ensure_triples_public(h, o);
@@ -487,7 +525,7 @@ te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precisio
     shares = W.shares;
     st = run_frag_fp64(h, c, cf, W, s);
   } else {
-    frag_oz_layout(o, v, B, base, &Z);
+    frag_oz_layout(h, o, v, B, base, &Z);
     shares = Z.shares;
     st = run_frag_oz(h, c, cf, Z, B, s);
   }

@@ -441,10 +441,13 @@ __device__ __forceinline__ void view_tc_body(const VtMaps& maps, const VtParams&
         for (int q = 0; q < COLS / 4; ++q) {
           if (4 * q < ncol && U.n0 + c_lo + 4 * q < J.N) {
             float h[4], l[4];
-            f2_get(hi[2 * q], h[0], h[1]);
-            f2_get(hi[2 * q + 1], h[2], h[3]);
-            f2_get(lo[2 * q], l[0], l[1]);
-            f2_get(lo[2 * q + 1], l[2], l[3]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {  // the low word can be the larger one
+              f2 H, L;
+              f2_two_sum(hi[2 * q + j], lo[2 * q + j], H, L);
+              f2_get(H, h[2 * j], h[2 * j + 1]);
+              f2_get(L, l[2 * j], l[2 * j + 1]);
+            }
             if (J.vec) {
               asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + 4 * q), "f"(h[0]), "f"(l[0]),
                            "f"(h[1]), "f"(l[1]), "f"(h[2]), "f"(l[2]), "f"(h[3]), "f"(l[3])

@@ -57,9 +57,8 @@ struct VtSeg {
   const int* eb;
 };
 
-// float64 +=, float64 =, or the unit's FP32 pair (hi, lo) as it is: relative to
-// 2^(the largest scale of the job's segments).  One kind per
-// launch; VT_PAIR on CTA pairs only.  VT_ADD (and VT_STORE on lone CTAs) sums a unit's blocks to 2^-48 of the sum;
+// float64 +=, float64 =, or the unit's FP32 pair (hi, lo), |lo| <= ulp(hi) / 2,
+// relative to 2^(the largest scale of the job's segments).  One kind per launch; VT_PAIR on CTA pairs only.  VT_ADD (and VT_STORE on lone CTAs) sums a unit's blocks to 2^-48 of the sum;
 // VT_STORE on pairs and VT_PAIR round the higher levels' part to FP32 against the low
 // word first (2^-38 of the operands' scale; few blocks per unit).  VT_STORE is the
 // adjoint's G, whose last bits decide how dW~ is cut.

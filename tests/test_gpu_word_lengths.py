@@ -88,3 +88,29 @@ def test_g_formats_in_one_batch(te):
     e = te.t_energy_batched(a, "ozaki")
     one = torch.stack([te.t_energy(x, "ozaki") for x in a])
     assert float(((e - one) / one).abs().max()) <= BAR
+
+
+# Random integers of 14 bits: nothing cancels, and every product of the contraction,
+# also with operands projected by 0 / 1 matrices, is exact.
+def random_integers(o, v, seed, **more):
+    rng = np.random.default_rng(seed)
+    n = lambda *shape: rng.integers(-8000, 8001, shape).astype(float)  # noqa: E731
+    t2 = n(o, o, v, v)
+    lower = np.arange(o)[:, None] > np.arange(o)
+    t2[lower] = np.swapaxes(np.swapaxes(t2, 0, 1), 2, 3)[lower]
+    base = tegen.make_cluster(o, v, 4 * (o + v), seed).arrays()
+    return dict(dict(eps_o=base["eps_o"], eps_v=base["eps_v"], ovvv=n(o, v, v, v), ooov=n(o, o, o, v),
+                     ovov=n(o, v, o, v), t1=n(o, v), t2=t2), **more)
+
+
+@pytest.mark.parametrize("v", [8, 17, 33])
+def test_projected_energy_with_a_gap_of_1e_7(te, v):
+    """D is a difference of orbital energies near 0.5 that leaves 3e-7: float64
+    orders of summation agree to rounding, 1e-16 per term of some v^3 / 6, where a
+    word of 48 bits would leave 1e-8 in 1 / D."""
+    rng = np.random.default_rng(v)
+    a = dev(random_integers(3, v, v, eps_o=-0.5 - 1e-7 * rng.random(3), eps_v=-0.5 + 1e-7 * (1.0 + rng.random(v))))
+    for cf in (np.eye(3), np.diag([1.0, 0.0, 1.0])):
+        _, e = te.t_energy_frag(a, cf, "ozaki", shares=True)
+        _, ref = te.t_energy_frag(a, cf, "fp64", shares=True)
+        assert float((e - ref).abs().max()) <= 1e-13 * float(ref.abs().max())
