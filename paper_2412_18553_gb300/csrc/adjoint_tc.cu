@@ -1,5 +1,5 @@
 // The exact-slice adjoint of E(T) (see vjp.cu for the formulas): contractions on
-// tcgen05 (view_tc.cu), what only enters sums in pairs of FP32.
+// tcgen05 (view_tc.cu), everything else in float64.
 //
 // Triples go in batches of consecutive canonical triples (up to eight, as many
 // as about a gigabyte of G, dW~ and layouts holds), and each stage is one launch
@@ -8,20 +8,12 @@
 // their work.  Contributions of a batch to one output block are segments of one
 // job, in triple order, so every accumulation has a fixed order.
 //
-// The epilogue forms G, W~, Y, R and dW~ in float64: dW~ is cut into slices next,
-// and a last bit decides a digit.  What only enters sums (dY, dD and the shares)
-// continues in FP32 pairs (h + l, about 48 bits): GB300's float64 rate is 1/64 of
-// its FP32 rate, and a pair operation takes five to thirteen FP32
-// instructions.  To keep FP32's range out of the picture the pairs are held
-// relative to a power of two: W~ and Y to 2^E, E the largest scale of the
-// triple's segments and of Y, and the gradients' factors carry the rest.
-//
 // What bounds the kernels around the contractions, one triple at nvir = 320: the
-// epilogue (1.06 ms; 1.85 with a warp along one orbit index, whose G reads touch 32
-// lines; 4 v^3 float64 values moved would take 0.16) its float64 operations; the dW~
-// slices (0.55 ms for all six layouts, cut once; 1.01 when cut for three at a time) and
-// the Y and denominator planes (0.39; 0.75 with one load in flight per thread)
-// memory.  The view GEMM launches take 5.6 of the 8.8 ms (view_tc.cu).
+// epilogue (1.27 ms; a warp along one orbit index, whose G reads touch 32 lines,
+// 1.85; 4 v^3 values moved would take 0.16) and the Y and denominator planes (0.65) their
+// float64 operations, about 106 per orbit and 8 per value at two lanes per SM and
+// cycle; the dW~ slices (0.55 ms for all six layouts, cut once; 1.01 when cut for three
+// at a time) memory.  The view GEMM launches take 5.6 of the 9.2 ms (view_tc.cu).
 //
 // Where the operand transposes of all occupied indices would take too much
 // memory (a large cluster: full = false) a triple goes alone, the transposes are
@@ -29,7 +21,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <cmath>
 #include <initializer_list>
 #include <map>
 #include <new>
@@ -63,31 +54,25 @@ struct AdjBatch {
   int n;             // triples (slots) of the batch
   Triple t[ADJ_MAX_BATCH];
   double w[ADJ_MAX_BATCH];  // gE m / 3
-  int we[ADJ_MAX_BATCH];    // its exponent
 };
 
 struct AdjEpi {
-  PairInputs in;
-  SliceExps ex;
-  AdjArgs a;          // float64 inputs; G of slot 0
+  AdjArgs a;          // inputs; G of slot 0
   double* dW;         // [slot][v^3]
-  float2 *dY, *dD;    // [slot][v^3] relative to 2^(E + we) and 2^(2 E + we)
-  int64_t g_stride, d_stride, w_stride;  // elements per slot of G; of dY and dD; of dW
-  int* eslot;         // [slot] E
+  double *dY, *dD;    // [slot][v^3]
+  int64_t g_stride, d_stride, w_stride;  // doubles per slot of G; of dY and dD; of dW
   unsigned long long* dwmax;  // [slot] bits of max |dW|
-  double *epart, *dpart;  // [slot][gridDim.x] sums of the share (m / 3 and 4^E apart) and of dD (2^(2 E + we) apart)
+  double *epart, *dpart;  // [slot][gridDim.x] sums of the share (m / 3 apart) and of dD
 };
 
 // Threads stride over the orbits a >= b >= c (v(v+1)(v+2)/6 of them): W~ and Y
 // are formed once per orbit and every distinct element of the orbit gets its
-// dW~, dY and dD.
+// dW~, dY and dD.  1/D: two Newton steps from an FP32 seed.
 __global__ void __launch_bounds__(256) k_adjoint_batch(const __grid_constant__ AdjEpi A,
                                                        const __grid_constant__ AdjBatch B) {
   __shared__ double red[8], redd[8], redw[8];
   const int slot = blockIdx.y;
   const Triple T = B.t[slot];
-  const int E = triple_scale(A.in, A.ex, T).E, we = B.we[slot];
-  if (blockIdx.x == 0 && threadIdx.x == 0) A.eslot[slot] = E;
   AdjArgs a = A.a;
   a.G += slot * A.g_stride;
   a.i = T.i;
@@ -97,11 +82,10 @@ __global__ void __launch_bounds__(256) k_adjoint_batch(const __grid_constant__ A
   const int64_t v = a.v, steps = orbit_steps(a.v);
   const OrbitTile tile = orbit_tile();
   double* dW = A.dW + slot * A.w_stride;
-  float2* dY = A.dY + slot * A.d_stride;
-  float2* dD = A.dD + slot * A.d_stride;
+  double* dY = A.dY + slot * A.d_stride;
+  double* dD = A.dD + slot * A.d_stride;
   const double eo = a.eps_o[T.i] + a.eps_o[T.j] + a.eps_o[T.k];
-  pr contrib{0.f, 0.f}, dsum{0.f, 0.f};
-  double wmax = 0.0;
+  double cs = 0.0, ds = 0.0, wmax = 0.0;
   for (int64_t t = blockIdx.x; t < steps; t += gridDim.x) {
     int x, y, z;
     if (!orbit_at(tile, t, (int)v, &x, &y, &z)) continue;
@@ -109,30 +93,29 @@ __global__ void __launch_bounds__(256) k_adjoint_batch(const __grid_constant__ A
     int64_t idx[6];
     orbit_values(a, x, y, z, W, Y);
     orbit_index(v, x, y, z, idx);
-    r_orbit(W, RW);
-    r_orbit(Y, RY);
+    r_orbit_sums(W, RW);
+    r_orbit_sums(Y, RY);
     const unsigned distinct = orbit_distinct(x, y, z);
     const double D = eo - a.eps_v[x] - a.eps_v[y] - a.eps_v[z];
     const double rD = recip_newton(D, recip_newton(D, recip_seed(D)));
     const double q = w * rD;
-    const pr qp = pr_bits(q, we), rp = pr_bits(rD, 0);
+    const double qr = -q * rD;
+    double se = 0.0;  // the orbit's W~ R[V]
 #pragma unroll
     for (int n = 0; n < 6; ++n) {
       if (!(distinct >> n & 1u)) continue;
-      const double dw = q * (2.0 * RW[n] + RY[n]);
+      const double dw = q * fma(2.0, RW[n], RY[n]);
       dW[idx[n]] = dw;
       const unsigned long long m = (unsigned long long)__double_as_longlong(dw) & 0x7FFFFFFFFFFFFFFFull;
       if (m > (unsigned long long)__double_as_longlong(wmax)) wmax = __longlong_as_double((long long)m);
-      const pr rw = pr_bits(RW[n], E);
-      const pr e = pr_mul(pr_mul(pr_bits(W[n], E), pr_add(rw, pr_bits(RY[n], E))), rp);
-      const pr dd = pr_mul(pr_neg(qp), e);
-      dY[idx[n]] = pr_norm2(pr_mul(qp, rw));
-      dD[idx[n]] = pr_norm2(dd);
-      dsum = pr_add(dsum, dd);
-      contrib = pr_add(contrib, e);
+      const double e = W[n] * (RW[n] + RY[n]);
+      dY[idx[n]] = q * RW[n];
+      dD[idx[n]] = qr * e;
+      se += e;
     }
+    cs = fma(se, rD, cs);
+    ds = fma(se, qr, ds);
   }
-  double cs = pr_double(contrib), ds = pr_double(dsum);
   for (int off = 16; off > 0; off >>= 1) {
     cs += __shfl_down_sync(0xffffffffu, cs, off);
     ds += __shfl_down_sync(0xffffffffu, ds, off);
@@ -161,7 +144,7 @@ __global__ void __launch_bounds__(256) k_adjoint_batch(const __grid_constant__ A
 // Y and denominator reductions
 // ---------------------------------------------------------------------------
 
-// Partial results of a slot, scaled to their true size, float64:
+// Partial results of a slot:
 //   s[m] [v][v]: d ovs of mode 0 (i,a; j,b), 1 (j,b; k,c), 2 (i,a; k,c)
 //   p[0], p[1] [v][v]: per first index a, the sums behind dt1 of k (at c) and of j (at b)
 //   p[2], p[3] [v][v]: per a, the sums of dD behind d eps_v at b and at c
@@ -172,107 +155,117 @@ struct YParts {
 };
 
 // sum over the warp, in lane 0
-__device__ __forceinline__ void warp_sum(pr& s) {
+__device__ __forceinline__ void warp_sum(double& s) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1)
-    s = pr_add(s, pr{__shfl_down_sync(0xffffffffu, s.h, off), __shfl_down_sync(0xffffffffu, s.l, off)});
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
 }
 
-// One block per plane a of a slot: its rows (warp per b, lanes along c), then its
-// columns (lanes along c, warps along b).  The plane is read twice, from L2.
+// The sums over the warp of 16 values: number i ends in the lanes l with
+// l >> 1 = bits of i reversed (warp_sum16_index).  Halves are exchanged and added, so
+// that 16 sums take 16 additions, not 80.
+__device__ __forceinline__ double warp_sum16(double (&x)[16], int lane) {
+#pragma unroll
+  for (int n = 8, off = 16; n >= 1; n >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const double mine = up ? x[i + n] : x[i], other = up ? x[i] : x[i + n];
+      x[i] = mine + __shfl_xor_sync(0xffffffffu, other, off);
+    }
+  }
+  return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
+}
+__device__ __forceinline__ int warp_sum16_index(int lane) {
+  return ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+}
+
+// One block per plane a of a slot: its rows (four per warp, lanes along c), then
+// its columns (lanes along c, warps along b).  The plane is read twice, from L2.
 __global__ void __launch_bounds__(256) k_y_planes(const __grid_constant__ AdjEpi A, const __grid_constant__ AdjBatch B,
                                                   const __grid_constant__ YParts Yp) {
   __shared__ double red[2][8];
   const int a = blockIdx.x, slot = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const Triple T = B.t[slot];
-  const int v = A.in.v, o = A.in.o;
+  const int v = A.a.v, o = A.a.o;
   const int64_t V = v, plane = (int64_t)a * V * V;
-  const float2* dY = A.dY + slot * A.d_stride + plane;
-  const float2* dD = A.dD + slot * A.d_stride + plane;
-  const int E = A.eslot[slot], we = B.we[slot];
-  const int Eo = *A.in.e_ovs, Et = *A.in.e_t1;
-  const double ft = ldexp(1.0, E + we + Et), fo = ldexp(1.0, E + we + Eo), fd = ldexp(1.0, 2 * E + we);
-  const pr* t1k = A.in.t1 + (int64_t)T.k * v;
-  const pr* t1j = A.in.t1 + (int64_t)T.j * v;
-  auto ovs = [&](int p1, int x, int p2) { return A.in.ovs + (((int64_t)p1 * v + x) * o + p2) * v; };
-  const pr* ovs_ik = ovs(T.i, a, T.k);
-  const pr* ovs_ij = ovs(T.i, a, T.j);
+  const double* dY = A.dY + slot * A.d_stride + plane;
+  const double* dD = A.dD + slot * A.d_stride + plane;
+  const double* t1k = A.a.t1 + (int64_t)T.k * v;
+  const double* t1j = A.a.t1 + (int64_t)T.j * v;
+  auto ovs = [&](int p1, int x, int p2) { return A.a.ovs + (((int64_t)p1 * v + x) * o + p2) * v; };
+  const double* ovs_ik = ovs(T.i, a, T.k);
+  const double* ovs_ij = ovs(T.i, a, T.j);
   const int64_t so = slot * Yp.stride;
-  pr all{0.f, 0.f}, alld{0.f, 0.f};
-  for (int b = warp; b < v; b += 8) {
-    const pr* ovs_jk = ovs(T.j, b, T.k);
-    const float2 *yr = dY + (int64_t)b * V, *dr = dD + (int64_t)b * V;
-    pr s0{0.f, 0.f}, s2{0.f, 0.f}, sd{0.f, 0.f};
-    for (int c0 = lane; c0 < v; c0 += 128) {  // four elements in flight
-      pr y[4], d[4];
+  double all = 0.0, alld = 0.0;
+  for (int b0 = warp; b0 < v; b0 += 32) {  // rows b0 + 8 u
+    double s[16] = {};  // [4 u + k]: sums behind d ovs of (i, j), dt1 of j and d eps_v at b
+    const double* ovs_jk[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ovs_jk[u] = ovs(T.j, min(b0 + 8 * u, v - 1), T.k);
+    for (int c = lane; c < v; c += 32) {
+      double y[4], d[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const bool in = c0 + 32 * u < v;
-        y[u] = in ? pr_load(yr + c0 + 32 * u) : pr{0.f, 0.f};
-        d[u] = in ? pr_load(dr + c0 + 32 * u) : pr{0.f, 0.f};
+        const bool in = b0 + 8 * u < v;
+        y[u] = in ? __ldg(dY + (int64_t)(b0 + 8 * u) * V + c) : 0.0;
+        d[u] = in ? __ldg(dD + (int64_t)(b0 + 8 * u) * V + c) : 0.0;
       }
+      const double tk = t1k[c], oik = ovs_ik[c];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int c = min(c0 + 32 * u, v - 1);
-        pr_fma(s0, y[u], t1k[c]);
-        pr_fma(s2, y[u], ovs_ik[c]);
-        pr_fma(all, y[u], ovs_jk[c]);
-        sd = pr_add(sd, d[u]);
+        if (b0 + 8 * u >= v) break;
+        s[4 * u] = fma(y[u], tk, s[4 * u]);
+        s[4 * u + 1] = fma(y[u], oik, s[4 * u + 1]);
+        s[4 * u + 2] += d[u];
+        all = fma(y[u], ovs_jk[u][c], all);
       }
     }
-    alld = pr_add(alld, sd);
-    warp_sum(s0);
-    warp_sum(s2);
-    warp_sum(sd);
-    if (lane == 0) {
-      Yp.s[0][so + a * V + b] = pr_double(s0) * ft;
-      Yp.p[1][so + a * V + b] = pr_double(s2) * fo;
-      Yp.p[2][so + a * V + b] = pr_double(sd) * fd;
-    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) alld += s[4 * u + 2];
+    const double t = warp_sum16(s, lane);
+    const int i = warp_sum16_index(lane), b = b0 + 8 * (i >> 2), k = i & 3;
+    if ((lane & 1) == 0 && k < 3 && b < v) (k == 0 ? Yp.s[0] : (k == 1 ? Yp.p[1] : Yp.p[2]))[so + a * V + b] = t;
   }
   // columns: 32 at a time, warp w takes the rows b = w, w + 8, ...
-  __shared__ float2 col[3][8][33];
+  __shared__ double col[3][8][33];
   for (int c0 = 0; c0 < v; c0 += 32) {
     const int c = c0 + lane;
     const bool in = c < v;
-    pr s2{0.f, 0.f}, p0{0.f, 0.f}, sd{0.f, 0.f};
+    double s2 = 0.0, p0 = 0.0, sd = 0.0;
     for (int b0 = warp; b0 < v; b0 += 32) {
-      pr y[4], d[4];
+      double y[4], d[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const bool ok = in && b0 + 8 * u < v;
-        y[u] = ok ? pr_load(dY + (int64_t)(b0 + 8 * u) * V + c) : pr{0.f, 0.f};
-        d[u] = ok ? pr_load(dD + (int64_t)(b0 + 8 * u) * V + c) : pr{0.f, 0.f};
+        y[u] = ok ? __ldg(dY + (int64_t)(b0 + 8 * u) * V + c) : 0.0;
+        d[u] = ok ? __ldg(dD + (int64_t)(b0 + 8 * u) * V + c) : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int b = min(b0 + 8 * u, v - 1);
-        pr_fma(s2, y[u], t1j[b]);
-        pr_fma(p0, y[u], ovs_ij[b]);
-        sd = pr_add(sd, d[u]);
+        if (b0 + 8 * u >= v) break;
+        s2 = fma(y[u], t1j[b0 + 8 * u], s2);
+        p0 = fma(y[u], ovs_ij[b0 + 8 * u], p0);
+        sd += d[u];
       }
     }
-    col[0][warp][lane] = make_float2(s2.h, s2.l);
-    col[1][warp][lane] = make_float2(p0.h, p0.l);
-    col[2][warp][lane] = make_float2(sd.h, sd.l);
+    col[0][warp][lane] = s2;
+    col[1][warp][lane] = p0;
+    col[2][warp][lane] = sd;
     __syncthreads();
     if (warp < 3 && in) {
-      pr t{0.f, 0.f};
+      double t = 0.0;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) t = pr_add(t, pr{col[warp][w][lane].x, col[warp][w][lane].y});
+      for (int w = 0; w < 8; ++w) t += col[warp][w][lane];
       double* out = warp == 0 ? Yp.s[2] : (warp == 1 ? Yp.p[0] : Yp.p[3]);
-      out[so + a * V + c] = pr_double(t) * (warp == 0 ? ft : (warp == 1 ? fo : fd));
+      out[so + a * V + c] = t;
     }
     __syncthreads();
   }
-  double x = pr_double(all), xd = pr_double(alld);
-  for (int off = 16; off > 0; off >>= 1) {
-    x += __shfl_down_sync(0xffffffffu, x, off);
-    xd += __shfl_down_sync(0xffffffffu, xd, off);
-  }
+  warp_sum(all);
+  warp_sum(alld);
   if (lane == 0) {
-    red[0][warp] = x;
-    red[1][warp] = xd;
+    red[0][warp] = all;
+    red[1][warp] = alld;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -281,23 +274,23 @@ __global__ void __launch_bounds__(256) k_y_planes(const __grid_constant__ AdjEpi
       t += red[0][w];
       td += red[1][w];
     }
-    Yp.q[0][so + a] = t * fo;
-    Yp.q[1][so + a] = td * fd;
+    Yp.q[0][so + a] = t;
+    Yp.q[1][so + a] = td;
   }
 }
 
 // s[1][b][c] = sum_a dY[a,b,c] t1[i,a]
 __global__ void __launch_bounds__(256) k_y_sum_a(const __grid_constant__ AdjEpi A, const __grid_constant__ AdjBatch B,
                                                  const __grid_constant__ YParts Yp) {
-  const int slot = blockIdx.y, v = A.in.v;
+  const int slot = blockIdx.y, v = A.a.v;
   const int64_t v2 = (int64_t)v * v, bc = blockIdx.x * 256LL + threadIdx.x;
   if (bc >= v2) return;
-  const float2* dY = A.dY + slot * A.d_stride + bc;
-  const pr* t1i = A.in.t1 + (int64_t)B.t[slot].i * v;
-  pr s{0.f, 0.f};
+  const double* dY = A.dY + slot * A.d_stride + bc;
+  const double* t1i = A.a.t1 + (int64_t)B.t[slot].i * v;
+  double s = 0.0;
 #pragma unroll 8
-  for (int a = 0; a < v; ++a) pr_fma(s, pr_load(dY + a * v2), t1i[a]);
-  Yp.s[1][slot * Yp.stride + bc] = pr_double(s) * ldexp(1.0, A.eslot[slot] + B.we[slot] + *A.in.e_t1);
+  for (int a = 0; a < v; ++a) s = fma(__ldg(dY + a * v2), t1i[a], s);
+  Yp.s[1][slot * Yp.stride + bc] = s;
 }
 
 // the p arrays summed over a: block (32 columns, slot, array), into rows 0 of p
@@ -355,20 +348,18 @@ __global__ void __launch_bounds__(256) k_y_small(const __grid_constant__ AdjEpi 
                                                  const __grid_constant__ YParts Yp, const __grid_constant__ AdjOut O,
                                                  int agrid) {
   __shared__ double red[8];
-  const int v = A.in.v;
+  const int v = A.a.v;
   if (blockIdx.x == 0) {
     for (int s = 0; s < B.n; ++s) {
       const Triple T = B.t[s];
-      const int E = A.eslot[s];
       const double e = block_sum(A.epart + (int64_t)s * agrid, agrid, red);
       const double d = block_sum(A.dpart + (int64_t)s * agrid, agrid, red);
       if (threadIdx.x == 0) {
-        O.shares[O.t0 + s] = e * ldexp((double)T.m / 3.0, 2 * E);
+        O.shares[O.t0 + s] = e * ((double)T.m / 3.0);
         if (O.eps_o) {
-          const double x = d * ldexp(1.0, 2 * E + B.we[s]);
-          O.eps_o[T.i] += x;
-          O.eps_o[T.j] += x;
-          O.eps_o[T.k] += x;
+          O.eps_o[T.i] += d;
+          O.eps_o[T.j] += d;
+          O.eps_o[T.k] += d;
         }
       }
     }
@@ -511,11 +502,9 @@ AdjPlan adj_plan(int64_t o, int64_t v, int num_sms, bool full) {
   const int64_t d_ooov = vt_split_doubles(rows_z * ((o + nto - 1) / nto), pair_blk, v * o, num_sms) + 8;
   const int64_t d_t2 = vt_split_doubles(rows_z * ((v + ntv - 1) / ntv), pair_blk, v * v, num_sms) + 8;
   z.part_cap = 6 * (d_t2 + d_ooov) + 1024;
-  const size_t small = al((size_t)o * v * o * v * 8) /* pairs of ovs */ + al((size_t)o * v * 8) + al((size_t)(o + v) * 8) + al(64) +
-                       al((size_t)o * v * o * v * 8) /* ovs */;
-  z.bytes = tc_slices_bytes((int)o, (int)v, z.ns) + 1024 + small + z.B * (al(z.region) + al((size_t)v3 * 8)) +
-            al((size_t)o * v * o * v * 8) + 2 * al((size_t)z.B * 8192 * 8) + al((size_t)std::max<int64_t>(1, nt) * 8) +
-            al(256) + al((size_t)z.B * z.ystride * 8) + z.ovt + z.t2t + z.t2p + z.noo +
+  z.bytes = tc_slices_bytes((int)o, (int)v, z.ns) + 1024 + 2 * al((size_t)o * v * o * v * 8) /* ovs, dOVS */ +
+            z.B * (al(z.region) + al((size_t)v3 * 8)) + 2 * al((size_t)z.B * adjoint_grid(num_sms) * 8) +
+            al((size_t)std::max<int64_t>(1, nt) * 8) + al(256) + al((size_t)z.B * z.ystride * 8) + z.ovt + z.t2t + z.t2p + z.noo +
             al((size_t)z.part_cap * 8) + 4096;
   return z;
 }
@@ -571,20 +560,15 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
     return r;
   };
   auto take = [&](int64_t n) { return reinterpret_cast<double*>(takeb((size_t)n * 8)); };
-  PairBuffers pb;
-  pb.ovs = reinterpret_cast<pr*>(takeb((size_t)o * v * o * v * 8));
-  pb.t1 = reinterpret_cast<pr*>(takeb((size_t)o * v * 8));
-  pb.eps = reinterpret_cast<pr*>(takeb((size_t)(o + v) * 8));
-  pb.hi = reinterpret_cast<unsigned int*>(takeb(64));
   double* ovs = take((int64_t)o * v * o * v);
   char* region = takeb(Z.B * al(Z.region));
   double* dW = reinterpret_cast<double*>(takeb(Z.B * al((size_t)v3 * 8)));
   double* dOVS = take((int64_t)o * v * o * v);
-  double* epart = take((int64_t)Z.B * 8192);
-  double* dpart = take((int64_t)Z.B * 8192);
+  const int agrid = adjoint_grid(h->num_sms);
+  double* epart = take((int64_t)Z.B * agrid);
+  double* dpart = take((int64_t)Z.B * agrid);
   double* shares = take(std::max<int64_t>(1, nt));
-  int* eslot = reinterpret_cast<int*>(takeb(256));
-  unsigned long long* dwmax = reinterpret_cast<unsigned long long*>(eslot + 16);
+  unsigned long long* dwmax = reinterpret_cast<unsigned long long*>(takeb(256));
   int* dwexp = reinterpret_cast<int*>(dwmax + ADJ_MAX_BATCH);
   double* ypart = take(Z.B * Z.ystride);
   bf* ovT = reinterpret_cast<bf*>(takeb(Z.ovt));
@@ -594,21 +578,14 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
   double* part = take(Z.part_cap);
   const int64_t reg_stride = (int64_t)al(Z.region);                // bytes per slot
   const int64_t lay_stride = (int64_t)al(Z.lay * 2) / 2;           // elements between layouts of a slot
-  const int agrid = adjoint_grid(h->num_sms);
 
-  // operand slices, and the epilogue's pairs; both from one pass over the inputs
-  cudaError_t e = cudaMemsetAsync(pb.hi, 0, 64, s);
-  if (e != cudaSuccess) return fail(TE_ECUDA, "memset: %s", cudaGetErrorString(e));
   SliceSet S;
-  st = tc_prepare_slices(c, base, &S, h->num_sms, s, ns, h->d_err, cluster, &h->n_launches, pb.hi);
+  st = tc_prepare_slices(c, base, &S, h->num_sms, s, ns, h->d_err, cluster, &h->n_launches);
   if (st != TE_OK) return st;
-  e = launch_pair_inputs(c, pb, s);
   Prepared P{};  // float64 ovs for the disconnected term
-  P.o = o;
-  P.v = v;
   P.ovs = ovs;
-  if (e == cudaSuccess) e = launch_prep_fp64(c, &P, s);
-  h->n_launches += 2;
+  cudaError_t e = launch_prep_fp64(c, &P, s);
+  ++h->n_launches;
 
   auto zero = [&](double* ptr, int64_t n) {
     if (ptr && e == cudaSuccess) e = cudaMemsetAsync(ptr, 0, sizeof(double) * n, s);
@@ -703,8 +680,6 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
   auto eN = [&](int p_, int r_) { return S.e_nooT + ((int64_t)p_ * o + r_); };
 
   AdjEpi A;
-  A.in = pair_inputs(c, pb, o, v);
-  A.ex = SliceExps{S.e_ovvv, S.e_t2, S.e_t2L, S.e_nooT};
   A.a = AdjArgs{};
   A.a.o = o;
   A.a.v = v;
@@ -713,12 +688,11 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
   A.a.t1 = c->t1;
   A.a.eps_o = c->eps_o;
   A.a.eps_v = c->eps_v;
-  A.dY = reinterpret_cast<float2*>(region + al((size_t)3 * v3 * 8));
+  A.dY = reinterpret_cast<double*>(region + al((size_t)3 * v3 * 8));
   A.dD = A.dY + al((size_t)v3 * 8) / 8;
   A.dW = dW;
   A.g_stride = A.d_stride = reg_stride / 8;
   A.w_stride = (int64_t)al((size_t)v3 * 8) / 8;
-  A.eslot = eslot;
   A.dwmax = dwmax;
   A.epart = epart;
   A.dpart = dpart;
@@ -763,9 +737,7 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
       const int q[3][3] = {{T.i, T.j, T.k}, {T.j, T.k, T.i}, {T.k, T.i, T.j}};
       for (int gi = 0; gi < 3; ++gi)
         for (int d = 0; d < 3; ++d) PQR[x][gi][d] = q[gi][d];
-      const double w = gE * (double)T.m / 3.0;
-      Bt.w[x] = w;
-      std::frexp(w, &Bt.we[x]);
+      Bt.w[x] = gE * (double)T.m / 3.0;
     }
     // lean: slots of the transposes this triple reads
     int pr_[6][2], npair = 0, occ[3], nocc_ = 0;

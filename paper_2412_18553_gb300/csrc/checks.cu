@@ -31,8 +31,8 @@ cudaError_t launch_check_inputs(const te_cluster* c, int64_t cluster, unsigned i
       {c->ooov, grp ? o * o * o : 1, grp ? v : o * o * o * v, grp ? (int)o : 0, m.ooov, nullptr, 0, 4u},
       {df ? df->Bov : nullptr, df ? 1 : 0, P * o * v, 0, m.bov, nullptr, 0, 9u},
       {df ? df->Bvv : nullptr, df ? 1 : 0, P * v * v, 0, m.bvv, nullptr, 0, 10u},
-      {c->ovov, 1, o * v * o * v, 0, m.ovov, nullptr, 0, 5u},
-      {c->t1, 1, o * v, 0, m.t1, nullptr, 0, 6u},
+      {c->ovov, 1, o * v * o * v, 0, nullptr, nullptr, 0, 5u},
+      {c->t1, 1, o * v, 0, nullptr, nullptr, 0, 6u},
       {c->eps_o, 1, o, 0, nullptr, nullptr, 0, 1u},
       {c->eps_v, 1, v, 0, nullptr, nullptr, 0, 2u}};
   MaxArray a[MAX_ARRAYS];

@@ -350,12 +350,7 @@ __global__ void __launch_bounds__(256, 4) k_proj_batch(const __grid_constant__ P
       V[n] = fma(ovs_jk[(int64_t)q1 * ox + q2], t1i[q0], V[n]);
       V[n] = fma(ovs_ik[(int64_t)q0 * ox + q2], t1j[q1], V[n]);
     }
-    {  // r_orbit with the class sums combined first
-      const double se = (V[0] + V[3]) + V[4], so = (V[1] + V[2]) + V[5];
-      const double ue = fma(-2.0, so, se), uo = fma(-2.0, se, so);
-#pragma unroll
-      for (int n = 0; n < 6; ++n) RV[n] = fma(3.0, V[n], n == 0 || n == 3 || n == 4 ? ue : uo);
-    }
+    r_orbit_sums(V, RV);
     orbit_w(SG, v3, es, at, S);
     const unsigned distinct = orbit_distinct(x, y, z);
     double e = 0.0;

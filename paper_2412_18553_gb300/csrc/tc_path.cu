@@ -1368,8 +1368,7 @@ size_t tc_slices_bytes(int o, int v, int ns) {
 }
 
 te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, int num_sms, cudaStream_t s,
-                            int ns, unsigned int* err, int64_t cluster, int64_t* launches,
-                            unsigned int* max_ovov_t1) {
+                            int ns, unsigned int* err, int64_t cluster, int64_t* launches) {
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int vp = round_up(v, 16), op = round_up(o, 16);
   if (ns != 4 && ns != 5) return fail(TE_EINVAL, "slice count %d (4 or 5)", ns);
@@ -1412,10 +1411,6 @@ te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, in
   mo.t2 = hi + o;
   mo.t2L = hi + o + oo;
   mo.ooov = hi + 2 * o + oo;
-  if (max_ovov_t1) {
-    mo.ovov = max_ovov_t1;
-    mo.t1 = max_ovov_t1 + 1;
-  }
   cudaError_t e = cudaMemsetAsync(hi, 0, (size_t)ng * 4, s);
   if (e == cudaSuccess) e = launch_check_inputs(c, cluster, err, num_sms, s, nullptr, &mo);
   const SplitScales sc{nullptr, nullptr, hi, exps, (int)ng};

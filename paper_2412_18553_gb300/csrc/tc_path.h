@@ -43,9 +43,7 @@ struct SliceSet {
 // (256-byte aligned) and launches the slicing on s.
 size_t tc_slices_bytes(int o, int v, int ns = 4);
 // With err set, the pass over the inputs that finds the scales also makes the
-// value checks of launch_check_inputs.  max_ovov_t1: also the high words of
-// max |ovov| and max |t1| (two words, cleared by the caller).
+// value checks of launch_check_inputs.
 te_status tc_prepare_slices(const te_cluster* c, void* base, SliceSet* out, int num_sms, cudaStream_t s,
-                            int ns, unsigned int* err, int64_t cluster, int64_t* launches,
-                            unsigned int* max_ovov_t1 = nullptr);
+                            int ns, unsigned int* err, int64_t cluster, int64_t* launches);
 }  // namespace te

@@ -32,7 +32,7 @@ enum : unsigned int {
 // arrays, or with `groups` of ovvv[p], t2[r,q], ooov[p,:,r,:] and, for t2L,
 // t2[:,q].
 struct MaxOut {
-  unsigned int *ovvv, *t2, *ooov, *bov, *bvv, *t2L, *ovov, *t1;
+  unsigned int *ovvv, *t2, *ooov, *bov, *bvv, *t2L;
   bool groups;
 };
 // err null: the magnitudes only, no checks.

@@ -114,3 +114,32 @@ def test_projected_energy_with_a_gap_of_1e_7(te, v):
         _, e = te.t_energy_frag(a, cf, "ozaki", shares=True)
         _, ref = te.t_energy_frag(a, cf, "fp64", shares=True)
         assert float((e - ref).abs().max()) <= 1e-13 * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("o,v", [(3, 12), (4, 33), (2, 201)])
+def test_gradient_of_decayed_integrals(te, o, v):
+    """W~ is 2^-80 of Y (integrals and amplitudes between distant orbitals): dY, and
+    with it d ovov and d t1, is a product with W~ alone.  The bar is the gradients'
+    1e-6 of a tensor's largest entry."""
+    a = tegen.make_cluster(o, v, 4 * (o + v), v).arrays()
+    for n in ("ovvv", "ooov", "t2"):
+        a[n] = a[n] * 2.0 ** -40
+    a["t1"] = a["t1"] * 50.0
+    a = dev(a)
+    ref, g64 = te.t_energy_vjp(a, precision="fp64")
+    e, g = te.t_energy_vjp(a, precision="ozaki")
+    assert abs(float(e) - float(ref)) <= 1e-6 * abs(float(ref))
+    for n in g:
+        top = float(g64[n].abs().max())
+        assert top > 0.0 and float((g[n] - g64[n]).abs().max()) <= 1e-6 * top, n
+
+
+@pytest.mark.parametrize("v", [8, 17, 33])
+def test_projected_energy_of_decayed_integrals(te, v):
+    a = tegen.make_cluster(3, v, 4 * (3 + v), v).arrays()
+    for n in ("ovvv", "ooov", "t2"):
+        a[n] = a[n] * 2.0 ** -40
+    a = dev(a)
+    _, e = te.t_energy_frag(a, np.eye(3), "ozaki", shares=True)
+    _, ref = te.t_energy_frag(a, np.eye(3), "fp64", shares=True)
+    assert float((e - ref).abs().max()) <= 1e-6 * float(ref.abs().max())
