@@ -177,9 +177,9 @@ struct Fp64Plan {
 };
 
 static int fp64_slots(const Handle* h, int64_t v, int64_t ntri) {
-  // about 32 CTAs per SM and launch (two to four run at a time): the last wave
-  // is then a small part of it; at most 512 MiB of G
-  const int64_t tiles = 3 * gemm_fp64_tiles(v);
+  // work of about 32 tiles of 128 x 64 per SM and launch: its last wave is then a
+  // small part of it; at most 512 MiB of G
+  const int64_t tiles = 3 * ((v * v + 127) / 128) * ((v + 63) / 64);
   int64_t want = (32LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
   const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(512LL << 20) / (24 * v * v * v));
   want = std::min<int64_t>({want, mem_cap, 4096, std::max<int64_t>(1, ntri)});
@@ -230,7 +230,7 @@ static te_status run_fp64(Handle* h, const te_cluster* c, int64_t t_begin, int64
   for (int64_t t0 = t_begin; t0 < t_end; t0 += nslots) {
     const int ns = (int)std::min<int64_t>(nslots, t_end - t0);
     size_t pm = prof_begin(h, 0, s);
-    e = launch_gemm_fp64(&P, h->d_triples, t0, ns, gbuf, s);
+    e = launch_gemm_fp64(&P, h->d_triples, t0, ns, gbuf, h->num_sms, s);
     prof_end(h, pm, s);
     h->gemm_flops += 2.0 * 3.0 * ns * (double)v * v * v * (2.0 * v + 2.0 * o);
     if (e == cudaSuccess) {

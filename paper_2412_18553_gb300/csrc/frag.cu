@@ -183,7 +183,7 @@ te_status run_frag_fp64(Handle* h, const te_cluster* c, const double* cf, const 
     const Triple T = trip[t];
     e = cudaMemsetAsync(W.SG, 0, sizeof(double) * 3 * v3, s);
     if (e != cudaSuccess) break;
-    e = launch_gemm_fp64(&P, h->d_triples, t, 1, W.G, s);
+    e = launch_gemm_fp64(&P, h->d_triples, t, 1, W.G, h->num_sms, s);
     ++h->n_launches;
     for (int gi = 0; gi < 3 && e == cudaSuccess; ++gi) {
       int pp, qq, rr;

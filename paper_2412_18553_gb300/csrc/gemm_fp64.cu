@@ -17,6 +17,8 @@
 // with t2L[q][x][y][l] = t2[l,q,x,y] and nooT[p][r][z][l] = -ooov[p,l,r,z].
 // Each of the six terms of the permutation operator P appears exactly once in
 // the three G blocks (S1/S2 carry the sum over d, S3/S4 the sum over l).
+#include <algorithm>
+
 #include "dfma_tile.cuh"
 #include "te_internal.h"
 
@@ -176,14 +178,14 @@ k_gemm_fp64(const double* __restrict__ ovvv, const double* __restrict__ t2,
   }
 }
 
-int64_t gemm_fp64_tiles(int64_t v) {
-  const DfmaPick t = dfma_pick(v * v, v);
-  return t.tiles_m * t.tiles_n;
+// (K = 2 (v + o): only its length against the staging matters to the pick)
+static DfmaPick gemm_fp64_pick(int64_t v, int nslots, int num_sms) {
+  return dfma_pick(v * v, v, 2 * v + 16, 3LL * nslots, std::max(1, num_sms), 0, false);
 }
 
 cudaError_t launch_gemm_fp64(const Prepared* P, const Triple* d_triples, int64_t t0, int nslots,
-                             double* gbuf, cudaStream_t s) {
-  const DfmaPick t = dfma_pick((int64_t)P->v * P->v, P->v);
+                             double* gbuf, int num_sms, cudaStream_t s) {
+  const DfmaPick t = gemm_fp64_pick(P->v, nslots, num_sms);
   const dim3 grid((unsigned)t.tiles_m, (unsigned)t.tiles_n, (unsigned)(3 * nslots));
   dfma_dispatch(t, [&](auto rm, auto nb) {
     k_gemm_fp64<decltype(rm)::value, decltype(nb)::value>

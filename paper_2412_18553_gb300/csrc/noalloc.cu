@@ -128,12 +128,16 @@ extern "C" te_status t_energy_fp64_noalloc(const te_cluster* c, double* e_out, t
   // Every scratch byte read below is first written by this call: the triple
   // table, the prepared copies, each G block (all x,y,z < v), each partial
   // and each share; nothing has to start at zero.
+  int dev = 0, num_sms = 0;  // for the tile of the contraction
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return fail(TE_ECUDA, "device query failed");
   k_noalloc_fill_triples<<<(unsigned)((o + 127) / 128), 128, 0, s>>>(triples, (int)o);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = launch_prep_fp64(c, &P, s);
   for (int64_t t0 = 0; e == cudaSuccess && t0 < nt; t0 += slots) {
     const int ns = (int)std::min<int64_t>(slots, nt - t0);
-    e = launch_gemm_fp64(&P, triples, t0, ns, gbuf, s);
+    e = launch_gemm_fp64(&P, triples, t0, ns, gbuf, num_sms, s);
     if (e == cudaSuccess) e = launch_energy_f64(&P, triples, t0, ns, gbuf, partials, nbt, s);
     if (e == cudaSuccess) e = launch_reduce_triples(partials, nbt, triples, t0, ns, shares + t0, s);
   }

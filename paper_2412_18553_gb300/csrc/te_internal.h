@@ -131,10 +131,8 @@ int64_t num_unique_triples(int64_t nocc);
 
 // launch wrappers (defined in the .cu files)
 cudaError_t launch_prep_fp64(const te_cluster* c, Prepared* P, cudaStream_t s);
-// CTAs of launch_gemm_fp64 per G block
-int64_t gemm_fp64_tiles(int64_t v);
 cudaError_t launch_gemm_fp64(const Prepared* P, const Triple* d_triples, int64_t t0,
-                             int nslots, double* gbuf, cudaStream_t s);
+                             int nslots, double* gbuf, int num_sms, cudaStream_t s);
 
 // energy over G buffers in float64
 cudaError_t launch_energy_f64(const Prepared* P, const Triple* d_triples, int64_t t0,

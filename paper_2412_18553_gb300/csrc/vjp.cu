@@ -197,24 +197,12 @@ __global__ void k_splitk_add(GemmView g, int nsplit, const double* __restrict__ 
   }
 }
 
-// Split count for a GEMM of `tiles` output tiles and K steps: about two
-// blocks per SM, each split at least 8 K steps; the scratch holds `cap`
-// doubles.
-static int num_splits(int64_t tiles, int64_t K, int64_t MN, int num_sms, int64_t cap) {
-  const int64_t steps = (K + DT_K - 1) / DT_K;
-  int64_t want = (2LL * num_sms + tiles - 1) / tiles;
-  want = std::min<int64_t>(want, std::max<int64_t>(1, steps / 8));
-  want = std::min<int64_t>(want, std::max<int64_t>(1, cap / std::max<int64_t>(1, MN)));
-  return (int)std::max<int64_t>(1, want);
-}
-
 cudaError_t gemm_strided(const GemmView& g, int num_sms, double* scratch, int64_t scratch_cap, cudaStream_t s,
                          int64_t* launches) {
   const int64_t M = g.M1 * g.M2, K = g.K1 * g.K2;
-  const DfmaPick t = dfma_pick(M, g.N);
-  const int ns = num_splits(t.tiles_m * t.tiles_n, K, M * g.N, num_sms, scratch_cap);
+  const DfmaPick t = dfma_pick(M, g.N, K, 1, std::max(1, num_sms), scratch_cap, g.symmetric);
   const int64_t steps = (K + DT_K - 1) / DT_K;
-  const int kchunk = (int)(((steps + ns - 1) / ns) * DT_K);
+  const int kchunk = (int)(((steps + t.nsplit - 1) / t.nsplit) * DT_K);
   const int nsplit = (int)((K + kchunk - 1) / kchunk);
   const dim3 grid((unsigned)t.tiles_m, (unsigned)t.tiles_n, (unsigned)nsplit);
   const bool a_fast = (g.K2 > 1 ? g.a_k2 : g.a_k1) == 1, b_fast = (g.K2 > 1 ? g.b_k2 : g.b_k1) == 1;
@@ -454,7 +442,7 @@ te_status run_vjp_fp64(Handle* h, const te_cluster* c, int64_t t_begin, int64_t 
   std::vector<Triple> trip = unique_triples(o);
   for (int64_t t = t_begin; t < t_end && e == cudaSuccess; ++t) {
     const Triple T = trip[t];
-    e = launch_gemm_fp64(&P, h->d_triples, t, 1, W.G, s);
+    e = launch_gemm_fp64(&P, h->d_triples, t, 1, W.G, h->num_sms, s);
     if (e != cudaSuccess) break;
     AdjArgs A{};
     A.o = o; A.v = v; A.i = T.i; A.j = T.j; A.k = T.k;
