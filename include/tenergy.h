@@ -223,8 +223,8 @@ te_status t_energy_frag(te_handle h, const te_cluster* c, const double* cf, te_p
  *
  * The slabs ovvv[i] are formed in groups on the tensor cores (Bov and Bvv cut
  * into five 7-bit BF16 slices with one power-of-two scale each, fifteen slice
- * products with exact level-0/1 sums over K blocks of at most 1024, float64
- * across blocks: each entry within naux 2^(ea + eb - 34) of the float64
+ * products with exact level-0/1 sums over K blocks of 128, which are added to
+ * 2^-48 of the sum: each entry within naux 2^(ea + eb - 34) of the float64
  * product, where 2^ea > max |Bov| and 2^eb > max |Bvv|) and written straight
  * into the contraction's operand form.  The
  * exact-slice modes need max |ovvv| before slicing, so the slabs are formed

@@ -10,7 +10,7 @@
 // The three contractions are GEMMs over two-index views (strided.h).  The
 // (ia|jb) contraction runs in float64 on the DFMA units or, in the exact-slice
 // mode, in exact BF16 slices on the tensor cores (Bov scaled by one power of
-// two and cut into four 7-bit slices; K blocks of at most 1024 keep the
+// two and cut into four 7-bit slices, K in blocks of 128 that keep the
 // level-0/1 sums exact).  The density contractions run in float64 in both
 // modes: their K spans the amplitudes' whole dynamic range (o^2 v and o v^2
 // terms), which one scale per array would resolve only to ~1e-6 of the
@@ -296,6 +296,7 @@ static size_t mp2_keep_bytes(int64_t o, int64_t v) {
   if (v > kEigSmemN) b += al256((size_t)v * v * 8);
   return b;
 }
+
 
 // Clusters per eigensolver launch: two matrices each, 64 jobs.
 constexpr int64_t kMp2Group = 32;

@@ -938,7 +938,7 @@ static te_status build_energy_maps(TcState* st, const TcPlan& pl, int o, int v, 
 // ovvv from density-fitting factors (t_energy_df):
 //   ovvv[p,x,y,d] = sum_P Bov[P,p,x] Bvv[P,y,d]
 // formed nst slabs at a time by the exact-slice view GEMM (five 7-bit slices
-// per factor, K in exact blocks of at most 1024) into a float64 staging block,
+// per factor, K in exact blocks of 128) into a float64 staging block,
 // then cut into the contraction's operand form.
 // ---------------------------------------------------------------------------
 

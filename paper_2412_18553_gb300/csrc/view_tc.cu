@@ -873,8 +873,10 @@ te_status vt_product(Handle* h, const void* a, int64_t a_plane, int64_t m, const
   if (!B) return fail(TE_ENOMEM, "view GEMM tables");
   vt_begin(B.get(), ns, false);
   const int none[3] = {0, 0, 0};
-  vt_job(B.get(), 1, (int)m, (int)n, 1, 128, NT, C, 0, n, 1, VT_STORE);
+  VtJob* j = vt_job(B.get(), 1, (int)m, (int)n, 1, 128, NT, C, 0, n, 1, VT_STORE);
   vt_seg(B.get(), vt_use(B.get(), bank, ma), vt_use(B.get(), bank, mb), 1, (int)K, none, none, ea, eb, 1);
+  j->bchunks = VT_PRODUCT_CHUNKS;
+  j->nblocks = vt_seg_blocks(1, (int)K, VT_PRODUCT_CHUNKS);
   st = vt_finish(B.get(), h->num_sms, nullptr, 0, nullptr);
   return st == TE_OK ? vt_launch(h, B.get(), s) : st;
 }

@@ -167,10 +167,14 @@ int vt_ntile(int64_t n, bool pair);
 
 // C[i][j] = 2^(ea + eb) sum_k A[i][k] B[j][k] (i < m, j < n; C has rows of n) over ns
 // slice planes with rows of Kp elements (Kp a multiple of 8, planes 16-byte aligned),
-// on lone CTAs: K of hundreds or more, so few drains.  The ovvv of nocc=16
-// nvir=160 from 704 auxiliary functions (five slices): 1.17 ms, 3.40 ms with mma.sync on
-// row-contiguous factors; batches of MP2 steps gain by as much (eight clusters of
-// nocc 8 .. 20, nvir = 8 nocc, exact slices: 18.0 ms a call).
+// on lone CTAs.  K is taken in blocks of VT_PRODUCT_CHUNKS stages: the third
+// accumulator cuts what every MMA adds at 2^-24 of its sum, and where the slices'
+// products have one sign (the diagonal of (ia|jb)) that error grows with the square
+// of a block's length: 1.7e-9 of the scale's square at K = 1024 in blocks of 128,
+// 2.4e-8 in one block.  The ovvv of nocc=16 nvir=160 from 704 auxiliary functions
+// (five slices): 1.84 ms, 1.17 in one block, 3.40 with mma.sync on row-contiguous
+// factors.
+constexpr int VT_PRODUCT_CHUNKS = 4;
 te_status vt_product(Handle* h, const void* a, int64_t a_plane, int64_t m, const void* b, int64_t b_plane, int64_t n,
                      int64_t K, int64_t Kp, int ns, const int* ea, const int* eb, double* C, cudaStream_t s);
 

@@ -143,3 +143,29 @@ def test_projected_energy_of_decayed_integrals(te, v):
     _, e = te.t_energy_frag(a, np.eye(3), "ozaki", shares=True)
     _, ref = te.t_energy_frag(a, np.eye(3), "fp64", shares=True)
     assert float((e - ref).abs().max()) <= 1e-6 * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("naux", [64, 1024, 2048, 5000])
+@pytest.mark.parametrize("low", [0.3, -1.0])
+def test_mp2_integrals_against_their_slices(te, naux, low):
+    """(ia|jb) of exact slices less the sum of the slice products that are kept.  The
+    level-0/1 sums are exact; the third accumulator loses at most half a unit on
+    average whenever an MMA adds to it: 56 times per 128 auxiliary functions (8 steps of
+    16, seven products of levels 2 and 3), a unit of 2^-34 (squares of the second slices,
+    64^2 / 3 on average, make its sum 2^-10.6 on the diagonal)."""
+    o, v = 2, 9
+    B = np.random.default_rng(naux).uniform(low, 1.0, (naux, o, v))
+    eo, ev = np.array([-1.0, -0.5]), np.linspace(0.5, 2.0, v)
+    t2 = te.mp2_bno_batched([(eo, ev, B)], "ozaki")[0]["t2"].cpu().numpy()
+    D = ev[:, None] + ev[None, :] - eo[:, None, None, None] - eo[:, None, None]
+    rest, m, ref = B.reshape(naux, o * v), [], 0.0
+    for _ in range(4):
+        m.append(np.rint(rest * 128.0))
+        rest = rest * 128.0 - m[-1]
+    for i in range(4):
+        for j in range(4 - i):
+            ref = ref + (m[i].T @ m[j]) * 2.0 ** (-7 * (i + j + 2))
+    err = (-t2 * D).transpose(0, 2, 1, 3).reshape(o * v, o * v) - ref
+    bar = max(1.0, naux / 128.0) * 56 * 2.0 ** -35
+    assert abs(float(np.diagonal(err).mean())) <= bar
+    assert float(np.abs(err).max()) <= 2.0 * bar
