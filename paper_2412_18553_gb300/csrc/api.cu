@@ -108,6 +108,19 @@ static te_status ensure_workspace(Handle* h, size_t bytes) {
   return TE_OK;
 }
 
+te_status acquire_workspace(Handle* h, const std::vector<size_t>& bytes, size_t* form) {
+  te_status st = TE_OK;
+  for (size_t k = 0; k < bytes.size(); ++k) {
+    *form = k;
+    const bool last = k + 1 == bytes.size();
+    if (bytes[k] <= h->ws_bytes) return TE_OK;
+    if (!last && (h->capturing || (h->ws_limit && bytes[k] > h->ws_limit))) continue;
+    st = ensure_workspace(h, bytes[k]);
+    if (st != TE_ENOMEM) return st;
+  }
+  return st;
+}
+
 // The canonical order is prefix-closed (the triples of nocc = n are the first
 // ones of any larger nocc), so one table for the largest nocc serves all.
 static te_status ensure_triples(Handle* h, int nocc) {
@@ -170,12 +183,6 @@ static te_status check_values(Handle* h, const te_cluster* c, cudaStream_t s, in
 // FP64 path
 // ---------------------------------------------------------------------------
 
-struct Fp64Plan {
-  int nslots;
-  int64_t nbt;
-  size_t bytes;
-};
-
 static int fp64_slots(const Handle* h, int64_t v, int64_t ntri) {
   // work of about 32 tiles of 128 x 64 per SM and launch: its last wave is then a
   // small part of it; at most 512 MiB of G
@@ -199,19 +206,38 @@ static size_t fp64_carve(Carver& cv, int64_t o, int64_t v, int nslots, int64_t n
   return cv.off;
 }
 
+// Triples per launch of the forms of a float64 energy, and their workspace: the
+// usual count, then halves of it down to one where memory is short.  A triple's
+// share has the same bits in all of them.
+struct Fp64Forms {
+  std::vector<int> slots;
+  std::vector<size_t> bytes;
+};
+static Fp64Forms fp64_forms(const Handle* h, int64_t o, int64_t v, int64_t nt) {
+  Fp64Forms f;
+  for (int n = fp64_slots(h, v, nt);; n /= 2) {
+    Prepared P{};
+    double *a, *b, *d;
+    Carver probe(nullptr);
+    f.slots.push_back(n);
+    f.bytes.push_back(fp64_carve(probe, o, v, n, energy_num_block_triples(v), num_unique_triples(o), &P, &a, &b, &d));
+    if (n == 1) return f;
+  }
+}
+
 static te_status run_fp64(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_end,
                           double* e_tri_out, double* e_total_out, cudaStream_t s) {
   const int64_t o = c->nocc, v = c->nvir;
   const int64_t ntri_all = num_unique_triples(o);
   const int64_t nt = t_end - t_begin;
-  const int nslots = fp64_slots(h, v, nt);
   const int64_t nbt = energy_num_block_triples(v);
+  const Fp64Forms forms = fp64_forms(h, o, v, nt);
+  size_t form = 0;
+  te_status st = acquire_workspace(h, forms.bytes, &form);
+  if (st != TE_OK) return st;
+  const int nslots = forms.slots[form];
   Prepared P{};
   double *gbuf, *partials, *etri;
-  Carver probe(nullptr);
-  const size_t bytes = fp64_carve(probe, o, v, nslots, nbt, ntri_all, &P, &gbuf, &partials, &etri);
-  te_status st = ensure_workspace(h, bytes);
-  if (st != TE_OK) return st;
   st = ensure_triples(h, (int)o);
   if (st != TE_OK) return st;
   Carver cv(h->ws);
@@ -520,20 +546,26 @@ te_status t_energy_batched(te_handle hh, const te_cluster* cs, int64_t n, te_pre
     }
   }
   // one workspace for the whole batch: float64 runs the members one after
-  // another; the tensor-core modes hold every member's operands and one G pool
-  size_t need = 0;
+  // another, each in the best form that fits it; the tensor-core modes hold every
+  // member's operands and one G pool
+  std::vector<size_t> need;
   if (p == TE_FP64) {
+    std::vector<std::vector<size_t>> f;
+    size_t levels = 1;
     for (int64_t x = 0; x < n; ++x) {
-      size_t b = 0;
-      st = te_workspace_bytes(hh, cs + x, p, &b);
-      if (st != TE_OK) return st;
-      need = std::max(need, b);
+      f.push_back(fp64_forms(h, cs[x].nocc, cs[x].nvir, num_unique_triples(cs[x].nocc)).bytes);
+      levels = std::max(levels, f.back().size());
     }
+    need.assign(levels, 0);
+    for (size_t k = 0; k < levels; ++k)
+      for (const auto& b : f) need[k] = std::max(need[k], b[std::min(k, b.size() - 1)]);
   } else {
-    st = tc_batched_bytes(h, cs, n, p, &need);
+    need.assign(1, 0);
+    st = tc_batched_bytes(h, cs, n, p, &need[0]);
     if (st != TE_OK) return st;
   }
-  st = ensure_workspace(h, need);
+  size_t form = 0;
+  st = acquire_workspace(h, need, &form);
   if (st != TE_OK) return st;
   // capture the batch's launches into one CUDA graph on an internal stream
   if (!h->cap_stream && cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -713,13 +745,11 @@ te_status te_workspace_bytes(te_handle hh, const te_cluster* c, te_precision p, 
   Handle* h = reinterpret_cast<Handle*>(hh);
   if (!h || !c || !bytes) return fail(TE_EINVAL, "null argument");
   if (c->nocc < 1 || c->nvir < 1) return fail(TE_EINVAL, "nocc and nvir must be >= 1");
-  const int64_t o = c->nocc, v = c->nvir;
-  const int64_t nt = num_unique_triples(o);
   if (p == TE_FP64) {
-    Prepared P{};
-    double *a, *b, *d;
-    Carver probe(nullptr);
-    *bytes = fp64_carve(probe, o, v, fp64_slots(h, v, nt), energy_num_block_triples(v), nt, &P, &a, &b, &d);
+    for (size_t b : fp64_forms(h, c->nocc, c->nvir, num_unique_triples(c->nocc)).bytes) {
+      *bytes = b;  // the first that the limit admits, else the smallest
+      if (!h->ws_limit || b <= h->ws_limit) break;
+    }
     return TE_OK;
   }
   return tc_workspace_bytes(h, c, p, bytes);

@@ -110,6 +110,11 @@ struct Handle {
   std::map<std::tuple<int, int, int>, std::pair<int, int>> tune_file;
 };
 
+// The workspace of a call that can run in several forms, `bytes` of them, best
+// first: the first form that the handle holds already or can have under its limit
+// and on the device.  Inside the library's graph capture nothing is allocated.
+te_status acquire_workspace(Handle* h, const std::vector<size_t>& bytes, size_t* form);
+
 void drop_graphs(Handle* h);
 
 // autotune cache file: first line of the format for this handle's GPU; write
