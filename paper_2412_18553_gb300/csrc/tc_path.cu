@@ -685,12 +685,17 @@ struct TcPlan {
   int stages;
   uint32_t stage_bytes, a_part_bytes, b_part_bytes, tmem_cols;
   int nbuf;
-  int nslots;
+  int nslots, par_slots;  // triples per launch, and per share reduction
+  int min_slots;          // triples per launch where memory is short
   int ldz;
   size_t smem;
 };
 
-constexpr int64_t MIN_SLOTS = 4;  // triples per launch where memory is short
+constexpr int64_t MIN_SLOTS = 4;          // triples per launch where memory is short,
+constexpr int64_t MIN_POOL = int64_t(3) << 30;  // as many as this holds
+// Triples whose energy partials wait for one share reduction (about 20 MB of
+// them) where memory is not short; a launch's own triples where it is.
+constexpr int64_t TC_PAR_SLOTS = 1024;
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -771,6 +776,10 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   want = std::max<int64_t>(want, MIN_SLOTS);
   want = std::min<int64_t>({want, mem_cap, 1024, std::max<int64_t>(1, ntri)});
   pl.nslots = (int)std::max<int64_t>(1, want);
+  pl.par_slots = (int)std::max<int64_t>(pl.nslots, std::min<int64_t>(TC_PAR_SLOTS, ntri));
+  // at the least, a tile for every pair of CTAs
+  const int64_t fill = (std::max(1, h->num_sms) / 2 + tiles - 1) / tiles;
+  pl.min_slots = (int)std::max<int64_t>(1, std::min<int64_t>({pl.nslots, std::max(MIN_SLOTS, fill), MIN_POOL / per_slot}));
   return pl;
 }
 
@@ -831,9 +840,6 @@ struct TcPool {
   int64_t max_slots;  // G slots per launch
   int64_t par_slots;  // energy partials held until their share reduction (at least max_slots)
 };
-
-// Triples whose partials wait for one share reduction: about 20 MB of them.
-constexpr int64_t TC_PAR_SLOTS = 1024;
 
 static size_t tc_partial_bytes(const TcPool& q, int num_sms) {
   return (size_t)q.par_slots * std::max(1, num_sms) * ENERGY_TC_WARPS * sizeof(double);
@@ -1339,23 +1345,30 @@ static TcPool single_pool(const TcPlan& pl, int v) {
   TcPool q;
   q.pool_floats = (int64_t)pl.nslots * g_slot_floats(v, pl.fmt);
   q.max_slots = pl.nslots;
-  q.par_slots = std::max<int64_t>(pl.nslots, TC_PAR_SLOTS);
+  q.par_slots = pl.par_slots;
   return q;
 }
 
-// Workspace of a single-cluster call; with `lean`, or a handle limit that the
-// usual G pool would pass, for MIN_SLOTS triples per launch (pl->nslots).
-static size_t single_bytes(const Handle* h, TcPlan* pl, int o, int v, const te_df* df, bool lean) {
+// The forms of a single-cluster call and their workspace: the usual one, then
+// half the triples per launch and again, down to min_slots, with a share
+// reduction per launch, where memory is short.  The shares have the same bits.
+struct SingleForms {
+  std::vector<TcPlan> plan;
+  std::vector<size_t> bytes;
+};
+static SingleForms single_forms(const Handle* h, TcPlan pl, int o, int v, const te_df* df) {
+  SingleForms f;
   TcBuffers b;
   DfScratch d;
-  const size_t fixed = tc_carve_cluster(nullptr, *pl, o, v, num_unique_triples(o), &b);
+  const size_t fixed = tc_carve_cluster(nullptr, pl, o, v, num_unique_triples(o), &b);
   const size_t form = df ? df_carve(nullptr, o, v, df->naux, &d) : size_t(0);
-  size_t bytes = fixed + std::max(tc_shared_bytes(single_pool(*pl, v), h->num_sms), form);
-  if ((lean || (h->ws_limit && bytes > h->ws_limit)) && pl->nslots > MIN_SLOTS) {
-    pl->nslots = (int)MIN_SLOTS;
-    bytes = fixed + std::max(tc_shared_bytes(single_pool(*pl, v), h->num_sms), form);
+  for (;;) {
+    f.plan.push_back(pl);
+    f.bytes.push_back(fixed + std::max(tc_shared_bytes(single_pool(pl, v), h->num_sms), form));
+    if (pl.nslots == pl.min_slots && pl.par_slots == pl.nslots) return f;
+    pl.nslots = std::max(pl.min_slots, pl.nslots / 2);
+    pl.par_slots = pl.nslots;
   }
-  return bytes;
 }
 
 size_t tc_slices_bytes(int o, int v, int ns) {
@@ -1446,8 +1459,11 @@ te_status tc_prepare_slices(const te_cluster* c, void* base_v, SliceSet* out, in
 
 te_status tc_workspace_bytes(Handle* h, const te_cluster* c, te_precision p, size_t* bytes, const te_df* df) {
   const int o = (int)c->nocc, v = (int)c->nvir;
-  TcPlan pl = make_plan(h, o, v, tc_mode_of(p, o, v, h->ozaki_bits), num_unique_triples(c->nocc));
-  *bytes = single_bytes(h, &pl, o, v, df, false);
+  const TcPlan pl = make_plan(h, o, v, tc_mode_of(p, o, v, h->ozaki_bits), num_unique_triples(c->nocc));
+  for (size_t b : single_forms(h, pl, o, v, df).bytes) {
+    *bytes = b;  // the first that the limit admits, else the smallest
+    if (!h->ws_limit || b <= h->ws_limit) break;
+  }
   return TE_OK;
 }
 
@@ -1499,7 +1515,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
   size_t need = 0;
   for (const auto& cd : cand) {
     TcPlan pl = make_plan(h, o, v, mode, nt, cd.first, cd.second);
-    pl.nslots = (int)std::min<int64_t>(pl.nslots, MIN_SLOTS);
+    pl.nslots = pl.par_slots = pl.min_slots;
     TcBuffers b;
     need = std::max(need, tc_carve_cluster(nullptr, pl, o, v, nt, &b) + tc_shared_bytes(single_pool(pl, v), h->num_sms));
   }
@@ -1517,7 +1533,7 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
   TcParams* P = new TcParams;
   for (const auto& cd : cand) {
     TcPlan pl = make_plan(h, o, v, mode, nt, cd.first, cd.second);
-    pl.nslots = (int)std::min<int64_t>(pl.nslots, MIN_SLOTS);
+    pl.nslots = pl.par_slots = pl.min_slots;
     if (pl.stages < 2) continue;
     TcJob& J = jobs[0];
     J = TcJob{};
@@ -1591,16 +1607,17 @@ te_status run_tc(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin
   if (pl.stages < 2) return fail(TE_EUNSUPPORTED, "not enough shared memory for two pipeline stages");
   rs = check_k(mode, o, v);
   if (rs != TE_OK) return rs;
-  size_t bytes = single_bytes(h, &pl, o, v, df, false);
+  const SingleForms forms = single_forms(h, pl, o, v, df);
+  size_t form = 0;
+  rs = acquire_workspace(h, forms.bytes, &form);
+  if (rs != TE_OK) return rs;
+  pl = forms.plan[form];
   if (h->log)
     std::fprintf(stderr,
                  "[tenergy] plan nocc=%d nvir=%d mode=%d: M tile %d x %d, N tile %d (%d per row block), %d stages "
                  "of %u bytes, %d triples per launch, %u TMEM columns (%d accumulator sets), workspace %zu bytes\n",
                  o, v, mode, pl.TA, pl.TB, pl.NT, pl.n_nt, pl.stages, pl.stage_bytes, pl.nslots, pl.tmem_cols,
-                 pl.nbuf, bytes);
-  rs = ensure_workspace_public(h, bytes);
-  if (rs == TE_ENOMEM && pl.nslots > MIN_SLOTS) rs = ensure_workspace_public(h, single_bytes(h, &pl, o, v, df, true));
-  if (rs != TE_OK) return rs;
+                 pl.nbuf, forms.bytes[form]);
   rs = ensure_triples_public(h, o);
   if (rs != TE_OK) return rs;
   TcBuffers b;

@@ -56,3 +56,22 @@ def test_float64_batch_under_its_old_limit(te):
     a = [cluster(o, 8 * o) for o in (4, 5, 6)]
     e = limited(te, 32538624, lambda h: te.t_energy_batched(a, "fp64", handle=h))
     assert torch.equal(e, te.t_energy_batched(a, "fp64", handle=te.Handle(0)))
+
+
+@pytest.mark.parametrize("prec,o,v,limit", [("ozaki", 2, 3, 202752), ("ozaki", 3, 9, 2297856), ("ozaki", 2, 17, 1775616),
+                                            ("ozaki", 4, 24, 13189120), ("ozaki", 2, 65, 31162368),
+                                            ("bf16x3", 2, 3, 124928), ("bf16x3", 4, 24, 6774784),
+                                            ("bf16x3", 8, 64, 43974656), ("tf32", 5, 81, 58589184),
+                                            ("tf32", 6, 161, 389021696)])
+def test_tensor_core_energy_under_its_old_limit(te, prec, o, v, limit):
+    a = cluster(o, v)
+    e = limited(te, limit, lambda h: te.t_energy_triples(a, precision=prec, handle=h))
+    assert torch.equal(e, te.t_energy_triples(a, precision=prec, handle=te.Handle(0)))
+
+
+@pytest.mark.parametrize("o,v,limit", [(2, 8, 140288), (4, 24, 1830912), (8, 64, 33554432), (4, 72, 29360128),
+                                       (16, 120, 365953024)])
+def test_one_triple_under_its_old_limit(te, o, v, limit):
+    a = cluster(o, v)
+    e = limited(te, limit, lambda h: te.t_energy_triples(a, 1, 2, "ozaki", handle=h))
+    assert torch.equal(e, te.t_energy_triples(a, 1, 2, "ozaki", handle=te.Handle(0)))
