@@ -496,12 +496,15 @@ AdjPlan adj_plan(int64_t o, int64_t v, int num_sms, bool full) {
   z.t2p = al((size_t)nocc * NS * o * v * vp * 2);
   z.noo = al((size_t)NS * o * o * o * vp * 2);
   z.ystride = rup(7 * v * v + 2 * v, 4);
-  // partials of the split jobs of one launch (an upper bound over the launches)
+  // partials of the split jobs of one launch: an upper bound over the launches, or
+  // in the lean form (one slab and three ooov blocks per launch) about that, less
+  // what the Y parts take; vt_finish fits its split counts to it
   const int64_t ntv = vt_ntile(v, false), nto = vt_ntile(o, false), rows_z = (v + 127) / 128;
-  const int64_t pair_blk = 6 * z.B * vt_seg_blocks((int)v, (int)v, VT_SPLIT_CHUNKS);
-  const int64_t d_ooov = vt_split_doubles(rows_z * ((o + nto - 1) / nto), pair_blk, v * o, num_sms) + 8;
-  const int64_t d_t2 = vt_split_doubles(rows_z * ((v + ntv - 1) / ntv), pair_blk, v * v, num_sms) + 8;
-  z.part_cap = 6 * (d_t2 + d_ooov) + 1024;
+  const int64_t pair_blk = (full ? 6 * z.B : 3) * vt_seg_blocks((int)v, (int)v, VT_SPLIT_CHUNKS);
+  const int64_t d_ooov = vt_split_doubles(rows_z * ((o + nto - 1) / nto), pair_blk, v * o, num_sms);
+  const int64_t d_t2 = vt_split_doubles(rows_z * ((v + ntv - 1) / ntv), pair_blk, v * v, num_sms);
+  if (full) z.part_cap = 6 * (d_t2 + d_ooov + 16) + 1024;
+  else z.part_cap = std::max<int64_t>(64, 3 * (d_t2 + d_ooov) + 1024 - z.ystride);
   z.bytes = tc_slices_bytes((int)o, (int)v, z.ns) + 1024 + 2 * al((size_t)o * v * o * v * 8) /* ovs, dOVS */ +
             z.B * (al(z.region) + al((size_t)v3 * 8)) + 2 * al((size_t)z.B * adjoint_grid(num_sms) * 8) +
             al((size_t)std::max<int64_t>(1, nt) * 8) + al(256) + al((size_t)z.B * z.ystride * 8) + z.ovt + z.t2t + z.t2p + z.noo +
@@ -509,11 +512,13 @@ AdjPlan adj_plan(int64_t o, int64_t v, int num_sms, bool full) {
   return z;
 }
 
-// All transposes at hand where they cost at most ADJ_FULL_BYTES more than the
-// lean form, and the handle's limit allows.
+// All transposes at hand where they (and six layouts for three) take at most
+// ADJ_FULL_BYTES more, and the handle's limit allows: per triple of nocc=32
+// nvir=320 7.6 ms against 9.7 in the lean form (13.3 before there were two).
 AdjPlan adj_choose(const Handle* h, int64_t o, int64_t v) {
   const AdjPlan lean = adj_plan(o, v, h->num_sms, false), full = adj_plan(o, v, h->num_sms, true);
-  if (full.bytes > lean.bytes + (size_t)ADJ_FULL_BYTES || (h->ws_limit && full.bytes > h->ws_limit)) return lean;
+  const int64_t more = (int64_t)(full.bytes - lean.bytes) - 8 * (full.part_cap - lean.part_cap);
+  if (more > ADJ_FULL_BYTES || (h->ws_limit && full.bytes > h->ws_limit)) return lean;
   return full;
 }
 

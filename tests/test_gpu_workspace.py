@@ -75,3 +75,25 @@ def test_one_triple_under_its_old_limit(te, o, v, limit):
     a = cluster(o, v)
     e = limited(te, limit, lambda h: te.t_energy_triples(a, 1, 2, "ozaki", handle=h))
     assert torch.equal(e, te.t_energy_triples(a, 1, 2, "ozaki", handle=te.Handle(0)))
+
+
+@pytest.mark.parametrize("o,v,limit", [(1, 1, 163840), (2, 8, 244736), (4, 24, 2412544), (8, 40, 15384576), (2, 65, 31358976),
+                                       (3, 80, 60227584), (3, 97, 119144448), (16, 120, 540016640), (3, 201, 914358272),
+                                       (4, 320, 3514826752)])
+def test_exact_slice_gradient_under_its_old_limit(te, o, v, limit):
+    """Less workspace sums the same slice products in other blocks (1e-8 of the
+    largest entry)."""
+    a = cluster(o, v)
+    _, g = limited(te, limit, lambda h: te.t_energy_vjp(a, precision="ozaki", handle=h))
+    _, ref = te.t_energy_vjp(a, precision="ozaki", handle=te.Handle(0))
+    for n in NAMES:
+        assert float((g[n] - ref[n]).abs().max()) <= 1e-8 * float(ref[n].abs().max()), n
+
+
+@pytest.mark.parametrize("o,v,limit", [(1, 1, 43008), (2, 3, 80896)])
+def test_exact_slice_projected_energy_under_its_old_limit(te, o, v, limit):
+    a = cluster(o, v)
+    cf = np.random.default_rng(v).standard_normal((o, o))
+    _, e = limited(te, limit, lambda h: te.t_energy_frag(a, cf, "ozaki", handle=h, shares=True))
+    _, ref = te.t_energy_frag(a, cf, "ozaki", handle=te.Handle(0), shares=True)
+    assert torch.equal(e, ref)
