@@ -763,14 +763,26 @@ te_status te_reserve(te_handle hh, const te_cluster* c, te_precision p, int what
     return fail(TE_EINVAL, "what must be a non-empty combination of TE_RESERVE_ENERGY, _VJP, _FRAG");
   if (p < TE_FP64 || p > TE_OZAKI) return fail(TE_EINVAL, "unknown precision %d", (int)p);
   DeviceGuard g(h->device);
-  size_t need = 0;
-  if (what & TE_RESERVE_ENERGY) {
-    te_status st = te_workspace_bytes(hh, c, p, &need);
-    if (st != TE_OK) return st;
-  }
-  if (what & TE_RESERVE_VJP)
-    need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(c->nocc, c->nvir) : vjp_tc_bytes(h, c->nocc, c->nvir));
-  if (what & TE_RESERVE_FRAG) need = std::max(need, frag_bytes(h, c->nocc, c->nvir, p));
+  // the form that a call of size (o, v) would choose
+  auto need_of = [&](int64_t o, int64_t v) {
+    size_t need = 0;
+    te_cluster x{};
+    x.nocc = o;
+    x.nvir = v;
+    if (what & TE_RESERVE_ENERGY) te_workspace_bytes(hh, &x, p, &need);
+    if (what & TE_RESERVE_VJP) need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(o, v) : vjp_tc_bytes(h, o, v));
+    if (what & TE_RESERVE_FRAG) need = std::max(need, frag_bytes(h, o, v, p));
+    return need;
+  };
+  size_t need = need_of(c->nocc, c->nvir);
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
+    return fail(TE_ECUDA, "memory query: %s", cudaGetErrorString(cudaGetLastError()));
+  // A smaller cluster can need more: another N tile, more triples per launch, all
+  // transposes of a gradient at hand.  (A size beyond the device fails as it is.)
+  if (need <= total_b)
+    for (int64_t o = 1; o <= c->nocc; ++o)
+      for (int64_t v = 1; v <= c->nvir; ++v) need = std::max(need, need_of(o, v));
   te_status st = ensure_workspace(h, need);
   if (st != TE_OK) return st;
   return ensure_triples(h, (int)c->nocc);

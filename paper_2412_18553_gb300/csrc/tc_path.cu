@@ -725,6 +725,7 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
       bestTB = TB;
     }
   }
+  const int defTB = bestTB;
   if (!force_tb) {
     auto it = h->tuned.find(std::make_tuple(o, v, mode));
     if (it != h->tuned.end()) {
@@ -738,7 +739,7 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   pl.n_my = (v + pl.TB - 1) / pl.TB;
   pl.n_mp = ((v + pl.TA - 1) / pl.TA * pl.n_my + 1) / 2;
   const int ntmax = std::min(256, (512 / (nacc * nbuf_max)) / 32 * 32);
-  pl.n_nt = (v + ntmax - 1) / ntmax;
+  const int def_nt = pl.n_nt = (v + ntmax - 1) / ntmax;
   // a tuned split: any count whose N tile fits three accumulators in TMEM (N <= 160)
   if (force_nnt > 0 && round_up((v + force_nnt - 1) / force_nnt, 32) <= (oz ? 160 : 256)) pl.n_nt = force_nnt;
   pl.NT = round_up((v + pl.n_nt - 1) / pl.n_nt, 32);  // cta_group::2: N in steps of 32
@@ -746,7 +747,8 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   // G's low words stay FP32 in tiles of at most 80 columns (two accumulator sets
   // up to 64, one set and three chunks per epilogue warp above), also where the
   // step of 32 pads the tile to 96; wider tiles round them to BF16.
-  pl.fmt = !oz ? G_F32 : ((v + pl.n_nt - 1) / pl.n_nt <= 80 ? G_PAIR : G_MIXED);
+  auto format = [&](int n_nt) { return !oz ? G_F32 : ((v + n_nt - 1) / n_nt <= 80 ? G_PAIR : G_MIXED); };
+  pl.fmt = format(pl.n_nt);
   pl.cbw = oz ? 64 : 128;
   pl.kw_elems = pl.cbw / pl.es;
   pl.kw_chunks = (pl.vp + pl.kw_elems - 1) / pl.kw_elems;
@@ -764,22 +766,26 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   while (cols < (uint32_t)(nacc * pl.nbuf * pl.NT)) cols <<= 1;
   pl.tmem_cols = cols;
   pl.ldz = round_up(v, 4);
-  const int64_t tiles = 3LL * pl.n_mp * pl.n_nt;  // pair tiles per triple
+  // pair tiles and G bytes per triple in the default shape; a tuned one gets the G
+  // pool that this makes, so that the workspace does not depend on the tuning
+  const int64_t def_m = (int64_t)((v + 128 / defTB - 1) / (128 / defTB)) * ((v + defTB - 1) / defTB);
+  const int64_t tiles = 3LL * ((def_m + 1) / 2) * def_nt;
+  const int64_t def_slot = g_slot_floats(v, format(def_nt)) * 4, per_slot = g_slot_floats(v, pl.fmt) * 4;
   // About 40 tiles per pair of CTAs and launch: a launch's fixed part (its
   // first loads, the last tile's epilogue, a last wave) is some 15 us, which at
   // nvir = 120 with four triples per launch was a sixth of the contraction
   // (nocc=16 nvir=120 energy: 33.9 ms with 4 triples per launch, 30.5 with 9,
   // 29.1 with 17).
   int64_t want = (20LL * std::max(1, h->num_sms) + tiles - 1) / tiles;
-  const int64_t per_slot = g_slot_floats(v, pl.fmt) * 4;
-  const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(6LL << 30) / per_slot);
+  const int64_t mem_cap = std::max<int64_t>(1, (int64_t)(6LL << 30) / def_slot);
   want = std::max<int64_t>(want, MIN_SLOTS);
-  want = std::min<int64_t>({want, mem_cap, 1024, std::max<int64_t>(1, ntri)});
-  pl.nslots = (int)std::max<int64_t>(1, want);
+  want = std::max<int64_t>(1, std::min<int64_t>({want, mem_cap, 1024, ntri}));
+  auto fit = [&](int64_t slots) { return (int)std::max<int64_t>(1, std::min<int64_t>(slots, slots * def_slot / per_slot)); };
+  pl.nslots = fit(want);
   pl.par_slots = (int)std::max<int64_t>(pl.nslots, std::min<int64_t>(TC_PAR_SLOTS, ntri));
   // at the least, a tile for every pair of CTAs
   const int64_t fill = (std::max(1, h->num_sms) / 2 + tiles - 1) / tiles;
-  pl.min_slots = (int)std::max<int64_t>(1, std::min<int64_t>({pl.nslots, std::max(MIN_SLOTS, fill), MIN_POOL / per_slot}));
+  pl.min_slots = fit(std::max<int64_t>(1, std::min<int64_t>({want, std::max(MIN_SLOTS, fill), MIN_POOL / def_slot})));
   return pl;
 }
 

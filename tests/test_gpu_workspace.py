@@ -97,3 +97,57 @@ def test_exact_slice_projected_energy_under_its_old_limit(te, o, v, limit):
     _, e = limited(te, limit, lambda h: te.t_energy_frag(a, cf, "ozaki", handle=h, shares=True))
     _, ref = te.t_energy_frag(a, cf, "ozaki", handle=te.Handle(0), shares=True)
     assert torch.equal(e, ref)
+
+
+def held(te, h):
+    """Device memory in use: the handle's workspace is the only thing that moves it."""
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+@pytest.mark.parametrize("what,prec,large,small", [
+    ("energy", "ozaki", (16, 161), (16, 160)), ("energy", "ozaki", (5, 161), (4, 160)),
+    ("energy", "bf16x3", (16, 257), (16, 256)), ("energy", "fp64", (10, 129), (10, 128)),
+    ("vjp", "ozaki", (33, 320), (32, 320)), ("vjp", "ozaki", (18, 400), (17, 400)), ("vjp", "ozaki", (4, 201), (4, 200)),
+    ("frag", "ozaki", (6, 97), (6, 96))])
+def test_reserve_covers_smaller_sizes(te, what, prec, large, small):
+    """Sizes across which the larger cluster needs less."""
+    h = te.Handle(0)
+    kinds = {k: k == what for k in ("energy", "vjp", "frag")}
+    h.reserve(*large, prec, **kinds)
+    before = held(te, h)
+    h.reserve(*small, prec, **kinds)
+    assert held(te, h) == before
+
+
+@pytest.mark.parametrize("prec", ["fp64", "ozaki"])
+def test_smaller_energy_is_capturable_after_reserve(te, prec):
+    h = te.Handle(0)
+    h.reserve(4, 161, prec)
+    before = held(te, h)
+    a = cluster(4, 160)
+    grown = held(te, h) - before  # the inputs
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        out = te.t_energy(a, prec, handle=h, stream=s)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert float(out) == float(te.t_energy(a, prec, handle=te.Handle(0)))
+    h.sync()
+    assert grown >= 0
+
+
+def test_smaller_gradient_allocates_nothing_after_reserve(te):
+    h = te.Handle(0)
+    h.reserve(4, 201, "ozaki", energy=False, vjp=True)
+    a = cluster(4, 200)
+    buf = torch.empty(a["ovvv"].numel() * 2, dtype=torch.float64, device="cuda")  # cached: room for the gradients
+    del buf
+    before = held(te, h)
+    te.t_energy_vjp(a, precision="ozaki", handle=h)
+    h.sync()
+    assert held(te, h) == before
