@@ -40,7 +40,11 @@
  *   records an error word and returns; te_sync() reports it as TE_ETIMEOUT.
  *   The error word is the handle's: it stays set until te_sync reads it.
  * - Results are deterministic: fixed-order reductions, no floating-point
- *   atomics; repeated calls give bitwise identical outputs.
+ *   atomics; repeated calls give bitwise identical outputs.  Calls run in a
+ *   smaller form where their usual workspace passes the handle's limit or what
+ *   the device has room for (a size it refused is not tried again before the
+ *   next te_reserve or te_set_workspace_limit); the form changes a gradient's
+ *   last bits in the exact-slice modes, and no other result.
  * - A handle owns its workspace (operand copies for the mixed modes, partial
  *   results); one handle must not be used from two host threads at once, and
  *   calls made on one handle with different streams must be ordered by the
@@ -318,9 +322,10 @@ te_status te_workspace_bytes(te_handle h, const te_cluster* c, te_precision p,
  * nvir are read; the array pointers may be NULL.  what: any non-empty
  * combination of TE_RESERVE_ENERGY (t_energy, t_energy_triples,
  * t_energy_batched), TE_RESERVE_VJP (t_energy_vjp) and TE_RESERVE_FRAG
- * (t_energy_frag).  TE_ENOMEM if the device cannot hold it (the handle keeps
- * what it had); TE_EUNSUPPORTED inside a stream capture.  Synchronises the
- * device when a smaller workspace is replaced. */
+ * (t_energy_frag).  Where the device cannot hold it, what the smallest form of
+ * those calls needs; TE_ENOMEM if not even that (the handle keeps what it had);
+ * TE_EUNSUPPORTED inside a stream capture.  Synchronises the device when a
+ * smaller workspace is replaced. */
 #define TE_RESERVE_ENERGY 1
 #define TE_RESERVE_VJP 2
 #define TE_RESERVE_FRAG 4

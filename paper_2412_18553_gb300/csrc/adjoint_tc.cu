@@ -35,7 +35,6 @@
 
 namespace te {
 
-te_status ensure_workspace_public(Handle* h, size_t bytes);
 te_status ensure_triples_public(Handle* h, int nocc);
 
 namespace {
@@ -512,19 +511,25 @@ AdjPlan adj_plan(int64_t o, int64_t v, int num_sms, bool full) {
   return z;
 }
 
-// All transposes at hand where they (and six layouts for three) take at most
-// ADJ_FULL_BYTES more, and the handle's limit allows: per triple of nocc=32
+// The forms of a gradient, best first.  All transposes at hand where they (and six
+// layouts for three) take at most ADJ_FULL_BYTES more: per triple of nocc=32
 // nvir=320 7.6 ms against 9.7 in the lean form (13.3 before there were two).
-AdjPlan adj_choose(const Handle* h, int64_t o, int64_t v) {
+std::vector<AdjPlan> adj_forms(const Handle* h, int64_t o, int64_t v) {
   const AdjPlan lean = adj_plan(o, v, h->num_sms, false), full = adj_plan(o, v, h->num_sms, true);
   const int64_t more = (int64_t)(full.bytes - lean.bytes) - 8 * (full.part_cap - lean.part_cap);
-  if (more > ADJ_FULL_BYTES || (h->ws_limit && full.bytes > h->ws_limit)) return lean;
-  return full;
+  if (more > ADJ_FULL_BYTES) return {lean};
+  return {full, lean};
+}
+
+std::vector<size_t> plan_bytes(const std::vector<AdjPlan>& f) {
+  std::vector<size_t> b;
+  for (const AdjPlan& z : f) b.push_back(z.bytes);
+  return b;
 }
 
 }  // namespace
 
-size_t vjp_tc_bytes(const Handle* h, int64_t o, int64_t v) { return adj_choose(h, o, v).bytes; }
+std::vector<size_t> vjp_tc_bytes(const Handle* h, int64_t o, int64_t v) { return plan_bytes(adj_forms(h, o, v)); }
 
 // The contractions of one triple (g = 0, 1, 2 the G blocks with occupied
 // indices (p, q, r) = (i, j, k), (j, k, i), (k, i, j); dG_g the views of dW~):
@@ -546,13 +551,11 @@ te_status run_vjp_tc(Handle* h, const te_cluster* c, int64_t t_begin, int64_t t_
                      double* e_out, te_cluster_grad* g, cudaStream_t s, int64_t cluster) {
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int64_t v2 = (int64_t)v * v, v3 = v2 * v, nt = num_unique_triples(o);
-  AdjPlan Z = adj_choose(h, o, v);
-  te_status st = ensure_workspace_public(h, Z.bytes);
-  if (st == TE_ENOMEM && Z.full) {
-    Z = adj_plan(o, v, h->num_sms, false);
-    st = ensure_workspace_public(h, Z.bytes);
-  }
+  const std::vector<AdjPlan> forms = adj_forms(h, o, v);
+  size_t form = 0;
+  te_status st = acquire_workspace(h, plan_bytes(forms), &form);
   if (st != TE_OK) return st;
+  const AdjPlan Z = forms[form];
   st = ensure_triples_public(h, o);
   if (st != TE_OK) return st;
   const int ns = Z.ns;

@@ -82,6 +82,7 @@ static te_status ensure_workspace(Handle* h, size_t bytes) {
                 h->ws_limit);
   if (h->capturing) return fail(TE_EUNSUPPORTED, "workspace growth inside a graph capture");
   drop_graphs(h);  // captured graphs hold the old workspace's addresses
+  const size_t held = h->ws_bytes;
   if (h->ws) {
     cudaDeviceSynchronize();  // no launch may still read the old workspace
     cudaFree(h->ws);
@@ -93,18 +94,25 @@ static te_status ensure_workspace(Handle* h, size_t bytes) {
   size_t want = bytes + std::min(bytes / 8, (size_t)1 << 30);
   if (h->ws_limit) want = std::min(want, h->ws_limit);
   if (h->log) std::fprintf(stderr, "[tenergy] workspace: %zu bytes (needed %zu)\n", want, bytes);
-  if (cudaMalloc(&h->ws, want) != cudaSuccess) {
+  cudaError_t e = cudaMalloc(&h->ws, want);
+  if (e != cudaSuccess && want > bytes) {
     cudaGetLastError();
+    e = cudaMalloc(&h->ws, want = bytes);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    if (e == cudaErrorMemoryAllocation && (!h->ws_refused || bytes < h->ws_refused)) h->ws_refused = bytes;
     h->ws = nullptr;
-    if (cudaMalloc(&h->ws, bytes) != cudaSuccess) {
+    if (held && cudaMalloc(&h->ws, held) == cudaSuccess) {
+      h->ws_bytes = held;  // what the handle had
+    } else {
       cudaGetLastError();
       h->ws = nullptr;
-      return fail(TE_ENOMEM, "workspace allocation of %zu bytes failed", bytes);
     }
-    h->ws_bytes = bytes;
-    return TE_OK;
+    return fail(TE_ENOMEM, "workspace allocation of %zu bytes failed", bytes);
   }
   h->ws_bytes = want;
+  if (want >= h->ws_refused) h->ws_refused = 0;
   return TE_OK;
 }
 
@@ -114,11 +122,22 @@ te_status acquire_workspace(Handle* h, const std::vector<size_t>& bytes, size_t*
     *form = k;
     const bool last = k + 1 == bytes.size();
     if (bytes[k] <= h->ws_bytes) return TE_OK;
-    if (!last && (h->capturing || (h->ws_limit && bytes[k] > h->ws_limit))) continue;
+    if (!last && (h->capturing || (h->ws_limit && bytes[k] > h->ws_limit) || (h->ws_refused && bytes[k] >= h->ws_refused)))
+      continue;
     st = ensure_workspace(h, bytes[k]);
     if (st != TE_ENOMEM) return st;
   }
   return st;
+}
+
+// Form by form the largest of several calls (the last form of one that has fewer).
+static std::vector<size_t> largest_forms(const std::vector<std::vector<size_t>>& f) {
+  size_t levels = 1;
+  for (const auto& b : f) levels = std::max(levels, b.size());
+  std::vector<size_t> need(levels, 0);
+  for (size_t k = 0; k < levels; ++k)
+    for (const auto& b : f) need[k] = std::max(need[k], b[std::min(k, b.size() - 1)]);
+  return need;
 }
 
 // The canonical order is prefix-closed (the triples of nocc = n are the first
@@ -551,14 +570,9 @@ te_status t_energy_batched(te_handle hh, const te_cluster* cs, int64_t n, te_pre
   std::vector<size_t> need;
   if (p == TE_FP64) {
     std::vector<std::vector<size_t>> f;
-    size_t levels = 1;
-    for (int64_t x = 0; x < n; ++x) {
+    for (int64_t x = 0; x < n; ++x)
       f.push_back(fp64_forms(h, cs[x].nocc, cs[x].nvir, num_unique_triples(cs[x].nocc)).bytes);
-      levels = std::max(levels, f.back().size());
-    }
-    need.assign(levels, 0);
-    for (size_t k = 0; k < levels; ++k)
-      for (const auto& b : f) need[k] = std::max(need[k], b[std::min(k, b.size() - 1)]);
+    need = largest_forms(f);
   } else {
     need.assign(1, 0);
     st = tc_batched_bytes(h, cs, n, p, &need[0]);
@@ -674,14 +688,15 @@ te_status t_energy_vjp_batched(te_handle hh, const te_cluster* cs, int64_t n, te
     }
   }
   // the workspace of the largest member, once
-  size_t need = 0;
+  std::vector<std::vector<size_t>> forms;
   int64_t maxo = 1;
   for (int64_t x = 0; x < n; ++x) {
-    need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(cs[x].nocc, cs[x].nvir)
-                                       : vjp_tc_bytes(h, cs[x].nocc, cs[x].nvir));
+    forms.push_back(p == TE_FP64 ? std::vector<size_t>{vjp_fp64_bytes(cs[x].nocc, cs[x].nvir)}
+                                 : vjp_tc_bytes(h, cs[x].nocc, cs[x].nvir));
     maxo = std::max<int64_t>(maxo, cs[x].nocc);
   }
-  te_status st = ensure_workspace(h, need);
+  size_t form = 0;
+  te_status st = acquire_workspace(h, largest_forms(forms), &form);
   if (st == TE_OK) st = ensure_triples(h, (int)maxo);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(ss);
   for (int64_t x = 0; x < n && st == TE_OK; ++x) {
@@ -763,28 +778,40 @@ te_status te_reserve(te_handle hh, const te_cluster* c, te_precision p, int what
     return fail(TE_EINVAL, "what must be a non-empty combination of TE_RESERVE_ENERGY, _VJP, _FRAG");
   if (p < TE_FP64 || p > TE_OZAKI) return fail(TE_EINVAL, "unknown precision %d", (int)p);
   DeviceGuard g(h->device);
-  // the form that a call of size (o, v) would choose
+  h->ws_refused = 0;
+  // the forms that a call of size (o, v) has under the limit: best and last
   auto need_of = [&](int64_t o, int64_t v) {
-    size_t need = 0;
-    te_cluster x{};
-    x.nocc = o;
-    x.nvir = v;
-    if (what & TE_RESERVE_ENERGY) te_workspace_bytes(hh, &x, p, &need);
-    if (what & TE_RESERVE_VJP) need = std::max(need, p == TE_FP64 ? vjp_fp64_bytes(o, v) : vjp_tc_bytes(h, o, v));
-    if (what & TE_RESERVE_FRAG) need = std::max(need, frag_bytes(h, o, v, p));
+    const int64_t nt = num_unique_triples(o);
+    std::pair<size_t, size_t> need{0, 0};
+    auto add = [&](const std::vector<size_t>& f) {
+      size_t k = 0;
+      while (k + 1 < f.size() && h->ws_limit && f[k] > h->ws_limit) ++k;
+      need.first = std::max(need.first, f[k]);
+      need.second = std::max(need.second, f.back());
+    };
+    if (what & TE_RESERVE_ENERGY) add(p == TE_FP64 ? fp64_forms(h, o, v, nt).bytes : tc_energy_bytes(h, o, v, p));
+    if (what & TE_RESERVE_VJP) add(p == TE_FP64 ? std::vector<size_t>{vjp_fp64_bytes(o, v)} : vjp_tc_bytes(h, o, v));
+    if (what & TE_RESERVE_FRAG) add(frag_bytes(h, o, v, p));
     return need;
   };
-  size_t need = need_of(c->nocc, c->nvir);
+  auto need = need_of(c->nocc, c->nvir);
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
     return fail(TE_ECUDA, "memory query: %s", cudaGetErrorString(cudaGetLastError()));
   // A smaller cluster can need more: another N tile, more triples per launch, all
   // transposes of a gradient at hand.  (A size beyond the device fails as it is.)
-  if (need <= total_b)
+  if (need.second <= total_b)
     for (int64_t o = 1; o <= c->nocc; ++o)
-      for (int64_t v = 1; v <= c->nvir; ++v) need = std::max(need, need_of(o, v));
-  te_status st = ensure_workspace(h, need);
+      for (int64_t v = 1; v <= c->nvir; ++v) {
+        const auto x = need_of(o, v);
+        need.first = std::max(need.first, x.first);
+        need.second = std::max(need.second, x.second);
+      }
+  size_t form = 0;
+  const te_status st = acquire_workspace(h, {need.first, need.second}, &form);
   if (st != TE_OK) return st;
+  // calls of these sizes stay within what there was room for
+  if (h->ws_refused) h->ws_refused = h->ws_bytes + 1;
   return ensure_triples(h, (int)c->nocc);
 }
 
@@ -844,6 +871,7 @@ te_status te_set_workspace_limit(te_handle hh, size_t bytes) {
   if (bytes && h->ws_bytes > bytes)
     return fail(TE_EINVAL, "the handle already holds %zu bytes of workspace, above %zu", h->ws_bytes, bytes);
   h->ws_limit = bytes;
+  h->ws_refused = 0;
   return TE_OK;
 }
 

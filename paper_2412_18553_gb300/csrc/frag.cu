@@ -15,7 +15,6 @@
 
 namespace te {
 
-te_status ensure_workspace_public(Handle* h, size_t bytes);
 te_status ensure_triples_public(Handle* h, int nocc);
 
 // ---------------------------------------------------------------------------
@@ -258,12 +257,6 @@ size_t frag_oz_layout(const Handle* h, int64_t o, int64_t v, int B, char* base, 
   return c.off + 1024;
 }
 
-int frag_oz_batch(const Handle* h, int64_t o, int64_t v) {
-  FragOz W;
-  const int B = frag_batch(o, v);
-  return h->ws_limit && frag_oz_layout(h, o, v, B, nullptr, &W) > h->ws_limit ? 1 : B;
-}
-
 struct ProjArgs {
   AdjArgs a;              // inputs
   SliceExps x0, xa, xb;   // scales of the input slices, of (ovvvC, t2C, ., ooovC) and of t2C2's t2L
@@ -489,27 +482,25 @@ te_status run_frag_oz(Handle* h, const te_cluster* c, const double* cf, const Fr
 
 }  // namespace
 
-size_t frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p) {
+// The usual batch, then triple by triple where memory is short.
+std::vector<size_t> frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p) {
   if (p == TE_FP64) {
     FragWork W;
-    return frag_layout(o, v, nullptr, &W);
+    return {frag_layout(o, v, nullptr, &W)};
   }
   FragOz W;
-  return frag_oz_layout(h, o, v, frag_oz_batch(h, o, v), nullptr, &W);
+  return {frag_oz_layout(h, o, v, frag_batch(o, v), nullptr, &W), frag_oz_layout(h, o, v, 1, nullptr, &W)};
 }
 
 te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precision p, double* e_out,
                    double* e_triples, cudaStream_t s) {
   const int o = (int)c->nocc, v = (int)c->nvir;
   const int64_t nt = num_unique_triples(o);
-  FragOz Z;
-  int B = p == TE_FP64 ? 1 : frag_oz_batch(h, o, v);
-  te_status st = ensure_workspace_public(h, frag_bytes(h, o, v, p));
-  if (st == TE_ENOMEM && B > 1) {
-    B = 1;
-    st = ensure_workspace_public(h, frag_oz_layout(h, o, v, B, nullptr, &Z));
-  }
+  size_t form = 0;
+  te_status st = acquire_workspace(h, frag_bytes(h, o, v, p), &form);
   if (st != TE_OK) return st;
+  FragOz Z;
+  const int B = form == 0 ? frag_batch(o, v) : 1;
   st = ensure_triples_public(h, o);
   if (st != TE_OK) return st;
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 1023) & ~uintptr_t(1023));

@@ -1473,6 +1473,10 @@ te_status tc_workspace_bytes(Handle* h, const te_cluster* c, te_precision p, siz
   return TE_OK;
 }
 
+std::vector<size_t> tc_energy_bytes(const Handle* h, int o, int v, te_precision p) {
+  return single_forms(h, make_plan(h, o, v, tc_mode_of(p, o, v, h->ozaki_bits), num_unique_triples(o)), o, v, nullptr).bytes;
+}
+
 te_status ensure_workspace_public(Handle* h, size_t bytes);
 te_status ensure_triples_public(Handle* h, int nocc);
 

@@ -8,6 +8,8 @@ te_status run_tc(Handle* h, const te_cluster* c, te_precision p, int64_t t_begin
                  double* e_tri_out, double* e_total_out, cudaStream_t s, const te_df* df = nullptr);
 te_status tc_workspace_bytes(Handle* h, const te_cluster* c, te_precision p, size_t* bytes,
                              const te_df* df = nullptr);
+// the same for an energy without df: its forms, best first
+std::vector<size_t> tc_energy_bytes(const Handle* h, int o, int v, te_precision p);
 // n clusters in rounds of multi-cluster launches (every member's operands
 // prepared first); e_out[x] = E(T) of cluster x.  tc_batched_bytes: the
 // workspace it needs (the tuned tile shapes must be known already).

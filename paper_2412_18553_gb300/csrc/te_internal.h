@@ -77,7 +77,8 @@ struct Handle {
   // workspace (grows, never shrinks until destroy)
   void* ws = nullptr;
   size_t ws_bytes = 0;
-  size_t ws_limit = 0;  // most workspace bytes the handle may hold (0: no limit)
+  size_t ws_limit = 0;    // most workspace bytes the handle may hold (0: no limit)
+  size_t ws_refused = 0;  // a size that the device could not give (0: none yet)
   bool log = false;     // TE_LOG=1: tile plans and autotune decisions on stderr
   // triple table cache
   Triple* d_triples = nullptr;
@@ -112,7 +113,10 @@ struct Handle {
 
 // The workspace of a call that can run in several forms, `bytes` of them, best
 // first: the first form that the handle holds already or can have under its limit
-// and on the device.  Inside the library's graph capture nothing is allocated.
+// and on the device.  What the device once refused is not asked for again while a
+// smaller form does (te_reserve and te_set_workspace_limit start afresh), so that
+// the form of a call does not change with the free memory of the moment.  Inside
+// the library's graph capture nothing is allocated.
 te_status acquire_workspace(Handle* h, const std::vector<size_t>& bytes, size_t* form);
 
 void drop_graphs(Handle* h);
@@ -155,12 +159,13 @@ te_status run_vjp_fp64(Handle* h, const te_cluster* c, int64_t t_begin, int64_t 
                        double* e_out, te_cluster_grad* g, cudaStream_t s);
 // fragment-projected E(T) (vjp.cu): cf device [nocc][nocc]; precision TE_FP64 or
 // exact slices; per-triple shares to e_triples (nullable), total to e_out (nullable)
-size_t frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p);
+std::vector<size_t> frag_bytes(const Handle* h, int64_t o, int64_t v, te_precision p);
 te_status run_frag(Handle* h, const te_cluster* c, const double* cf, te_precision p, double* e_out,
                    double* e_triples, cudaStream_t s);
-// workspace bytes of the two adjoints (vjp.cu, adjoint_tc.cu)
+// workspace bytes of the two adjoints (vjp.cu, adjoint_tc.cu); of their forms, best
+// first, where there are several
 size_t vjp_fp64_bytes(int64_t o, int64_t v);
-size_t vjp_tc_bytes(const Handle* h, int64_t o, int64_t v);
+std::vector<size_t> vjp_tc_bytes(const Handle* h, int64_t o, int64_t v);
 // threads of the adjoint epilogues stride over the orbits on this many blocks
 int adjoint_grid(int num_sms);
 // dovov[P1,x,P2,y] = (dOVS[P1,x,P2,y] + dOVS[P2,y,P1,x]) / 2

@@ -151,3 +151,53 @@ def test_smaller_gradient_allocates_nothing_after_reserve(te):
     te.t_energy_vjp(a, precision="ozaki", handle=h)
     h.sync()
     assert held(te, h) == before
+
+
+@pytest.fixture
+def little_memory(te):
+    """Leaves `room` bytes of the device free, beside what torch has cached."""
+    kept = []
+
+    def fill(room):
+        torch.cuda.synchronize()
+        kept.append(torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda"))
+
+    yield fill
+    kept.clear()
+    torch.cuda.empty_cache()
+
+
+def test_gradients_and_reservation_where_only_the_lean_form_fits(te, little_memory):
+    """nocc=8 nvir=64: 49 MB do (the limit above); what the usual form takes is
+    measured here."""
+    o, v = 8, 64
+    a = cluster(o, v)
+    h = te.Handle(0)
+    before = held(te, h)
+    h.reserve(o, v, "ozaki", energy=False, vjp=True)
+    usual = held(te, h) - before
+    h.close()
+    room = 64 << 20
+    assert usual > 2 * room
+    ref, g = te.t_energy_vjp(a, precision="ozaki", handle=te.Handle(0))  # and torch's cache for the gradients
+    g = {n: x.cpu() for n, x in g.items()}
+    h1, h2 = te.Handle(0), te.Handle(0)
+    e, grads = te.t_energy_vjp_batched([a], precision="fp64", handle=te.Handle(0))
+    del e, grads
+    little_memory(room)
+    e, grads = te.t_energy_vjp_batched([a], precision="ozaki", handle=h1)
+    h1.sync()
+    assert abs(float(e[0]) - float(ref)) <= 1e-12 * abs(float(ref))
+    for n in NAMES:
+        assert float((grads[0][n].cpu() - g[n]).abs().max()) <= 1e-8 * float(g[n].abs().max())
+    first = held(te, h1)
+    del e, grads
+    te.t_energy_vjp_batched([a], precision="ozaki", handle=h1)  # the same form, nothing allocated
+    h1.sync()
+    assert held(te, h1) == first
+    h1.close()
+    h2.reserve(o, v, "ozaki", energy=False, vjp=True)
+    first = held(te, h2)
+    te.t_energy_vjp(a, precision="ozaki", handle=h2)
+    h2.sync()
+    assert held(te, h2) == first
