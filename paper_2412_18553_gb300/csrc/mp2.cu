@@ -279,24 +279,30 @@ static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Bytes of workspace one cluster uses while its contractions run (the largest
 // is allocated; the next cluster reuses it).
+static size_t mp2_shared_bytes(int64_t o, int64_t v, int64_t naux, bool oz) {
+  // split-K partial tiles of the densities; before them, of (ia|jb) or (4 x 2 B per
+  // element) the slices of Bov
+  return al256((size_t)std::max<int64_t>(mp2_scratch(o, v), oz ? mp2_pitch(naux) * o * v : 0) * 8);
+}
 static size_t mp2_bytes(int64_t o, int64_t v, int64_t naux, bool oz) {
   const size_t ovov = (size_t)o * v * o * v, t2n = (size_t)o * o * v * v;
-  size_t b = al256(ovov * 8) + 2 * al256(t2n * 8);                       // ovov, t2 (own copy), T~
-  b += al256((size_t)mp2_scratch(o, v) * 8);                             // split-K partial tiles
-  if (oz) b += al256((size_t)mp2_pitch(naux) * o * v * 8) + al256(64);   // slices of Bov (4 x 2 B per element), scale
-  return b;
+  return al256(ovov * 8) + 2 * al256(t2n * 8) + mp2_shared_bytes(o, v, naux, oz) + (oz ? al256(64) : 0);
 }
 
 // Bytes one cluster keeps until its group's eigensolver launch: the gamma
-// blocks (when the caller did not ask for them), the tridiagonal forms and
-// global working copies for orders above kEigSmemN.
+// blocks (when the caller did not ask for them) and global working copies for
+// orders above kEigSmemN.
 static size_t mp2_keep_bytes(int64_t o, int64_t v) {
-  size_t b = al256((size_t)o * o * 8) + al256((size_t)v * v * 8) + al256((size_t)o * 16) + al256((size_t)v * 16);
+  size_t b = al256((size_t)o * o * 8) + al256((size_t)v * v * 8);
   if (o > kEigSmemN) b += al256((size_t)o * o * 8);
   if (v > kEigSmemN) b += al256((size_t)v * v * 8);
   return b;
 }
 
+
+// The tridiagonal forms of one cluster.  A group's live where its contractions had
+// their transient arrays: the eigensolver runs after the last of them.
+static size_t mp2_tri_bytes(int64_t o, int64_t v) { return al256((size_t)o * 16) + al256((size_t)v * 16); }
 
 // Clusters per eigensolver launch: two matrices each, 64 jobs.
 constexpr int64_t kMp2Group = 32;
@@ -337,7 +343,7 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
   if (p == TE_OZAKI && h->cc_major != 10 && h->cc_major != 11)
     return fail(TE_EUNSUPPORTED, "exact-slice contractions need an sm_100-family GPU");
   const bool oz = p == TE_OZAKI;
-  size_t need_tr = 0, need_keep = 0, group_keep = 0;
+  size_t need_tr = 0, need_keep = 0, group_keep = 0, group_tri = 0;
   for (int64_t x = 0; x < n; ++x) {  // every descriptor before any launch
     const te_mp2_cluster& c = cs[x];
     if (c.nocc < 1 || c.nvir < 1 || c.naux < 1)
@@ -349,7 +355,9 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     if (!q.t2 && !q.gamma_oo && !q.gamma_vv && !q.pop_o && !q.pop_v)
       return fail(TE_EINVAL, "cluster %lld: no output requested", (long long)x);
     need_tr = std::max(need_tr, mp2_bytes(c.nocc, c.nvir, c.naux, oz));
-    if (x % kMp2Group == 0) group_keep = 0;
+    if (x % kMp2Group == 0) group_keep = group_tri = 0;
+    group_tri += mp2_tri_bytes(c.nocc, c.nvir);
+    need_tr = std::max(need_tr, group_tri);
     group_keep += mp2_keep_bytes(c.nocc, c.nvir);
     need_keep = std::max(need_keep, group_keep);
   }
@@ -370,13 +378,17 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
   cudaError_t e = cudaSuccess;
   char* const ws0 = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 255) & ~uintptr_t(255));
   char* keep = ws0;                       // kept blocks of the current group
-  char* const transient = ws0 + need_keep;  // one cluster's contractions
+  char* const transient = ws0 + need_keep;  // one cluster's contractions, then
+  char* tri = transient;                    // the group's tridiagonal forms
   for (int64_t x = 0; x < n && e == cudaSuccess; ++x) {
     const te_mp2_cluster& c = cs[x];
     const te_mp2_out& q = outs[x];
     const int64_t o = c.nocc, v = c.nvir, P = c.naux;
     const int64_t ov = o * v, t2n = o * o * v * v;
-    if (x % kMp2Group == 0) keep = ws0;
+    if (x % kMp2Group == 0) {
+      keep = ws0;
+      tri = transient;
+    }
     auto take_from = [](char*& base, size_t bytes) {
       char* r = base;
       base += al256(bytes);
@@ -389,18 +401,18 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
     double* tt = reinterpret_cast<double*>(take((size_t)t2n * 8));
     double* goo = reinterpret_cast<double*>(take_from(keep, (size_t)o * o * 8));
     double* gvv = reinterpret_cast<double*>(take_from(keep, (size_t)v * v * 8));
-    double* eo_tri = reinterpret_cast<double*>(take_from(keep, (size_t)o * 16));
-    double* ev_tri = reinterpret_cast<double*>(take_from(keep, (size_t)v * 16));
+    double* eo_tri = reinterpret_cast<double*>(take_from(tri, (size_t)o * 16));
+    double* ev_tri = reinterpret_cast<double*>(take_from(tri, (size_t)v * 16));
     double* eo_work = o > kEigSmemN ? reinterpret_cast<double*>(take_from(keep, (size_t)o * o * 8)) : nullptr;
     double* ev_work = v > kEigSmemN ? reinterpret_cast<double*>(take_from(keep, (size_t)v * v * 8)) : nullptr;
     const int64_t cap = mp2_scratch(o, v);
-    double* scratch = reinterpret_cast<double*>(take((size_t)cap * 8));
+    double* scratch = reinterpret_cast<double*>(take(mp2_shared_bytes(o, v, P, oz)));
     if (q.t2) t2 = q.t2;
     if (q.gamma_oo) goo = q.gamma_oo;
     if (q.gamma_vv) gvv = q.gamma_vv;
     // input values: finite, max eps_o < min eps_v (reported by te_sync); the
     // same pass finds max |Bov|, the scale of its slices
-    __nv_bfloat16* bs = oz ? reinterpret_cast<__nv_bfloat16*>(take((size_t)mp2_pitch(P) * ov * 8)) : nullptr;
+    __nv_bfloat16* bs = reinterpret_cast<__nv_bfloat16*>(scratch);
     unsigned int* mx = oz ? reinterpret_cast<unsigned int*>(take(64)) : nullptr;
     if (oz) e = cudaMemsetAsync(mx, 0, 4, s);
     if (e == cudaSuccess)

@@ -201,3 +201,24 @@ def test_gradients_and_reservation_where_only_the_lean_form_fits(te, little_memo
     te.t_energy_vjp(a, precision="ozaki", handle=h2)
     h2.sync()
     assert held(te, h2) == first
+
+
+@pytest.mark.parametrize("o,v,naux,prec,limit", [(2, 10, 50, "fp64", 76288), (2, 10, 50, "ozaki", 84736)])
+def test_mp2_under_its_old_limit(te, o, v, naux, prec, limit):
+    c = tegen.mp2_inputs(o, v, naux, 5)
+    out = limited(te, limit, lambda h: te.mp2_bno_batched([c], prec, handle=h))[0]
+    ref = te.mp2_bno_batched([c], prec, handle=te.Handle(0))[0]
+    for n in ref:
+        assert torch.equal(out[n], ref[n]), n
+
+
+def test_mp2_groups_of_many_clusters(te):
+    """More than one group of the eigensolver, sizes that grow and shrink: the
+    tridiagonal forms and the transient arrays of other clusters share memory."""
+    sizes = [(1 + x % 3, 1 + (7 * x) % 23) for x in range(67)] + [(3, 40)]
+    cs = [tegen.mp2_inputs(o, v, 2 * (o + v), x) for x, (o, v) in enumerate(sizes)]
+    out = te.mp2_bno_batched(cs, "fp64", handle=te.Handle(0))
+    for x in (0, 1, 30, 31, 32, 33, 63, 64, 66, 67):
+        one = te.mp2_bno_batched([cs[x]], "fp64", handle=te.Handle(0))[0]
+        for n in one:
+            assert torch.equal(out[x][n], one[n]), (x, n)
