@@ -26,8 +26,8 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <cstring>
-#include <vector>
+#include <memory>
+#include <new>
 
 #include "strided.h"
 #include "te_internal.h"
@@ -373,8 +373,9 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
   } restore{prev, h->device};
   te_status st = ensure_workspace_public(h, need);
   if (st != TE_OK) return st;
-  EigJobs* jobs = new EigJobs;
-  std::memset(jobs, 0, sizeof(*jobs));
+  const std::unique_ptr<EigJobs> owned(new (std::nothrow) EigJobs{});
+  EigJobs* const jobs = owned.get();
+  if (!jobs) return fail(TE_ENOMEM, "eigensolver tables");
   cudaError_t e = cudaSuccess;
   char* const ws0 = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(h->ws) + 255) & ~uintptr_t(255));
   char* keep = ws0;                       // kept blocks of the current group
@@ -429,7 +430,7 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
       const int64_t Pp = mp2_pitch(P);
       if (e == cudaSuccess) e = slice_rows(c.Bov, ov, P, Pp, 4, mx, ex, bs, s, &h->n_launches);
       if (e == cudaSuccess) {
-        const te_status st = vt_product(h, bs, ov * Pp, ov, bs, ov * Pp, ov, P, Pp, 4, ex, ex, ovov, s);
+        st = vt_product(h, bs, ov * Pp, ov, bs, ov * Pp, ov, P, Pp, 4, ex, ex, ovov, s);
         if (st != TE_OK) return st;
       }
     }
@@ -466,7 +467,6 @@ extern "C" te_status t_mp2_bno_batched(te_handle hh, const te_mp2_cluster* cs, c
       }
     }
   }
-  delete jobs;
   if (e != cudaSuccess) return fail(TE_ECUDA, "MP2 step launch: %s", cudaGetErrorString(e));
   return TE_OK;
 }
