@@ -217,8 +217,6 @@ static size_t fp64_carve(Carver& cv, int64_t o, int64_t v, int nslots, int64_t n
   P->t2L = cv.take<double>(o * v * v * o);
   P->nooT = cv.take<double>(o * o * v * o);
   P->ovs = cv.take<double>(o * v * o * v);
-  P->ovs32 = nullptr;
-  P->t1_32 = nullptr;
   *gbuf = cv.take<double>((size_t)nslots * 3 * v * v * v);
   *partials = cv.take<double>((size_t)nslots * nbt);
   *etri = cv.take<double>((size_t)std::max<int64_t>(1, ntri));
@@ -411,6 +409,7 @@ te_status te_create(te_handle* out, int device, const char* autotune_cache_path)
   h->device = device;
   h->num_sms = prop.multiProcessorCount;
   h->smem_optin = prop.sharedMemPerBlockOptin;
+  h->total_mem = prop.totalGlobalMem;
   h->cc_major = prop.major;
   h->cc_minor = prop.minor;
   if (cudaMalloc(&h->d_err, sizeof(unsigned int) * 4) != cudaSuccess ||
@@ -795,12 +794,9 @@ te_status te_reserve(te_handle hh, const te_cluster* c, te_precision p, int what
     return need;
   };
   auto need = need_of(c->nocc, c->nvir);
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
-    return fail(TE_ECUDA, "memory query: %s", cudaGetErrorString(cudaGetLastError()));
   // A smaller cluster can need more: another N tile, more triples per launch, all
   // transposes of a gradient at hand.  (A size beyond the device fails as it is.)
-  if (need.second <= total_b)
+  if (need.second <= h->total_mem)
     for (int64_t o = 1; o <= c->nocc; ++o)
       for (int64_t v = 1; v <= c->nvir; ++v) {
         const auto x = need_of(o, v);

@@ -44,9 +44,9 @@ __device__ __forceinline__ void decode_block_triple(int64_t bt, int& X, int& Y, 
   Z = (int)(rem - (int64_t)y * (y + 1) / 2);
 }
 
-template <typename T, int N>
-__device__ __forceinline__ void position(const T* cube, const T* ovsS, const T* t1S, const int* l,
-                                         T& Wn, T& Vn) {
+template <int N>
+__device__ __forceinline__ void position(const double* cube, const double* ovsS, const double* t1S, const int* l,
+                                         double& Wn, double& Vn) {
   constexpr int TB = ENERGY_TB, TB3 = TB * TB * TB;
   constexpr int s0 = Rot<N>::s0, s1 = Rot<N>::s1, s2 = Rot<N>::s2;
   const int x = l[s0], y = l[s1], z = l[s2];
@@ -55,24 +55,23 @@ __device__ __forceinline__ void position(const T* cube, const T* ovsS, const T* 
      + cube[(1 * 6 + Rot<N>::r1) * TB3 + (y * TB + z) * TB + x]
      + cube[(2 * 6 + Rot<N>::r2) * TB3 + (z * TB + x) * TB + y];
   // Y[x,y,z] = ovs(i,x,j,y) t1(k,z) + ovs(j,y,k,z) t1(i,x) + ovs(i,x,k,z) t1(j,y)
-  const T yv = ovsS[((0 * 3 + s0) * 3 + s1) * TB * TB + x * TB + y] * t1S[(2 * 3 + s2) * TB + z]
+  const double yv = ovsS[((0 * 3 + s0) * 3 + s1) * TB * TB + x * TB + y] * t1S[(2 * 3 + s2) * TB + z]
              + ovsS[((1 * 3 + s1) * 3 + s2) * TB * TB + y * TB + z] * t1S[(0 * 3 + s0) * TB + x]
              + ovsS[((2 * 3 + s0) * 3 + s2) * TB * TB + x * TB + z] * t1S[(1 * 3 + s1) * TB + y];
   Vn = Wn + yv;
 }
 
-template <typename T>
 __global__ void __launch_bounds__(256)
-k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __restrict__ triples, int64_t t0,
+k_energy(const double* __restrict__ gbuf, int o, int v, const Triple* __restrict__ triples, int64_t t0,
          const double* __restrict__ eps_o, const double* __restrict__ eps_v,
-         const T* __restrict__ ovs, const T* __restrict__ t1, double* __restrict__ partials,
+         const double* __restrict__ ovs, const double* __restrict__ t1, double* __restrict__ partials,
          int64_t nbt) {
   constexpr int TB = ENERGY_TB, TB3 = TB * TB * TB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* cube = reinterpret_cast<T*>(smem_raw);  // [3 G][6 block orders][TB^3]
-  T* ovsS = cube + 18 * TB3;                 // [3 pairs ij,jk,ik][3][3][TB][TB]
-  T* t1S = ovsS + 27 * TB * TB;              // [3 i,j,k][3][TB]
-  double* epsS = reinterpret_cast<double*>(t1S + 9 * TB + (sizeof(T) == 4 ? 8 : 0));  // [3][TB]
+  double* cube = reinterpret_cast<double*>(smem_raw);  // [3 G][6 block orders][TB^3]
+  double* ovsS = cube + 18 * TB3;                 // [3 pairs ij,jk,ik][3][3][TB][TB]
+  double* t1S = ovsS + 27 * TB * TB;              // [3 i,j,k][3][TB]
+  double* epsS = reinterpret_cast<double*>(t1S + 9 * TB);  // [3][TB]
   __shared__ double red[8];
 
   const int tid = threadIdx.x;
@@ -82,8 +81,8 @@ k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __rest
   decode_block_triple(bt, blk[0], blk[1], blk[2]);
   const Triple tr = triples[t0 + slot];
   const int64_t v2 = (int64_t)v * v;
-  const int64_t gstride = v2 * ldz;  // one G block: [v][v][ldz]
-  const T* G = gbuf + (int64_t)slot * 3 * gstride;
+  const int64_t gstride = v2 * v;  // one G block: [v][v][v]
+  const double* G = gbuf + (int64_t)slot * 3 * gstride;
 
   for (int idx = tid; idx < 18 * TB3; idx += blockDim.x) {
     const int e = idx % TB3, cp = idx / TB3;
@@ -92,8 +91,8 @@ k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __rest
     const int x = blk[c_perm[pid][0]] * TB + u;
     const int y = blk[c_perm[pid][1]] * TB + w;
     const int zz = blk[c_perm[pid][2]] * TB + z;
-    T val = T(0);
-    if (x < v && y < v && zz < v) val = G[g * gstride + ((int64_t)x * v + y) * ldz + zz];
+    double val = 0.0;
+    if (x < v && y < v && zz < v) val = G[g * gstride + ((int64_t)x * v + y) * v + zz];
     cube[idx] = val;
   }
   for (int idx = tid; idx < 27 * TB * TB; idx += blockDim.x) {
@@ -104,7 +103,7 @@ k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __rest
     const int P1 = (pair == 1) ? tr.j : tr.i;
     const int P2 = (pair == 0) ? tr.j : tr.k;
     const int x = blk[sx] * TB + u, y = blk[sy] * TB + w;
-    T val = T(0);
+    double val = 0.0;
     if (x < v && y < v) val = ovs[(((int64_t)P1 * v + x) * o + P2) * v + y];
     ovsS[idx] = val;
   }
@@ -112,7 +111,7 @@ k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __rest
     const int which = tid / (3 * TB), s = (tid / TB) % 3, u = tid % TB;
     const int occ = (which == 0) ? tr.i : (which == 1) ? tr.j : tr.k;
     const int x = blk[s] * TB + u;
-    t1S[tid] = (x < v) ? t1[(int64_t)occ * v + x] : T(0);
+    t1S[tid] = (x < v) ? t1[(int64_t)occ * v + x] : 0.0;
   }
   if (tid < 3 * TB) {
     const int s = tid / TB, u = tid % TB;
@@ -130,20 +129,20 @@ k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __rest
     if (blk[0] == blk[1] && la < lb) continue;
     if (blk[1] == blk[2] && lb < lc) continue;
     const int l[3] = {la, lb, lc};
-    T W0, W1, W2, W3, W4, W5, V0, V1, V2, V3, V4, V5;
-    position<T, 0>(cube, ovsS, t1S, l, W0, V0);
-    position<T, 1>(cube, ovsS, t1S, l, W1, V1);
-    position<T, 2>(cube, ovsS, t1S, l, W2, V2);
-    position<T, 3>(cube, ovsS, t1S, l, W3, V3);
-    position<T, 4>(cube, ovsS, t1S, l, W4, V4);
-    position<T, 5>(cube, ovsS, t1S, l, W5, V5);
-    const T Ae = W0 + W3 + W4, Ao = W1 + W2 + W5;
-    const T Se = V0 + V3 + V4, So = V1 + V2 + V5;
-    const T dot = W0 * V0 + W1 * V1 + W2 * V2 + W3 * V3 + W4 * V4 + W5 * V5;
-    const T Tv = T(3) * dot + Ae * Se + Ao * So - T(2) * (Ae * So + Ao * Se);
+    double W0, W1, W2, W3, W4, W5, V0, V1, V2, V3, V4, V5;
+    position<0>(cube, ovsS, t1S, l, W0, V0);
+    position<1>(cube, ovsS, t1S, l, W1, V1);
+    position<2>(cube, ovsS, t1S, l, W2, V2);
+    position<3>(cube, ovsS, t1S, l, W3, V3);
+    position<4>(cube, ovsS, t1S, l, W4, V4);
+    position<5>(cube, ovsS, t1S, l, W5, V5);
+    const double Ae = W0 + W3 + W4, Ao = W1 + W2 + W5;
+    const double Se = V0 + V3 + V4, So = V1 + V2 + V5;
+    const double dot = W0 * V0 + W1 * V1 + W2 * V2 + W3 * V3 + W4 * V4 + W5 * V5;
+    const double Tv = 3.0 * dot + Ae * Se + Ao * So - 2.0 * (Ae * So + Ao * Se);
     const double wA = (a == b && b == c) ? (1.0 / 6.0) : ((a == b || b == c) ? 0.5 : 1.0);
     const double D = eo - epsS[la] - epsS[TB + lb] - epsS[2 * TB + lc];
-    acc = fma(wA * (double)Tv, __drcp_rn(D), acc);
+    acc = fma(wA * Tv, __drcp_rn(D), acc);
   }
   // fixed-order block reduction
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
@@ -156,30 +155,15 @@ k_energy(const T* __restrict__ gbuf, int o, int v, int ldz, const Triple* __rest
   }
 }
 
-template <typename T>
-static cudaError_t launch_energy(const Prepared* P, const Triple* d_triples, int64_t t0, int nslots,
-                                 const T* gbuf, int ldz, const T* ovs, const T* t1, double* partials,
-                                 int64_t nbt, cudaStream_t s) {
-  constexpr int TB = ENERGY_TB, TB3 = TB * TB * TB;
-  const size_t smem = sizeof(T) * (18 * TB3 + 27 * TB * TB + 9 * TB + (sizeof(T) == 4 ? 8 : 0)) +
-                      sizeof(double) * 3 * TB;
-  static bool attr_set[2] = {false, false};
-  bool& done = attr_set[sizeof(T) == 8];
-  if (!done) {
-    cudaError_t e = cudaFuncSetAttribute(k_energy<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    done = true;
-  }
-  dim3 grid((unsigned)nbt, (unsigned)nslots);
-  k_energy<T><<<grid, 256, smem, s>>>(gbuf, P->o, P->v, ldz, d_triples, t0, P->eps_o, P->eps_v, ovs, t1,
-                                      partials, nbt);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_energy_f64(const Prepared* P, const Triple* d_triples, int64_t t0, int nslots,
                               const double* gbuf, double* partials, int64_t nbt, cudaStream_t s) {
-  return launch_energy<double>(P, d_triples, t0, nslots, gbuf, P->v, P->ovs, P->t1, partials, nbt, s);
+  constexpr int TB = ENERGY_TB, TB3 = TB * TB * TB;
+  const size_t smem = sizeof(double) * (18 * TB3 + 27 * TB * TB + 9 * TB + 3 * TB);
+  const cudaError_t e = cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)nbt, (unsigned)nslots);
+  k_energy<<<grid, 256, smem, s>>>(gbuf, P->o, P->v, d_triples, t0, P->eps_o, P->eps_v, P->ovs, P->t1, partials, nbt);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -128,8 +128,7 @@ struct EnergyMaps {
 };
 
 struct EnergyParams {
-  int ncl, npieces;
-  int64_t items;
+  int npieces;
   EnergyCl cl[TC_MAX_CL];
   TcPiece pc[TC_MAX_PIECES];  // G: orbit-major [slot][bt][g][pid][cube] from pc.gbuf
   const Triple* triples;
@@ -455,10 +454,8 @@ __global__ void __launch_bounds__(Layout<FMT>::threads, 1)
 
 }  // namespace
 
-int64_t energy_tc_grid(int num_sms, int64_t items) {
-  (void)items;  // one block per SM whatever the launch holds: the item-to-block map is fixed per triple
-  return std::max(1, num_sms);
-}
+// one block per SM whatever the launch holds: the item-to-block map is fixed per triple
+int64_t energy_tc_grid(int num_sms) { return std::max(1, num_sms); }
 
 template <int FMT>
 static cudaError_t launch_fmt(const EnergyMaps& M, const EnergyParams& P, int64_t grid, cudaStream_t s) {
@@ -478,16 +475,14 @@ cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s) {
   }
   EnergyParams P;
   std::memset(&P, 0, sizeof(P));
-  P.ncl = e.ncl;
   P.npieces = e.npieces;
-  P.items = e.items;
   for (int c = 0; c < e.ncl; ++c) P.cl[c] = e.cl[c];
   for (int q = 0; q < e.npieces; ++q) P.pc[q] = e.pc[q];
   P.triples = e.triples;
   P.partials = e.partials;
   P.err = e.err;
   P.wait_ns = e.wait_ns;
-  const int64_t grid = energy_tc_grid(e.num_sms, P.items);
+  const int64_t grid = energy_tc_grid(e.num_sms);
   if (e.fmt == G_MIXED) return launch_fmt<G_MIXED>(M, P, grid, s);
   if (e.fmt == G_PAIR) return launch_fmt<G_PAIR>(M, P, grid, s);
   return launch_fmt<G_F32>(M, P, grid, s);

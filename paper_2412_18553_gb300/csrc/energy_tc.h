@@ -21,7 +21,6 @@ struct TcPiece {
   int slot0;       // first G slot, counted over the launch's pieces
   int64_t t0;      // first canonical triple
   int64_t tile0;   // first contraction tile of the piece
-  int64_t item0;   // first energy item of the piece
   int64_t nbt;     // energy items per triple (the cluster's block triples)
   float* gbuf;     // G of the piece's first slot
   double* shares;  // per-triple shares of the piece (ns doubles)
@@ -36,14 +35,13 @@ struct EnergyCl {
 };
 
 struct EnergyLaunch {
-  int ncl, npieces, fmt, num_sms, nslots;  // fmt: the G format; nslots: G slots over all pieces
-  int64_t items;                          // sum over pieces of ns * nbt
+  int ncl, npieces, fmt, num_sms;  // fmt: the G format
   EnergyCl cl[TC_MAX_CL];
   TcPiece pc[TC_MAX_PIECES];
   const CUtensorMap* map_ovs[TC_MAX_CL];  // ovs32 [o][v][o][vq], 4D (b, j, a, i), box (8, 1, 8, 1)
   const CUtensorMap* map_t1[TC_MAX_CL];   // t1 [o][vq], 2D (a, i), box (8, 1)
   const Triple* triples;
-  double* partials;  // [slot][energy_tc_grid(num_sms, items)][ENERGY_TC_WARPS]
+  double* partials;  // [slot][energy_tc_grid(num_sms)][ENERGY_TC_WARPS]
   unsigned int* err;
   unsigned long long wait_ns;
 };
@@ -105,7 +103,7 @@ __host__ __device__ __forceinline__ int64_t g_slot_floats(int v, int fmt) {
 }
 
 constexpr int ENERGY_TC_WARPS = 16;
-int64_t energy_tc_grid(int num_sms, int64_t items);
+int64_t energy_tc_grid(int num_sms);
 cudaError_t launch_energy_tc(const EnergyLaunch& e, cudaStream_t s);
 
 }  // namespace te

@@ -56,8 +56,7 @@ __global__ void k_prep_nooT(const double* __restrict__ ooov, double* __restrict_
   }
 }
 
-__global__ void k_prep_ovs(const double* __restrict__ ovov, double* __restrict__ ovs,
-                           float* __restrict__ ovs32, int o, int v) {
+__global__ void k_prep_ovs(const double* __restrict__ ovov, double* __restrict__ ovs, int o, int v) {
   const int64_t n = (int64_t)o * v * o * v;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -67,16 +66,8 @@ __global__ void k_prep_ovs(const double* __restrict__ ovov, double* __restrict__
     rest /= o;
     const int a = (int)(rest % v);
     const int i = (int)(rest / v);
-    const double s = 0.5 * (ovov[idx] + ovov[(((int64_t)j * v + b) * o + i) * v + a]);
-    if (ovs) ovs[idx] = s;
-    if (ovs32) ovs32[idx] = (float)s;
+    ovs[idx] = 0.5 * (ovov[idx] + ovov[(((int64_t)j * v + b) * o + i) * v + a]);
   }
-}
-
-__global__ void k_to_f32(const double* __restrict__ x, float* __restrict__ y, int64_t n) {
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x)
-    y[idx] = (float)x[idx];
 }
 
 static int grid_for(int64_t n) {
@@ -91,8 +82,7 @@ cudaError_t launch_prep_fp64(const te_cluster* c, Prepared* P, cudaStream_t s) {
   // the tensor-core adjoint reads its own slice planes: no float64 t2L / nooT copies
   if (P->t2L) k_prep_t2L<<<grid_for((int64_t)o * v * v * o), 256, 0, s>>>(c->t2, P->t2L, o, v);
   if (P->nooT) k_prep_nooT<<<grid_for((int64_t)o * o * v * o), 256, 0, s>>>(c->ooov, P->nooT, o, v);
-  k_prep_ovs<<<grid_for((int64_t)o * v * o * v), 256, 0, s>>>(c->ovov, P->ovs, P->ovs32, o, v);
-  if (P->t1_32) k_to_f32<<<grid_for((int64_t)o * v), 256, 0, s>>>(c->t1, P->t1_32, (int64_t)o * v);
+  k_prep_ovs<<<grid_for((int64_t)o * v * o * v), 256, 0, s>>>(c->ovov, P->ovs, o, v);
   return cudaGetLastError();
 }
 

@@ -236,7 +236,8 @@ __global__ void __launch_bounds__(32) k_bisect(const __grid_constant__ EigJobs J
   const double pad = 1e-15 * fmax(fabs(lo), fabs(hi)) + 1e-300;
   lo -= pad;
   hi += pad;
-  // 2^-58 of the first interval, itself at most a few times the largest entry
+  // to 2^-58 of the first interval, the matrix's norm: up to n times its largest
+  // entry (all entries equal), 2^-46 of it at the largest order
   for (int it = 0; it < 58; ++it) {
     const double x = 0.5 * (lo + hi);
     int below = 0;

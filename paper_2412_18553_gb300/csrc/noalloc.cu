@@ -115,8 +115,6 @@ extern "C" te_status t_energy_fp64_noalloc(const te_cluster* c, double* e_out, t
   P.t2L = static_cast<double*>(take(sizeof(double) * (size_t)(o * v * v * o)));
   P.nooT = static_cast<double*>(take(sizeof(double) * (size_t)(o * o * v * o)));
   P.ovs = static_cast<double*>(take(sizeof(double) * (size_t)(o * v * o * v)));
-  P.ovs32 = nullptr;
-  P.t1_32 = nullptr;
   double* gbuf = static_cast<double*>(take(sizeof(double) * (size_t)(slots * 3 * v * v * v)));
   double* partials = static_cast<double*>(take(sizeof(double) * (size_t)(slots * nbt)));
   double* shares = static_cast<double*>(take(sizeof(double) * (size_t)std::max<int64_t>(1, nt)));

@@ -683,12 +683,10 @@ struct TcPlan {
   int TA, TB, NT, n_my, n_mp, n_nt;
   int kw_chunks, ko_chunks, kw_elems, ko_elems, cbw, cbo;
   int stages;
-  uint32_t stage_bytes, a_part_bytes, b_part_bytes, tmem_cols;
+  uint32_t stage_bytes, tmem_cols;
   int nbuf;
   int nslots, par_slots;  // triples per launch, and per share reduction
   int min_slots;          // triples per launch where memory is short
-  int ldz;
-  size_t smem;
 };
 
 constexpr int64_t MIN_SLOTS = 4;          // triples per launch where memory is short,
@@ -756,16 +754,13 @@ static TcPlan make_plan(const Handle* h, int o, int v, int mode, int64_t ntri, i
   pl.cbo = obytes <= 32 ? 32 : (obytes <= 64 ? 64 : std::min(128, pl.cbw));
   pl.ko_elems = pl.cbo / pl.es;
   pl.ko_chunks = (pl.op + pl.ko_elems - 1) / pl.ko_elems;
-  pl.a_part_bytes = 128u * (uint32_t)pl.cbw;
-  pl.b_part_bytes = (uint32_t)(pl.NT / 2) * (uint32_t)pl.cbw;  // a CTA's half of the B tile
-  pl.stage_bytes = (uint32_t)pl.nparts * (pl.a_part_bytes + pl.b_part_bytes);
+  // 128 rows of A and this CTA's half of the B tile, every part
+  pl.stage_bytes = (uint32_t)pl.nparts * (128u + (uint32_t)(pl.NT / 2)) * (uint32_t)pl.cbw;
   const size_t avail = h->smem_optin > 2048 ? h->smem_optin - 2048 : 0;
   pl.stages = (int)std::min<size_t>(8, avail / pl.stage_bytes);
-  pl.smem = (size_t)pl.stages * pl.stage_bytes + 1024 + 256;
   uint32_t cols = 32;
   while (cols < (uint32_t)(nacc * pl.nbuf * pl.NT)) cols <<= 1;
   pl.tmem_cols = cols;
-  pl.ldz = round_up(v, 4);
   // pair tiles and G bytes per triple in the default shape; a tuned one gets the G
   // pool that this makes, so that the workspace does not depend on the tuning
   const int64_t def_m = (int64_t)((v + 128 / defTB - 1) / (128 / defTB)) * ((v + defTB - 1) / defTB);
@@ -1185,7 +1180,7 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
   TcParams* P = new TcParams;
   EnergyLaunch* EL = new EnergyLaunch;
   te_status st = TE_OK;
-  const int egrid = (int)energy_tc_grid(h->num_sms, 0);
+  const int egrid = (int)energy_tc_grid(h->num_sms);
   std::vector<TcPiece> held;  // runs of triples whose partials wait for the share reduction
   int nheld = 0;              // their slots
   auto reduce_held = [&]() {
@@ -1204,7 +1199,7 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     if (j >= jobs.size()) break;
     int jl[TC_MAX_CL];
     int ncl = 0, nbuf = -1, fmt = 0, nslots = 0;
-    int64_t used = 0, tiles = 0, items = 0;
+    int64_t used = 0, tiles = 0;
     double flops = 0.0;
     pcs.clear();
     while (j < jobs.size() && (int)pcs.size() < TC_MAX_PIECES) {
@@ -1235,7 +1230,6 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
       pc.slot0 = nslots;
       pc.t0 = t;
       pc.tile0 = tiles;
-      pc.item0 = items;
       pc.nbt = J.nbt;
       pc.gbuf = pool + used;
       pc.shares = J.shares + (t - J.t_begin);
@@ -1243,7 +1237,6 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
       used += (int64_t)ns * J.slot_floats;
       nslots += ns;
       tiles += (int64_t)ns * J.tiles_per_triple;
-      items += (int64_t)ns * J.nbt;
       t += ns;
       const double kpad = 2.0 * J.pl.kw_chunks * J.pl.kw_elems + 2.0 * J.pl.ko_chunks * J.pl.ko_elems;
       flops += 2.0 * nprod * (double)ns * J.tiles_per_triple * 256.0 * J.pl.NT * kpad;
@@ -1272,8 +1265,6 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     EL->npieces = (int)pcs.size();
     EL->fmt = jobs[jl[0]].pl.fmt;
     EL->num_sms = h->num_sms;
-    EL->nslots = nslots;
-    EL->items = items;
     for (int q = 0; q < ncl; ++q) {
       const TcJob& J = jobs[jl[q]];
       EL->cl[q] = EnergyCl{J.o, J.v, (int)energy_num_blocks(J.v), J.nbt, J.c->eps_o, J.c->eps_v};
@@ -1287,8 +1278,8 @@ static te_status run_rounds(Handle* h, std::vector<TcJob>& jobs, int mode, float
     EL->err = h->d_err;
     EL->wait_ns = h->wait_limit_ns;
     if (h->log)
-      std::fprintf(stderr, "[tenergy] round: %d clusters, %zu pieces, %d triples, %lld tiles, %lld energy items\n",
-                   ncl, pcs.size(), nslots, (long long)tiles, (long long)items);
+      std::fprintf(stderr, "[tenergy] round: %d clusters, %zu pieces, %d triples, %lld tiles\n",
+                   ncl, pcs.size(), nslots, (long long)tiles);
     size_t pm = prof_begin(h, 0, s);
     cudaError_t e = launch_gemm_any(mode, *MS, *P, smem, h->num_sms, s);
     prof_end(h, pm, s);
@@ -1501,12 +1492,8 @@ te_status tc_autotune(Handle* h, const te_cluster* c, te_precision p, cudaStream
     const int64_t rows = (int64_t)round_up(v, TA) * round_up(v, TB);
     if (rows * 100 > best_rows * 115) continue;
     cand.emplace_back(TB, base.n_nt);
-    // one more N split (smaller N tiles re-read the A operand more often), and
-    // in the exact-slice modes the fewer splits of 160-column tiles, which do
-    // not rotate their TMEM blocks
+    // one more N split (smaller N tiles re-read the A operand more often)
     if (round_up((v + base.n_nt) / (base.n_nt + 1), 32) < base.NT) cand.emplace_back(TB, base.n_nt + 1);
-    const int n160 = (v + 159) / 160;
-    if (is_ozaki(mode) && n160 < base.n_nt) cand.emplace_back(TB, n160);
   }
   if (cand.size() <= 1) {
     if (!cand.empty()) h->tuned[key] = cand[0];

@@ -62,8 +62,6 @@ struct Prepared {
   double* t2L;   // [o][v][v][o]  t2L[q][a][b][l] = t2[l,q,a,b]
   double* nooT;  // [o][o][v][o]  nooT[p][r][g][l] = -ooov[p,l,r,g]
   double* ovs;   // [o][v][o][v]  1/2 (ovov[i,a,j,b] + ovov[j,b,i,a])
-  float* ovs32;  // same, float32 (mixed modes)
-  float* t1_32;  // t1 as float32 (mixed modes)
 };
 
 struct Handle {
@@ -71,6 +69,7 @@ struct Handle {
   int num_sms = 0;
   int cc_major = 0, cc_minor = 0;
   size_t smem_optin = 0;
+  size_t total_mem = 0;  // of the device
   uint64_t wait_limit_ns = 4000000000ull;
   int ozaki_bits = 0;                // exact-slice width: 0 automatic, 6 or 7
   unsigned int* d_err = nullptr;     // device error word
