@@ -66,9 +66,10 @@
  *              rounding in the tensor-core accumulation), and the G blocks
  *              are kept as FP32 pairs.  Meets 1e-7 Ha where FP32
  *              accumulation does not.
- *   In every mode D, 1/D, the products with 1/D and all sums are float64;
- *   the tensor-core modes form the orbit sum of R from differences of W~ in
- *   FP32 pairs (no cancellation of the part of W~ that R annihilates).
+ *   In every mode D, 1/D, the products with 1/D and all sums over orbits are
+ *   float64; in the tensor-core modes the energies form the orbit sum of R from
+ *   differences of W~ in FP32 pairs (no cancellation of the part of W~ that R
+ *   annihilates), the gradient and the projected energy in float64.
  */
 #ifndef TENERGY_H
 #define TENERGY_H
@@ -163,8 +164,7 @@ te_status t_energy_batched(te_handle h, const te_cluster* cs, int64_t n,
  * receives E(T) (one device double).  TE_FP64 runs every contraction in
  * float64; the other modes run them on the tcgen05 tensor cores in exact
  * 7-bit BF16 slices (the TE_OZAKI scheme; gradients to ~1e-7 of each tensor's
- * largest entry), with W~, its adjoint and their slices from float64 and what
- * only enters sums in FP32 pairs.  Deterministic. */
+ * largest entry), with everything else in float64.  Deterministic. */
 te_status t_energy_vjp(te_handle h, const te_cluster* c, te_precision p,
                        double gE, double* e_out, te_cluster_grad* g,
                        te_stream_t s);

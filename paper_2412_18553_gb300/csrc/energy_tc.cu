@@ -174,8 +174,8 @@ __device__ __forceinline__ void cursor_settle(const EnergyParams& P, ItemCursor&
   }
 }
 
-// Bound by instruction issue (59% of cycles; float64 pipe and HBM 45% each).
-// nocc=32 nvir=320: 177 us per triple; 272 us with the assembled area, 8-byte G
+// Bound by instruction issue (60% of cycles; float64 pipe and HBM 44% each).
+// nocc=32 nvir=320: 185 us per triple (177 without the renormalisations); 272 us with the assembled area, 8-byte G
 // and one producer warp, 240 us with one producer for three buffers.
 template <int FMT>
 __global__ void __launch_bounds__(Layout<FMT>::threads, 1)

@@ -90,7 +90,7 @@ cudaError_t launch_prep_fp64(const te_cluster* c, Prepared* P, cudaStream_t s) {
 // DFMA GEMM: one CTA = 32 RM rows (x,y) x 8 NB columns z of one G block
 // (dfma_tile.cuh).  The float64 units bound it: 12 v^3 (v + o) flops per triple
 // at 1.25 TFLOP/s (3.3 ms).  nocc=8 nvir=40, whole energy: 8.18 ms with 64 x 64 tiles
-// (40 columns on 64, K of 40 and 8 on 48 and 16), 4.01 ms with 128 x 40.
+// (40 columns on 64, K of 40 and 8 on 48 and 16), 3.85 ms with the picked one.
 // ---------------------------------------------------------------------------
 
 template <int RM, int NB>

@@ -20,7 +20,8 @@
 // neither 16 epilogue warps nor a sum of four instructions changes it much.
 // Eight triples of a gradient at nvir = 120, one set of 128 columns -> two of 64:
 // G 671 -> 520 us, ovvv and t2 479 -> 384; one triple at nvir = 320: 1981 -> 1561,
-// 2057 -> 1503 (the projected energy's pairs, which convert nothing: 1096 -> 1105).
+// 2057 -> 1503.  The projected energy's pairs, which convert nothing, gain nothing
+// from it (1096 -> 1105); one rule serves all.
 // Lone CTAs have K of nvir^2: few drains, so one set of 128 columns, whose operands
 // from L2 bound them (tensor pipe 49% active at nvir = 320).
 //

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) k_adjoint(AdjArgs A) {
 // mirrored bits are those the other half would have had.  The float64 units
 // bound every launch; eight clusters' MP2 step (nocc 8 .. 20, nvir = 8 nocc,
 // three contractions each): 56.1 ms with 64 x 64 tiles and both halves of
-// (ia|jb), 29.1 ms now.
+// (ia|jb), 26 ms now.
 template <int RM, int NB>
 __global__ void __launch_bounds__(DT_THREADS) k_gemm_strided(const __grid_constant__ GemmView g, int kchunk,
                                                              double* __restrict__ part, int a_fast, int b_fast,

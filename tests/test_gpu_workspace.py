@@ -145,8 +145,10 @@ def test_smaller_gradient_allocates_nothing_after_reserve(te):
     h = te.Handle(0)
     h.reserve(4, 201, "ozaki", energy=False, vjp=True)
     a = cluster(4, 200)
-    buf = torch.empty(a["ovvv"].numel() * 2, dtype=torch.float64, device="cuda")  # cached: room for the gradients
-    del buf
+    h0 = te.Handle(0)
+    te.t_energy_vjp(a, precision="ozaki", handle=h0)  # torch then has the gradients' memory in its cache
+    h0.sync()
+    h0.close()
     before = held(te, h)
     te.t_energy_vjp(a, precision="ozaki", handle=h)
     h.sync()
