@@ -309,7 +309,7 @@ __device__ __forceinline__ void orbit_w(const float2* G, int64_t v3, const int* 
 
 // per-block sums of (S W~) R[V] / D over the orbits of each slot, in float64 from
 // the pairs on.  Its two lanes per SM and cycle bound it, some 70 operations per
-// orbit, 30 of the 47 ms it takes at nocc=16 nvir=120 (161 ms in all; with W~, D and
+// orbit, 30 of the 47 ms it takes at nocc=16 nvir=120 (160 ms in all; with W~, D and
 // the sums in FP32 pairs 30 and 143, at 48 bits; one thread per element of v^3, a
 // sixth of them an orbit, 102 of 320).  Four blocks per SM: 47 ms, two 52.
 __global__ void __launch_bounds__(256, 4) k_proj_batch(const __grid_constant__ ProjArgs A) {
